@@ -7,8 +7,8 @@
 //   warp 8           TMA producer and scheduler: the Q tiles, then through a 5-slot ring K_j, V_j
 //                    for every key tile, then W_phi_q^T, the raw Q tiles again and the bf16
 //                    copy of the state S
-//   warp 9 / 10      MMA issuer of tile 0 / 1 (one thread each): S_t = Q~_t K_j^T and
-//                    O_t += P_t V_j into TMEM
+//   warp 9 / 10      MMA issuer of tile 0 / 1 (the warp walks the loop, one elected lane issues):
+//                    S_t = Q~_t K_j^T and O_t += P_t V_j into TMEM
 // TMEM (512 columns): S_0 | S_1 | O_0 | O_1, 128 fp32 columns each; the bf16 probabilities P_t
 // overwrite the first 64 columns of S_t and feed the second MMA straight from TMEM.
 // RoPE(Q) is applied in place in shared memory by the softmax groups; K arrives rotated.
@@ -50,7 +50,7 @@ enum Bar : int {
     kBarSFull0 = kBarEmpty0 + kStages, kBarSFull1,
     kBarPFull0, kBarPFull1,
     kBarOFinal0, kBarOFinal1,
-    kBarTok0, kBarTok1,                         // softmax groups take turns in the exponential phase
+    kBarTurn0, kBarTurn1,                       // the MMA issuers take turns on the tensor pipe
     kBarDrain0, kBarDrain1,                     // an MMA issuer that gives up waits here for its MMAs in flight
     kNumBars
 };
@@ -202,7 +202,6 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
     const int n_kv = p.n_kv;
     uint32_t s_cnt = 0;   // phases of bar_s consumed so far
     uint32_t of_cnt = 0;  // phases of this tile's final-O barrier consumed so far
-    uint32_t tok_cnt = 0; // turns taken in the exponential phase
     uint32_t sreg[128];
 
     for (uint32_t item = 0;; ++item) {
@@ -296,13 +295,6 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
                     }
                 }
                 const uint64_t neg_m2 = pack2(-m_ref, -m_ref);
-                if (it.ntile == 2) {
-                    // the two groups alternate in the exponential phase, so that one group's
-                    // exponentials overlap the other tile's MMAs instead of its exponentials
-                    const uint32_t par = (t == 0) ? ((tok_cnt + 1) & 1) : (tok_cnt & 1);
-                    if (!wait_bar(bars + 8 * (kBarTok0 + t), par, ab, 24 + t)) return;
-                    ++tok_cnt;
-                }
 #pragma unroll
                 for (int c = 0; c < 64; ++c) {
                     float x0, x1, p0, p1;
@@ -313,7 +305,6 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
                     l2 = add2(l2, pack2(p0, p1));
                     sreg[c] = pack_bf16(p0, p1);
                 }
-                if (it.ntile == 2) mbar_arrive(bars + 8 * (kBarTok0 + (t ^ 1)));
                 tmem_st32(s_addr, *reinterpret_cast<uint32_t(*)[32]>(&sreg[0]));
                 tmem_st32(s_addr + 32, *reinterpret_cast<uint32_t(*)[32]>(&sreg[32]));
                 tmem_wait_st();
@@ -522,8 +513,8 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         mbar_init(bars + 8 * kBarPFull1, 128);
         mbar_init(bars + 8 * kBarOFinal0, 1);
         mbar_init(bars + 8 * kBarOFinal1, 1);
-        mbar_init(bars + 8 * kBarTok0, 128);
-        mbar_init(bars + 8 * kBarTok1, 128);
+        mbar_init(bars + 8 * kBarTurn0, 1);
+        mbar_init(bars + 8 * kBarTurn1, 1);
         mbar_init(bars + 8 * kBarDrain0, 1);
         mbar_init(bars + 8 * kBarDrain1, 1);
         *abort_flag = 0;
@@ -616,13 +607,25 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         }
     } else if (warp == 9 || warp == 10) {
         // ---------------- MMA issuers: warp 9 drives query tile 0, warp 10 tile 1 ----------------
-        // Issuing a tcgen05.mma holds the thread until the tensor pipe accepts it, and every
-        // wait / commit between two MMAs is time the pipe may idle; with one issuer per tile the
-        // synchronisation of one tile overlaps the MMAs of the other.  Both issuers walk the
-        // same sequence of ring entries and both release every entry (the empty barriers count
-        // two arrivals), whether or not they read it.
-        if (lane == 0) {
-            const int t = warp - 9;
+        // Both issuers walk the same sequence of ring entries and both release every entry (the empty
+        // barriers count two arrivals), whether or not they read it.
+        //
+        // The serial chain of a tile -- S ready, softmax, P ready, P V and the next S -- sets the time of a
+        // key iteration, so what an issuer adds to it counts.  (1) The whole warp walks the loop and one
+        // elected lane issues: with operands in uniform registers the 16 MMAs of an iteration are issued in
+        // 770 clk and run back to back (1275 clk from P ready to S ready); issued by a single live lane they
+        // took 1125 to 1385, more the busier the softmax warps were, because every operand of every MMA was
+        // first moved to a uniform register.  (2) The issuers take turns, 16 MMAs each: interleaved, both
+        // tiles' MMAs end late and the two softmax groups fall into step (0.57 ms for L = 4680, 40 heads;
+        // the turn the groups used to take in the exponential phase instead left the exponential unit idle
+        // between them).  Key iteration 3790 -> 3310 clk; that shape 0.447 -> 0.423 ms per pass at full clocks,
+        // 0.502 -> 0.479 under the power cap; 4680 queries against a cache of 18720 tokens, 12 heads: 0.548 -> 0.514.
+        {
+            const uint32_t lead = elect_one();
+            const int t = __shfl_sync(0xffffffffu, warp - 9, 0);
+            const uint32_t smem_base = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
+            const uint32_t bars = smem_base + kOffBars;
+            const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
             constexpr uint32_t idesc_qk = idesc_bf16(kTile, kTile, 0, 0);  // A, B K-major
             constexpr uint32_t idesc_pv = idesc_bf16(kTile, kTile, 0, 1);  // A in TMEM, B N-contiguous
             const uint32_t q_tile = smem_base + kOffQ + t * kTileBytes;
@@ -647,7 +650,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
                     const uint32_t koff = (uint32_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
-                    mma_ss(s_col, desc64(a_lo + koff), desc64(b_lo + koff), idesc_qk, ks > 0);
+                    mma_ss_if(lead, s_col, desc64(a_lo + koff), desc64(b_lo + koff), idesc_qk, ks > 0);
                 }
             };
             // O_t (+)= P_t * V with P in TMEM and V rows = contraction index, 8 k-steps of 16
@@ -655,23 +658,24 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 const uint32_t v_lo = (v_tile >> 4) | kLboMN;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
-                    mma_ts(o_col, s_col + ks * 8, desc64(v_lo + (uint32_t)(ks * (2048 >> 4))), idesc_pv,
+                    mma_ts_if(lead, o_col, s_col + ks * 8, desc64(v_lo + (uint32_t)(ks * (2048 >> 4))), idesc_pv,
                            (accumulate || ks > 0) ? 1u : 0u);
             };
             auto slot_addr = [&](uint32_t entry) { return smem_base + kOffRing + (entry % kStages) * kTileBytes; };
             auto wait_full = [&](uint32_t entry, int site) {
-                return wait_bar(bars + 8 * (kBarFull0 + entry % kStages), (entry / kStages) & 1, ab, site);
+                return wait_bar_warp(bars + 8 * (kBarFull0 + entry % kStages), (entry / kStages) & 1, ab, site);
             };
-            auto release = [&](uint32_t entry) { mma_commit(bars + 8 * (kBarEmpty0 + entry % kStages)); };
+            auto release = [&](uint32_t entry) { mma_commit_if(lead, bars + 8 * (kBarEmpty0 + entry % kStages)); };
 
             uint32_t cons = 0;        // ring entries consumed so far (all items)
             uint32_t p_cnt = 0;       // phases of bar_p consumed
             uint32_t qrot_cnt = 0, of_cnt = 0;
+            uint32_t turn = 0;        // turns taken on the tensor pipe
             bool ok = true;
             for (uint32_t item = 0; ok; ++item) {
-                ok = wait_bar(bars + 8 * kBarQFull, item & 1, ab, 60);
+                ok = wait_bar_warp(bars + 8 * kBarQFull, item & 1, ab, 60);
                 if (!ok) break;
-                const int id = item_slots[item & 1];
+                const int id = __shfl_sync(0xffffffffu, item_slots[item & 1], 0);
                 if (id < 0) break;
                 const Item it = decode_item<kSplit>(id, p);
                 const int nj = kSplit ? it.nj : n_kv;   // key tiles of this item (a part walks its own range)
@@ -686,11 +690,11 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     if (exclusive) release(e);
                 };
                 auto q_free = [&]() {
-                    mma_commit(bars + 8 * kBarQFree);
-                    if (ntile == 1) mma_commit(bars + 8 * kBarQFree);   // on behalf of the idle issuer
+                    mma_commit_if(lead, bars + 8 * kBarQFree);
+                    if (ntile == 1) mma_commit_if(lead, bars + 8 * kBarQFree);   // on behalf of the idle issuer
                 };
                 if (active) {
-                    ok = wait_bar(bars + 8 * (kBarQRot0 + t), qrot_cnt & 1, ab, 61);
+                    ok = wait_bar_warp(bars + 8 * (kBarQRot0 + t), qrot_cnt & 1, ab, 61);
                     ++qrot_cnt;
                     if (!ok) break;
                     // S_t(0) = Q~_t K_0^T
@@ -699,7 +703,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     if (!ok) break;
                     tc_fence_after();
                     issue_qk(q_tile, slot_addr(e_k));
-                    mma_commit(bar_s);
+                    mma_commit_if(lead, bar_s);
                     release_mine(e_k, !shared);
                     if (nj == 1) q_free();
                 }
@@ -717,13 +721,20 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                         if (ok) ok = wait_full(e_b, 66);
                         if (ok && last) ok = wait_full(e_q, 68);
                         if (!ok) break;
-                        ok = wait_bar(bar_p, p_cnt & 1, ab, 64 + t);
+                        if (ntile == 2) {
+                            ok = wait_bar_warp(bars + 8 * (kBarTurn0 + t), (t == 0) ? ((turn + 1) & 1) : (turn & 1), ab,
+                                               24 + t);
+                            ++turn;
+                            if (!ok) break;
+                        }
+                        ok = wait_bar_warp(bar_p, p_cnt & 1, ab, 64 + t);
                         ++p_cnt;
                         if (!ok) break;
                         tc_fence_after();
                         issue_pv(slot_addr(e_v), j > 0);
                         issue_qk(last ? slot_addr(e_q) : q_tile, slot_addr(e_b));
-                        mma_commit(bar_s);
+                        mma_commit_if(lead, bar_s);
+                        if (ntile == 2) mbar_arrive_if(lead, bars + 8 * (kBarTurn0 + (t ^ 1)));
                         release_mine(e_v, !shared);
                         release_mine(e_b, !shared);
                         if (last) release_mine(e_q, true);
@@ -736,7 +747,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 if (active) {
                     const uint32_t e_s = cons + (shared ? 0 : t);
                     ok = wait_full(e_s, 69);
-                    if (ok) ok = wait_bar(bar_p, p_cnt & 1, ab, 70 + t);
+                    if (ok) ok = wait_bar_warp(bar_p, p_cnt & 1, ab, 70 + t);
                     ++p_cnt;
                     if (!ok) break;
                     tc_fence_after();
@@ -746,7 +757,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                         constexpr uint32_t idesc_x = idesc_bf16(kTile, 64, 0, 1);
                         for (int hv = 0; hv < 2 && ok; ++hv) {
                             if (hv == 1) {
-                                ok = wait_bar(bar_p, p_cnt & 1, ab, 72 + t);   // first half consumed
+                                ok = wait_bar_warp(bar_p, p_cnt & 1, ab, 72 + t);   // first half consumed
                                 ++p_cnt;
                                 if (!ok) break;
                                 tc_fence_after();
@@ -754,25 +765,25 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                             const uint32_t x_lo = ((slot_addr(e_s) + hv * kHalfBytes) >> 4) | kLboMN;
 #pragma unroll
                             for (int ks = 0; ks < 8; ++ks)
-                                mma_ts(s_col + 64, s_col + ks * 8, desc64(x_lo + (uint32_t)(ks * (2048 >> 4))), idesc_x,
+                                mma_ts_if(lead, s_col + 64, s_col + ks * 8, desc64(x_lo + (uint32_t)(ks * (2048 >> 4))), idesc_x,
                                        ks > 0 ? 1u : 0u);
-                            mma_commit(bar_s);
+                            mma_commit_if(lead, bar_s);
                         }
                         if (!ok) break;
                         release_mine(e_s, !shared);
                     } else {
                         issue_pv(slot_addr(e_s), true);
                         release_mine(e_s, !shared);
-                        mma_commit(bars + 8 * (kBarOFinal0 + t));
+                        mma_commit_if(lead, bars + 8 * (kBarOFinal0 + t));
                         ++of_cnt;
                     }
                 }
                 cons += shared ? 1 : ntile;
             }
             (void)of_cnt;
-            if (!ok || *abort_flag) {
+            if (!ok || __any_sync(0xffffffffu, *abort_flag)) {
                 // tensor memory is freed below: none of this thread's MMAs may still be running
-                mma_commit(bars + 8 * (kBarDrain0 + t));
+                mma_commit_if(lead, bars + 8 * (kBarDrain0 + t));
                 drain_bar(bars + 8 * (kBarDrain0 + t), 0);
             }
         }

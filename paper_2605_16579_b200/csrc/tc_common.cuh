@@ -40,6 +40,20 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, const Ab
     return false;
 }
 
+// The same for a whole warp in uniform control flow: every lane gets the same answer, so that the warp
+// never splits, not even when the wait expires.
+__device__ __forceinline__ bool wait_bar_warp(uint32_t bar, uint32_t parity, const Abort& ab, int site)
+{
+    for (uint32_t it = 0; it < ab.limit; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if ((it & 255u) == 255u && __any_sync(0xffffffffu, *ab.flag)) return false;
+    }
+    *ab.flag = 1;
+    if (atomicCAS(ab.status + kStatusError, 0u, (uint32_t)(-ARL2_ERR_TIMEOUT)) == 0u)
+        ab.status[kStatusWhere] = (uint32_t)site;
+    return false;
+}
+
 // Bounded wait that ignores the abort flag: used on the way out, for copies still in flight.
 __device__ __forceinline__ void drain_bar(uint32_t bar, uint32_t parity)
 {
