@@ -806,7 +806,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 //   U_k, U_v (MMA) -> K' -> Gram matrix K' K'^T (MMA) -> A (fp32, shared memory) -> T by forward
 //   substitution (thread = column), stored as a bf16 block-diagonal 128 x 128 operand -> W and U1
 //   (MMA, both chunks at once) -> global: W, Khat, U1 in bf16, chunk decays g in fp32.
-// tc_token_scan_kernel: one CTA per (stream, head) walks the chunks in order (further down).
+// tc_token_scan_kernel: walks the chunks of a head in order (further down).
 // ---------------------------------------------------------------------------------------------
 constexpr int kTPOffWk = 0;                        // maps; later the fp32 matrix A (2 x 64 x 65)
 constexpr int kTPOffWv = kTileBytes;
@@ -1109,242 +1109,256 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     }
 }
 
-// tc_token_scan_kernel: one CTA (256 threads) per (stream, head); the fp32 state lives in TMEM
-// (row = key dim d, 128 columns) for the whole walk.  Per chunk:
-//   Y = W_c S            MMA, A = W tile (128 rows fetched, the first 64 are the chunk), B = bf16 copy of S
-//   U = U1_c - Y         two threads per token (64 columns each), written as a bf16 operand tile
-//   S += Khat_c^T U      MMA over the chunk's 64 tokens, accumulating on g_c S (scaled beforehand)
-//   bf16 copy of the new S for the next chunk; S scaled by g_{c+1} in the same pass (two threads
-//                        per state row, 64 columns each)
-// The tiles of chunk c + 2 are fetched by TMA as soon as chunk c has released its buffers.
-constexpr int kTSOffS = 0;                           // bf16 S, [d][e], 128 rows
-constexpr int kTSOffW = kTileBytes;                  // 2 x 32 KB: W tiles (128 rows)
-constexpr int kTSOffKh = 3 * kTileBytes;             // 2 x 16 KB: Khat chunks (64 rows)
-constexpr int kTSOffU1 = 4 * kTileBytes;             // 2 x 16 KB: U1 chunks
-constexpr int kTSOffU = 5 * kTileBytes;              // 16 KB: U operand
-constexpr int kTSOffBars = 5 * kTileBytes + kHalfBytes;
-constexpr int kTSSmemBytes = kTSOffBars + 128 + 1024;
+// tc_token_scan_kernel: the ordered walk over the chunks.  The columns of S never mix (U = U1 - W S and
+// S <- g S + Khat^T U act on each value column alone), so a head's 128 columns are cut into slabs of 16, each
+// walked by a group of four warps; a CTA holds kSlabs of them and the W, Khat and U1 tiles they share.
+// The walk is a chain of ceil(L / 64) dependent chunks: what counts is the latency of one, not throughput.
+// Everything is kept transposed (row = value column e), so that the warp-level tensor instruction
+// hands every result on in the layout the next product needs:
+//   U^T[16 x 64]  = U1^T - S^T W^T     A = S^T (bf16, 4 KB of shared memory), B = W as it lies; warp w: 16 tokens
+//   S^T[16 x 128] = g S^T + U^T Khat   A = U^T (bf16, 2 KB of shared memory), B = Khat;         warp w: 32 keys d
+// The fp32 state stays in registers for the whole walk (16 per thread).  Per chunk a warp runs 16 + 16
+// instructions in four independent chains each and meets its group twice (named barriers, 128 threads);
+// the B fragments of the next chunk are fetched while this chunk's products run.  A fifth warp per CTA
+// streams the tiles through a TMA ring.  12 heads x 4680 tokens: 162 us with one CTA per head and the state in
+// TMEM (3.8 k clk per chunk: two MMAs, two passes through registers, four CTA-wide meetings) -> 32 us
+// (0.8 k clk; the 34 KB per chunk and SM that come from L2 are about 0.65 k of that).
 constexpr int kChunkHalf = kTokC * 128;              // bytes of a 64-row, 64-column box
-constexpr uint32_t kChunkTx = kTileBytes + 4 * kChunkHalf;   // W tile + Khat + U1 per chunk
+constexpr int kScanLdS = kTile + 8, kScanLdU = kTokC + 8;   // padded rows: conflict-free 8 x 8 loads
+constexpr int kScanSlab = 16;
+constexpr int kScanMaxStages = 6;
+// kSlabs slabs per CTA; kShared: two CTAs share an SM (two stages each, fragments fetched when needed)
+template <int kSlabs, bool kShared>
+struct ScanCfg {
+    static constexpr int kStages = kShared ? 2 : kSlabs == 1 ? 6 : 5;
+    static constexpr int kStageBytes = 4 * kChunkHalf + kSlabs * kTokC * kScanSlab * 2;
+    static constexpr int kOffS = kStages * kStageBytes;
+    static constexpr int kOffBars = kOffS + kSlabs * kScanSlab * (kScanLdS + kScanLdU) * 2;
+    static constexpr int kSmemBytes = kOffBars + 2 * kScanMaxStages * 8 + 8 + 1024;
+    static constexpr int kThreads = kSlabs * 128 + 32;
+    static_assert(kSmemBytes <= (kShared ? 115712 : 232448), "shared memory");
+};
 
-enum TSBar : int { kTSBarS0 = 0, kTSBarFull0, kTSBarFull1, kTSBarY, kTSBarS2, kTSBarDrain, kTSNumBars };
-
-constexpr int kTSThreads = 256;
-__global__ void __launch_bounds__(kTSThreads, 1)
-tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_kh,
-                     const __grid_constant__ CUtensorMap tm_u1, const __grid_constant__ CUtensorMap tm_s,
-                     const TcTokenParams p)
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr)
 {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+template <int kSlabs, bool kShared>
+__global__ void __launch_bounds__(kSlabs * 128 + 32, kShared ? 2 : 1)
+tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_kh,
+                     const __grid_constant__ CUtensorMap tm_u1, const TcTokenParams p)
+{
+    using Cfg = ScanCfg<kSlabs, kShared>;
+    constexpr int kS = Cfg::kStages;
+    constexpr uint32_t kStageBytes = (uint32_t)Cfg::kStageBytes;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                ~static_cast<uintptr_t>(1023));
     const uint32_t smem_base = smem_u32(smem);
-    const uint32_t bars = smem_base + kTSOffBars;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kTSOffBars + kTSNumBars * 8);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kTSOffBars + kTSNumBars * 8 + 4);
+    const uint32_t bar_full = smem_base + Cfg::kOffBars;
+    const uint32_t bar_free = bar_full + 8 * kScanMaxStages;
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + Cfg::kOffBars + 16 * kScanMaxStages);
     const Abort ab{abort_flag, p.status, p.spin_limit};
 
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int h = blockIdx.x, b = blockIdx.y;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int h = blockIdx.y, b = blockIdx.z;
     const size_t bh = (size_t)b * p.s.H + h;
-    const int rows_pad = p.ntile * kTile;
     const int nchunk = p.nchunk;
-    const float* gc = p.gc + bh * 2 * p.ntile;
+    const int e0 = blockIdx.x * kSlabs * kScanSlab;      // first value column of this CTA
 
     if (tid == 0) {
-        for (int i = 0; i < kTSNumBars; ++i) mbar_init(bars + 8 * i, 1);
+        for (int i = 0; i < kS; ++i) {
+            mbar_init(bar_full + 8 * i, 1);
+            mbar_init(bar_free + 8 * i, kSlabs * 4);
+        }
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
     }
-    if (warp == 0) {
-        tmem_alloc(smem_u32(tmem_slot), 256);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    // warps w and w + 4 own the same 32 TMEM lanes (rows) and split the 128 columns in two
-    const int rowid = (warp & 3) * 32 + (tid & 31);
-    const int chalf = warp >> 2;
-    const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(chalf * 64);
+    // (one answer for the whole CTA) after an error the chunk factors are not all there: S stays as it is
+    if (__syncthreads_or(*reinterpret_cast<volatile uint32_t*>(p.status + kStatusError) != 0u)) return;
 
-    int loads_issued = 0;
-    auto load_chunk = [&](int c) {
-        const uint32_t bar = bars + 8 * (kTSBarFull0 + (c & 1));
-        const int r0 = (int)(bh * rows_pad) + c * kTokC;
-        mbar_expect_tx(bar, kChunkTx);
+    if (warp == kSlabs * 4) {
+        // ---------------- TMA producer ----------------
+        if (lane == 0) {
+            const int r0 = (int)(bh * p.ntile * kTile);
+            bool ok = true;
+            int c = 0;
+            for (; c < nchunk; ++c) {
+                const int s = c % kS;
+                if (c >= kS) ok = wait_bar(bar_free + 8 * s, (uint32_t)(c / kS - 1) & 1u, ab, 100);
+                if (!ok) break;
+                const uint32_t bar = bar_full + 8 * s, dst = smem_base + s * kStageBytes;
+                mbar_expect_tx(bar, kStageBytes);
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            tma_load_2d(smem_base + kTSOffW + (c & 1) * kTileBytes + half * kHalfBytes, &tm_w, bar, half * 64, r0);
-            tma_load_2d(smem_base + kTSOffKh + (c & 1) * kHalfBytes + half * kChunkHalf, &tm_kh, bar, half * 64, r0);
-            tma_load_2d(smem_base + kTSOffU1 + (c & 1) * kHalfBytes + half * kChunkHalf, &tm_u1, bar, half * 64, r0);
-        }
-        ++loads_issued;
-    };
-    if (tid == 0) {
-        mbar_expect_tx(bars + 8 * kTSBarS0, kTileBytes);
-        tma_load_2d(smem_base + kTSOffS, &tm_s, bars + 8 * kTSBarS0, 0, (int)bh * kTile);
-        tma_load_2d(smem_base + kTSOffS + kHalfBytes, &tm_s, bars + 8 * kTSBarS0, 64, (int)bh * kTile);
-        load_chunk(0);
-        if (nchunk > 1) load_chunk(1);
-    }
-
-    // fp32 state row d = rowid (this thread's 64 columns) into TMEM columns 128-255, already scaled
-    // by the first chunk's decay
-    float* srow = p.state + (bh * kTile + rowid) * kTile + chalf * 64;
-    {
-        const float g0 = __ldg(gc);
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            uint32_t x[32];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float4 v = *reinterpret_cast<const float4*>(srow + c * 32 + e * 4);
-                x[e * 4 + 0] = __float_as_uint(v.x * g0);
-                x[e * 4 + 1] = __float_as_uint(v.y * g0);
-                x[e * 4 + 2] = __float_as_uint(v.z * g0);
-                x[e * 4 + 3] = __float_as_uint(v.w * g0);
+                for (int half = 0; half < 2; ++half) {
+                    tma_load_2d(dst + half * kChunkHalf, &tm_w, bar, half * 64, r0 + c * kTokC);
+                    tma_load_2d(dst + (2 + half) * kChunkHalf, &tm_kh, bar, half * 64, r0 + c * kTokC);
+                }
+                tma_load_2d(dst + 4 * kChunkHalf, &tm_u1, bar, e0, r0 + c * kTokC);
             }
-            tmem_st32(lane_base + kTile + c * 32, x);
+            // no bulk copy may be in flight into this CTA's shared memory when it ends, whatever the walkers do
+            for (int m = (c > kS ? c - kS : 0); m < c; ++m) drain_bar(bar_full + 8 * (m % kS), (uint32_t)(m / kS) & 1u);
         }
-        tmem_wait_st();
+        return;
     }
-    tc_fence_before();
-    __syncthreads();
 
-    constexpr uint32_t kLboK = 1u << 16;
-    constexpr uint32_t kLboMN = (uint32_t)(kHalfBytes >> 4) << 16;     // 128-row tiles
-    constexpr uint32_t kLboMN64 = (uint32_t)(kChunkHalf >> 4) << 16;   // 64-row tiles
-    const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0, 0) >> 32);
-    auto desc64 = [&](uint32_t lo) {
-        uint64_t d;
-        asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(desc_hi));
-        return d;
+    // ---------------- the walk: slab `slab` of this CTA, warp wq of its four ----------------
+    const int slab = warp >> 2, wq = warp & 3;
+    const int mi = lane >> 3, mr = lane & 7;             // 8 x 8 block and row this lane addresses in a load
+    const int ge = lane >> 2, gk = (lane & 3) * 2;       // fragment row (value column) and column pair
+    __nv_bfloat16* s_s = reinterpret_cast<__nv_bfloat16*>(smem + Cfg::kOffS) + slab * kScanSlab * (kScanLdS + kScanLdU);
+    __nv_bfloat16* u_s = s_s + kScanSlab * kScanLdS;
+    const uint32_t a_s = smem_u32(s_s) + (uint32_t)((((mi & 1) * 8 + mr) * kScanLdS + (mi >> 1) * 8) * 2);
+    const uint32_t a_u = smem_u32(u_s) + (uint32_t)((((mi & 1) * 8 + mr) * kScanLdU + (mi >> 1) * 8) * 2);
+    // offsets inside a stage (128-byte swizzle: the 16-byte piece index is xored with the row)
+    const uint32_t w_row = (uint32_t)(wq * 16 + (mi >> 1) * 8 + mr);
+    const uint32_t u1_off = 4 * kChunkHalf + (w_row * kSlabs * kScanSlab + (uint32_t)(slab * kScanSlab + (mi & 1) * 8)) * 2;
+    auto group_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(slab + 1) : "memory"); };
+
+    // state: st[n][0..1] = S[d][e], S[d + 1][e], st[n][2..3] the same for e + 8, d = 32 wq + 8 n + gk
+    float st[4][4];
+    float* srow = p.state + (bh * kTile + wq * 32 + gk) * kTile + e0 + slab * kScanSlab + ge;
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) st[n][x] = srow[(size_t)(n * 8 + (x & 1)) * kTile + (x >> 1) * 8];
+    auto put_s = [&]() {
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            *reinterpret_cast<uint32_t*>(s_s + ge * kScanLdS + wq * 32 + n * 8 + gk) = pack_bf16(st[n][0], st[n][1]);
+            *reinterpret_cast<uint32_t*>(s_s + (ge + 8) * kScanLdS + wq * 32 + n * 8 + gk) = pack_bf16(st[n][2], st[n][3]);
+        }
     };
-    constexpr uint32_t idesc_kn = idesc_bf16(kTile, kTile, 0, 1);
-    constexpr uint32_t idesc_nn = idesc_bf16(kTile, kTile, 1, 1);
+    put_s();
+    const float* gc = p.gc + bh * 2 * p.ntile;
+    float g_cur = lane < nchunk ? __ldg(gc + lane) : 1.0f;   // decays of 32 chunks, one per lane
 
-    bool ok = true, alive = true;
+    bool dead = false;
+    // On a wait that expires the warp goes on without waiting: the barriers of the group keep their
+    // counts, the loop is finite, and nothing is stored at the end.
+    auto landed = [&](int c) {
+        if (!dead) dead = !wait_bar_warp(bar_full + 8 * (c % kS), (uint32_t)(c / kS) & 1u, ab, 101);
+    };
+    auto release = [&](int c) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_free + 8 * (c % kS));
+    };
+    auto stage = [&](int c) { return smem_base + (uint32_t)(c % kS) * kStageBytes; };
+    auto load_w = [&](uint32_t (&f)[4], uint32_t base, int ks) {
+        ldsm4(f, base + (uint32_t)(ks >> 2) * kChunkHalf + w_row * 128 + ((((uint32_t)(ks & 3) * 2 + (mi & 1)) ^ (w_row & 7)) << 4));
+    };
+    auto load_k = [&](uint32_t (&f)[4], uint32_t base, int ks, int j) {
+        const uint32_t row = (uint32_t)(ks * 16 + (mi & 1) * 8 + mr);
+        ldsm4t(f, base + (uint32_t)(2 + (wq >> 1)) * kChunkHalf + row * 128 +
+                      ((((uint32_t)(wq & 1) * 4 + j * 2 + (mi >> 1)) ^ (row & 7)) << 4));
+    };
+    // fragments of the chunk at hand; kShared: filled just before their use instead of a chunk ahead
+    uint32_t wf[kShared ? 1 : 8][4], kf[kShared ? 1 : 4][2][4], uf[4];
+    auto load_all_w = [&](int c) {
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks) load_w(wf[kShared ? 0 : ks], stage(c), ks);
+    };
+    auto load_all_k = [&](int c) {
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) load_k(kf[kShared ? 0 : ks][j], stage(c), ks, j);
+        ldsm4t(uf, stage(c) + u1_off);
+    };
+
+    if (!kShared) {
+        landed(0);
+        load_all_w(0);
+        load_all_k(0);
+        release(0);
+    }
+    group_sync();
     for (int c = 0; c < nchunk; ++c) {
-        const int s = c & 1;
-        const uint32_t par = (uint32_t)((c >> 1) & 1);
-        // ---- Y = W_c S
-        if (tid == 0) {
-            if (c == 0) ok = wait_bar(bars + 8 * kTSBarS0, 0, ab, 100);
-            if (ok) ok = wait_bar(bars + 8 * (kTSBarFull0 + s), par, ab, 101);
-            if (ok) {
-                tc_fence_after();
-                const uint32_t a_lo = ((smem_base + kTSOffW + s * kTileBytes) >> 4) | kLboK;
-                const uint32_t b_lo = ((smem_base + kTSOffS) >> 4) | kLboMN;
+        const bool more = c + 1 < nchunk;
+        if (kShared) {
+            landed(c);
+            ldsm4t(uf, stage(c) + u1_off);
+        }
+        // ---- Y^T = S^T W^T for this warp's 16 tokens: even and odd k-steps in chains of their own
+        float y[2][2][4] = {};
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint32_t koff = (uint32_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4);
-                    mma_ss(tmem_base, desc64(a_lo + koff), desc64(b_lo + (uint32_t)(ks * (2048 >> 4))), idesc_kn, ks > 0);
-                }
-                mma_commit(bars + 8 * kTSBarY);
+        for (int ks = 0; ks < 8; ++ks) {
+            uint32_t a[4];
+            ldsm4(a, a_s + ks * 32);
+            if (kShared) load_w(wf[0], stage(c), ks);
+            const uint32_t(&w)[4] = wf[kShared ? 0 : ks];
+#pragma unroll
+            for (int n = 0; n < 2; ++n) mma_16816(y[ks & 1][n], a, w[2 * n], w[2 * n + 1]);
+        }
+        if (!kShared && more) {
+            landed(c + 1);
+            load_all_w(c + 1);
+        }
+        // ---- U^T = U1^T - Y^T
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const uint32_t u1 = uf[2 * n + half];
+                const float lo = __uint_as_float(u1 << 16) - (y[0][n][2 * half] + y[1][n][2 * half]);
+                const float hi = __uint_as_float(u1 & 0xFFFF0000u) - (y[0][n][2 * half + 1] + y[1][n][2 * half + 1]);
+                *reinterpret_cast<uint32_t*>(u_s + (ge + 8 * half) * kScanLdU + wq * 16 + n * 8 + gk) = pack_bf16(lo, hi);
             }
-        }
-        alive = wait_bar(bars + 8 * kTSBarY, (uint32_t)(c & 1), ab, 102);
-        // the chunk's tiles landed before the MMA above was issued; waiting here as well makes
-        // the bulk copy's writes visible to this thread
-        if (alive) alive = wait_bar(bars + 8 * (kTSBarFull0 + s), par, ab, 103);
-        tc_fence_after();
-        // ---- U = U1_c - Y for the chunk's 64 tokens (threads 0-63), as a bf16 operand tile
-        if (alive && rowid < kTokC) {
-            const uint8_t* u1t = smem + kTSOffU1 + s * kHalfBytes + chalf * kChunkHalf;
-            uint8_t* ut = smem + kTSOffU + chalf * kChunkHalf;
-            uint32_t y[64];
-            tmem_ld32(lane_base, *reinterpret_cast<uint32_t(*)[32]>(&y[0]));
-            tmem_ld32(lane_base + 32, *reinterpret_cast<uint32_t(*)[32]>(&y[32]));
-            tmem_wait_ld();
+        const float g = __shfl_sync(0xffffffffu, g_cur, c & 31);
+        if ((c & 31) == 31) g_cur = c + 1 + lane < nchunk ? __ldg(gc + c + 1 + lane) : 1.0f;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {   // 16-byte chunk of this thread's 64-column half
-                const int off = rowid * 128 + ((q ^ (rowid & 7)) << 4);
-                const uint4 u1 = *reinterpret_cast<const uint4*>(u1t + off);
-                const uint32_t uw[4] = {u1.x, u1.y, u1.z, u1.w};
-                uint32_t o[4];
+        for (int n = 0; n < 4; ++n)
 #pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const float lo = __uint_as_float(uw[m] << 16) - __uint_as_float(y[q * 8 + 2 * m]);
-                    const float hi = __uint_as_float(uw[m] & 0xFFFF0000u) - __uint_as_float(y[q * 8 + 2 * m + 1]);
-                    o[m] = pack_bf16(lo, hi);
-                }
-                *reinterpret_cast<uint4*>(ut + off) = make_uint4(o[0], o[1], o[2], o[3]);
+            for (int x = 0; x < 4; ++x) st[n][x] *= g;
+        group_sync();
+        // ---- S^T = g S^T + U^T Khat for this warp's 32 keys
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+            uint32_t a[4];
+            ldsm4(a, a_u + ks * 32);
+            if (kShared) {
+                load_k(kf[0][0], stage(c), ks, 0);
+                load_k(kf[0][1], stage(c), ks, 1);
             }
+            const uint32_t(&kk)[2][4] = kf[kShared ? 0 : ks];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) mma_16816(st[n], a, kk[n >> 1][(n & 1) * 2], kk[n >> 1][(n & 1) * 2 + 1]);
         }
-        fence_proxy_async_smem();
-        tc_fence_before();
-        if (__syncthreads_or(!alive)) break;   // every thread leaves together
-        // ---- S += Khat_c^T U
-        if (tid == 0 && ok) {
-            tc_fence_after();
-            const uint32_t a_lo = ((smem_base + kTSOffKh + s * kHalfBytes) >> 4) | kLboMN64;
-            const uint32_t b_lo = ((smem_base + kTSOffU) >> 4) | kLboMN64;
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-                mma_ss(tmem_base + kTile, desc64(a_lo + (uint32_t)(ks * (2048 >> 4))),
-                       desc64(b_lo + (uint32_t)(ks * (2048 >> 4))), idesc_nn, 1u);
-            mma_commit(bars + 8 * kTSBarS2);
-        }
-        alive = wait_bar(bars + 8 * kTSBarS2, (uint32_t)(c & 1), ab, 104);
-        tc_fence_after();
-        if (alive && tid == 0 && c + 2 < nchunk) load_chunk(c + 2);   // both MMAs that read slot s are done
-        // ---- the new S: bf16 operand copy, and the fp32 rows scaled for the next chunk (or stored)
-        const bool last = c + 1 == nchunk;
-        const float gn = last ? 1.0f : __ldg(gc + c + 1);
-        if (alive) {
-            uint32_t x[64];
-            tmem_ld32(lane_base + kTile, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
-            tmem_ld32(lane_base + kTile + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
-            tmem_wait_ld();
-            if (!last) {
-                uint8_t* sb = smem + kTSOffS + chalf * kHalfBytes + rowid * 128;
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *reinterpret_cast<uint4*>(sb + ((q ^ (rowid & 7)) << 4)) =
-                        make_uint4(pack_bf16(__uint_as_float(x[q * 8 + 0]), __uint_as_float(x[q * 8 + 1])),
-                                   pack_bf16(__uint_as_float(x[q * 8 + 2]), __uint_as_float(x[q * 8 + 3])),
-                                   pack_bf16(__uint_as_float(x[q * 8 + 4]), __uint_as_float(x[q * 8 + 5])),
-                                   pack_bf16(__uint_as_float(x[q * 8 + 6]), __uint_as_float(x[q * 8 + 7])));
-#pragma unroll
-                for (int e = 0; e < 64; ++e) x[e] = __float_as_uint(__uint_as_float(x[e]) * gn);
-                tmem_st32(lane_base + kTile, *reinterpret_cast<uint32_t(*)[32]>(&x[0]));
-                tmem_st32(lane_base + kTile + 32, *reinterpret_cast<uint32_t(*)[32]>(&x[32]));
-            } else {
-                __nv_bfloat16* mrow = p.state_bf16 + (bh * kTile + rowid) * kTile + chalf * 64;
-#pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    *reinterpret_cast<uint4*>(srow + e * 4) = make_uint4(x[e * 4], x[e * 4 + 1], x[e * 4 + 2], x[e * 4 + 3]);
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *reinterpret_cast<uint4*>(mrow + q * 8) =
-                        make_uint4(pack_bf16(__uint_as_float(x[q * 8 + 0]), __uint_as_float(x[q * 8 + 1])),
-                                   pack_bf16(__uint_as_float(x[q * 8 + 2]), __uint_as_float(x[q * 8 + 3])),
-                                   pack_bf16(__uint_as_float(x[q * 8 + 4]), __uint_as_float(x[q * 8 + 5])),
-                                   pack_bf16(__uint_as_float(x[q * 8 + 6]), __uint_as_float(x[q * 8 + 7])));
+        if (kShared) release(c);
+        if (more) {
+            if (!kShared) {
+                load_all_k(c + 1);
+                release(c + 1);   // chunk c + 1 is in registers
             }
+            put_s();
+            group_sync();
         }
-        tmem_wait_st();
-        fence_proxy_async_smem();
-        tc_fence_before();
-        if (__syncthreads_or(!alive)) break;
     }
-    if (tid == 0 && (!ok || *abort_flag)) {
-        // leave no bulk copy in flight into this CTA's shared memory
-        drain_bar(bars + 8 * kTSBarS0, 0);
-        for (int m = (loads_issued > 2 ? loads_issued - 2 : 0); m < loads_issued; ++m)
-            drain_bar(bars + 8 * (kTSBarFull0 + (m & 1)), (uint32_t)((m >> 1) & 1));
-        mma_commit(bars + 8 * kTSBarDrain);    // no MMA still writing tensor memory when it is freed
-        drain_bar(bars + 8 * kTSBarDrain, 0);
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tc_fence_after();
-        tmem_dealloc(tmem_base, 256);
-    }
+    if (dead || *abort_flag || *reinterpret_cast<volatile uint32_t*>(p.status + kStatusError) != 0u) return;
+    __nv_bfloat16* mrow = p.state_bf16 + (srow - p.state);
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+            const size_t at = (size_t)(n * 8 + (x & 1)) * kTile + (x >> 1) * 8;
+            srow[at] = st[n][x];
+            mrow[at] = __float2bfloat16_rn(st[n][x]);
+        }
 }
 
 // The rotation table in the form the step kernel reads: half2 (cos, sin) per pair, 16 vectors of
@@ -1474,7 +1488,9 @@ int device_setup(int* num_sms)
         if (e == cudaSuccess) e = opt_in_smem(tc_step_kernel<true, false>, kSmemBytes);
         if (e == cudaSuccess) e = opt_in_smem(tc_step_kernel<false, true>, kSmemBytes);
         if (e == cudaSuccess) e = opt_in_smem(tc_token_prepare_kernel, kTPSmemBytes);
-        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel, kTSSmemBytes);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<1, false>, ScanCfg<1, false>::kSmemBytes);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<2, false>, ScanCfg<2, false>::kSmemBytes);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<2, true>, ScanCfg<2, true>::kSmemBytes);
         return e;
     }, num_sms);
 }
@@ -1606,7 +1622,6 @@ int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const
 {
     int num_sms = 0;
     if (int r = device_setup(&num_sms)) return r;
-    (void)num_sms;
     if (a.state_bf16 == nullptr) { set_error("tc_commit_tokens: needs the bf16 copy of the state"); return ARL2_ERR_INVALID_ARG; }
     TcTokenParams p;
     p.s = a.s;
@@ -1626,21 +1641,31 @@ int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const
     p.decayed = a.decayed ? 1 : 0;
     const size_t rows = (size_t)a.s.B * a.s.H * p.ntile * kTile;
     if (rows >= ((size_t)1 << 31)) { set_error("tc_commit_tokens: too many rows"); return ARL2_ERR_UNSUPPORTED; }
-    CUtensorMap tm_k, tm_v, tm_wk, tm_wv, tm_w, tm_kh, tm_u1, tm_s;
+    // Value columns per scan CTA: 16 while that leaves one CTA per SM (the walk is a latency chain), 32
+    // beyond (half the L2 traffic), two such CTAs per SM when even those do not fit beside one another (40 heads:
+    // 157 -> 113 us for the walk; four slabs in one CTA took 205: its 16 warps load 139 KB of fragments per chunk).
+    const long heads = (long)a.s.B * a.s.H;
+    const int slabs = heads * 8 <= num_sms ? 1 : 2;
+    const bool shared_sm = heads * 4 > num_sms;
+    CUtensorMap tm_k, tm_v, tm_wk, tm_wv, tm_w, tm_kh, tm_u1;
     if (int r = make_map_blhd(&tm_k, a.k, a.s)) return r;
     if (int r = make_map_blhd(&tm_v, a.v, a.s)) return r;
     if (int r = make_map_rows(&tm_wk, wk_op, (size_t)a.s.H * kTile)) return r;
     if (int r = make_map_rows(&tm_wv, wv_op, (size_t)a.s.H * kTile)) return r;
-    if (int r = make_map_rows(&tm_w, p.w, rows)) return r;
+    if (int r = make_map_rows(&tm_w, p.w, rows, kTokC)) return r;
     if (int r = make_map_rows(&tm_kh, p.kh, rows, kTokC)) return r;
-    if (int r = make_map_rows(&tm_u1, p.u1, rows, kTokC)) return r;
-    if (int r = make_map_rows(&tm_s, a.state_bf16, (size_t)a.s.B * a.s.H * kTile)) return r;
+    if (int r = make_map_rows(&tm_u1, p.u1, rows, kTokC, slabs * kScanSlab, false)) return r;
     dim3 grid1(p.ntile, a.s.H, a.s.B);
     tc_token_prepare_kernel<<<grid1, 128, kTPSmemBytes, st>>>(tm_k, tm_v, tm_wk, tm_wv, p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("launch of tc_token_prepare_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
-    dim3 grid2(a.s.H, a.s.B);
-    tc_token_scan_kernel<<<grid2, kTSThreads, kTSSmemBytes, st>>>(tm_w, tm_kh, tm_u1, tm_s, p);
+    dim3 grid2(kTile / (slabs * kScanSlab), a.s.H, a.s.B);
+    if (slabs == 1)
+        tc_token_scan_kernel<1, false><<<grid2, ScanCfg<1, false>::kThreads, ScanCfg<1, false>::kSmemBytes, st>>>(tm_w, tm_kh, tm_u1, p);
+    else if (!shared_sm)
+        tc_token_scan_kernel<2, false><<<grid2, ScanCfg<2, false>::kThreads, ScanCfg<2, false>::kSmemBytes, st>>>(tm_w, tm_kh, tm_u1, p);
+    else
+        tc_token_scan_kernel<2, true><<<grid2, ScanCfg<2, true>::kThreads, ScanCfg<2, true>::kSmemBytes, st>>>(tm_w, tm_kh, tm_u1, p);
     e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("launch of tc_token_scan_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 2;

@@ -178,17 +178,17 @@ int make_map_blhd(CUtensorMap* m, const void* base, const Shape& s)
     return 0;
 }
 
-// [rows, 128] bf16 row-major; box = 64 columns x 128 rows.
-int make_map_rows(CUtensorMap* m, const void* base, size_t rows, int box_rows = kTile)
+// [rows, 128] bf16 row-major; box = 64 columns x 128 rows unless said otherwise.
+int make_map_rows(CUtensorMap* m, const void* base, size_t rows, int box_rows = kTile, int box_cols = 64, bool swizzle = true)
 {
     EncodeTiledFn fn = encode_fn();
     if (fn == nullptr) { set_error("cuTensorMapEncodeTiled is not available from the driver"); return ARL2_ERR_CUDA; }
     cuuint64_t dims[2] = {(cuuint64_t)kTile, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)kTile * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+    cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { set_error("cuTensorMapEncodeTiled([rows,128]) failed with %d", (int)r); return ARL2_ERR_CUDA; }
     return 0;

@@ -101,3 +101,38 @@ def test_token_commit_with_the_prediction_against_the_decayed_state(oracle, dtyp
     # the two readings do differ on these inputs
     a, b = pair.layer.get_state().numpy(), plain.layer.get_state().numpy()
     assert np.abs(a - b).max() > 1e-3 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("B,H,L", [
+    (1, 18, 65),      # the most heads with one 16-column slab per CTA; a second chunk of one token
+    (1, 19, 449),     # two slabs per CTA; more chunks than its ring has stages
+    (1, 37, 128),     # the most heads with one CTA per SM
+    (2, 19, 330),     # two CTAs per SM
+    (1, 2, 2117),     # more chunks than one load of decays covers (32), a ragged last one
+])
+def test_token_commit_over_the_cuts_of_the_walk(oracle, B, H, L):
+    cfg = workload.custom(B=B, H=H, D=128, L=L, dtype="bf16", cfg_id=47)
+    pair = Pair(oracle, cfg, flags=FLAG)
+    for blk in range(2):
+        kc, vc, _ = workload.commit_inputs(cfg, blk)
+        alpha, beta = workload.token_gate_logits(cfg, blk)
+        err = pair.commit_tokens(kc, vc, alpha, beta)
+        assert err <= pair.tol, f"block {blk}: error {err:.3e} > {pair.tol}"
+
+
+def test_token_commit_that_timed_out_leaves_the_state(oracle):
+    cfg = workload.custom(B=1, H=3, D=128, L=700, dtype="bf16", cfg_id=48)
+    pair = Pair(oracle, cfg, flags=FLAG)
+    kc, vc, _ = workload.commit_inputs(cfg, 0)
+    alpha, beta = workload.token_gate_logits(cfg, 0)
+    assert pair.commit_tokens(kc, vc, alpha, beta) <= pair.tol
+    before = pair.layer.get_state().numpy()
+    d = pair.dev
+    pair.layer.debug_set_wait_limit(0)
+    pair.layer.commit_tokens(kc.to(d), vc.to(d), alpha.to(d), beta.to(d))
+    with pytest.raises(arl2.Arl2Error, match="wait"):
+        pair.layer.sync_status()
+    np.testing.assert_array_equal(pair.layer.get_state().numpy(), before)
+    pair.layer.debug_set_wait_limit(-1)
+    kc, vc, _ = workload.commit_inputs(cfg, 1)
+    assert pair.commit_tokens(kc, vc, alpha, beta) <= pair.tol
