@@ -19,6 +19,8 @@
 //
 // Every wait is bounded: when a limit expires the thread records ARL2_ERR_TIMEOUT in the
 // device status block, raises the CTA's abort flag and every role falls through to the exit.
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace arl2 {
@@ -802,25 +804,31 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 // Notation as in the plain-FMA version: for a chunk of C = 64 tokens entering with state S_0,
 //   U = U1 - W S_0,  S_C = g S_0 + Khat^T U,  U1 = T diag(beta) V',  W = T diag(beta g_{j-1}) K',
 //   T = (I + A)^-1,  A_ji = beta_j (g_{j-1} / g_i) <K'_j, K'_i> (i < j),  Khat_i = (g / g_i) K'_i.
-// tc_token_prepare_kernel: one CTA (128 threads, thread = token) per 128-token tile = two chunks.
-//   U_k, U_v (MMA) -> K' -> Gram matrix K' K'^T (MMA) -> A (fp32, shared memory) -> T by forward
-//   substitution (thread = column), stored as a bf16 block-diagonal 128 x 128 operand -> W and U1
-//   (MMA, both chunks at once) -> global: W, Khat, U1 in bf16, chunk decays g in fp32.
+// tc_token_prepare_kernel: one CTA per 128-token tile = two chunks; 256 threads, two per token row
+// (thread 0 also issues the copies and MMAs).  A tile is a chain of dependent stages, so two CTAs share an SM (96 KB of
+// tiles and 256 TMEM columns each) and hide each other's latencies:
+//   U_k = K W_k -> K' (bf16, over K);  U_v = V W_v -> diag(beta) V' (bf16, over V)        W_v replaces W_k
+//   Gram matrix K' K'^T -> A (fp32, column by column, over W_v);  diag(beta g) K' over K'
+//   T = (I + A)^-1 in place: the four 16 x 16 diagonal blocks of a chunk by forward substitution (thread =
+//   column), then T21 = -T22 A21 T11 for blocks of 16 and of 32 (all threads)
+//   T as a bf16 operand (over A): 128 rows x 64, each chunk's block in its own rows
+//   W = T diag(beta g) K', then U1 = T diag(beta) V': one MMA per chunk over all 128 rows, each token row
+//   read from its own chunk's result -> global: W, U1 (and Khat on the way) in bf16, chunk decays g in fp32.
+// 12 heads x 4680 tokens (444 tiles): 74 us with one 128-thread CTA per SM, T by one 64-step substitution per column
+// and row-wise stores -> 42 us; 40 heads 205 -> 112.
 // tc_token_scan_kernel: walks the chunks of a head in order (further down).
 // ---------------------------------------------------------------------------------------------
-constexpr int kTPOffWk = 0;                        // maps; later the fp32 matrix A (2 x 64 x 65)
-constexpr int kTPOffWv = kTileBytes;
-constexpr int kTPOffK = 2 * kTileBytes;            // raw K tile -> K' (bf16)
-constexpr int kTPOffV = 3 * kTileBytes;            // raw V tile -> diag(beta) V'
-constexpr int kTPOffKs = 4 * kTileBytes;           // diag(beta g_{j-1}) K'
-constexpr int kTPOffT = 5 * kTileBytes;            // block-diagonal T
-constexpr int kTPOffBars = 6 * kTileBytes;
-constexpr int kTPSmemBytes = kTPOffBars + 1024 + 1024;   // barriers, gate scratch, alignment slack
+constexpr int kTPOffK = 0;                         // raw K tile -> K' -> diag(beta g) K'
+constexpr int kTPOffV = kTileBytes;                // raw V tile -> diag(beta) V'
+constexpr int kTPOffW = 2 * kTileBytes;            // W_k; then W_v; then A -> T (2 x 64 x 68 fp32); then T (bf16)
 constexpr int kTokC = 64;                          // tokens per chunk
-constexpr int kLdA = kTokC + 4;   // 16-byte aligned rows, conflict-free 16-byte stores
-static_assert(2 * kTokC * kLdA * 4 <= 2 * kTileBytes, "A fits over the two maps");
+constexpr int kLdA = kTokC + 4;                    // column stride of A: 16-byte aligned, columns spread over the banks
+constexpr int kTPOffBars = kTPOffW + 2 * kTokC * kLdA * 4;
+constexpr int kTPSmemBytes = kTPOffBars + 1024 + 1024;   // barriers, gate scratch, alignment slack
+constexpr int kTPThreads = 256;
+static_assert(2 * kTokC * kLdA * 4 >= kTileBytes && kTPSmemBytes <= 115712, "two CTAs per SM");
 
-enum TPBar : int { kTPBarLoad = 0, kTPBarU, kTPBarG, kTPBarW, kTPBarDrain, kTPNumBars };
+enum TPBar : int { kTPBarLoadK = 0, kTPBarLoadV, kTPBarLoadW, kTPBarUk, kTPBarUv, kTPBarG, kTPBarW, kTPBarU1, kTPBarDrain, kTPNumBars };
 
 struct TcTokenParams {
     Shape s;
@@ -840,9 +848,10 @@ struct TcTokenParams {
     int decayed;               // prediction against alpha_j S_{j-1}
 };
 
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kTPThreads, 2)
 tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                         const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_wv,
+                        const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_u1,
                         const TcTokenParams p)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -852,75 +861,45 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     const uint32_t bars = smem_base + kTPOffBars;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kTPOffBars + kTPNumBars * 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kTPOffBars + kTPNumBars * 8 + 4);
-    float* cl_s = reinterpret_cast<float*>(smem + kTPOffBars + 64);          // [128] log g_j (inclusive)
-    float* wsum = reinterpret_cast<float*>(smem + kTPOffBars + 64 + 512);    // [4] warp totals
+    float* cl_s = reinterpret_cast<float*>(smem + kTPOffBars + 128);         // [128] log g_j (inclusive)
+    float* wsum = reinterpret_cast<float*>(smem + kTPOffBars + 128 + 512);   // [8] warp totals
     const Abort ab{abort_flag, p.status, p.spin_limit};
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tile = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int L = p.s.L, H = p.s.H;
-    const int row = tile * kTile + tid;          // this thread's token
-    const int chunk = tid >> 6, jj = tid & 63;   // chunk of the tile, index in the chunk
+    // two threads per token row: warps w and w + 4 own the same 32 TMEM lanes and split the 128 columns
+    const int r = (warp & 3) * 32 + lane;        // token row of the tile
+    const int hf = warp >> 2;                    // which 64 of the 128 columns
+    const int row = tile * kTile + r;            // this thread's token
+    const int chunk = r >> 6, jj = r & 63;       // chunk of the tile, index in the chunk
 
     if (tid == 0) {
         for (int i = 0; i < kTPNumBars; ++i) mbar_init(bars + 8 * i, 1);
         *abort_flag = 0;
         fence_barrier_init();
+        fence_proxy_async_smem();
+        const uint32_t bar_k = bars + 8 * kTPBarLoadK, bar_v = bars + 8 * kTPBarLoadV;
+        mbar_expect_tx(bar_k, 2 * kTileBytes);
+        mbar_expect_tx(bar_v, kTileBytes);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            tma_load_2d(smem_base + kTPOffW + half * kHalfBytes, &tm_wk, bar_k, half * 64, h * kTile);
+            tma_load_4d(smem_base + kTPOffK + half * kHalfBytes, &tm_k, bar_k, half * 64, h, tile * kTile, b);
+        }
+#pragma unroll
+        for (int half = 0; half < 2; ++half)
+            tma_load_4d(smem_base + kTPOffV + half * kHalfBytes, &tm_v, bar_v, half * 64, h, tile * kTile, b);
     }
-    // the off-diagonal blocks of T stay zero
-    for (int i = tid; i < kTileBytes / 16; i += 128)
-        reinterpret_cast<uint4*>(smem + kTPOffT)[i] = make_uint4(0u, 0u, 0u, 0u);
-    fence_proxy_async_smem();
     if (warp == 0) {
-        tmem_alloc(smem_u32(tmem_slot), 512);
+        tmem_alloc(smem_u32(tmem_slot), 256);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    const uint32_t lane_base = tmem_base + ((uint32_t)(warp * 32) << 16);
-
-    bool ok = true;
-    if (tid == 0) {
-        const uint32_t bar = bars + 8 * kTPBarLoad;
-        mbar_expect_tx(bar, 4 * kTileBytes);
-        tma_load_2d(smem_base + kTPOffWk, &tm_wk, bar, 0, h * kTile);
-        tma_load_2d(smem_base + kTPOffWk + kHalfBytes, &tm_wk, bar, 64, h * kTile);
-        tma_load_2d(smem_base + kTPOffWv, &tm_wv, bar, 0, h * kTile);
-        tma_load_2d(smem_base + kTPOffWv + kHalfBytes, &tm_wv, bar, 64, h * kTile);
-        tma_load_4d(smem_base + kTPOffK, &tm_k, bar, 0, h, tile * kTile, b);
-        tma_load_4d(smem_base + kTPOffK + kHalfBytes, &tm_k, bar, 64, h, tile * kTile, b);
-        tma_load_4d(smem_base + kTPOffV, &tm_v, bar, 0, h, tile * kTile, b);
-        tma_load_4d(smem_base + kTPOffV + kHalfBytes, &tm_v, bar, 64, h, tile * kTile, b);
-    }
-
-    // ---- gates: log alpha_j, beta_j, cumulative decay within the chunk (tokens past L: 1 and 0)
-    float la = 0.0f, be = 0.0f;
-    if (row < L) {
-        const size_t gi = ((size_t)b * L + row) * H + h;
-        if (p.alpha != nullptr) {
-            const float x = __ldg(p.alpha + gi);
-            la = x >= 0.0f ? -log1pf(expf(-x)) : x - log1pf(expf(x));
-        }
-        be = p.beta != nullptr ? 1.0f / (1.0f + expf(-__ldg(p.beta + gi))) : 1.0f;
-    }
-    float cl = la;   // inclusive scan over the 64 tokens of the chunk (two warps)
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float up = __shfl_up_sync(0xffffffffu, cl, off);
-        if (lane >= off) cl += up;
-    }
-    if (lane == 31) wsum[warp] = cl;
-    __syncthreads();
-    if (warp & 1) cl += wsum[warp - 1];
-    cl_s[tid] = cl;
-    __syncthreads();
-    const float cl_total = cl_s[chunk * kTokC + kTokC - 1];
-    const float cl_excl = cl - la;
-    // log of the factor on K'_j S_0: g_{j-1} for Eq. 4 as printed, g_j when the token's prediction is made
-    // against the state after its own forget gate
-    const float cl_pred = p.decayed ? cl : cl_excl;
+    const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
 
     constexpr uint32_t kLboK = 1u << 16;
     constexpr uint32_t kLboMN = (uint32_t)(kHalfBytes >> 4) << 16;
@@ -933,179 +912,354 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     constexpr uint32_t idesc_kk = idesc_bf16(kTile, kTile, 0, 0);   // both operands d-major
     constexpr uint32_t idesc_kn = idesc_bf16(kTile, kTile, 0, 1);   // A K-major, B rows = contraction index
     auto koff_k = [](int ks) { return (uint32_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4); };
+    const bool issuer = tid == 0;
+    bool ok = true;                              // the issuer's waits
+    bool alive = true;                           // the row threads' waits
+    bool w_loaded = false;
+    // D[128 x 128] = A[128 x 128] B^T, both d-major
+    auto issue_kk = [&](uint32_t col, int a_off, int b_off) {
+        const uint32_t a_lo = ((smem_base + a_off) >> 4) | kLboK, b_lo = ((smem_base + b_off) >> 4) | kLboK;
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks)
+            mma_ss(tmem_base + col, desc64(a_lo + koff_k(ks)), desc64(b_lo + koff_k(ks)), idesc_kk, ks > 0);
+    };
+    // columns c * 128: T (all 128 rows) times the 64 token rows of chunk c of a tile
+    auto issue_t = [&](int b_off) {
+        const uint32_t t_lo = ((smem_base + kTPOffW) >> 4) | kLboK, b_lo = ((smem_base + b_off) >> 4) | kLboMN;
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+                mma_ss(tmem_base + c * kTile, desc64(t_lo + (uint32_t)(ks * 32 >> 4)),
+                       desc64(b_lo + (uint32_t)((c * 4 + ks) * (2048 >> 4))), idesc_kn, ks > 0);
+    };
 
-    // ---- U_k = K W_phi_k, U_v = V W_phi_v
-    if (tid == 0) {
-        ok = wait_bar(bars + 8 * kTPBarLoad, 0, ab, 90);
+    if (issuer) {
+        // ---- U_k = K W_phi_k -> columns 0-127
+        ok = wait_bar(bars + 8 * kTPBarLoadK, 0, ab, 90);
         if (ok) {
             tc_fence_after();
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const uint32_t a_lo = ((smem_base + (u ? kTPOffV : kTPOffK)) >> 4) | kLboK;
-                const uint32_t b_lo = ((smem_base + (u ? kTPOffWv : kTPOffWk)) >> 4) | kLboK;
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    mma_ss(tmem_base + u * kTile, desc64(a_lo + koff_k(ks)), desc64(b_lo + koff_k(ks)), idesc_kk, ks > 0);
-            }
-            mma_commit(bars + 8 * kTPBarU);
+            issue_kk(0, kTPOffK, kTPOffW);
+            mma_commit(bars + 8 * kTPBarUk);
         }
     }
-    uint32_t sreg[128];
-    bool alive = wait_bar(bars + 8 * kTPBarU, 0, ab, 91);
-    const size_t grow = (((size_t)b * H + h) * p.ntile + tile) * kTile + tid;   // row of the scratch tensors
+
+    // ---- gates: log alpha_j, beta_j, cumulative decay within the chunk (tokens past L: 1 and 0)
+    float la = 0.0f, be = 0.0f, cl = 0.0f;
+    uint4 cs[8];
+    if (row < L) {
+        const size_t gi = ((size_t)b * L + row) * H + h;
+        if (p.alpha != nullptr) {
+            const float x = __ldg(p.alpha + gi);
+            la = x >= 0.0f ? -log1pf(expf(-x)) : x - log1pf(expf(x));
+        }
+        be = p.beta != nullptr ? 1.0f / (1.0f + expf(-__ldg(p.beta + gi))) : 1.0f;
+    }
+    if (p.rope_h != nullptr) {
+        const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16 + hf * 8) * 32 + (row & 31);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) cs[c] = __ldg(tab + c * 32);
+    }
+    cl = la;   // inclusive scan over the 64 tokens of the chunk (two warps)
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const float up = __shfl_up_sync(0xffffffffu, cl, off);
+        if (lane >= off) cl += up;
+    }
+    if (lane == 31) wsum[warp] = cl;
+    __syncthreads();
+    if (warp & 1) cl += wsum[warp - 1];
+    if (hf == 0) cl_s[r] = cl;
+    __syncthreads();
+    const float cl_total = cl_s[chunk * kTokC + kTokC - 1];
+    const float cl_excl = cl - la;
+    // log of the factor on K'_j S_0: g_{j-1} for Eq. 4 as printed, g_j when the token's prediction is made
+    // against the state after its own forget gate
+    const float cl_pred = p.decayed ? cl : cl_excl;
+
+    // 32 columns of this thread's half row (piece q of 2) into a swizzled tile, times f
+    auto put32 = [&](int off, int q, const uint32_t (&y)[32], float f) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            uint32_t w[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                w[m] = pack_bf16(__uint_as_float(y[c * 8 + 2 * m]) * f, __uint_as_float(y[c * 8 + 2 * m + 1]) * f);
+            *reinterpret_cast<uint4*>(smem + off + hf * kHalfBytes + r * 128 + (((q * 4 + c) ^ (r & 7)) << 4)) =
+                make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    };
+    alive = wait_bar(bars + 8 * kTPBarUk, 0, ab, 96);
+    if (issuer && ok && alive) {
+        // the value map takes the key map's place while the rows of K' are worked out
+        const uint32_t bar = bars + 8 * kTPBarLoadW;
+        mbar_expect_tx(bar, kTileBytes);
+        tma_load_2d(smem_base + kTPOffW, &tm_wv, bar, 0, h * kTile);
+        tma_load_2d(smem_base + kTPOffW + kHalfBytes, &tm_wv, bar, 64, h * kTile);
+        w_loaded = true;
+    }
+    float ss4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (alive) {
         tc_fence_after();
-        // ---- K' = L2Norm(RoPE(U_k)); three copies: K' (Gram), scaled for W, scaled for the scan
+        // ---- K' = L2Norm(RoPE(U_k)): the norm over the whole row first (a rotation leaves it as it is), then
+        // this thread's half, 32 columns at a time (with whole half rows in registers the kernel spilled at two
+        // CTAs per SM: 4.5 k clk for this pass against 1.5 k): K' for the Gram matrix, Khat to global memory,
+        // and K' in fp32 back to the columns of U_k for diag(beta g) K'
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            tmem_ld32(lane_base + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sreg[c * 32]));
-        tmem_wait_ld();
-        if (p.rope_h != nullptr) {
-            const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16) * 32 + (row & 31);
-            uint4 cs[16];
+        for (int q = 0; q < 4; ++q) {
+            uint32_t y[32];
+            tmem_ld32(lane_base + q * 32, y);
+            tmem_wait_ld();
 #pragma unroll
-            for (int c = 0; c < 16; ++c) cs[c] = __ldg(tab + c * 32);
+            for (int c = 0; c < 32; ++c) ss4[c & 3] = fmaf(__uint_as_float(y[c]), __uint_as_float(y[c]), ss4[c & 3]);
+        }
+    }
+    __syncthreads();   // the other thread of the row is done with the norm before this half is overwritten
+    if (alive) {
+        const float f = rsqrtf((ss4[0] + ss4[1]) + (ss4[2] + ss4[3]) + p.s.eps);
+        const float f_kh = expf(cl_total - cl);
+        __nv_bfloat16* kh = p.kh + ((((size_t)b * H + h) * p.ntile + tile) * kTile + r) * kTile + hf * 64;
 #pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                const uint32_t h2[4] = {cs[c].x, cs[c].y, cs[c].z, cs[c].w};
+        for (int q = 0; q < 2; ++q) {
+            uint32_t y[32];
+            tmem_ld32(lane_base + hf * 64 + q * 32, y);
+            tmem_wait_ld();
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const uint4 v = p.rope_h != nullptr ? cs[q * 4 + c] : make_uint4(0x3C00u, 0x3C00u, 0x3C00u, 0x3C00u);   // cos 1, sin 0
+                const uint32_t h2[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
                     float cc, s1;
                     unpack_cs(h2[m], cc, s1);
-                    const float x0 = __uint_as_float(sreg[c * 8 + 2 * m]);
-                    const float x1 = __uint_as_float(sreg[c * 8 + 2 * m + 1]);
-                    sreg[c * 8 + 2 * m] = __float_as_uint(x0 * cc - x1 * s1);
-                    sreg[c * 8 + 2 * m + 1] = __float_as_uint(x0 * s1 + x1 * cc);
+                    const float x0 = __uint_as_float(y[c * 8 + 2 * m]) * f, x1 = __uint_as_float(y[c * 8 + 2 * m + 1]) * f;
+                    y[c * 8 + 2 * m] = __float_as_uint(x0 * cc - x1 * s1);
+                    y[c * 8 + 2 * m + 1] = __float_as_uint(x0 * s1 + x1 * cc);
+                }
+            }
+            tmem_st32(lane_base + hf * 64 + q * 32, y);
+            put32(kTPOffK, q, y, 1.0f);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                uint32_t w[8];
+#pragma unroll
+                for (int m = 0; m < 8; ++m)
+                    w[m] = pack_bf16(__uint_as_float(y[e * 16 + 2 * m]) * f_kh, __uint_as_float(y[e * 16 + 2 * m + 1]) * f_kh);
+                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(kh + q * 32 + e * 16),
+                             "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                             : "memory");
+            }
+        }
+        tmem_wait_st();
+        if (issuer && ok) {
+            // ---- U_v = V W_phi_v -> columns 128-255
+            ok = wait_bar(bars + 8 * kTPBarLoadW, 0, ab, 94);
+            if (ok) ok = wait_bar(bars + 8 * kTPBarLoadV, 0, ab, 95);
+            if (ok) {
+                tc_fence_after();
+                issue_kk(kTile, kTPOffV, kTPOffW);
+                mma_commit(bars + 8 * kTPBarUv);
+            }
+        }
+        alive = wait_bar(bars + 8 * kTPBarUv, 0, ab, 97);
+        if (alive) {
+            tc_fence_after();
+            // ---- diag(beta) V'
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t y[32];
+                tmem_ld32(lane_base + kTile + hf * 64 + q * 32, y);
+                tmem_wait_ld();
+                put32(kTPOffV, q, y, be);
+            }
+        }
+    }
+    fence_proxy_async_smem();
+    tc_fence_before();
+    __syncthreads();
+
+    // ---- Gram matrix K' K'^T -> columns 128-255 (row = token j, column = token i)
+    if (issuer && ok && !*abort_flag) {
+        tc_fence_after();
+        issue_kk(kTile, kTPOffK, kTPOffK);
+        mma_commit(bars + 8 * kTPBarG);
+    }
+    float* As = reinterpret_cast<float*>(smem + kTPOffW);   // the maps are dead: U_k, U_v are complete
+    alive = alive && wait_bar(bars + 8 * kTPBarG, 0, ab, 92);
+    if (alive) {
+        tc_fence_after();
+        // diag(beta g) K' replaces K', which the Gram matrix was the last to read
+        const float f_w = be * expf(cl_pred);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            uint32_t y[32];
+            tmem_ld32(lane_base + hf * 64 + q * 32, y);
+            tmem_wait_ld();
+            put32(kTPOffK, q, y, f_w);
+        }
+        // this token's row of A: the columns of its own chunk, strictly below the diagonal (zero elsewhere),
+        // stored column by column (a warp's 32 rows side by side).  All values before the first store: the
+        // compiler may not move the reads of cl_s across stores to shared memory.
+        uint32_t g[32];
+        tmem_ld32(lane_base + kTile + chunk * kTokC + hf * 32, g);
+        tmem_wait_ld();
+        const float* cl_c = cl_s + chunk * kTokC + hf * 32;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            g[i] = __float_as_uint(hf * 32 + i < jj ? be * __expf(cl_pred - cl_c[i]) * __uint_as_float(g[i]) : 0.0f);
+        float* a_out = As + (chunk * kTokC + hf * 32) * kLdA + jj;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) a_out[i * kLdA] = __uint_as_float(g[i]);
+    }
+    tc_fence_before();
+    __syncthreads();
+    // ---- T = (I + A)^-1, in place (element (i, j) of chunk c at X[(c * 64 + j) * kLdA + i])
+    {
+        // diagonal blocks: thread = (chunk, block, column) for the first 128 threads
+        const int o = (tid >> 4 & 3) * 16, cc = tid & 15;
+        float* Xd = As + ((tid >> 6) * kTokC + o) * kLdA + o;
+        float t[16];
+        if (tid < 128) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) t[i] = i == cc ? 1.0f : 0.0f;
+#pragma unroll
+            for (int j = 0; j < 15; ++j) {
+                // as soon as t_j is known it is taken out of all later rows: a step is one FMA deep
+#pragma unroll
+                for (int i4 = (j + 1) / 4; i4 < 4; ++i4) {
+                    const float4 a4 = *reinterpret_cast<const float4*>(Xd + j * kLdA + i4 * 4);
+                    const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (i4 * 4 + k > j) t[i4 * 4 + k] = fmaf(-av[k], t[j], t[i4 * 4 + k]);
                 }
             }
         }
-        float ss4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        __syncthreads();
+        if (tid < 128) {
 #pragma unroll
-        for (int c = 0; c < 128; c += 4) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                ss4[k] = fmaf(__uint_as_float(sreg[c + k]), __uint_as_float(sreg[c + k]), ss4[k]);
+            for (int i4 = 0; i4 < 4; ++i4)
+                *reinterpret_cast<float4*>(Xd + cc * kLdA + i4 * 4) = make_float4(t[i4 * 4], t[i4 * 4 + 1], t[i4 * 4 + 2], t[i4 * 4 + 3]);
         }
-        const float f = rsqrtf((ss4[0] + ss4[1]) + (ss4[2] + ss4[3]) + p.s.eps);
-        store_row_bf16_swizzled(smem + kTPOffK, tid, sreg, f);
-        store_row_bf16_swizzled(smem + kTPOffKs, tid, sreg, f * be * expf(cl_pred));
-        store_row_bf16_global(p.kh + grow * kTile, sreg, f * expf(cl_total - cl));
-        // ---- diag(beta) V'
+        __syncthreads();
+        // out(i, j0 .. j0 + NJ) = sum over k < N of P(i, k) Q(k, j): each operand given by its first
+        // element; i runs over the lanes, k is contiguous in Q
+        auto product = [&](auto n_tag, auto nj_tag, const float* P, const float* Q, float* out, float sign, int i, int j0) {
+            constexpr int N = decltype(n_tag)::value, NJ = decltype(nj_tag)::value;
+            float acc[NJ] = {};
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            tmem_ld32(lane_base + kTile + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sreg[c * 32]));
-        tmem_wait_ld();
-        store_row_bf16_swizzled(smem + kTPOffV, tid, sreg, be);
+            for (int k4 = 0; k4 < N; k4 += 4) {
+                float pv[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) pv[k] = P[(k4 + k) * kLdA + i];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    const float4 q = *reinterpret_cast<const float4*>(Q + (j0 + j) * kLdA + k4);
+                    acc[j] = fmaf(pv[0], q.x, fmaf(pv[1], q.y, fmaf(pv[2], q.z, fmaf(pv[3], q.w, acc[j]))));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) out[(j0 + j) * kLdA + i] = sign * acc[j];
+        };
+        {
+            // blocks of 16: rows 32 m + 16 .., columns 32 m ..; the intermediate A21 T11 goes to the unused
+            // rows 0-15 of columns 32 + 16 m ..
+            const int c = tid >> 7, m = tid >> 6 & 1, u = tid & 63;
+            float* X = As + c * kTokC * kLdA;
+            float* low = X + (m * 32) * kLdA + m * 32 + 16;
+            float* tmp = X + (32 + m * 16) * kLdA;
+            product(std::integral_constant<int, 16>(), std::integral_constant<int, 4>(), low, X + (m * 32) * kLdA + m * 32, tmp, 1.0f,
+                    u & 15, (u >> 4) * 4);
+            __syncthreads();
+            product(std::integral_constant<int, 16>(), std::integral_constant<int, 4>(), X + (m * 32 + 16) * kLdA + m * 32 + 16, tmp, low,
+                    -1.0f, u & 15, (u >> 4) * 4);
+            __syncthreads();
+        }
+        {
+            // blocks of 32: rows 32 .., columns 0 ..; the intermediate in rows 0-31 of columns 32 ..
+            const int c = tid >> 7, u = tid & 127;
+            float* X = As + c * kTokC * kLdA;
+            float* low = X + 32;
+            float* tmp = X + 32 * kLdA;
+            product(std::integral_constant<int, 32>(), std::integral_constant<int, 8>(), low, X, tmp, 1.0f, u & 31, (u >> 5) * 8);
+            __syncthreads();
+            product(std::integral_constant<int, 32>(), std::integral_constant<int, 8>(), X + 32 * kLdA + 32, tmp, low, -1.0f, u & 31,
+                    (u >> 5) * 8);
+            __syncthreads();
+        }
+        // T as a K-major swizzled operand (row = token, 64 columns), over the fp32 matrix
+        uint4 tv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c16 = hf * 4 + q;
+            uint32_t w[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const int j = c16 * 8 + 2 * m;
+                const float lo = As[(chunk * kTokC + j) * kLdA + jj], hi = As[(chunk * kTokC + j + 1) * kLdA + jj];
+                w[m] = pack_bf16(j <= jj ? lo : 0.0f, j + 1 <= jj ? hi : 0.0f);
+            }
+            tv[q] = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<uint4*>(smem + kTPOffW + r * 128 + (((hf * 4 + q) ^ (r & 7)) << 4)) = tv[q];
     }
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
 
-    // ---- Gram matrix K' K'^T -> TMEM columns 256-383 (row = token j, column = token i)
-    if (tid == 0 && ok && !*abort_flag) {
-        tc_fence_after();
-        const uint32_t k_lo = ((smem_base + kTPOffK) >> 4) | kLboK;
+    // ---- W = T diag(beta g) K', then U1 = T diag(beta) V': chunk c's rows in columns c * 128 ..
+#pragma unroll 1
+    for (int u = 0; u < 2; ++u) {
+        const uint32_t bar = bars + 8 * (u == 0 ? kTPBarW : kTPBarU1);
+        if (issuer && ok && !*abort_flag) {
+            tc_fence_after();
+            issue_t(u == 0 ? kTPOffK : kTPOffV);
+            mma_commit(bar);
+        }
+        alive = alive && wait_bar(bar, 0, ab, 93);
+        if (alive) {
+            tc_fence_after();
+            // staged in the tile that this product was the last to read
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks)
-            mma_ss(tmem_base + 2 * kTile, desc64(k_lo + koff_k(ks)), desc64(k_lo + koff_k(ks)), idesc_kk, ks > 0);
-        mma_commit(bars + 8 * kTPBarG);
-    }
-    alive = alive && wait_bar(bars + 8 * kTPBarG, 0, ab, 92);
-    float* As = reinterpret_cast<float*>(smem + kTPOffWk);   // the maps are dead: U_k, U_v are complete
-    if (alive) {
-        tc_fence_after();
-        // this token's row of A: only the columns of its own chunk, strictly below the diagonal
-        uint32_t g[64];
-        tmem_ld32(lane_base + 2 * kTile + chunk * kTokC, *reinterpret_cast<uint32_t(*)[32]>(&g[0]));
-        tmem_ld32(lane_base + 2 * kTile + chunk * kTokC + 32, *reinterpret_cast<uint32_t(*)[32]>(&g[32]));
-        tmem_wait_ld();
-        float* arow = As + (chunk * kTokC + jj) * kLdA;
-#pragma unroll
-        for (int i4 = 0; i4 < kTokC / 4; ++i4) {
-            float v[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = i4 * 4 + k;
-                const float w = be * __expf(cl_pred - cl_s[chunk * kTokC + i]);
-                v[k] = i < jj ? w * __uint_as_float(g[i]) : 0.0f;
+            for (int q = 0; q < 2; ++q) {
+                uint32_t y[32];
+                tmem_ld32(lane_base + chunk * kTile + hf * 64 + q * 32, y);
+                tmem_wait_ld();
+                put32(u == 0 ? kTPOffK : kTPOffV, q, y, 1.0f);
             }
-            *reinterpret_cast<float4*>(arow + i4 * 4) = make_float4(v[0], v[1], v[2], v[3]);
         }
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
     }
-    __syncthreads();
-    // ---- T = (I + A)^-1 by forward substitution; this thread owns column jj of its chunk's T
-    if (alive) {
-        const float* Ac = As + chunk * kTokC * kLdA;
-        float t[kTokC];
+    // ---- W and U1 leave as whole tiles
+    const bool all_ok = ok && alive && !*abort_flag;
+    if (issuer && all_ok) {
+        const int r0 = (int)((((size_t)b * H + h) * p.ntile + tile) * kTile);
 #pragma unroll
-        for (int j = 0; j < kTokC; ++j) {
-            // row j of A in 16-byte pieces (the same address for the whole chunk: a broadcast),
-            // four independent partial sums
-            float acc[4] = {j == jj ? 1.0f : 0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-            for (int i4 = 0; i4 < (j + 3) / 4; ++i4) {
-                const float4 a4 = *reinterpret_cast<const float4*>(Ac + j * kLdA + i4 * 4);
-                const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (i4 * 4 + k < j) acc[k] -= av[k] * t[i4 * 4 + k];
-            }
-            t[j] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        for (int half = 0; half < 2; ++half) {
+            tma_store_2d(&tm_w, smem_base + kTPOffK + half * kHalfBytes, half * 64, r0);
+            tma_store_2d(&tm_u1, smem_base + kTPOffV + half * kHalfBytes, half * 64, r0);
         }
-        // element (row r = chunk*64 + j, column c = chunk*64 + jj) of the K-major swizzled bf16 tile
-        const int cglob = chunk * kTokC + jj;
-        uint8_t* tt = smem + kTPOffT + (cglob >> 6) * kHalfBytes + (cglob & 7) * 2;
-        const int c16 = (cglob & 63) >> 3;
-#pragma unroll
-        for (int j = 0; j < kTokC; ++j) {
-            const int r = chunk * kTokC + j;
-            *reinterpret_cast<__nv_bfloat16*>(tt + r * 128 + ((c16 ^ (r & 7)) << 4)) = __float2bfloat16_rn(t[j]);
-        }
+        tma_store_wait_read();
     }
-    fence_proxy_async_smem();
-    tc_fence_before();
-    __syncthreads();
-
-    // ---- W = T diag(beta g_{j-1}) K' -> columns 0-127, U1 = T diag(beta) V' -> columns 128-255
-    if (tid == 0 && ok && !*abort_flag) {
-        tc_fence_after();
-        const uint32_t t_lo = ((smem_base + kTPOffT) >> 4) | kLboK;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const uint32_t b_lo = ((smem_base + (u ? kTPOffV : kTPOffKs)) >> 4) | kLboMN;
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                mma_ss(tmem_base + u * kTile, desc64(t_lo + koff_k(ks)), desc64(b_lo + (uint32_t)(ks * (2048 >> 4))),
-                       idesc_kn, ks > 0);
-        }
-        mma_commit(bars + 8 * kTPBarW);
-    }
-    alive = alive && wait_bar(bars + 8 * kTPBarW, 0, ab, 93);
-    if (alive) {
-        tc_fence_after();
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            tmem_ld32(lane_base + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sreg[c * 32]));
-        tmem_wait_ld();
-        store_row_bf16_global(p.w + grow * kTile, sreg, 1.0f);
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            tmem_ld32(lane_base + kTile + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&sreg[c * 32]));
-        tmem_wait_ld();
-        store_row_bf16_global(p.u1 + grow * kTile, sreg, 1.0f);
-        if (jj == kTokC - 1)
-            p.gc[(((size_t)b * H + h) * p.ntile + tile) * 2 + chunk] = expf(cl_total);
-    }
-    if (tid == 0 && (!ok || *abort_flag)) {
-        drain_bar(bars + 8 * kTPBarLoad, 0);   // no bulk copy left in flight
-        mma_commit(bars + 8 * kTPBarDrain);    // and no MMA still writing tensor memory
+    if (hf == 0 && alive && jj == kTokC - 1)
+        p.gc[(((size_t)b * H + h) * p.ntile + tile) * 2 + chunk] = expf(cl_total);
+    if (issuer && (!ok || *abort_flag)) {
+        drain_bar(bars + 8 * kTPBarLoadK, 0);   // no bulk copy left in flight
+        drain_bar(bars + 8 * kTPBarLoadV, 0);
+        if (w_loaded) drain_bar(bars + 8 * kTPBarLoadW, 0);
+        mma_commit(bars + 8 * kTPBarDrain);     // and no MMA still writing tensor memory
         drain_bar(bars + 8 * kTPBarDrain, 0);
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc(tmem_base, 256);
     }
 }
 
@@ -1652,11 +1806,14 @@ int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const
     if (int r = make_map_blhd(&tm_v, a.v, a.s)) return r;
     if (int r = make_map_rows(&tm_wk, wk_op, (size_t)a.s.H * kTile)) return r;
     if (int r = make_map_rows(&tm_wv, wv_op, (size_t)a.s.H * kTile)) return r;
+    CUtensorMap out_w, out_u1;   // whole tiles, written by the prepare kernel
+    if (int r = make_map_rows(&out_w, p.w, rows)) return r;
+    if (int r = make_map_rows(&out_u1, p.u1, rows)) return r;
     if (int r = make_map_rows(&tm_w, p.w, rows, kTokC)) return r;
     if (int r = make_map_rows(&tm_kh, p.kh, rows, kTokC)) return r;
     if (int r = make_map_rows(&tm_u1, p.u1, rows, kTokC, slabs * kScanSlab, false)) return r;
     dim3 grid1(p.ntile, a.s.H, a.s.B);
-    tc_token_prepare_kernel<<<grid1, 128, kTPSmemBytes, st>>>(tm_k, tm_v, tm_wk, tm_wv, p);
+    tc_token_prepare_kernel<<<grid1, kTPThreads, kTPSmemBytes, st>>>(tm_k, tm_v, tm_wk, tm_wv, out_w, out_u1, p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { set_error("launch of tc_token_prepare_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     dim3 grid2(kTile / (slabs * kScanSlab), a.s.H, a.s.B);
