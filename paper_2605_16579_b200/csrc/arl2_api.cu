@@ -375,6 +375,42 @@ int arl2_denoise_step(arl2_ctx* ctx, const void* d_q, const void* d_k, const voi
     return launch_step(ctx, d_q, k_rot, d_v, d_gate_logits, d_out, st);
 }
 
+namespace {
+
+// Argument block of a commit on this context (mode: 0 gated linear, 1 delta rule, 2 per-token weights).
+bool fill_commit(arl2_ctx* ctx, CommitArgs& a, const void* d_k_clean, const void* d_v_clean,
+                 const float* d_decay_logits, int mode, const float* d_beta, bool decay_direct)
+{
+    if (!d_k_clean || !d_v_clean || !d_decay_logits) {
+        set_error("commit: k_clean, v_clean and decay_logits must not be NULL");
+        return false;
+    }
+    if ((reinterpret_cast<uintptr_t>(d_k_clean) | reinterpret_cast<uintptr_t>(d_v_clean)) % 16 != 0) {
+        set_error("commit: k_clean and v_clean must be 16-byte aligned");
+        return false;
+    }
+    a.s = ctx->shape;
+    a.k = d_k_clean; a.v = d_v_clean; a.decay = d_decay_logits;
+    a.wk = ctx->wk; a.wv = ctx->wv;
+    a.rope_cos = ctx->rope_cos; a.rope_sin = ctx->rope_sin;
+    a.state = ctx->state;
+    a.partials = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials);
+    a.partials_g = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials_g);
+    a.state_bf16 = ctx->use_tc ? mirror_of(ctx) : nullptr;
+    a.state_bf16_next = ctx->use_tc ? mirror_of(ctx, 1) : nullptr;
+    a.nsplit = ctx->lay.nsplit;
+    a.nslot = ctx->lay.nslot;
+    a.rope_h = (ctx->use_tc && ctx->rope_cos != nullptr) ? ctx->ws + ctx->lay.rope_h : nullptr;
+    a.status = reinterpret_cast<uint32_t*>(ctx->ws + ctx->lay.status);
+    a.mode = mode;
+    a.wait_limit = ctx->wait_limit;
+    a.beta = d_beta;
+    a.decay_direct = decay_direct;
+    return true;
+}
+
+}  // namespace
+
 int arl2_denoise_step_token_level(arl2_ctx* ctx, const void* d_q, const void* d_k, const void* d_v,
                                   const float* d_gate_logits, const float* d_alpha_logits, void* d_out,
                                   void* stream)
@@ -390,7 +426,31 @@ int arl2_denoise_step_token_level(arl2_ctx* ctx, const void* d_q, const void* d_
     const void* k_rot = nullptr;
     if (int r = rotate_k(ctx, d_k, &k_rot, st)) return r;
     if (int r = launch_step(ctx, d_q, k_rot, d_v, nullptr, d_out, st)) return r;
-    // 2. ... then the causal readout adds sigmoid(g_i) Q'_i S^(i) to it
+    // 2. ... then the state at the start of every run of tiles ...
+    const __nv_bfloat16* wk_op = reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wk_op);
+    float* w = reinterpret_cast<float*>(ctx->ws + ctx->lay.dec_w);
+    float* totals = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials_g);   // the delta rule's sums are not in use here
+    CommitArgs seg;
+    if (!fill_commit(ctx, seg, d_k, d_v, w, d_alpha_logits != nullptr ? 2 : 0, d_alpha_logits != nullptr ? w : nullptr, true))
+        return ARL2_ERR_INVALID_ARG;
+    int share = 0, ntile = 0;
+    if (int r = tc_commit_run_share(ctx->shape, seg.nslot, &share, &ntile)) return r;
+    // A walked tile takes about 10 us, the three launches before the walk 25 us and 1 us per tile of a run: heads
+    // of no more tiles than that are walked whole, from the state itself (one tile: 35 us per pass against 60,
+    // three tiles: 61 against 73; 13 tiles in runs of 2: 197 against 97).
+    const bool whole_heads = 10 * ntile <= 11 * share + 30;
+    if (whole_heads) {
+        seg.partials = nullptr;
+        seg.run_share = seg.run_ntile = ntile;
+    }
+    if (!whole_heads && d_alpha_logits != nullptr) {
+        if (int r = account(ctx, run_decay_weights(ctx->shape, d_alpha_logits, w, totals, share, ntile, seg.nslot, st))) return r;
+    }
+    if (!whole_heads) {
+        if (int r = account(ctx, tc_commit_partials(seg, wk_op, st))) return r;
+        if (int r = account(ctx, tc_run_prefix(seg, d_alpha_logits != nullptr ? totals : nullptr, st))) return r;
+    }
+    // 3. ... from which the causal readout adds sigmoid(g_i) Q'_i S^(i) to it
     StepArgs a;
     a.s = ctx->shape;
     a.q = d_q; a.k_rot = d_k; a.v = d_v; a.gate = d_gate_logits;
@@ -401,9 +461,8 @@ int arl2_denoise_step_token_level(arl2_ctx* ctx, const void* d_q, const void* d_
     a.status = reinterpret_cast<uint32_t*>(ctx->ws + ctx->lay.status);
     a.launch_parity = 0;
     a.rope_h = ctx->rope_cos != nullptr ? ctx->ws + ctx->lay.rope_h : nullptr;
-    return account(ctx, tc_token_readout(a, d_alpha_logits,
-                                         reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wq_op),
-                                         reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wk_op),
+    return account(ctx, tc_token_readout(a, d_alpha_logits, seg,
+                                         reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wq_op), wk_op,
                                          reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wv_op), st));
 }
 
@@ -480,38 +539,6 @@ int arl2_set_profile_events(arl2_ctx* ctx, void* ev_before, void* ev_after)
 }
 
 namespace {
-
-// Argument block of a commit on this context (mode: 0 gated linear, 1 delta rule, 2 per-token weights).
-bool fill_commit(arl2_ctx* ctx, CommitArgs& a, const void* d_k_clean, const void* d_v_clean,
-                 const float* d_decay_logits, int mode, const float* d_beta, bool decay_direct)
-{
-    if (!d_k_clean || !d_v_clean || !d_decay_logits) {
-        set_error("commit: k_clean, v_clean and decay_logits must not be NULL");
-        return false;
-    }
-    if ((reinterpret_cast<uintptr_t>(d_k_clean) | reinterpret_cast<uintptr_t>(d_v_clean)) % 16 != 0) {
-        set_error("commit: k_clean and v_clean must be 16-byte aligned");
-        return false;
-    }
-    a.s = ctx->shape;
-    a.k = d_k_clean; a.v = d_v_clean; a.decay = d_decay_logits;
-    a.wk = ctx->wk; a.wv = ctx->wv;
-    a.rope_cos = ctx->rope_cos; a.rope_sin = ctx->rope_sin;
-    a.state = ctx->state;
-    a.partials = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials);
-    a.partials_g = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials_g);
-    a.state_bf16 = ctx->use_tc ? mirror_of(ctx) : nullptr;
-    a.state_bf16_next = ctx->use_tc ? mirror_of(ctx, 1) : nullptr;
-    a.nsplit = ctx->lay.nsplit;
-    a.nslot = ctx->lay.nslot;
-    a.rope_h = (ctx->use_tc && ctx->rope_cos != nullptr) ? ctx->ws + ctx->lay.rope_h : nullptr;
-    a.status = reinterpret_cast<uint32_t*>(ctx->ws + ctx->lay.status);
-    a.mode = mode;
-    a.wait_limit = ctx->wait_limit;
-    a.beta = d_beta;
-    a.decay_direct = decay_direct;
-    return true;
-}
 
 // The second half of a tensor-core commit: the new state goes to S and to the mirror that was not
 // current, which becomes the current one.

@@ -119,6 +119,11 @@ int simt_commit(const CommitArgs& a, int dtype, cudaStream_t st);
 int commit_reduce(const CommitArgs& a, cudaStream_t st);  // fixed-order sum + gated decay
 // w[b,l,h] = prod_{i>l} sigmoid(alpha[b,i,h]), total[b,h] = prod_l sigmoid(alpha[b,l,h])
 int decay_weights(const Shape& s, const float* alpha_logits, float* w, float* total, cudaStream_t st);
+// The same per run of `share` tiles over the flattened tile sequence (a "segment" is what a run holds of one
+// head; segment i of a head is its i-th run): w = product of the forget gates after the token inside its
+// segment, total[bh, segment] (row stride nslot) = product over the segment.
+int run_decay_weights(const Shape& s, const float* alpha_logits, float* w, float* total, int share, int ntile, int nslot,
+                      cudaStream_t st);
 int simt_commit_tokens(const TokenCommitArgs& a, int dtype, cudaStream_t st);
 int fill_zero(void* p, size_t bytes, cudaStream_t st);
 int state_to_bf16(const float* state, __nv_bfloat16* dst, size_t n, cudaStream_t st);
@@ -136,11 +141,16 @@ int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* 
 // partial sums on tensor cores (fills a.run_share / a.run_ntile for the finishing kernel) ...
 int tc_commit_partials(CommitArgs& a, const __nv_bfloat16* wk_op, cudaStream_t st);
 // ... then S <- alpha S + (sum of slots) W_phi_v [- (sum of G slots) S_old], mirror written to state_bf16_next
+// tiles per run that tc_commit_partials cuts the flattened tile sequence into
+int tc_commit_run_share(const Shape& s, int nslot, int* share, int* ntile);
+// after tc_commit_partials: replaces the sums of segment i of every head by the state at the segment's start,
+//   S_0 = state, S_{i+1} = total_i S_i + (sums_i) W_phi_v   (total == nullptr: 1)
+int tc_run_prefix(const CommitArgs& a, const float* total, cudaStream_t st);
 int tc_commit_finish(const CommitArgs& a, cudaStream_t st);
 
 // out += sigmoid(g) Q' S^(i): token-level state access (a.k_rot holds the RAW K here; a.out already holds the
-// softmax branch); alpha_logits [B, L, H] or nullptr
-int tc_token_readout(const StepArgs& a, const float* alpha_logits, const __nv_bfloat16* wq_op,
+// softmax branch); alpha_logits [B, L, H] or nullptr; seg: after tc_commit_partials and tc_run_prefix
+int tc_token_readout(const StepArgs& a, const float* alpha_logits, const CommitArgs& seg, const __nv_bfloat16* wq_op,
                      const __nv_bfloat16* wk_op, const __nv_bfloat16* wv_op, cudaStream_t st);
 
 int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const __nv_bfloat16* wv_op,

@@ -930,12 +930,61 @@ __global__ void __launch_bounds__(1024) decay_weights_kernel(const float* __rest
     if (tid == 0) total[(size_t)b * H + h] = expf(carry);
 }
 
+// Segment (run, head) of the flattened tile sequence: one block walks its tokens backwards, 256 at a time.
+__global__ void __launch_bounds__(256) run_decay_weights_kernel(const float* __restrict__ alpha, float* __restrict__ w,
+                                                                float* __restrict__ total, int L, int H, int share, int ntile,
+                                                                int nslot)
+{
+    __shared__ float warp_tot[8];
+    const int slot = blockIdx.x, h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int bh = b * H + h, g_head = bh * ntile, run = g_head / share + slot;
+    const int g0 = max(g_head, run * share), g1 = min(g_head + ntile, (run + 1) * share);
+    if (g0 >= g1) return;
+    const int l0 = (g0 - g_head) * 128, l1 = min(L, (g1 - g_head) * 128);
+    const size_t base = (size_t)b * L * H + h;
+    float carry = 0.0f;   // log-product of all later tokens of the segment
+    for (int at = l0 + (l1 - 1 - l0) / 256 * 256; at >= l0; at -= 256) {
+        const int l = at + tid;
+        float la = 0.0f;
+        if (l < l1) {
+            const float x = alpha[base + (size_t)l * H];
+            la = x >= 0.0f ? -log1pf(expf(-x)) : x - log1pf(expf(x));   // log sigmoid(x)
+        }
+        float incl = la;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float dn = __shfl_down_sync(0xffffffffu, incl, off);
+            if (lane + off < 32) incl += dn;
+        }
+        if (lane == 0) warp_tot[wid] = incl;
+        __syncthreads();
+        float later = 0.0f, all = 0.0f;
+#pragma unroll
+        for (int q = 7; q >= 0; --q) {
+            if (q == wid) later = all;
+            all += warp_tot[q];
+        }
+        if (l < l1) w[base + (size_t)l * H] = expf(carry + later + (incl - la));
+        carry += all;
+        __syncthreads();
+    }
+    if (tid == 0) total[(size_t)bh * nslot + slot] = expf(carry);
+}
+
 int decay_weights(const Shape& s, const float* alpha_logits, float* w, float* total, cudaStream_t st)
 {
     int seg = (s.L + 1023) / 1024;
     seg = seg < 1 ? 1 : seg > 8 ? 8 : seg;
     decay_weights_kernel<<<dim3(s.H, s.B), 1024, 0, st>>>(alpha_logits, w, total, s.L, s.H, seg);
     if (int r = check_launch("decay_weights_kernel")) return r;
+    return 1;
+}
+
+int run_decay_weights(const Shape& s, const float* alpha_logits, float* w, float* total, int share, int ntile, int nslot,
+                      cudaStream_t st)
+{
+    run_decay_weights_kernel<<<dim3(nslot, s.H, s.B), 256, 0, st>>>(alpha_logits, w, total, s.L, s.H, share, ntile, nslot);
+    if (int r = check_launch("run_decay_weights_kernel")) return r;
     return 1;
 }
 

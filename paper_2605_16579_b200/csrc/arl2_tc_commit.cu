@@ -637,6 +637,83 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* __restrict__ par
     }
 }
 
+// The state at the start of every segment (what a run holds of one head), in place of the segment's sums:
+// S_{i+1} = total_i S_i + (sums_i) W_phi_v.  Geometry, products and the layout inside a slot as in the finishing
+// kernel; a CTA owns 16 rows of a head and walks the head's segments in order, the sums of the next segment
+// under way while this one's are multiplied.
+__global__ void __launch_bounds__(kFinThreads)
+tc_run_prefix_kernel(float* __restrict__ slots, const float* __restrict__ state, const __nv_bfloat16* __restrict__ wv,
+                     const float* __restrict__ total, int H, int share, int ntile, int nslot)
+{
+    extern __shared__ __align__(16) uint8_t fin_smem[];
+    __nv_bfloat16* Ws = reinterpret_cast<__nv_bfloat16*>(fin_smem);
+    float* As = reinterpret_cast<float*>(fin_smem + kFinMatBytes);   // two buffers of 16 x 128 sums
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int srow = lane >> 1, shalf = lane & 1;
+    const int bh = (int)(blockIdx.x / (kTile / kFinRows)), h = bh % H;
+    const int cta_row0 = (int)(blockIdx.x % (kTile / kFinRows)) * kFinRows;
+    if (wv != nullptr) fin_load_matrix(Ws, wv + (size_t)h * kTile * kTile, tid);
+    const int nparts = (bh * ntile + ntile - 1) / share - (bh * ntile) / share + 1;
+    float* head_slots = slots + (size_t)bh * nslot * kTile * kTile;
+    const size_t read0 = ((size_t)(warp * 4) * kTile + cta_row0 + srow) * 8 + shalf * 4;
+    const int g = lane >> 2, t = lane & 3;
+    const size_t write0 = ((size_t)(warp * 4) * kTile + cta_row0 + g) * 8 + 2 * t;
+    const size_t state0 = ((size_t)bh * kTile + cta_row0 + g) * kTile + warp * 32 + 2 * t;
+    float S[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const float2 v = *reinterpret_cast<const float2*>(state + state0 + j * 8 + (size_t)half * 8 * kTile);
+            S[j][2 * half] = v.x;
+            S[j][2 * half + 1] = v.y;
+        }
+    float4 cur[4];
+    auto fetch = [&](int i) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            cur[c] = *reinterpret_cast<const float4*>(head_slots + (size_t)i * kTile * kTile + read0 + (size_t)c * kTile * 8);
+    };
+    if (nparts > 1) fetch(0);
+    fin_matrices_landed();
+    for (int i = 0; i < nparts; ++i) {
+        float* A = As + (i & 1) * kFinRows * kFinLdA;
+        const bool more = i + 1 < nparts;   // the last segment's sums lead nowhere
+        float gamma = 1.0f;
+        if (more) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) *reinterpret_cast<float4*>(A + srow * kFinLdA + (warp * 4 + c) * 8 + shalf * 4) = cur[c];
+            if (i + 2 < nparts) fetch(i + 1);
+            if (total != nullptr) gamma = __ldg(total + (size_t)bh * nslot + i);
+        }
+        __syncthreads();   // the CTA's rows of this slot have been read
+        float* out = head_slots + (size_t)i * kTile * kTile + write0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int half = 0; half < 2; ++half)
+                *reinterpret_cast<float2*>(out + ((size_t)j * kTile + half * 8) * 8) = make_float2(S[j][2 * half], S[j][2 * half + 1]);
+        if (!more) break;
+        float inc[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (wv == nullptr) {
+                const float2 lo = *reinterpret_cast<const float2*>(A + g * kFinLdA + warp * 32 + j * 8 + 2 * t);
+                const float2 hi = *reinterpret_cast<const float2*>(A + (g + 8) * kFinLdA + warp * 32 + j * 8 + 2 * t);
+                inc[j][0] = lo.x; inc[j][1] = lo.y; inc[j][2] = hi.x; inc[j][3] = hi.y;
+            } else {
+                inc[j][0] = inc[j][1] = inc[j][2] = inc[j][3] = 0.0f;
+            }
+        }
+        if (wv != nullptr) fin_multiply<false>(inc, A, Ws, warp, lane);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) S[j][x] = gamma * S[j][x] + inc[j][x];
+    }
+}
+constexpr int kPrefixSmemBytes = kFinMatBytes + 2 * kFinRowBytes;
+
 std::mutex g_setup_mutex;
 DeviceSetup g_setup[kMaxDevices];
 
@@ -648,16 +725,42 @@ int device_setup(int* num_sms)
         if (e == cudaSuccess) e = opt_in_smem(tc_commit_kernel<2>, kCommitSmemBytes);
         if (e == cudaSuccess) e = opt_in_smem(tc_commit_finish_kernel<0>, fin_smem_bytes(0));
         if (e == cudaSuccess) e = opt_in_smem(tc_commit_finish_kernel<1>, fin_smem_bytes(1));
+        if (e == cudaSuccess) e = opt_in_smem(tc_run_prefix_kernel, kPrefixSmemBytes);
         return e;
     }, num_sms);
 }
 
 }  // namespace
 
-int tc_commit_partials(CommitArgs& a, const __nv_bfloat16* wk_op, cudaStream_t st)
+// equal runs of the flattened tile sequence, at least 2 tiles each and long enough for a head's
+// partial sums (one per run it falls into, at most ceil(ntile / share) + 1) to fit the slots
+int tc_commit_run_share(const Shape& s, int nslot, int* share, int* ntile)
 {
     int num_sms = 0;
     if (int r = device_setup(&num_sms)) return r;
+    if (nslot < 2) {
+        set_error("tc_commit: needs at least two partial-sum slots per head (got %d)", nslot);
+        return ARL2_ERR_WORKSPACE;
+    }
+    *ntile = (s.L + kTile - 1) / kTile;
+    const int total = s.B * s.H * *ntile;
+    *share = (total + num_sms - 1) / num_sms;
+    if (*share < 2) *share = 2;
+    if ((*ntile + *share - 1) / *share + 1 > nslot) *share = (*ntile + nslot - 2) / (nslot - 1);
+    return 0;
+}
+
+int tc_run_prefix(const CommitArgs& a, const float* total, cudaStream_t st)
+{
+    tc_run_prefix_kernel<<<(unsigned)(a.s.B * a.s.H) * (kTile / kFinRows), kFinThreads, kPrefixSmemBytes, st>>>(
+        a.partials, a.state, static_cast<const __nv_bfloat16*>(a.wv), total, a.s.H, a.run_share, a.run_ntile, a.nslot);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) { set_error("launch of tc_run_prefix_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
+    return 1;
+}
+
+int tc_commit_partials(CommitArgs& a, const __nv_bfloat16* wk_op, cudaStream_t st)
+{
     if (a.mode == 1 && (a.partials_g == nullptr || a.state_bf16 == nullptr)) {
         set_error("tc_commit: the delta rule needs the second accumulator and the bf16 copy of the state");
         return ARL2_ERR_INVALID_ARG;
@@ -675,18 +778,9 @@ int tc_commit_partials(CommitArgs& a, const __nv_bfloat16* wk_op, cudaStream_t s
     p.k_rot = a.rope_h != nullptr ? static_cast<__nv_bfloat16*>(a.k_rot_out) : nullptr;
     p.status = a.status;
     p.spin_limit = a.wait_limit ? a.wait_limit - 1 : kSpinLimit;
-    // equal runs of the flattened tile sequence, at least 2 tiles each and long enough for a head's
-    // partial sums (one per run it falls into, at most ceil(ntile / share) + 1) to fit the slots
-    p.ntile = (a.s.L + kTile - 1) / kTile;
-    p.total_tiles = a.s.B * a.s.H * p.ntile;
-    p.share = (p.total_tiles + num_sms - 1) / num_sms;
-    if (p.share < 2) p.share = 2;
     p.nslot = a.nslot;
-    if (p.nslot < 2) {
-        set_error("tc_commit: needs at least two partial-sum slots per head (got %d)", p.nslot);
-        return ARL2_ERR_WORKSPACE;
-    }
-    if ((p.ntile + p.share - 1) / p.share + 1 > p.nslot) p.share = (p.ntile + p.nslot - 2) / (p.nslot - 1);
+    if (int r = tc_commit_run_share(a.s, a.nslot, &p.share, &p.ntile)) return r;
+    p.total_tiles = a.s.B * a.s.H * p.ntile;
     const unsigned grid = (unsigned)((p.total_tiles + p.share - 1) / p.share);
     if (a.mode == 1)
         tc_commit_kernel<1><<<grid, kCThreads, kCommitSmemBytes, st>>>(tm_k, tm_v, tm_wk, p);

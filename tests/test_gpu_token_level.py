@@ -88,3 +88,26 @@ def test_token_level_needs_the_tensor_core_context(oracle):
     q, k, v, g = (t.to(pair.dev) for t in workload.step_inputs(cfg, 0, 0))
     with pytest.raises(arl2.Arl2Error, match="status -2"):
         pair.layer.denoise_step_token_level(q, k, v, g)
+
+
+@pytest.mark.parametrize("B,H,L,gates", [
+    (1, 2, 640, "forgetting"),     # the longest heads that are walked whole at two tiles per run
+    (1, 38, 1030, "near one"),     # runs of three tiles that cross from one head into the next, ragged last tile
+    (2, 19, 1030, "none"),
+])
+def test_token_level_over_runs_that_cross_heads(oracle, B, H, L, gates):
+    cfg = workload.custom(B=B, H=H, D=128, L=L, dtype="bf16", cfg_id=63)
+    pair = Pair(oracle, cfg)
+    kc, vc, a = workload.commit_inputs(cfg, 0)
+    assert pair.commit(kc, vc, a) <= pair.tol
+    q, k, v, g = workload.step_inputs(cfg, 1, 0)
+    alpha = None
+    if gates != "none":
+        alpha = workload.token_gate_logits(cfg, 1, alpha_mean=7.0 if gates == "near one" else 1.5)[0]
+    before = pair.layer.get_state().numpy().tobytes()
+    got = run(pair, q, k, v, g, alpha)
+    ref = oracle.step_token_level(q, k, v, g, pair.S_ref, alpha, pair.wq, pair.wk, pair.wv, pair.cos, pair.sin)
+    err = float(head_errors(got, ref).max())
+    assert err <= pair.tol, f"{err:.3e} > {pair.tol}"
+    assert pair.layer.get_state().numpy().tobytes() == before
+    pair.layer.sync_status()
