@@ -342,6 +342,7 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
         // really went out moves on to the other one
         if (r == ARL2_OK) ++ctx->step_calls;
     } else {
+        a.k_raw = simt_step_rotates_k(ctx->shape, ctx->wq);
         r = account(ctx, simt_step(a, ctx->cfg.io_dtype, st));
     }
     if (e1 != nullptr) cudaEventRecord(e1, st);
@@ -352,7 +353,7 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
 int rotate_k(arl2_ctx* ctx, const void* d_k, const void** k_rot, cudaStream_t st)
 {
     *k_rot = d_k;
-    if (ctx->rope_cos == nullptr) return ARL2_OK;
+    if (ctx->rope_cos == nullptr || (!ctx->use_tc && simt_step_rotates_k(ctx->shape, ctx->wq))) return ARL2_OK;
     void* buf = ctx->ws + ctx->lay.k_rot;
     int r = ctx->use_tc
                 ? account(ctx, tc_rope_k(ctx->shape, d_k, ctx->ws + ctx->lay.rope_h, buf, st))

@@ -34,7 +34,7 @@ struct Shape {
 struct StepArgs {
     Shape s;
     const void* q;
-    const void* k_rot;      // K after RoPE (or the caller's K when there is no rotation)
+    const void* k_rot;      // K after RoPE (or the caller's K when there is no rotation, or with k_raw)
     const void* v;
     const float* gate;      // [B, L, H]
     const float* state;     // [B, H, D, D] fp32, read only
@@ -46,6 +46,7 @@ struct StepArgs {
     int launch_parity;      // step launches so far on this context, mod 2 (scheduler counters)
     const void* rope_h;     // [L, D/2] half2 (cos, sin) copy of the tables (tensor-core path), or nullptr
     int Lk = 0;             // > 0: K and V hold Lk tokens (a cache), [B, Lk, H, D]; 0: L
+    bool k_raw = false;     // plain-FMA path: k_rot is the caller's K, rotated by the step kernel itself
     int gate_mode = 0;      // 0: gate [B, L, H]; 1: [B, L]; 2: [B, L, H, D]
     uint32_t wait_limit = 0;  // 0: default; n > 0: bounded waits give up after n - 1 polls (test hook)
     // key-range split of the last wave of work items (tensor-core path), or nullptr: never split
@@ -114,6 +115,8 @@ constexpr int kTokenChunk = 64;
 // Each returns the number of kernels it launched (>= 0) or a negative arl2_status.
 int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, const float* sin_t,
                 void* k_rot, cudaStream_t st);
+// whether the step kernel that serves this shape rotates K itself (then StepArgs::k_raw must be set)
+bool simt_step_rotates_k(const Shape& s, const void* wq);
 int simt_step(const StepArgs& a, int dtype, cudaStream_t st);
 int simt_commit(const CommitArgs& a, int dtype, cudaStream_t st);
 int commit_reduce(const CommitArgs& a, cudaStream_t st);  // fixed-order sum + gated decay

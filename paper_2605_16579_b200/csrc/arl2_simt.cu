@@ -330,6 +330,302 @@ __global__ void __launch_bounds__(NT) simt_step_kernel(StepArgs a)
     }
 }
 
+// The step for D = 128, and for shapes whose 64-row tiles would leave most SMs idle (a 16 x 16 latent frame: 8
+// tiles).  16 query rows per CTA, and the eight warps split the keys: a warp scores its share of each key tile
+// against all rows, keeps its own running maximum, sum and O, and the eight partial results are merged at the end,
+// so that the loop over the keys has no CTA-wide exchange.  K is rotated while it is loaded (no separate launch).
+// Lane (rg, kg) holds a 4 x KJ block of scores, rows 4 i + rg, keys 8 j + kg: every shared-memory read of the
+// products is a 16-byte one without bank conflicts, 8 (KJ = 4) or 6 (KJ = 2) of them per 4 columns for 64 or
+// 32 FMAs.
+constexpr int SR = 16;
+template <int D>
+struct SmallCfg {
+    static constexpr int KT = D == 64 ? 256 : 128;     // keys per tile
+    static constexpr int KW = KT / 8, KJ = KW / 8;     // keys per warp, per lane
+    static constexpr int LD = D + 4, LP = KW + 4;
+    static constexpr int kFloats = SR * LD + KT * LD + KT * D + 8 * SR * LP + 2 * 8 * SR;
+};
+
+template <int D, typename T>
+__global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
+{
+    using C = SmallCfg<D>;
+    constexpr int KT = C::KT, KW = C::KW, KJ = C::KJ, LD = C::LD, LP = C::LP, CN = D / 32;
+    extern __shared__ __align__(16) float smem[];
+    float* Qs = smem;                  // [16][LD] rotated Q; later raw Q, then Q'
+    float* Ks = Qs + SR * LD;          // [KT][LD] rotated K tile; later the warps' O, then W_phi_q
+    float* Vs = Ks + KT * LD;          // [KT][D]  V tile; later S
+    float* Ps = Vs + KT * D;           // [8][16][LP] probabilities, one block per warp
+    float* Ms = Ps + 8 * SR * LP;      // [8][16] reference maxima, then [8][16] row sums
+    float* Ls = Ms + 8 * SR;
+
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int rg = lane >> 3, kg = lane & 7;
+    const int L = a.s.L, H = a.s.H;
+    const int i0 = blockIdx.x * SR, h = blockIdx.y, b = blockIdx.z;
+    const T* q = static_cast<const T*>(a.q);
+    const T* k = static_cast<const T*>(a.k_rot);
+    const T* v = static_cast<const T*>(a.v);
+
+    auto load4 = [](const T* src) {
+        if constexpr (sizeof(T) == 4) {
+            return *reinterpret_cast<const float4*>(src);
+        } else {
+            const uint2 u = *reinterpret_cast<const uint2*>(src);
+            return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                               __uint_as_float(u.y & 0xFFFF0000u));
+        }
+    };
+    // 4 columns of a row, rotated (and rounded to the io type, as a rotated operand in memory would be)
+    auto rotated4 = [&](const T* t, int row, int c4) {
+        float4 x = load4(t + (((size_t)b * L + row) * H + h) * D + c4 * 4);
+        if (a.rope_cos != nullptr) {
+            const float2 c = *reinterpret_cast<const float2*>(a.rope_cos + (size_t)row * (D / 2) + c4 * 2);
+            const float2 s = *reinterpret_cast<const float2*>(a.rope_sin + (size_t)row * (D / 2) + c4 * 2);
+            x = make_float4(x.x * c.x - x.y * s.x, x.x * s.x + x.y * c.x, x.z * c.y - x.w * s.y, x.z * s.y + x.w * c.y);
+            if (sizeof(T) == 2) {
+                x.x = __bfloat162float(__float2bfloat16_rn(x.x)); x.y = __bfloat162float(__float2bfloat16_rn(x.y));
+                x.z = __bfloat162float(__float2bfloat16_rn(x.z)); x.w = __bfloat162float(__float2bfloat16_rn(x.w));
+            }
+        }
+        return x;
+    };
+    const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+
+    for (int idx = tid; idx < SR * (D / 4); idx += NT) {
+        const int r = idx / (D / 4), c4 = idx % (D / 4);
+        *reinterpret_cast<float4*>(Qs + r * LD + c4 * 4) = i0 + r < L ? rotated4(q, i0 + r, c4) : zero4;
+    }
+    float o[4][CN * 4];
+    float mrun[4], lrun[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        mrun[i] = -INFINITY;
+        lrun[i] = 0.0f;
+#pragma unroll
+        for (int e = 0; e < CN * 4; ++e) o[i][e] = 0.0f;
+    }
+    float* Pw = Ps + w * SR * LP;
+
+    for (int j0 = 0; j0 < L; j0 += KT) {
+        __syncthreads();   // previous tile fully consumed
+        constexpr int kPer = KT * (D / 4) / NT;
+#pragma unroll 4
+        for (int it = 0; it < kPer; ++it) {
+            const int idx = tid + it * NT, r = idx / (D / 4), c4 = idx % (D / 4), row = j0 + r;
+            float4 kv = zero4, vv = zero4;
+            if (row < L) {
+                kv = rotated4(k, row, c4);
+                vv = load4(v + (((size_t)b * L + row) * H + h) * D + c4 * 4);
+            }
+            *reinterpret_cast<float4*>(Ks + r * LD + c4 * 4) = kv;
+            *reinterpret_cast<float4*>(Vs + r * D + c4 * 4) = vv;
+        }
+        __syncthreads();
+
+        float s[4][KJ];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < KJ; ++j) s[i][j] = 0.0f;
+        const float* kb = Ks + (w * KW + kg) * LD;
+        const float* qb = Qs + rg * LD;
+#pragma unroll 4
+        for (int d = 0; d < D; d += 4) {
+            float4 qv[4], kv[KJ];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) qv[i] = *reinterpret_cast<const float4*>(qb + i * 4 * LD + d);
+#pragma unroll
+            for (int j = 0; j < KJ; ++j) kv[j] = *reinterpret_cast<const float4*>(kb + j * 8 * LD + d);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < KJ; ++j)
+                    s[i][j] = fmaf(qv[i].x, kv[j].x, fmaf(qv[i].y, kv[j].y, fmaf(qv[i].z, kv[j].z, fmaf(qv[i].w, kv[j].w, s[i][j]))));
+        }
+        // online softmax over this warp's keys (base 2; keys past L are masked out).  A warp whose share lies
+        // past L altogether keeps a maximum of -inf and weights of 0.
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float mx = -INFINITY;
+#pragma unroll
+            for (int j = 0; j < KJ; ++j) {
+                s[i][j] = j0 + w * KW + j * 8 + kg < L ? s[i][j] * a.s.scale_log2 : -INFINITY;
+                mx = fmaxf(mx, s[i][j]);
+            }
+#pragma unroll
+            for (int off = 4; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            const float mnew = fmaxf(mrun[i], mx);
+            const float mref = mnew == -INFINITY ? 0.0f : mnew;
+            const float corr = exp2f(mrun[i] - mref);
+            float sum = 0.0f;
+#pragma unroll
+            for (int j = 0; j < KJ; ++j) {
+                s[i][j] = exp2f(s[i][j] - mref);
+                sum += s[i][j];
+                Pw[(i * 4 + rg) * LP + j * 8 + kg] = s[i][j];
+            }
+#pragma unroll
+            for (int off = 4; off >= 1; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            lrun[i] = lrun[i] * corr + sum;
+            mrun[i] = mnew;
+#pragma unroll
+            for (int e = 0; e < CN * 4; ++e) o[i][e] *= corr;
+        }
+        __syncwarp();
+        // O += P V over this warp's keys: rows 4 i + rg, columns 32 c + 4 kg ..
+        const float* vb = Vs + (w * KW) * D + kg * 4;
+#pragma unroll 2
+        for (int kk = 0; kk < KW; kk += 4) {
+            float4 p4[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) p4[i] = *reinterpret_cast<const float4*>(Pw + (i * 4 + rg) * LP + kk);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+#pragma unroll
+                for (int c = 0; c < CN; ++c) {
+                    const float4 vv = *reinterpret_cast<const float4*>(vb + (kk + e) * D + c * 32);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float pv = e == 0 ? p4[i].x : e == 1 ? p4[i].y : e == 2 ? p4[i].z : p4[i].w;
+                        o[i][c * 4 + 0] = fmaf(pv, vv.x, o[i][c * 4 + 0]);
+                        o[i][c * 4 + 1] = fmaf(pv, vv.y, o[i][c * 4 + 1]);
+                        o[i][c * 4 + 2] = fmaf(pv, vv.z, o[i][c * 4 + 2]);
+                        o[i][c * 4 + 3] = fmaf(pv, vv.w, o[i][c * 4 + 3]);
+                    }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    // ---- merge of the warps' results
+    float* Ow = Ks;                    // [8][16][D]
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int r = i * 4 + rg;
+        if (kg == 0) {
+            Ms[w * SR + r] = mrun[i];
+            Ls[w * SR + r] = lrun[i];
+        }
+#pragma unroll
+        for (int c = 0; c < CN; ++c)
+            *reinterpret_cast<float4*>(Ow + (w * SR + r) * D + c * 32 + kg * 4) =
+                make_float4(o[i][c * 4], o[i][c * 4 + 1], o[i][c * 4 + 2], o[i][c * 4 + 3]);
+    }
+    // (raw Q for the other branch takes the place of the rotated rows, S that of the last V tile)
+    for (int idx = tid; idx < SR * (D / 4); idx += NT) {
+        const int r = idx / (D / 4), c4 = idx % (D / 4);
+        *reinterpret_cast<float4*>(Qs + r * LD + c4 * 4) =
+            i0 + r < L ? load4(q + (((size_t)b * L + i0 + r) * H + h) * D + c4 * 4) : zero4;
+    }
+    const float* Sh = a.state + ((size_t)b * H + h) * D * D;
+#pragma unroll 4
+    for (int idx = tid; idx < D * D / 4; idx += NT)
+        *reinterpret_cast<float4*>(Vs + idx * 4) = *reinterpret_cast<const float4*>(Sh + idx * 4);
+    __syncthreads();
+    // from here: thread = row r, columns 64 c + 4 t16 ..; the 16 threads of a row sit in one half warp
+    const int r = tid >> 4, t16 = tid & 15, row = i0 + r;
+    float oi[D / 16];
+    {
+        float m_all = -INFINITY;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) m_all = fmaxf(m_all, Ms[x * SR + r]);
+        float l_all = 0.0f;
+#pragma unroll
+        for (int e = 0; e < D / 16; ++e) oi[e] = 0.0f;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            const float f = exp2f(Ms[x * SR + r] - m_all);
+            l_all = fmaf(f, Ls[x * SR + r], l_all);
+#pragma unroll
+            for (int c = 0; c < D / 64; ++c) {
+                const float4 ov = *reinterpret_cast<const float4*>(Ow + (x * SR + r) * D + c * 64 + t16 * 4);
+                oi[c * 4 + 0] = fmaf(f, ov.x, oi[c * 4 + 0]);
+                oi[c * 4 + 1] = fmaf(f, ov.y, oi[c * 4 + 1]);
+                oi[c * 4 + 2] = fmaf(f, ov.z, oi[c * 4 + 2]);
+                oi[c * 4 + 3] = fmaf(f, ov.w, oi[c * 4 + 3]);
+            }
+        }
+        const float inv = 1.0f / l_all;
+#pragma unroll
+        for (int e = 0; e < D / 16; ++e) oi[e] *= inv;
+    }
+    // y = (row r of Qs) M for this thread's columns; M row-major [D][D] in shared memory
+    auto row_times = [&](const float* M, float (&y)[D / 16]) {
+#pragma unroll
+        for (int e = 0; e < D / 16; ++e) y[e] = 0.0f;
+#pragma unroll 4
+        for (int d = 0; d < D; d += 4) {
+            const float4 x4 = *reinterpret_cast<const float4*>(Qs + r * LD + d);
+            const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+                for (int c = 0; c < D / 64; ++c) {
+                    const float4 m4 = *reinterpret_cast<const float4*>(M + (d + e) * D + c * 64 + t16 * 4);
+                    y[c * 4 + 0] = fmaf(xv[e], m4.x, y[c * 4 + 0]);
+                    y[c * 4 + 1] = fmaf(xv[e], m4.y, y[c * 4 + 1]);
+                    y[c * 4 + 2] = fmaf(xv[e], m4.z, y[c * 4 + 2]);
+                    y[c * 4 + 3] = fmaf(xv[e], m4.w, y[c * 4 + 3]);
+                }
+        }
+    };
+    // ---- inter branch: Q' = L2Norm(RoPE(Q W_phi_q)), then Q' S
+    float u[D / 16];
+    if (a.wq != nullptr) {
+        __syncthreads();               // the warps' O has been read
+        const T* W = static_cast<const T*>(a.wq) + (size_t)h * D * D;
+#pragma unroll 4
+        for (int idx = tid; idx < D * D / 4; idx += NT) *reinterpret_cast<float4*>(Ks + idx * 4) = load4(W + idx * 4);
+        __syncthreads();
+        row_times(Ks, u);
+    } else {
+#pragma unroll
+        for (int c = 0; c < D / 64; ++c) {
+            const float4 x4 = *reinterpret_cast<const float4*>(Qs + r * LD + c * 64 + t16 * 4);
+            u[c * 4 + 0] = x4.x; u[c * 4 + 1] = x4.y; u[c * 4 + 2] = x4.z; u[c * 4 + 3] = x4.w;
+        }
+    }
+    float ss = 0.0f;
+#pragma unroll
+    for (int c = 0; c < D / 64; ++c) {
+        if (a.rope_cos != nullptr && row < L) {
+            const size_t at = (size_t)row * (D / 2) + c * 32 + t16 * 2;
+            const float2 cs = *reinterpret_cast<const float2*>(a.rope_cos + at);
+            const float2 sn = *reinterpret_cast<const float2*>(a.rope_sin + at);
+            const float x0 = u[c * 4], x1 = u[c * 4 + 1], x2 = u[c * 4 + 2], x3 = u[c * 4 + 3];
+            u[c * 4 + 0] = x0 * cs.x - x1 * sn.x;
+            u[c * 4 + 1] = x0 * sn.x + x1 * cs.x;
+            u[c * 4 + 2] = x2 * cs.y - x3 * sn.y;
+            u[c * 4 + 3] = x2 * sn.y + x3 * cs.y;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) ss = fmaf(u[c * 4 + e], u[c * 4 + e], ss);
+    }
+#pragma unroll
+    for (int off = 8; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+    const float rn = 1.0f / sqrtf(ss + a.s.eps);
+    __syncwarp();                      // the half warp has read its row of Qs
+#pragma unroll
+    for (int c = 0; c < D / 64; ++c)
+        *reinterpret_cast<float4*>(Qs + r * LD + c * 64 + t16 * 4) =
+            make_float4(u[c * 4] * rn, u[c * 4 + 1] * rn, u[c * 4 + 2] * rn, u[c * 4 + 3] * rn);
+    __syncwarp();
+    row_times(Vs, u);
+    if (row >= L) return;
+    const size_t rh = ((size_t)b * L + row) * H + h;
+    float gate = a.gate_mode == 2 ? 0.0f : sigmoidf_(a.gate[a.gate_mode == 1 ? (size_t)b * L + row : rh]);
+    T* out = static_cast<T*>(a.out) + rh * D;
+#pragma unroll
+    for (int c = 0; c < D / 64; ++c)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int col = c * 64 + t16 * 4 + e;
+            if (a.gate_mode == 2) gate = sigmoidf_(a.gate[rh * D + col]);
+            from_f(out[col], oi[c * 4 + e] + gate * u[c * 4 + e]);
+        }
+}
+
 // partial[b, h, split] = K'^T V' over tokens [split*chunk, min(L, (split+1)*chunk)).
 template <int D, typename T>
 __global__ void __launch_bounds__(NT) simt_commit_partial_kernel(CommitArgs a)
@@ -851,6 +1147,13 @@ int check_launch(const char* what)
 template <int D, typename T>
 int launch_step(const StepArgs& a, cudaStream_t st)
 {
+    if (a.k_raw) {
+        constexpr size_t small_smem = sizeof(float) * SmallCfg<D>::kFloats;
+        if (int r = set_smem(simt_step_small_kernel<D, T>, small_smem)) return r;
+        simt_step_small_kernel<D, T><<<dim3((a.s.L + SR - 1) / SR, a.s.H, a.s.B), NT, small_smem, st>>>(a);
+        if (int r = check_launch("simt_step_small_kernel")) return r;
+        return 1;
+    }
     size_t smem = sizeof(float) * (2 * D * (BM + PAD) + BN * D + BM * (BM + PAD));
     if (int r = set_smem(simt_step_kernel<D, T>, smem)) return r;
     dim3 grid((a.s.L + BM - 1) / BM, a.s.H, a.s.B);
@@ -1013,6 +1316,17 @@ int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, co
             s.L, s.H, s.D, total8);
     if (int r = check_launch("rope_k_kernel")) return r;
     return 1;
+}
+
+// 16-row tiles with the keys split over the warps: always for D = 128 (fp32, 12 heads: 777 tokens 489 -> 304 us,
+// 1560 tokens 1571 -> 1251, 4680 tokens x 2 streams 20.8 -> 16.0 ms -- the 64-row kernel's transposing stores
+// meet in the same banks); for D = 64 while 64-row tiles leave SMs idle (8 tiles: 48.6 -> 15.5 us per pass
+// including the launch that the rotation of K took, 52: 115 -> 71, 156: 151 -> 140; at 192 tiles 184 -> 223, at
+// 300 462 -> 501: one CTA per SM).  The maps are read in 16-byte pieces.
+bool simt_step_rotates_k(const Shape& s, const void* wq)
+{
+    const long tiles = (long)((s.L + BM - 1) / BM) * s.H * s.B;
+    return (s.D == 128 || tiles <= 156) && reinterpret_cast<uintptr_t>(wq) % 16 == 0;
 }
 
 int simt_step(const StepArgs& a, int dtype, cudaStream_t st)

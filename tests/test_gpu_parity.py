@@ -265,3 +265,34 @@ def test_key_range_split_bf16(oracle, B, H, L):
     pair.layer.sync_status()
     assert torch.equal(outs[0].view(torch.int16), outs[1].view(torch.int16))
     assert torch.equal(outs[0].view(torch.int16), outs[2].view(torch.int16))
+
+
+@pytest.mark.parametrize("dtype,D,B,H,L", [
+    ("fp32", 64, 1, 2, 15), ("fp32", 64, 1, 2, 17),      # one row tile and a remainder
+    ("fp32", 64, 2, 1, 255), ("fp32", 64, 1, 2, 257),    # a key tile of 256, and one key more
+    ("fp32", 128, 1, 2, 16), ("fp32", 128, 1, 3, 129),   # a key tile of 128, and one key more
+    ("fp32", 64, 1, 39, 256), ("fp32", 64, 1, 40, 256),  # both sides of the choice of kernel (156, 160 tiles)
+    ("bf16", 64, 1, 2, 300),
+])
+@pytest.mark.parametrize("rope", [True, False])
+def test_plain_fma_step_over_its_tiles(oracle, dtype, D, B, H, L, rope):
+    cfg = workload.custom(B=B, H=H, D=D, L=L, dtype=dtype, cfg_id=71)
+    pair = Pair(oracle, cfg, rope=rope)
+    kc, vc, a = workload.commit_inputs(cfg, 0)
+    assert pair.commit(kc, vc, a) <= pair.tol
+    q, k, v, g = workload.step_inputs(cfg, 1, 0)
+    assert pair.step_full(q, k, v, g) <= pair.tol
+    assert pair.step_full(q, k, v, torch.full_like(g, -40.0)) <= pair.tol
+
+
+def test_plain_fma_step_with_a_map_that_is_not_16_byte_aligned(oracle):
+    cfg = workload.custom(B=1, H=2, D=128, L=100, dtype="fp32", cfg_id=72)
+    pair = Pair(oracle, cfg)
+    kc, vc, a = workload.commit_inputs(cfg, 0)
+    assert pair.commit(kc, vc, a) <= pair.tol
+    odd = torch.empty(pair.wq.numel() + 1, device=pair.dev)[1:].view(pair.wq.shape)
+    odd.copy_(pair.wq)
+    assert odd.data_ptr() % 16 == 4
+    pair.layer.set_params(odd, pair.wk.to(pair.dev), pair.wv.to(pair.dev), pair.cos.to(pair.dev), pair.sin.to(pair.dev))
+    q, k, v, g = workload.step_inputs(cfg, 1, 0)
+    assert pair.step_full(q, k, v, g) <= pair.tol
