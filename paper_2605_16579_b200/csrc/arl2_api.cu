@@ -322,6 +322,7 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
     StepArgs a;
     a.s = ctx->shape;
     a.q = d_q; a.k_rot = k_rot; a.v = d_v; a.gate = d_gate_logits;
+    a.k_made_before = k_rot == ctx->ws + ctx->lay.k_rot;   // by rotate_k, or by the commit kernel of a clean pass
     a.gate_mode = (ctx->cfg.flags & ARL2_FLAG_GATE_ELEMENTWISE) ? 2 : (ctx->cfg.flags & ARL2_FLAG_GATE_SCALAR) ? 1 : 0;
     a.state = ctx->state; a.wq = ctx->wq;
     a.rope_cos = ctx->rope_cos; a.rope_sin = ctx->rope_sin;

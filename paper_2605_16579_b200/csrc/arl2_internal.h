@@ -46,6 +46,7 @@ struct StepArgs {
     int launch_parity;      // step launches so far on this context, mod 2 (scheduler counters)
     const void* rope_h;     // [L, D/2] half2 (cos, sin) copy of the tables (tensor-core path), or nullptr
     int Lk = 0;             // > 0: K and V hold Lk tokens (a cache), [B, Lk, H, D]; 0: L
+    bool k_made_before = false;   // the launch just before on the stream wrote k_rot and nothing else this step reads
     bool k_raw = false;     // plain-FMA path: k_rot is the caller's K, rotated by the step kernel itself
     int gate_mode = 0;      // 0: gate [B, L, H]; 1: [B, L]; 2: [B, L, H, D]
     uint32_t wait_limit = 0;  // 0: default; n > 0: bounded waits give up after n - 1 polls (test hook)
