@@ -111,7 +111,8 @@ int arl2_create(const arl2_config* cfg, void* d_state, void* d_workspace,
 /*
  * Feature maps phi_q, phi_k, phi_v (Eq. 3: per-head grouped 1x1 maps, read here as
  * bias-free linear maps applied as row-vector times matrix) and the rotary tables.
- *   d_wphi_*   [H, D, D] indexed [head][in][out], io_dtype; NULL = identity map.
+ *   d_wphi_*   [H, D, D] indexed [head][in][out], io_dtype, at any element-aligned address (16-byte
+ *              aligned maps are read faster); NULL = identity map.
  *   d_rope_cos, d_rope_sin  [L, D/2] fp32: cos / sin of the angle of pair (2m, 2m+1) at
  *              token l; both NULL = no rotation.  The same tables serve Q and K and both
  *              branches.

@@ -444,9 +444,15 @@ constexpr int fin_smem_bytes(int mode) { return (mode == 1 ? 2 : 1) * (kFinMatBy
 
 // a [128][128] bf16 matrix from global memory into padded rows of shared memory, as asynchronous
 // 16-byte copies (no registers, and the thread goes on to request its other loads at once);
-// fin_matrices_landed() before the matrix is read
+// fin_matrices_landed() before the matrix is read.  The value map is the caller's own array, which need
+// not start on a 16-byte boundary: element by element then.
 __device__ __forceinline__ void fin_load_matrix(__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, int tid)
 {
+    if ((reinterpret_cast<uintptr_t>(src) & 15) != 0) {
+#pragma unroll 8
+        for (int c = tid; c < kTile * kTile; c += kFinThreads) dst[(c >> 7) * kFinLdM + (c & 127)] = src[c];
+        return;
+    }
     constexpr int kPer = kTile * kTile / 8 / kFinThreads;   // 16-byte pieces per thread
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {

@@ -111,3 +111,28 @@ def test_token_level_over_runs_that_cross_heads(oracle, B, H, L, gates):
     assert err <= pair.tol, f"{err:.3e} > {pair.tol}"
     assert pair.layer.get_state().numpy().tobytes() == before
     pair.layer.sync_status()
+
+
+@pytest.mark.parametrize("H,L", [(2, 300), (2, 1030)])   # heads walked whole; heads cut into runs
+def test_tensor_core_calls_with_maps_that_are_not_16_byte_aligned(oracle, H, L):
+    cfg = workload.custom(B=1, H=H, D=128, L=L, dtype="bf16", cfg_id=64)
+    pair = Pair(oracle, cfg)
+    odd = []
+    for w in (pair.wq, pair.wk, pair.wv):
+        t = torch.empty(w.numel() + 1, dtype=torch.bfloat16, device=pair.dev)[1:].view(w.shape)
+        t.copy_(w)
+        assert t.data_ptr() % 16 == 2
+        odd.append(t)
+    pair.layer.set_params(*odd, pair.cos.to(pair.dev), pair.sin.to(pair.dev))
+    kc, vc, a = workload.commit_inputs(cfg, 0)
+    assert pair.commit(kc, vc, a) <= pair.tol
+    kc, vc, a = workload.commit_inputs(cfg, 1)
+    assert pair.commit_delta(kc, vc, a, workload.beta_logits(cfg, 1)) <= pair.tol
+    kc, vc, _ = workload.commit_inputs(cfg, 2)
+    assert pair.commit_decay_tokens(kc, vc, workload.token_gate_logits(cfg, 2)[0]) <= pair.tol
+    q, k, v, g = workload.step_inputs(cfg, 3, 0)
+    alpha = workload.token_gate_logits(cfg, 3)[0]
+    got = run(pair, q, k, v, g, alpha)
+    ref = oracle.step_token_level(q, k, v, g, pair.S_ref, alpha, pair.wq, pair.wk, pair.wv, pair.cos, pair.sin)
+    assert float(head_errors(got, ref).max()) <= pair.tol
+    pair.layer.sync_status()
