@@ -230,6 +230,7 @@ int arl2_commit_decay_tokens(arl2_ctx* ctx, const void* d_k_clean, const void* d
  * pass over the chunks); bitwise reproducible.  With fp32 I/O, or D = 64, the arithmetic is fp32
  * throughout; with bf16 I/O and D = 128 the chunk factors are bf16 tensor-core operands with fp32
  * accumulation, the state itself staying fp32.
+ * After a wait that expired (arl2_sync_status) S is what it was before the call, in every head.
  * d_alpha_logits, d_beta_logits: [B, L, H] fp32, each may be NULL (gate = 1).  The context must
  * have been created with ARL2_FLAG_TOKEN_GATES (else ARL2_ERR_WORKSPACE).  K', V' as in
  * arl2_commit; calls of the three commit entry points may be mixed on one context.
@@ -285,6 +286,9 @@ int arl2_sync_status(arl2_ctx* ctx, void* stream);
  * follows it sees the recorded error and does nothing).
  */
 int arl2_debug_set_wait_limit(arl2_ctx* ctx, int32_t polls);
+/* The same for one wait only: the first one of the last thread block of arl2_commit_tokens' ordered walk
+   (tensor-core contexts), which expires after the kernel before it, and other thread blocks, have done their work. */
+int arl2_debug_set_walk_wait_limit(arl2_ctx* ctx, int32_t polls);
 
 /*
  * Measurement hook (no counterpart in the paper).  `ev_before` / `ev_after` are

@@ -30,7 +30,7 @@ EXPORTS = (
     "arl2_workspace_bytes", "arl2_create", "arl2_set_params", "arl2_denoise_step", "arl2_commit",
     "arl2_reset", "arl2_get_state", "arl2_set_state", "arl2_sync_status", "arl2_launch_count",
     "arl2_set_profile_events", "arl2_commit_static_scratch", "arl2_commit_delta", "arl2_commit_tokens", "arl2_teacher_step", "arl2_commit_decay_tokens",
-    "arl2_step_kernel_name", "arl2_destroy", "arl2_last_error", "arl2_version", "arl2_debug_set_wait_limit", "arl2_clean_pass", "arl2_denoise_step_token_level",
+    "arl2_step_kernel_name", "arl2_destroy", "arl2_last_error", "arl2_version", "arl2_debug_set_wait_limit", "arl2_debug_set_walk_wait_limit", "arl2_clean_pass", "arl2_denoise_step_token_level",
     "arl2_projection_workspace_bytes", "arl2_set_projections", "arl2_project_in", "arl2_project_out",
 )
 
@@ -108,6 +108,8 @@ def load(build_if_missing: bool = False) -> ctypes.CDLL:
     lib.arl2_sync_status.argtypes = [vp, vp]
     lib.arl2_debug_set_wait_limit.restype = ctypes.c_int
     lib.arl2_debug_set_wait_limit.argtypes = [vp, ctypes.c_int32]
+    lib.arl2_debug_set_walk_wait_limit.restype = ctypes.c_int
+    lib.arl2_debug_set_walk_wait_limit.argtypes = [vp, ctypes.c_int32]
     lib.arl2_set_profile_events.restype = ctypes.c_int
     lib.arl2_set_profile_events.argtypes = [vp, vp, vp]
     lib.arl2_commit_static_scratch.restype = ctypes.c_int
@@ -382,6 +384,10 @@ class Layer:
     def debug_set_wait_limit(self, polls: int):
         """Test hook: bounded waits in the tensor-core kernels give up after ``polls`` polls (< 0: default)."""
         _check(load().arl2_debug_set_wait_limit(self._ctx, polls), "arl2_debug_set_wait_limit")
+
+    def debug_set_walk_wait_limit(self, polls: int):
+        """Test hook: the same for the first wait of the last thread block of ``commit_tokens``' walk alone."""
+        _check(load().arl2_debug_set_walk_wait_limit(self._ctx, polls), "arl2_debug_set_walk_wait_limit")
 
     def set_profile_events(self, before: "torch.cuda.Event", after: "torch.cuda.Event"):
         """The next denoise_step records these events around its dominant kernel."""

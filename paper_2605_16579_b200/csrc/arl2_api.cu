@@ -144,6 +144,7 @@ struct arl2_ctx {
     int mirror;            // which of the two bf16 copies of S is current
     cudaEvent_t ev_before, ev_after;  // one-shot timing hook around the step kernel
     uint32_t wait_limit;   // 0: the kernels' default bound; n: waits give up after n - 1 polls (test hook)
+    uint32_t walk_limit;   // the same for the first wait of the last thread block of arl2_commit_tokens' walk
     // projections around the core (arl2_set_projections)
     const void* w_pack;    // [d, 3 d + gate pad] bf16: W_q | W_k | W_v | W_g (zero padded)
     const void* w_o;       // [d, d] bf16
@@ -234,6 +235,7 @@ int arl2_create(const arl2_config* cfg, void* d_state, void* d_workspace, size_t
     ctx->w_pack = ctx->w_o = nullptr;
     ctx->pack_cols = 0;
     ctx->wait_limit = cfg->flags >> ARL2_FLAG_DEBUG_WAIT_LIMIT_SHIFT;
+    ctx->walk_limit = 0;
     ctx->ev_before = ctx->ev_after = nullptr;
     int r = account(ctx, fill_zero(ctx->ws + lay.status, kStatusWords * sizeof(uint32_t),
                                    as_stream(stream)));
@@ -532,6 +534,17 @@ int arl2_debug_set_wait_limit(arl2_ctx* ctx, int32_t polls)
     return ARL2_OK;
 }
 
+int arl2_debug_set_walk_wait_limit(arl2_ctx* ctx, int32_t polls)
+{
+    if (!check_ctx(ctx)) return ARL2_ERR_INVALID_ARG;
+    if (polls > 65534) {
+        set_error("debug_set_walk_wait_limit: polls must be <= 65534, or negative for the default (got %d)", polls);
+        return ARL2_ERR_INVALID_ARG;
+    }
+    ctx->walk_limit = polls < 0 ? 0u : (uint32_t)polls + 1u;
+    return ARL2_OK;
+}
+
 int arl2_set_profile_events(arl2_ctx* ctx, void* ev_before, void* ev_after)
 {
     if (!check_ctx(ctx)) return ARL2_ERR_INVALID_ARG;
@@ -628,9 +641,11 @@ int arl2_commit_tokens(arl2_ctx* ctx, const void* d_k_clean, const void* d_v_cle
     a.u1 = reinterpret_cast<float*>(ctx->ws + ctx->lay.tok_u1);
     a.kh = reinterpret_cast<float*>(ctx->ws + ctx->lay.tok_kh);
     a.gc = reinterpret_cast<float*>(ctx->ws + ctx->lay.tok_gc);
+    a.next = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials);   // a [D, D] slot per head and more, not in use here
     a.nchunk = ctx->lay.nchunk;
     a.decayed = (ctx->cfg.flags & ARL2_FLAG_DELTA_DECAYED_PREDICTION) != 0;
     a.wait_limit = ctx->wait_limit;
+    a.walk_limit = ctx->walk_limit;
     if ((reinterpret_cast<uintptr_t>(d_k_clean) | reinterpret_cast<uintptr_t>(d_v_clean)) % 16 != 0) {
         set_error("commit_tokens: k_clean and v_clean must be 16-byte aligned");
         return ARL2_ERR_INVALID_ARG;

@@ -106,9 +106,11 @@ struct TokenCommitArgs {
     float* u1;              // same shape
     float* kh;              // same shape
     float* gc;              // [B, H, nchunk] decay of a whole chunk
+    float* next;            // [B, H, D, D] fp32 scratch: the walk's result before it is published (tensor-core path)
     int nchunk;             // ceil(L / 64)
     bool decayed = false;   // each token predicts against alpha_j S_{j-1} instead of S_{j-1}
     uint32_t wait_limit = 0;   // as in StepArgs
+    uint32_t walk_limit = 0;   // the same for the first wait of the walk's last thread block alone
 };
 constexpr int kTokenChunk = 64;
 
@@ -158,7 +160,7 @@ int tc_token_readout(const StepArgs& a, const float* alpha_logits, const CommitA
                      const __nv_bfloat16* wk_op, const __nv_bfloat16* wv_op, cudaStream_t st);
 
 int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const __nv_bfloat16* wv_op,
-                     const void* rope_h, uint32_t* status, cudaStream_t st);   // prepare + ordered scan
+                     const void* rope_h, uint32_t* status, cudaStream_t st);   // prepare + ordered scan + publish
 
 // C[M, N] = A[M, K] B[K, N] on tensor cores (bf16 operands, row-major); the columns of C are routed to up to
 // four bf16 tensors of seg_cols columns each (row stride ld_out) and, after them, one fp32 tensor.

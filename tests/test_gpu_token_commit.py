@@ -120,7 +120,34 @@ def test_token_commit_over_the_cuts_of_the_walk(oracle, B, H, L):
         assert err <= pair.tol, f"block {blk}: error {err:.3e} > {pair.tol}"
 
 
+@pytest.mark.parametrize("B,H,L", [
+    (1, 3, 700),      # one slab per CTA
+    (1, 30, 200),     # two slabs per CTA
+    (5, 20, 130),     # two CTAs per SM and more CTAs than fit at once: the last one starts after others have finished
+])
+def test_token_commit_whose_walk_timed_out_leaves_the_whole_state(oracle, B, H, L):
+    cfg = workload.custom(B=B, H=H, D=128, L=L, dtype="bf16", cfg_id=49)
+    pair = Pair(oracle, cfg, flags=FLAG)
+    kc, vc, _ = workload.commit_inputs(cfg, 0)
+    alpha, beta = workload.token_gate_logits(cfg, 0)
+    assert pair.commit_tokens(kc, vc, alpha, beta) <= pair.tol
+    q, k, v, g = workload.step_inputs(cfg, 1, 0)
+    before, out = pair.layer.get_state().numpy(), pair.step_gpu(q, k, v, g)
+    d = pair.dev
+    pair.layer.debug_set_walk_wait_limit(0)
+    pair.layer.commit_tokens(kc.to(d), vc.to(d), alpha.to(d), beta.to(d))
+    with pytest.raises(arl2.Arl2Error, match="site 101"):
+        pair.layer.sync_status()
+    np.testing.assert_array_equal(pair.layer.get_state().numpy(), before)
+    np.testing.assert_array_equal(pair.step_gpu(q, k, v, g), out)     # nor has the operand copy of S moved on
+    pair.layer.debug_set_walk_wait_limit(-1)
+    kc, vc, _ = workload.commit_inputs(cfg, 1)
+    assert pair.commit_tokens(kc, vc, alpha, beta) <= pair.tol
+    pair.layer.sync_status()
+
+
 def test_token_commit_that_timed_out_leaves_the_state(oracle):
+    # every wait expires, those of the kernel that makes the chunk factors first: the walk does not begin
     cfg = workload.custom(B=1, H=3, D=128, L=700, dtype="bf16", cfg_id=48)
     pair = Pair(oracle, cfg, flags=FLAG)
     kc, vc, _ = workload.commit_inputs(cfg, 0)
