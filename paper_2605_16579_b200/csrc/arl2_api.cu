@@ -139,6 +139,7 @@ struct arl2_ctx {
     const void *wq, *wk, *wv;
     const float *rope_cos, *rope_sin;
     bool use_tc;
+    bool simt_16_rows;     // plain-FMA step: the 16-row kernel is the faster one for this shape on this device
     uint64_t launches;
     uint32_t step_calls;   // parity selects the scheduler counter of the next step launch
     int mirror;            // which of the two bf16 copies of S is current
@@ -166,6 +167,12 @@ __nv_bfloat16* mirror_of(const arl2_ctx* ctx, int which = 0)
 {
     const size_t off = ((ctx->mirror ^ which) & 1) ? ctx->lay.state_bf16_b : ctx->lay.state_bf16;
     return reinterpret_cast<__nv_bfloat16*>(ctx->ws + off);
+}
+
+// whether the plain-FMA step of this context runs on the 16-row kernel, which rotates K itself
+bool step_rotates_k(const arl2_ctx* ctx)
+{
+    return !ctx->use_tc && ctx->simt_16_rows && reinterpret_cast<uintptr_t>(ctx->wq) % 16 == 0;
 }
 
 // adds the launches of a helper to the context's counter; passes errors through
@@ -229,6 +236,18 @@ int arl2_create(const arl2_config* cfg, void* d_state, void* d_workspace, size_t
     ctx->wq = ctx->wk = ctx->wv = nullptr;
     ctx->rope_cos = ctx->rope_sin = nullptr;
     ctx->use_tc = tc_supported(*cfg);
+    ctx->simt_16_rows = false;
+    if (!ctx->use_tc) {
+        int dev = 0, num_sms = 0;
+        e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess || num_sms < 1) {
+            set_error("cannot read the device's SM count: %s", cudaGetErrorString(e));
+            delete ctx;
+            return ARL2_ERR_CUDA;
+        }
+        ctx->simt_16_rows = simt_step_prefers_16_rows(ctx->shape, cfg->io_dtype, num_sms);
+    }
     ctx->launches = 0;
     ctx->step_calls = 0;
     ctx->mirror = 0;
@@ -345,7 +364,7 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
         // really went out moves on to the other one
         if (r == ARL2_OK) ++ctx->step_calls;
     } else {
-        a.k_raw = simt_step_rotates_k(ctx->shape, ctx->wq);
+        a.k_raw = step_rotates_k(ctx);
         r = account(ctx, simt_step(a, ctx->cfg.io_dtype, st));
     }
     if (e1 != nullptr) cudaEventRecord(e1, st);
@@ -356,7 +375,7 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
 int rotate_k(arl2_ctx* ctx, const void* d_k, const void** k_rot, cudaStream_t st)
 {
     *k_rot = d_k;
-    if (ctx->rope_cos == nullptr || (!ctx->use_tc && simt_step_rotates_k(ctx->shape, ctx->wq))) return ARL2_OK;
+    if (ctx->rope_cos == nullptr || step_rotates_k(ctx)) return ARL2_OK;
     void* buf = ctx->ws + ctx->lay.k_rot;
     int r = ctx->use_tc
                 ? account(ctx, tc_rope_k(ctx->shape, d_k, ctx->ws + ctx->lay.rope_h, buf, st))

@@ -47,7 +47,7 @@ struct StepArgs {
     const void* rope_h;     // [L, D/2] half2 (cos, sin) copy of the tables (tensor-core path), or nullptr
     int Lk = 0;             // > 0: K and V hold Lk tokens (a cache), [B, Lk, H, D]; 0: L
     bool k_made_before = false;   // the launch just before on the stream wrote k_rot and nothing else this step reads
-    bool k_raw = false;     // plain-FMA path: k_rot is the caller's K, rotated by the step kernel itself
+    bool k_raw = false;     // plain-FMA path: the 16-row kernel; k_rot is the caller's K, which it rotates itself
     int gate_mode = 0;      // 0: gate [B, L, H]; 1: [B, L]; 2: [B, L, H, D]
     uint32_t wait_limit = 0;  // 0: default; n > 0: bounded waits give up after n - 1 polls (test hook)
     // key-range split of the last wave of work items (tensor-core path), or nullptr: never split
@@ -118,8 +118,9 @@ constexpr int kTokenChunk = 64;
 // Each returns the number of kernels it launched (>= 0) or a negative arl2_status.
 int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, const float* sin_t,
                 void* k_rot, cudaStream_t st);
-// whether the step kernel that serves this shape rotates K itself (then StepArgs::k_raw must be set)
-bool simt_step_rotates_k(const Shape& s, const void* wq);
+// whether the 16-row step kernel is the faster one for this shape on a device of num_sms SMs.  It rotates K itself
+// (StepArgs::k_raw) and reads W_phi_q in 16-byte pieces.
+bool simt_step_prefers_16_rows(const Shape& s, int dtype, int num_sms);
 int simt_step(const StepArgs& a, int dtype, cudaStream_t st);
 int simt_commit(const CommitArgs& a, int dtype, cudaStream_t st);
 int commit_reduce(const CommitArgs& a, cudaStream_t st);  // fixed-order sum + gated decay

@@ -330,8 +330,8 @@ __global__ void __launch_bounds__(NT) simt_step_kernel(StepArgs a)
     }
 }
 
-// The step for D = 128, and for shapes whose 64-row tiles would leave most SMs idle (a 16 x 16 latent frame: 8
-// tiles).  16 query rows per CTA, and the eight warps split the keys: a warp scores its share of each key tile
+// The step for shapes whose 64-row tiles would leave SMs idle (a 16 x 16 latent frame: 8 tiles) or fill a last
+// round badly (simt_step_prefers_16_rows).  16 query rows per CTA, and the eight warps split the keys: a warp scores its share of each key tile
 // against all rows, keeps its own running maximum, sum and O, and the eight partial results are merged at the end,
 // so that the loop over the keys has no CTA-wide exchange.  K is rotated while it is loaded (no separate launch).
 // Lane (rg, kg) holds a 4 x KJ block of scores, rows 4 i + rg, keys 8 j + kg: every shared-memory read of the
@@ -1318,15 +1318,38 @@ int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, co
     return 1;
 }
 
-// 16-row tiles with the keys split over the warps: always for D = 128 (fp32, 12 heads: 777 tokens 489 -> 304 us,
-// 1560 tokens 1571 -> 1251, 4680 tokens x 2 streams 20.8 -> 16.0 ms -- the 64-row kernel's transposing stores
-// meet in the same banks); for D = 64 while 64-row tiles leave SMs idle (8 tiles: 48.6 -> 15.5 us per pass
-// including the launch that the rotation of K took, 52: 115 -> 71, 156: 151 -> 140; at 192 tiles 184 -> 223, at
-// 300 462 -> 501: one CTA per SM).  The maps are read in 16-byte pieces.
-bool simt_step_rotates_k(const Shape& s, const void* wq)
+// Which of the two step kernels serves a shape: the one whose rounds of CTAs take less time on this device.
+// A 16-row CTA fills an SM; of the 64-row CTAs an SM holds one at D = 128, two (fp32) or three (bf16) at
+// D = 64.  So a shape that is one round of 64-row tiles can be four of 16-row tiles, and neither kernel is the
+// faster one over a whole range: with L = 777 and fp32, us per pass of the 16-row / 64-row kernel (its
+// rotation of K included) at 1, 6, 9, 11, 12, 20 and 24 heads
+//   D = 128:  72 / 236, 144 / 237, 214 / 238, 282 / 238, 285 / 460, 490 / 484, 565 / 700
+//   D = 64:   37 / 114,  72 / 117, 107 / 117, 140 / 117, 141 / 150, 242 / 155, 277 / 254
+// The model (us: once per call, then per round a fixed part and a part per key tile; the time of 1, 2, 3 64-row
+// CTAs on an SM relative to one) was fitted to 130 shapes of 48 to 4614 tokens with 1 to 192 heads.  There it
+// picks the slower kernel nowhere by more than 8 %, in the mean by 0.2 % (always the 64-row kernel: 53 %; the 16-row
+// kernel at D = 128 and up to 156 tiles at D = 64: 3 %, 47 % at most).  At even times the 64-row kernel is taken.
+bool simt_step_prefers_16_rows(const Shape& s, int dtype, int num_sms)
 {
-    const long tiles = (long)((s.L + BM - 1) / BM) * s.H * s.B;
-    return (s.D == 128 || tiles <= 156) && reinterpret_cast<uintptr_t>(wq) % 16 == 0;
+    struct Model {
+        float call16, fixed16, tile16;
+        float call64, fixed64, tile64;
+        int together;            // 64-row CTAs per SM
+        float time_of[3];
+    };
+    static constexpr Model kModel[2][2] = {
+        {{1.6f, 2.0f, 10.9f, 5.1f, 17.2f, 9.8f, 3, {1.0f, 1.21f, 1.48f}}, {3.0f, 9.6f, 12.0f, 5.0f, 28.1f, 16.1f, 1, {1.0f}}},   // bf16
+        {{1.9f, 4.0f, 7.9f, 4.7f, 16.3f, 7.25f, 2, {1.0f, 1.34f}}, {1.7f, 13.1f, 8.44f, 0.0f, 31.8f, 16.2f, 1, {1.0f}}}};        // fp32
+    const Model& m = kModel[dtype == ARL2_FP32][s.D == 128];
+    const long units = (long)s.H * s.B;
+    const long rounds16 = ((s.L + SR - 1) / SR * units + num_sms - 1) / num_sms;
+    const long per_sm64 = ((s.L + BM - 1) / BM * units + num_sms - 1) / num_sms;
+    const int keys16 = s.D == 64 ? SmallCfg<64>::KT : SmallCfg<128>::KT;
+    const float t16 = m.call16 + rounds16 * (m.fixed16 + m.tile16 * ((s.L + keys16 - 1) / keys16));
+    const long rest = per_sm64 % m.together;
+    const float t64 = m.call64 + (per_sm64 / m.together * m.time_of[m.together - 1] + (rest ? m.time_of[rest - 1] : 0.0f)) *
+                                     (m.fixed64 + m.tile64 * ((s.L + BN - 1) / BN));
+    return t16 < 0.98f * t64;
 }
 
 int simt_step(const StepArgs& a, int dtype, cudaStream_t st)

@@ -39,6 +39,7 @@ def _run(oracle, cfg, gate_mode, flags):
     ("bf16", 128, 2, 3, 333),      # tensor-core kernels, ragged tiles packed across units
     ("bf16", 128, 1, 2, 640),
     ("bf16", 64, 1, 2, 130),       # plain-FMA kernels with bf16 I/O
+    ("fp32", 64, 2, 28, 256),      # the 64-row plain-FMA kernel
 ])
 @pytest.mark.parametrize("gate_mode", [1, 2])
 def test_gate_granularities_match_oracle(oracle, gate_mode, dtype, D, B, H, L):

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2605_16579_b200 import workload
+from paper_2605_16579_b200 import arl2, workload
 from parity_util import Pair, head_errors
 
 pytestmark = pytest.mark.gpu
@@ -271,7 +271,7 @@ def test_key_range_split_bf16(oracle, B, H, L):
     ("fp32", 64, 1, 2, 15), ("fp32", 64, 1, 2, 17),      # one row tile and a remainder
     ("fp32", 64, 2, 1, 255), ("fp32", 64, 1, 2, 257),    # a key tile of 256, and one key more
     ("fp32", 128, 1, 2, 16), ("fp32", 128, 1, 3, 129),   # a key tile of 128, and one key more
-    ("fp32", 64, 1, 39, 256), ("fp32", 64, 1, 40, 256),  # both sides of the choice of kernel (156, 160 tiles)
+    ("fp32", 64, 1, 39, 256), ("fp32", 64, 1, 40, 256),  # just past one round of 64-row tiles
     ("bf16", 64, 1, 2, 300),
 ])
 @pytest.mark.parametrize("rope", [True, False])
@@ -296,3 +296,25 @@ def test_plain_fma_step_with_a_map_that_is_not_16_byte_aligned(oracle):
     pair.layer.set_params(odd, pair.wk.to(pair.dev), pair.wv.to(pair.dev), pair.cos.to(pair.dev), pair.sin.to(pair.dev))
     q, k, v, g = workload.step_inputs(cfg, 1, 0)
     assert pair.step_full(q, k, v, g) <= pair.tol
+
+
+@pytest.mark.parametrize("dtype,D,H,L,rows", [
+    # both sides of the choice on 148 SMs: by rounds (three or four of 16-row tiles against one of 64-row tiles; one
+    # 64-row tile more than an SM each), at both head dimensions, and where several 64-row CTAs share an SM
+    ("fp32", 128, 24, 256, 16), ("fp32", 128, 30, 256, 64), ("fp32", 128, 38, 256, 16),
+    ("fp32", 64, 24, 256, 16), ("fp32", 64, 56, 256, 64),
+    ("bf16", 64, 24, 256, 16), ("bf16", 64, 56, 256, 64),
+    ("bf16", 128, 4, 300, 16), ("bf16", 128, 30, 256, 64),      # (forced onto the plain-FMA kernels)
+])
+def test_plain_fma_step_is_chosen_by_rounds(oracle, dtype, D, H, L, rows):
+    cfg = workload.custom(B=1, H=H, D=D, L=L, dtype=dtype, cfg_id=73)
+    pair = Pair(oracle, cfg, flags=arl2.ARL2_FLAG_FORCE_SIMT)
+    kc, vc, a = workload.commit_inputs(cfg, 0)
+    assert pair.commit(kc, vc, a) <= pair.tol
+    q, k, v, g = workload.step_inputs(cfg, 1, 0)
+    before = pair.layer.launch_count
+    assert pair.step_full(q, k, v, g) <= pair.tol
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        # the 64-row kernel has K rotated by a launch of its own
+        assert pair.layer.launch_count - before == (1 if rows == 16 else 2)
+    assert pair.step_full(q, k, v, torch.full_like(g, -40.0)) <= pair.tol
