@@ -1742,14 +1742,17 @@ int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* 
     // The last wave: `rem` items on num_sms SMs.  Cut into k key ranges, the wave takes
     // ceil(rem k / SMs) rounds of one part each; a part costs its share of the key iterations plus
     // what every item costs (the readout iteration, the hand-over between items) plus the exchange
-    // of the partial rows -- measured: 3.7 k clk per iteration, 10.8 k per item, about 6 k for the
+    // of the partial rows -- measured: 3.3 k clk per iteration, 10.8 k per item, about 6 k for the
     // exchange.  Take the k that makes the wave shortest, if that is shorter than leaving it whole.
+    // (At 3.7 k, what an iteration took before the issuers took turns, 26 to 28 key tiles were still cut in three
+    // where a third costs more than it saves: 6 heads x 3300 tokens 68 us, whole 62; 29 x 3456 218, 204;
+    // 17 x 3584 139, 125.)
     p.n_whole = p.n_items;
     p.k_split = 1;
     if (!elem_gate && a.split_o != nullptr) {
         const int waves = (p.n_items + num_sms - 1) / num_sms;
         const int rem = p.n_items - (waves - 1) * num_sms;
-        const float iter = 3.74f, fixed = 10.8f, exchange = 6.0f;
+        const float iter = 3.31f, fixed = 10.8f, exchange = 6.0f;
         float best = (p.n_kv + 1) * iter + fixed;
         for (int k = 2; k <= kMaxSplit; ++k) {
             if (p.n_kv < 4 * k || (long)rem * k * 2 > a.split_tile_parts) break;
