@@ -148,12 +148,13 @@ int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* 
 // partial sums on tensor cores (fills a.run_share / a.run_ntile for the finishing kernel) ...
 int tc_commit_partials(CommitArgs& a, const __nv_bfloat16* wk_op, cudaStream_t st);
 // ... then S <- alpha S + (sum of slots) W_phi_v [- (sum of G slots) S_old], mirror written to state_bf16_next
+int tc_commit_finish(const CommitArgs& a, cudaStream_t st);
 // tiles per run that tc_commit_partials cuts the flattened tile sequence into
 int tc_commit_run_share(const Shape& s, int nslot, int* share, int* ntile);
 // after tc_commit_partials: replaces the sums of segment i of every head by the state at the segment's start,
-//   S_0 = state, S_{i+1} = total_i S_i + (sums_i) W_phi_v   (total == nullptr: 1)
+//   S_0 = state, S_{i+1} = total_i S_i + (sums_i) W_phi_v   (total == nullptr: 1).  It does not look at the status
+// word: what it writes is scratch, read by a pass whose output is undefined after a time-out anyway.
 int tc_run_prefix(const CommitArgs& a, const float* total, cudaStream_t st);
-int tc_commit_finish(const CommitArgs& a, cudaStream_t st);
 
 // out += sigmoid(g) Q' S^(i): token-level state access (a.k_rot holds the RAW K here; a.out already holds the
 // softmax branch); alpha_logits [B, L, H] or nullptr; seg: after tc_commit_partials and tc_run_prefix

@@ -571,8 +571,9 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     tma_load_4d(dst, &tm_q, bar_q, 0, it.h[t], it.row0[t], it.b[t]);
                     tma_load_4d(dst + kHalfBytes, &tm_q, bar_q, 64, it.h[t], it.row0[t], it.b[t]);
                 }
-                // K comes from the kernel before this one (the rotation, or the commit of a clean pass): up to
-                // here everything ran beside its last CTAs
+                // K comes from the kernel before this one: up to here everything ran beside the end of the rotation,
+                // which lets this grid start early (the commit kernel of a clean pass does not: after it this
+                // grid starts when its last CTA has left, and only the launch itself is hidden)
                 if (item == 0) grid_dependency_wait();
                 const int entries = item_entries(it, nj);
                 for (int e = 0; e < entries && ok; ++e, ++n) {
@@ -617,10 +618,10 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         //
         // The serial chain of a tile -- S ready, softmax, P ready, P V and the next S -- sets the time of a
         // key iteration, so what an issuer adds to it counts.  (1) The whole warp walks the loop and one
-        // elected lane issues: with operands in uniform registers the 16 MMAs of an iteration are issued in
-        // 770 clk and run back to back (1275 clk from P ready to S ready); issued by a single live lane they
-        // took 1125 to 1385, more the busier the softmax warps were, because every operand of every MMA was
-        // first moved to a uniform register.  (2) The issuers take turns, 16 MMAs each: interleaved, both
+        // elected lane issues: the 16 MMAs of an iteration are then issued in 770 clk and run back to back (1275
+        // clk from P ready to S ready); issued by a single live lane they took 1125 to 1385, more the busier the
+        // softmax warps were (presumably because a warp in uniform control flow can keep descriptors and
+        // addresses in uniform registers; measured is the issue time only).  (2) The issuers take turns, 16 MMAs each: interleaved, both
         // tiles' MMAs end late and the two softmax groups fall into step (0.57 ms for L = 4680, 40 heads;
         // the turn the groups used to take in the exponential phase instead left the exponential unit idle
         // between them).  Key iteration 3790 -> 3310 clk; that shape 0.447 -> 0.423 ms per pass at full clocks,
@@ -817,8 +818,8 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 //   T as a bf16 operand (over A): 128 rows x 64, each chunk's block in its own rows
 //   W = T diag(beta g) K', then U1 = T diag(beta) V': one MMA per chunk over all 128 rows, each token row
 //   read from its own chunk's result -> global: W, U1 (and Khat on the way) in bf16, chunk decays g in fp32.
-// 12 heads x 4680 tokens (444 tiles): 74 us with one 128-thread CTA per SM, T by one 64-step substitution per column
-// and row-wise stores -> 42 us; 40 heads 205 -> 112.
+// 12 heads x 4680 tokens (444 tiles), inside the call: 66 us with one 128-thread CTA per SM, T by one 64-step
+// substitution per column and row-wise stores -> 42 us; 40 heads 205 -> 112 (each alone).
 // tc_token_scan_kernel: walks the chunks of a head in order (further down).
 // ---------------------------------------------------------------------------------------------
 constexpr int kTPOffK = 0;                         // raw K tile -> K' -> diag(beta g) K'
@@ -1279,9 +1280,9 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
 // The fp32 state stays in registers for the whole walk (16 per thread).  Per chunk a warp runs 16 + 16
 // instructions in four independent chains each and meets its group twice (named barriers, 128 threads);
 // the B fragments of the next chunk are fetched while this chunk's products run.  A fifth warp per CTA
-// streams the tiles through a TMA ring.  12 heads x 4680 tokens: 162 us with one CTA per head and the state in
-// TMEM (3.8 k clk per chunk: two MMAs, two passes through registers, four CTA-wide meetings) -> 32 us
-// (0.8 k clk; the 34 KB per chunk and SM that come from L2 are about 0.65 k of that).
+// streams the tiles through a TMA ring.  12 heads x 4680 tokens, inside the call: 162 us with one CTA per head and the
+// state in TMEM (two MMAs, two passes through registers, four CTA-wide meetings per chunk) -> 46 us (1.2 k clk per
+// chunk; the 34 KB per chunk and SM that come from L2 are about 0.65 k of that).
 constexpr int kChunkHalf = kTokC * 128;              // bytes of a 64-row, 64-column box
 constexpr int kScanLdS = kTile + 8, kScanLdU = kTokC + 8;   // padded rows: conflict-free 8 x 8 loads
 constexpr int kScanSlab = 16;
@@ -1766,10 +1767,11 @@ int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* 
     p.split_o = a.split_o;
     p.split_ml = a.split_ml;
     const int grid = p.n_sched < num_sms ? p.n_sched : num_sms;
-    // After a kernel of this library that made K, the launch overlaps that kernel's end: barriers, tensor memory,
-    // the first Q tiles and their rotation need nothing from it.  (After anything else -- K as the caller gave
-    // it -- the kernel before may be the one that makes Q, and the launch is an ordinary one.)
-    // 12 heads x 1560 tokens 44.1 -> 41.7 us per pass, 3 x 12 x 1001 38.8 -> 34.8, 2 heads x 300 22.5 -> 18.4.
+    // After the rotation of K the launch overlaps that kernel's end: barriers, tensor memory, the first Q tiles and
+    // their rotation need nothing from it.  (After the commit kernel of a clean pass, which does not release its
+    // dependents early, only the launch is hidden.  After anything else -- K as the caller gave it -- the kernel
+    // before may be the one that makes Q, and the launch is an ordinary one.)
+    // 12 heads x 1560 tokens 44.1 -> 42.5 us per pass, 3 x 12 x 1001 38.8 -> 34.9, 2 heads x 300 22.5 -> 18.4.
     cudaLaunchConfig_t scfg = {};
     scfg.gridDim = dim3((unsigned)grid);
     scfg.blockDim = dim3(kThreads);

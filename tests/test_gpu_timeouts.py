@@ -8,7 +8,7 @@ import pytest
 import torch
 
 from paper_2605_16579_b200 import arl2, workload
-from parity_util import Pair
+from parity_util import Pair, head_errors
 
 pytestmark = pytest.mark.gpu
 
@@ -50,6 +50,33 @@ def test_expired_wait_is_reported_and_the_context_recovers(oracle):
         assert pair.step_full(q, k, v, g) <= pair.tol
         kc, vc, a = workload.commit_inputs(cfg, blk)
         assert pair.commit(kc, vc, a) <= pair.tol
+    pair.layer.sync_status()
+
+
+def test_token_level_pass_through_runs_that_timed_out(oracle):
+    """Six launches whose waits all expire (attention, partial sums of the runs, readout): the time-out is
+    reported, S is untouched, and the next pass on the context matches the oracle."""
+    cfg = workload.custom(B=1, H=2, D=128, L=1030, dtype="bf16", cfg_id=84)
+    pair = Pair(oracle, cfg)
+    kc, vc, a = workload.commit_inputs(cfg, 0)
+    assert pair.commit(kc, vc, a) <= pair.tol
+    saved = pair.layer.get_state()
+    q, k, v, g = workload.step_inputs(cfg, 1, 0)
+    alpha = workload.token_gate_logits(cfg, 1)[0]
+    on = [t.to(pair.dev) for t in (q, k, v, g, alpha)]
+    before = pair.layer.launch_count
+    pair.layer.denoise_step_token_level(*on, out=pair.g_out.t)
+    assert pair.layer.launch_count - before >= 6          # heads cut into runs
+    pair.layer.debug_set_wait_limit(0)
+    pair.layer.denoise_step_token_level(*on, out=pair.g_out.t)
+    expect_timeout(pair.layer)
+    pair.check_guards()
+    assert torch.equal(pair.layer.get_state(), saved)
+    pair.layer.debug_set_wait_limit(-1)
+    pair.g_out.t.fill_(float("nan"))
+    got = pair.layer.denoise_step_token_level(*on, out=pair.g_out.t).float().cpu().numpy()
+    ref = oracle.step_token_level(q, k, v, g, pair.S_ref, alpha, pair.wq, pair.wk, pair.wv, pair.cos, pair.sin)
+    assert float(head_errors(got, ref).max()) <= pair.tol
     pair.layer.sync_status()
 
 
