@@ -169,6 +169,7 @@ __device__ __forceinline__ void feature_tile(float* xs, float* ws, const T* __re
 template <int D, typename T>
 __global__ void __launch_bounds__(NT) simt_step_kernel(StepArgs a)
 {
+    grid_dependency_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LD = D + PAD;       // row-major [64][D] matrices
     constexpr int LT = BM + PAD;      // transposed [D][64] matrices
@@ -349,6 +350,7 @@ struct SmallCfg {
 template <int D, typename T>
 __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
 {
+    grid_dependency_sync();
     using C = SmallCfg<D>;
     constexpr int KT = C::KT, KW = C::KW, KJ = C::KJ, LD = C::LD, LP = C::LP, CN = D / 32;
     extern __shared__ __align__(16) float smem[];
@@ -630,6 +632,7 @@ __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
 template <int D, typename T>
 __global__ void __launch_bounds__(NT) simt_commit_partial_kernel(CommitArgs a)
 {
+    grid_dependency_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LD = D + PAD;
     float* Ks = smem;             // [64][LD]  K tile -> K'
@@ -759,6 +762,7 @@ constexpr int LA = kTokChunk + 4;   // row stride of the C x C matrices
 template <int D, typename T>
 __global__ void __launch_bounds__(NT) token_prepare_kernel(TokenCommitArgs a)
 {
+    grid_dependency_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LD = D + PAD;
     float* Ks = smem;                       // [64][LD]  K tile -> K'
@@ -904,6 +908,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int D, int kScanCols>
 __global__ void __launch_bounds__(NT) token_scan_kernel(TokenCommitArgs a)
 {
+    grid_dependency_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LD = D + PAD;
     constexpr int CG = kScanCols / 4;           // float4 column groups
@@ -1026,6 +1031,7 @@ __global__ void commit_reduce_kernel(float* __restrict__ state, const float* __r
                                      size_t total4, int run_share, int run_ntile, int nslot,
                                      const uint32_t* __restrict__ status)
 {
+    grid_dependency_sync();
     size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total4) return;
     // a partial-sum kernel that gave up on a bounded wait left its slots unwritten: S stays as it was
@@ -1069,6 +1075,7 @@ __global__ void rope_k_kernel(const T* __restrict__ k, const float* __restrict__
                               const float* __restrict__ sin_t, T* __restrict__ out, int L, int H,
                               int D, size_t total8)
 {
+    grid_dependency_sync();
     size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total8) return;
     size_t e = t * 8;
@@ -1134,9 +1141,8 @@ int set_smem(K kernel, size_t bytes)
     return 0;
 }
 
-int check_launch(const char* what)
+int check_launch(const char* what, cudaError_t e)
 {
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("launch of %s failed: %s", what, cudaGetErrorString(e));
         return ARL2_ERR_CUDA;
@@ -1150,15 +1156,15 @@ int launch_step(const StepArgs& a, cudaStream_t st)
     if (a.k_raw) {
         constexpr size_t small_smem = sizeof(float) * SmallCfg<D>::kFloats;
         if (int r = set_smem(simt_step_small_kernel<D, T>, small_smem)) return r;
-        simt_step_small_kernel<D, T><<<dim3((a.s.L + SR - 1) / SR, a.s.H, a.s.B), NT, small_smem, st>>>(a);
-        if (int r = check_launch("simt_step_small_kernel")) return r;
+        if (int r = check_launch("simt_step_small_kernel",
+                                 launch_kernel(simt_step_small_kernel<D, T>, dim3((a.s.L + SR - 1) / SR, a.s.H, a.s.B), NT, small_smem, st, a)))
+            return r;
         return 1;
     }
     size_t smem = sizeof(float) * (2 * D * (BM + PAD) + BN * D + BM * (BM + PAD));
     if (int r = set_smem(simt_step_kernel<D, T>, smem)) return r;
     dim3 grid((a.s.L + BM - 1) / BM, a.s.H, a.s.B);
-    simt_step_kernel<D, T><<<grid, NT, smem, st>>>(a);
-    if (int r = check_launch("simt_step_kernel")) return r;
+    if (int r = check_launch("simt_step_kernel", launch_kernel(simt_step_kernel<D, T>, grid, NT, smem, st, a))) return r;
     return 1;
 }
 
@@ -1168,8 +1174,7 @@ int launch_commit(const CommitArgs& a, cudaStream_t st)
     size_t smem = sizeof(float) * (2 * BM * (D + PAD) + BN * D);
     if (int r = set_smem(simt_commit_partial_kernel<D, T>, smem)) return r;
     dim3 grid(a.nsplit, a.s.H, a.s.B);
-    simt_commit_partial_kernel<D, T><<<grid, NT, smem, st>>>(a);
-    if (int r = check_launch("simt_commit_partial_kernel")) return r;
+    if (int r = check_launch("simt_commit_partial_kernel", launch_kernel(simt_commit_partial_kernel<D, T>, grid, NT, smem, st, a))) return r;
     return 1;
 }
 
@@ -1185,6 +1190,7 @@ __global__ void __launch_bounds__(1024) decay_weights_kernel(const float* __rest
                                                              float* __restrict__ w, float* __restrict__ total,
                                                              int L, int H, int seg)
 {
+    grid_dependency_sync();
     constexpr int kMaxSeg = 8;
     __shared__ float warp_tot[32];
     const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -1238,6 +1244,7 @@ __global__ void __launch_bounds__(256) run_decay_weights_kernel(const float* __r
                                                                 float* __restrict__ total, int L, int H, int share, int ntile,
                                                                 int nslot)
 {
+    grid_dependency_sync();
     __shared__ float warp_tot[8];
     const int slot = blockIdx.x, h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int bh = b * H + h, g_head = bh * ntile, run = g_head / share + slot;
@@ -1278,16 +1285,18 @@ int decay_weights(const Shape& s, const float* alpha_logits, float* w, float* to
 {
     int seg = (s.L + 1023) / 1024;
     seg = seg < 1 ? 1 : seg > 8 ? 8 : seg;
-    decay_weights_kernel<<<dim3(s.H, s.B), 1024, 0, st>>>(alpha_logits, w, total, s.L, s.H, seg);
-    if (int r = check_launch("decay_weights_kernel")) return r;
+    if (int r = check_launch("decay_weights_kernel",
+                             launch_kernel(decay_weights_kernel, dim3(s.H, s.B), 1024, 0, st, alpha_logits, w, total, s.L, s.H, seg)))
+        return r;
     return 1;
 }
 
 int run_decay_weights(const Shape& s, const float* alpha_logits, float* w, float* total, int share, int ntile, int nslot,
                       cudaStream_t st)
 {
-    run_decay_weights_kernel<<<dim3(nslot, s.H, s.B), 256, 0, st>>>(alpha_logits, w, total, s.L, s.H, share, ntile, nslot);
-    if (int r = check_launch("run_decay_weights_kernel")) return r;
+    if (int r = check_launch("run_decay_weights_kernel", launch_kernel(run_decay_weights_kernel, dim3(nslot, s.H, s.B), 256, 0, st, alpha_logits, w,
+                                                                       total, s.L, s.H, share, ntile, nslot)))
+        return r;
     return 1;
 }
 
@@ -1295,10 +1304,10 @@ int commit_reduce(const CommitArgs& a, cudaStream_t st)
 {
     int DD = a.s.D * a.s.D;
     size_t total4 = (size_t)a.s.B * a.s.H * DD / 4;
-    commit_reduce_kernel<<<(unsigned)((total4 + 255) / 256), 256, 0, st>>>(
-        a.state, a.partials, a.decay, a.decay_direct ? 1 : 0, a.state_bf16, a.nsplit, DD, total4,
-        a.run_share, a.run_ntile, a.nslot, a.status);
-    if (int r = check_launch("commit_reduce_kernel")) return r;
+    if (int r = check_launch("commit_reduce_kernel",
+                             launch_kernel(commit_reduce_kernel, dim3((unsigned)((total4 + 255) / 256)), 256, 0, st, a.state, a.partials, a.decay,
+                                           a.decay_direct ? 1 : 0, a.state_bf16, a.nsplit, DD, total4, a.run_share, a.run_ntile, a.nslot, a.status)))
+        return r;
     return 1;
 }
 
@@ -1307,14 +1316,14 @@ int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, co
 {
     size_t total8 = (size_t)s.B * s.L * s.H * s.D / 8;
     unsigned blocks = (unsigned)((total8 + 255) / 256);
+    cudaError_t e;
     if (dtype == ARL2_FP32)
-        rope_k_kernel<float><<<blocks, 256, 0, st>>>(static_cast<const float*>(k), cos_t, sin_t,
-                                                     static_cast<float*>(k_rot), s.L, s.H, s.D, total8);
+        e = launch_kernel(rope_k_kernel<float>, dim3(blocks), 256, 0, st, static_cast<const float*>(k), cos_t, sin_t,
+                          static_cast<float*>(k_rot), s.L, s.H, s.D, total8);
     else
-        rope_k_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(
-            static_cast<const __nv_bfloat16*>(k), cos_t, sin_t, static_cast<__nv_bfloat16*>(k_rot),
-            s.L, s.H, s.D, total8);
-    if (int r = check_launch("rope_k_kernel")) return r;
+        e = launch_kernel(rope_k_kernel<__nv_bfloat16>, dim3(blocks), 256, 0, st, static_cast<const __nv_bfloat16*>(k), cos_t, sin_t,
+                          static_cast<__nv_bfloat16*>(k_rot), s.L, s.H, s.D, total8);
+    if (int r = check_launch("rope_k_kernel", e)) return r;
     return 1;
 }
 
@@ -1368,14 +1377,12 @@ int launch_commit_tokens(const TokenCommitArgs& a, cudaStream_t st)
     size_t smem1 = sizeof(float) * (2 * BM * (D + PAD) + BN * D + 2 * kTokChunk * LA + 3 * kTokChunk + 8);
     if (int r = set_smem(token_prepare_kernel<D, T>, smem1)) return r;
     dim3 grid1(a.nchunk, a.s.H, a.s.B);
-    token_prepare_kernel<D, T><<<grid1, NT, smem1, st>>>(a);
-    if (int r = check_launch("token_prepare_kernel")) return r;
+    if (int r = check_launch("token_prepare_kernel", launch_kernel(token_prepare_kernel<D, T>, grid1, NT, smem1, st, a))) return r;
     constexpr int kScanCols = D / 4;   // 4 CTAs per (stream, head)
     size_t smem2 = sizeof(float) * (2 * kTokChunk * (D + PAD) + 2 * kTokChunk * kScanCols + D * kScanCols);
     if (int r = set_smem(token_scan_kernel<D, kScanCols>, smem2)) return r;
     dim3 grid2(D / kScanCols, a.s.H, a.s.B);
-    token_scan_kernel<D, kScanCols><<<grid2, NT, smem2, st>>>(a);
-    if (int r = check_launch("token_scan_kernel")) return r;
+    if (int r = check_launch("token_scan_kernel", launch_kernel(token_scan_kernel<D, kScanCols>, grid2, NT, smem2, st, a))) return r;
     return 2;
 }
 
@@ -1411,7 +1418,7 @@ int fill_zero(void* p, size_t bytes, cudaStream_t st)
     size_t n16 = bytes / 16;  // callers pass multiples of 16 bytes
     if (n16 == 0) return 0;
     fill_zero_kernel<<<(unsigned)((n16 + 255) / 256), 256, 0, st>>>(static_cast<uint4*>(p), n16);
-    if (int r = check_launch("fill_zero_kernel")) return r;
+    if (int r = check_launch("fill_zero_kernel", cudaGetLastError())) return r;
     return 1;
 }
 
@@ -1419,7 +1426,7 @@ int state_to_bf16(const float* state, __nv_bfloat16* dst, size_t n, cudaStream_t
 {
     size_t n4 = n / 4;
     state_to_bf16_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(state, dst, n4);
-    if (int r = check_launch("state_to_bf16_kernel")) return r;
+    if (int r = check_launch("state_to_bf16_kernel", cudaGetLastError())) return r;
     return 1;
 }
 

@@ -68,6 +68,7 @@ struct TcStepParams {
     __nv_bfloat16* out;
     uint32_t* status;
     uint32_t spin_limit;       // polls a bounded wait makes before it gives up
+    int k_made_before;         // the kernel before this one made K and nothing else that is read or written here
     uint32_t* sched_counter;   // this launch's item counter (zero on entry)
     uint32_t* sched_next;      // the next launch's counter: cleared by this launch
     int gate_mode;             // 0: gate logits [B, L, H]; 1: [B, L] (one per token); 2: [B, L, H, D] (per channel)
@@ -500,6 +501,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_kv = p.n_kv;
 
+    if (!p.k_made_before) grid_dependency_sync();
     if (threadIdx.x == 0) {
         mbar_init(bars + 8 * kBarQFull, 1);
         mbar_init(bars + 8 * kBarQFree, 2);
@@ -571,10 +573,8 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     tma_load_4d(dst, &tm_q, bar_q, 0, it.h[t], it.row0[t], it.b[t]);
                     tma_load_4d(dst + kHalfBytes, &tm_q, bar_q, 64, it.h[t], it.row0[t], it.b[t]);
                 }
-                // K comes from the kernel before this one: up to here everything ran beside the end of the rotation,
-                // which lets this grid start early (the commit kernel of a clean pass does not: after it this
-                // grid starts when its last CTA has left, and only the launch itself is hidden)
-                if (item == 0) grid_dependency_wait();
+                // K comes from the kernel before this one: up to here everything ran beside its end
+                if (item == 0 && p.k_made_before) grid_dependency_sync();
                 const int entries = item_entries(it, nj);
                 for (int e = 0; e < entries && ok; ++e, ++n) {
                     const uint32_t slot = n % kStages;
@@ -885,6 +885,7 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
+        grid_dependency_wait();
         const uint32_t bar_k = bars + 8 * kTPBarLoadK, bar_v = bars + 8 * kTPBarLoadV;
         mbar_expect_tx(bar_k, 2 * kTileBytes);
         mbar_expect_tx(bar_v, kTileBytes);
@@ -906,6 +907,7 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    grid_dependency_sync();
 
     constexpr uint32_t kLboK = 1u << 16;
     constexpr uint32_t kLboMN = (uint32_t)(kHalfBytes >> 4) << 16;
@@ -1349,6 +1351,7 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
         fence_barrier_init();
         fence_proxy_async_smem();
     }
+    grid_dependency_sync();
     // (one answer for the whole CTA) after an error the chunk factors are not all there, and nothing is published
     if (__syncthreads_or(*reinterpret_cast<volatile uint32_t*>(p.status + kStatusError) != 0u)) return;
 
@@ -1528,7 +1531,7 @@ constexpr int kPublishThreads = 256;   // four values each
 __global__ void __launch_bounds__(kPublishThreads) tc_token_publish_kernel(const TcTokenParams p)
 {
     const size_t i = ((size_t)blockIdx.x * kPublishThreads + threadIdx.x) * 4;
-    grid_dependency_wait();
+    grid_dependency_sync();
     const uint32_t err = p.status[kStatusError];
     const float4 v = *reinterpret_cast<const float4*>(p.next + i);   // (on its way beside the status word)
     if (err != 0u) return;
@@ -1558,7 +1561,7 @@ __global__ void pack_rope_kernel(const float* __restrict__ cos_t, const float* _
 __global__ void tc_rope_k_kernel(const uint4* __restrict__ k, const uint4* __restrict__ rope_h,
                                  uint4* __restrict__ out, int L, int H, size_t total8)
 {
-    grid_dependents_launch();
+    grid_dependency_sync();
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total8) return;
     const int c = (int)(t & 15);                     // vector of the 128-element row
@@ -1610,7 +1613,7 @@ tc_split_merge_kernel(const TcStepParams p)
     if (in_range) it = decode_item<false>(p.n_whole + slot, p);
     const int k = p.k_split;
     const size_t tp0 = ((size_t)slot * 2 + t) * k;
-    asm volatile("griddepcontrol.wait;" ::: "memory");   // the step kernel has finished, its writes are visible
+    grid_dependency_sync();   // the step kernel has finished, its writes are visible
     if (!in_range || t >= it.ntile || p.status[kStatusError] != 0u) return;
     const int row0 = it.row0[t] + r0;
     __nv_bfloat16* obase = p.out + (((size_t)it.b[t] * p.s.L + row0) * p.s.H + it.h[t]) * kTile + lane * 4;
@@ -1691,9 +1694,8 @@ int tc_prepare_map(const void* w, __nv_bfloat16* w_op, int H, cudaStream_t st)
 int tc_rope_k(const Shape& s, const void* k, const void* rope_h, void* k_rot, cudaStream_t st)
 {
     const size_t total8 = (size_t)s.B * s.L * s.H * kTile / 8;
-    tc_rope_k_kernel<<<(unsigned)((total8 + 255) / 256), 256, 0, st>>>(
-        static_cast<const uint4*>(k), static_cast<const uint4*>(rope_h), static_cast<uint4*>(k_rot), s.L, s.H, total8);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(tc_rope_k_kernel, dim3((unsigned)((total8 + 255) / 256)), 256, 0, st, static_cast<const uint4*>(k),
+                                        static_cast<const uint4*>(rope_h), static_cast<uint4*>(k_rot), s.L, s.H, total8);
     if (e != cudaSuccess) { set_error("launch of tc_rope_k_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 1;
 }
@@ -1767,40 +1769,18 @@ int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* 
     p.split_o = a.split_o;
     p.split_ml = a.split_ml;
     const int grid = p.n_sched < num_sms ? p.n_sched : num_sms;
-    // After the rotation of K the launch overlaps that kernel's end: barriers, tensor memory, the first Q tiles and
-    // their rotation need nothing from it.  (After the commit kernel of a clean pass, which does not release its
-    // dependents early, only the launch is hidden.  After anything else -- K as the caller gave it -- the kernel
-    // before may be the one that makes Q, and the launch is an ordinary one.)
-    // 12 heads x 1560 tokens 44.1 -> 42.5 us per pass, 3 x 12 x 1001 38.8 -> 34.9, 2 heads x 300 22.5 -> 18.4.
-    cudaLaunchConfig_t scfg = {};
-    scfg.gridDim = dim3((unsigned)grid);
-    scfg.blockDim = dim3(kThreads);
-    scfg.dynamicSmemBytes = kSmemBytes;
-    scfg.stream = st;
-    cudaLaunchAttribute sattr[1];
-    sattr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    sattr[0].val.programmaticStreamSerializationAllowed = 1;
-    scfg.attrs = sattr;
-    scfg.numAttrs = a.k_made_before ? 1 : 0;
+    // After the kernel that makes K (the rotation, or the commit kernel of a clean pass) barriers, tensor memory, the first Q
+    // tiles and their rotation run ahead of the wait; with K as the caller gave it the kernel before may be the one that
+    // makes Q.  12 heads x 1560 tokens 44.1 -> 42.5 us per pass, 3 x 12 x 1001 38.8 -> 34.9, 2 heads x 300 22.5 -> 18.4.
+    p.k_made_before = a.k_made_before ? 1 : 0;
     auto kernel = elem_gate ? tc_step_kernel<true, false> : p.k_split > 1 ? tc_step_kernel<false, true> : tc_step_kernel<false, false>;
-    cudaError_t e = cudaLaunchKernelEx(&scfg, kernel, tm_q, tm_k, tm_v, tm_w, tm_s, p);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    cudaError_t e = launch_kernel(kernel, dim3((unsigned)grid), kThreads, kSmemBytes, st, tm_q, tm_k, tm_v, tm_w, tm_s, p);
     if (e != cudaSuccess) { set_error("launch of tc_step_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     if (p.k_split == 1) return 1;
     // the parts' rows are combined by a second, small kernel (one warp per row); it may start
     // before the step kernel ends and waits for it at its griddepcontrol.wait
     const long warps = (long)(p.n_items - p.n_whole) * 2 * (kTile / kMergeRows);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((warps + 7) / 8));
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, tc_split_merge_kernel, p);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    e = launch_kernel(tc_split_merge_kernel, dim3((unsigned)((warps + 7) / 8)), 256, 0, st, p);
     if (e != cudaSuccess) { set_error("launch of tc_split_merge_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 2;
 }
@@ -1851,30 +1831,17 @@ int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const
     if (int r = make_map_rows(&tm_kh, p.kh, rows, kTokC)) return r;
     if (int r = make_map_rows(&tm_u1, p.u1, rows, kTokC, slabs * kScanSlab, false)) return r;
     dim3 grid1(p.ntile, a.s.H, a.s.B);
-    tc_token_prepare_kernel<<<grid1, kTPThreads, kTPSmemBytes, st>>>(tm_k, tm_v, tm_wk, tm_wv, out_w, out_u1, p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_kernel(tc_token_prepare_kernel, grid1, kTPThreads, kTPSmemBytes, st, tm_k, tm_v, tm_wk, tm_wv, out_w, out_u1, p);
     if (e != cudaSuccess) { set_error("launch of tc_token_prepare_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     dim3 grid2(kTile / (slabs * kScanSlab), a.s.H, a.s.B);
     if (slabs == 1)
-        tc_token_scan_kernel<1, false><<<grid2, ScanCfg<1, false>::kThreads, ScanCfg<1, false>::kSmemBytes, st>>>(tm_w, tm_kh, tm_u1, p);
+        e = launch_kernel(tc_token_scan_kernel<1, false>, grid2, ScanCfg<1, false>::kThreads, ScanCfg<1, false>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
     else if (!shared_sm)
-        tc_token_scan_kernel<2, false><<<grid2, ScanCfg<2, false>::kThreads, ScanCfg<2, false>::kSmemBytes, st>>>(tm_w, tm_kh, tm_u1, p);
+        e = launch_kernel(tc_token_scan_kernel<2, false>, grid2, ScanCfg<2, false>::kThreads, ScanCfg<2, false>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
     else
-        tc_token_scan_kernel<2, true><<<grid2, ScanCfg<2, true>::kThreads, ScanCfg<2, true>::kSmemBytes, st>>>(tm_w, tm_kh, tm_u1, p);
-    e = cudaGetLastError();
+        e = launch_kernel(tc_token_scan_kernel<2, true>, grid2, ScanCfg<2, true>::kThreads, ScanCfg<2, true>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
     if (e != cudaSuccess) { set_error("launch of tc_token_scan_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
-    // staged while the walk ends; the kernel itself waits for it
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(heads * (kTile * kTile / 4 / kPublishThreads)));
-    cfg.blockDim = dim3(kPublishThreads);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, tc_token_publish_kernel, p);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    e = launch_kernel(tc_token_publish_kernel, dim3((unsigned)(heads * (kTile * kTile / 4 / kPublishThreads))), kPublishThreads, 0, st, p);
     if (e != cudaSuccess) { set_error("launch of tc_token_publish_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 3;
 }

@@ -121,6 +121,7 @@ tc_commit_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
+        grid_dependency_wait();
         // this thread is the TMA producer: the run's first map and first tile are requested now, while
         // tensor memory is still being allocated (nothing else can start before they land)
         if (n_my > 0) {
@@ -147,6 +148,7 @@ tc_commit_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    grid_dependency_sync();
     // TMEM columns: U buffer 0 | U buffer 1 | dS | G
     constexpr uint32_t kColDS = 2 * kTile, kColG = 3 * kTile;
 
@@ -547,7 +549,7 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* __restrict__ par
     if (wv != nullptr) fin_load_matrix(Ws, wv + (size_t)h * kTile * kTile, tid);
     if (kMode == 1) fin_load_matrix(Ss, mirror_cur + head, tid);
     const float decay_v = decay[bh];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    grid_dependency_sync();
     const uint32_t err = status != nullptr ? status[kStatusError] : 0u;
     const int first = (bh * ntile) / share, last = (bh * ntile + ntile - 1) / share;
     const int nparts = last - first + 1;
@@ -659,6 +661,7 @@ tc_run_prefix_kernel(float* __restrict__ slots, const float* __restrict__ state,
     const int bh = (int)(blockIdx.x / (kTile / kFinRows)), h = bh % H;
     const int cta_row0 = (int)(blockIdx.x % (kTile / kFinRows)) * kFinRows;
     if (wv != nullptr) fin_load_matrix(Ws, wv + (size_t)h * kTile * kTile, tid);
+    grid_dependency_sync();
     const int nparts = (bh * ntile + ntile - 1) / share - (bh * ntile) / share + 1;
     float* head_slots = slots + (size_t)bh * nslot * kTile * kTile;
     const size_t read0 = ((size_t)(warp * 4) * kTile + cta_row0 + srow) * 8 + shalf * 4;
@@ -758,9 +761,8 @@ int tc_commit_run_share(const Shape& s, int nslot, int* share, int* ntile)
 
 int tc_run_prefix(const CommitArgs& a, const float* total, cudaStream_t st)
 {
-    tc_run_prefix_kernel<<<(unsigned)(a.s.B * a.s.H) * (kTile / kFinRows), kFinThreads, kPrefixSmemBytes, st>>>(
-        a.partials, a.state, static_cast<const __nv_bfloat16*>(a.wv), total, a.s.H, a.run_share, a.run_ntile, a.nslot);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(tc_run_prefix_kernel, dim3((unsigned)(a.s.B * a.s.H) * (kTile / kFinRows)), kFinThreads, kPrefixSmemBytes, st,
+                                        a.partials, a.state, static_cast<const __nv_bfloat16*>(a.wv), total, a.s.H, a.run_share, a.run_ntile, a.nslot);
     if (e != cudaSuccess) { set_error("launch of tc_run_prefix_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 1;
 }
@@ -788,13 +790,8 @@ int tc_commit_partials(CommitArgs& a, const __nv_bfloat16* wk_op, cudaStream_t s
     if (int r = tc_commit_run_share(a.s, a.nslot, &p.share, &p.ntile)) return r;
     p.total_tiles = a.s.B * a.s.H * p.ntile;
     const unsigned grid = (unsigned)((p.total_tiles + p.share - 1) / p.share);
-    if (a.mode == 1)
-        tc_commit_kernel<1><<<grid, kCThreads, kCommitSmemBytes, st>>>(tm_k, tm_v, tm_wk, p);
-    else if (a.mode == 2)
-        tc_commit_kernel<2><<<grid, kCThreads, kCommitSmemBytes, st>>>(tm_k, tm_v, tm_wk, p);
-    else
-        tc_commit_kernel<0><<<grid, kCThreads, kCommitSmemBytes, st>>>(tm_k, tm_v, tm_wk, p);
-    cudaError_t e = cudaGetLastError();
+    auto kernel = a.mode == 1 ? tc_commit_kernel<1> : a.mode == 2 ? tc_commit_kernel<2> : tc_commit_kernel<0>;
+    const cudaError_t e = launch_kernel(kernel, dim3(grid), kCThreads, kCommitSmemBytes, st, tm_k, tm_v, tm_wk, p);
     if (e != cudaSuccess) { set_error("launch of tc_commit_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     a.run_share = p.share;
     a.run_ntile = p.ntile;
@@ -803,32 +800,11 @@ int tc_commit_partials(CommitArgs& a, const __nv_bfloat16* wk_op, cudaStream_t s
 
 int tc_commit_finish(const CommitArgs& a, cudaStream_t st)
 {
-    // programmatic stream serialisation: the grid is staged while the kernel before it in the stream
-    // (the partial sums) is still running; the kernel itself waits for that kernel where it must
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(a.s.B * a.s.H) * (kTile / kFinRows));
-    cfg.blockDim = dim3(kFinThreads);
-    cfg.dynamicSmemBytes = (size_t)fin_smem_bytes(a.mode == 1 ? 1 : 0);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const __nv_bfloat16* wv = static_cast<const __nv_bfloat16*>(a.wv);
-    const float* partials = a.partials;
-    const float* partials_g = a.partials_g;
-    const __nv_bfloat16* cur = a.state_bf16;
-    const uint32_t* status = a.status;
-    const int direct = a.decay_direct ? 1 : 0;
-    cudaError_t e;
-    if (a.mode == 1)
-        e = cudaLaunchKernelEx(&cfg, tc_commit_finish_kernel<1>, a.state, partials, partials_g, wv, a.decay, direct, cur,
-                               a.state_bf16_next, a.s.H, a.run_share, a.run_ntile, a.nslot, status);
-    else
-        e = cudaLaunchKernelEx(&cfg, tc_commit_finish_kernel<0>, a.state, partials, partials_g, wv, a.decay, direct, cur,
-                               a.state_bf16_next, a.s.H, a.run_share, a.run_ntile, a.nslot, status);
-    if (e == cudaSuccess) e = cudaGetLastError();
+    auto kernel = a.mode == 1 ? tc_commit_finish_kernel<1> : tc_commit_finish_kernel<0>;
+    const cudaError_t e = launch_kernel(kernel, dim3((unsigned)(a.s.B * a.s.H) * (kTile / kFinRows)), kFinThreads,
+                                        (size_t)fin_smem_bytes(a.mode == 1 ? 1 : 0), st, a.state, a.partials, a.partials_g,
+                                        static_cast<const __nv_bfloat16*>(a.wv), a.decay, a.decay_direct ? 1 : 0, a.state_bf16, a.state_bf16_next,
+                                        a.s.H, a.run_share, a.run_ntile, a.nslot, a.status);
     if (e != cudaSuccess) { set_error("launch of tc_commit_finish_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 1;
 }

@@ -111,6 +111,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    grid_dependency_sync();
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
@@ -327,17 +328,9 @@ int tc_gemm(const GemmArgs& a, cudaStream_t st)
     p.spin_limit = a.wait_limit ? a.wait_limit - 1 : kSpinLimit;
     const int total = p.m_tiles * p.n_tiles;
     const int grid = total < num_sms ? total : num_sms;
-    if (mh == 2 && p.bn == 256)
-        tc_gemm_kernel<256, 2><<<grid, kGThreads, kGemmSmemBytes, st>>>(tm_a, tm_b, p);
-    else if (mh == 2)
-        tc_gemm_kernel<192, 2><<<grid, kGThreads, kGemmSmemBytes, st>>>(tm_a, tm_b, p);
-    else if (p.bn == 256)
-        tc_gemm_kernel<256, 1><<<grid, kGThreads, kGemmSmemBytes, st>>>(tm_a, tm_b, p);
-    else if (p.bn == 192)
-        tc_gemm_kernel<192, 1><<<grid, kGThreads, kGemmSmemBytes, st>>>(tm_a, tm_b, p);
-    else
-        tc_gemm_kernel<128, 1><<<grid, kGThreads, kGemmSmemBytes, st>>>(tm_a, tm_b, p);
-    cudaError_t e = cudaGetLastError();
+    auto kernel = mh == 2 ? (p.bn == 256 ? tc_gemm_kernel<256, 2> : tc_gemm_kernel<192, 2>)
+                          : p.bn == 256 ? tc_gemm_kernel<256, 1> : p.bn == 192 ? tc_gemm_kernel<192, 1> : tc_gemm_kernel<128, 1>;
+    const cudaError_t e = launch_kernel(kernel, dim3((unsigned)grid), kGThreads, kGemmSmemBytes, st, tm_a, tm_b, p);
     if (e != cudaSuccess) { set_error("launch of tc_gemm_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 1;
 }

@@ -165,6 +165,8 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         const uint32_t par = (uint32_t)(g - g_begin) & 1u;
         const int row = tl * kTile + r;                // this thread's token
         if (seg_first) {
+            // The maps, Q, K and V are of the caller, not of the kernel before; the states and the output are not.
+            if (g == g_begin) grid_dependency_sync();
             // the segment's state (fp32) into TMEM: row d = r, this thread's 64 columns
             const bool whole = p.entry == nullptr;
             const float* src = whole ? p.state + (bh * kTile + r) * kTile + hf * 64
@@ -424,8 +426,8 @@ int tc_token_readout(const StepArgs& a, const float* alpha_logits, const CommitA
     p.nslot = seg.nslot;
     p.total_tiles = a.s.B * a.s.H * p.ntile;
     const int grid = (p.total_tiles + p.share - 1) / p.share;
-    tc_token_readout_kernel<<<grid, kTRThreads, kTRSmemBytes, st>>>(tm_q, tm_k, tm_v, tm_wq, tm_wk, tm_wv, p);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_kernel(tc_token_readout_kernel, dim3((unsigned)grid), kTRThreads, kTRSmemBytes, st, tm_q, tm_k, tm_v, tm_wq,
+                                        tm_wk, tm_wv, p);
     if (e != cudaSuccess) { set_error("launch of tc_token_readout_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 1;
 }

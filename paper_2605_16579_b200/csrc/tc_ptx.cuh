@@ -229,13 +229,6 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
         : "memory");
 }
 
-// ---- programmatic dependent launch --------------------------------------------------------
-// Returns once the kernel before this one in the stream has finished and its writes are visible (at once
-// when this kernel was launched without the attribute).
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Lets the next kernel's CTAs start as soon as this one's have all started and leave room.
-__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 __device__ __forceinline__ float ex2_approx(float x)
 {
     float y;
