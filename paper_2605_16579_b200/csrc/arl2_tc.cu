@@ -208,8 +208,10 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
     uint32_t sreg[128];
 
     for (uint32_t item = 0;; ++item) {
-        if (!wait_bar(bars + 8 * kBarQFull, item & 1, ab, 10)) return;
-        const int id = item_slots[item & 1];
+        // the first item is known without the producer: its rotation table is fetched while Q is on its way (a rotation
+        // that asked for the table once Q had landed ended 1.2 us later)
+        if (item > 0 && !wait_bar(bars + 8 * kBarQFull, item & 1, ab, 10)) return;
+        const int id = item > 0 ? item_slots[item & 1] : (int)blockIdx.x;
         if (id < 0) return;
         const Item it = decode_item<kSplit>(id, p);
         const int j0 = kSplit ? it.j0 : 0, nj = kSplit ? it.nj : n_kv;
@@ -217,6 +219,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
         const int row = it.row0[t] + r;
         const bool valid_row = row < L;
         const bool active = t < it.ntile;
+        if (item == 0 && !active && !wait_bar(bars + 8 * kBarQFull, 0, ab, 10)) return;   // (no phase is left out)
 
         if (active) {
             // ---- Q~ = RoPE(Q): rotate this thread's row of the tile in place          (Eq. 2)
@@ -227,6 +230,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
                 uint4 cs[16];
 #pragma unroll
                 for (int c = 0; c < 16; ++c) cs[c] = __ldg(tab + c * 32);
+                if (item == 0 && !wait_bar(bars + 8 * kBarQFull, 0, ab, 10)) return;
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     int off = (c >> 3) * kHalfBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4);
@@ -244,6 +248,8 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
                     *reinterpret_cast<uint4*>(tile + off) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
                 fence_proxy_async_smem();
+            } else if (item == 0 && !wait_bar(bars + 8 * kBarQFull, 0, ab, 10)) {
+                return;
             }
             mbar_arrive(bars + 8 * (kBarQRot0 + t));
 
@@ -502,7 +508,19 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     const int n_kv = p.n_kv;
 
     if (!p.k_made_before) grid_dependency_sync();
-    if (threadIdx.x == 0) {
+    // a work item's Q tiles (and its id) for everyone who waits on kBarQFull
+    auto request_q = [&](uint32_t slot, int id, const Item& it) {
+        item_slots[slot] = id;
+        const uint32_t bar_q = bars + 8 * kBarQFull;
+        mbar_expect_tx(bar_q, it.ntile * kTileBytes);
+        for (int t = 0; t < it.ntile; ++t) {
+            const uint32_t dst = smem_base + kOffQ + t * kTileBytes;
+            tma_load_4d(dst, &tm_q, bar_q, 0, it.h[t], it.row0[t], it.b[t]);
+            tma_load_4d(dst + kHalfBytes, &tm_q, bar_q, 64, it.h[t], it.row0[t], it.b[t]);
+        }
+    };
+    if (threadIdx.x == 8 * 32) {   // the TMA producer
+        prefetch_tensormap(&tm_q);
         mbar_init(bars + 8 * kBarQFull, 1);
         mbar_init(bars + 8 * kBarQFree, 2);
         mbar_init(bars + 8 * kBarQRot0, 128);
@@ -524,6 +542,10 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
+        // the first item's Q goes out now, beside the allocation of tensor memory
+        request_q(0, (int)blockIdx.x, decode_item<kSplit>((int)blockIdx.x, p));
+        prefetch_tensormap(&tm_k);
+        prefetch_tensormap(&tm_v);
         if (blockIdx.x == 0) *p.sched_next = 0;   // the next launch starts from a clean counter
     }
     if (warp == 9) {
@@ -544,15 +566,10 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
     if (warp == 8) {
         // ---------------- TMA producer and scheduler ----------------
         if (lane == 0) {
-            prefetch_tensormap(&tm_q);
-            prefetch_tensormap(&tm_k);
-            prefetch_tensormap(&tm_v);
-            prefetch_tensormap(&tm_w);
-            prefetch_tensormap(&tm_s);
             const uint32_t bar_q = bars + 8 * kBarQFull;
             uint32_t n = 0;       // ring entries produced so far (all items)
             bool ok = true;
-            int q_item = -1;      // item whose Q tiles were requested last
+            int q_item = 0;       // item whose Q tiles were requested last
             int id = (int)blockIdx.x;
             for (uint32_t item = 0; ok; ++item) {
                 if (item > 0) ok = wait_bar(bars + 8 * kBarQFree, (item - 1) & 1, ab, 50);
@@ -562,19 +579,16 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     mbar_arrive(bar_q);
                     break;
                 }
-                item_slots[item & 1] = id;
                 const Item it = decode_item<kSplit>(id, p);
                 const int j0 = kSplit ? it.j0 : 0, nj = kSplit ? it.nj : n_kv;
-                const int ntile = it.ntile;
-                mbar_expect_tx(bar_q, ntile * kTileBytes);
+                if (item > 0) request_q(item & 1, id, it);
                 q_item = (int)item;
-                for (int t = 0; t < ntile; ++t) {
-                    uint32_t dst = smem_base + kOffQ + t * kTileBytes;
-                    tma_load_4d(dst, &tm_q, bar_q, 0, it.h[t], it.row0[t], it.b[t]);
-                    tma_load_4d(dst + kHalfBytes, &tm_q, bar_q, 64, it.h[t], it.row0[t], it.b[t]);
-                }
                 // K comes from the kernel before this one: up to here everything ran beside its end
-                if (item == 0 && p.k_made_before) grid_dependency_sync();
+                if (item == 0) {
+                    if (p.k_made_before) grid_dependency_sync();
+                    prefetch_tensormap(&tm_w);
+                    prefetch_tensormap(&tm_s);
+                }
                 const int entries = item_entries(it, nj);
                 for (int e = 0; e < entries && ok; ++e, ++n) {
                     const uint32_t slot = n % kStages;
@@ -606,7 +620,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             }
             if (!ok || *abort_flag) {
                 // do not leave the CTA while bulk copies into its shared memory are in flight
-                if (q_item >= 0) drain_bar(bar_q, (uint32_t)q_item & 1);
+                drain_bar(bar_q, (uint32_t)q_item & 1);
                 for (uint32_t m = (n > (uint32_t)kStages ? n - kStages : 0); m < n; ++m)
                     drain_bar(bars + 8 * (kBarFull0 + m % kStages), (m / kStages) & 1);
             }
@@ -1556,29 +1570,47 @@ __global__ void pack_rope_kernel(const float* __restrict__ cos_t, const float* _
     out[dst] = l < L ? __floats2half2_rn(cos_t[t], sin_t[t]) : __floats2half2_rn(0.0f, 0.0f);
 }
 
-// k_rot = RoPE(k) for bf16 [B, L, H, 128] from the packed half2 table: 8 elements (4 rotation pairs,
-// one 16-byte table vector) per thread.  The same table rotates Q inside the step kernel.
-__global__ void tc_rope_k_kernel(const uint4* __restrict__ k, const uint4* __restrict__ rope_h,
-                                 uint4* __restrict__ out, int L, int H, size_t total8)
+// k_rot = RoPE(k) for bf16 [B, L, H, 128] from the packed half2 table: 16 threads per row (8 elements, 4 rotation
+// pairs, one 16-byte table vector each), kRopeRows rows per thread with all loads ahead of the first use.  The same table
+// rotates Q inside the step kernel.  Bound by memory, and where it is short by its latencies.  (With one row per thread,
+// 64-bit index divisions and the step kernel's first Q tiles requested 0.6 us later and rotated 1.2 us later: 40.2 us per
+// pass of 12 heads x 1560 tokens against 38.8, 3 x 12 x 1001 33.0 against 32.2.)
+constexpr int kRopeRows = 4;
+__global__ void __launch_bounds__(256) tc_rope_k_kernel(const uint4* __restrict__ k, const uint4* __restrict__ rope_h,
+                                                        uint4* __restrict__ out, uint32_t L, uint32_t H, uint32_t rows)
 {
-    grid_dependency_sync();
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= total8) return;
-    const int c = (int)(t & 15);                     // vector of the 128-element row
-    const int l = (int)((t >> 4) / H % L);           // token
-    const uint4 raw = __ldg(k + t);
-    const uint4 cs = __ldg(rope_h + ((size_t)(l >> 5) * 16 + c) * 32 + (l & 31));
-    uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-    const uint32_t h2[4] = {cs.x, cs.y, cs.z, cs.w};
+    const uint32_t c = threadIdx.x & 15;             // vector of the 128-element row
+    const uint32_t row0 = blockIdx.x * (16 * kRopeRows) + (threadIdx.x >> 4);
+    const uint4* tab[kRopeRows];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        float cc, ss;
-        unpack_cs(h2[m], cc, ss);
-        const float x0 = __uint_as_float(w[m] << 16);
-        const float x1 = __uint_as_float(w[m] & 0xFFFF0000u);
-        w[m] = pack_bf16(x0 * cc - x1 * ss, x0 * ss + x1 * cc);
+    for (int i = 0; i < kRopeRows; ++i) {
+        const uint32_t l = (row0 + i * 16) / H % L;  // token
+        tab[i] = rope_h + ((size_t)(l >> 5) * 16 + c) * 32 + (l & 31);
     }
-    out[t] = make_uint4(w[0], w[1], w[2], w[3]);
+    grid_dependency_sync();
+    uint4 raw[kRopeRows], cs[kRopeRows];
+#pragma unroll
+    for (int i = 0; i < kRopeRows; ++i) {
+        if (row0 + i * 16 < rows) {
+            raw[i] = __ldg(k + (size_t)(row0 + i * 16) * 16 + c);
+            cs[i] = __ldg(tab[i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kRopeRows; ++i) {
+        if (row0 + i * 16 >= rows) return;
+        uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+        const uint32_t h2[4] = {cs[i].x, cs[i].y, cs[i].z, cs[i].w};
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            float cc, ss;
+            unpack_cs(h2[m], cc, ss);
+            const float x0 = __uint_as_float(w[m] << 16);
+            const float x1 = __uint_as_float(w[m] & 0xFFFF0000u);
+            w[m] = pack_bf16(x0 * cc - x1 * ss, x0 * ss + x1 * cc);
+        }
+        out[(size_t)(row0 + i * 16) * 16 + c] = make_uint4(w[0], w[1], w[2], w[3]);
+    }
 }
 
 // out[h][o][i] = w[h][i][o] (bf16), or the identity when w is null: the K-major B operand of
@@ -1693,9 +1725,11 @@ int tc_prepare_map(const void* w, __nv_bfloat16* w_op, int H, cudaStream_t st)
 
 int tc_rope_k(const Shape& s, const void* k, const void* rope_h, void* k_rot, cudaStream_t st)
 {
-    const size_t total8 = (size_t)s.B * s.L * s.H * kTile / 8;
-    const cudaError_t e = launch_kernel(tc_rope_k_kernel, dim3((unsigned)((total8 + 255) / 256)), 256, 0, st, static_cast<const uint4*>(k),
-                                        static_cast<const uint4*>(rope_h), static_cast<uint4*>(k_rot), s.L, s.H, total8);
+    const size_t rows = (size_t)s.B * s.L * s.H;
+    if (rows >= ((size_t)1 << 32) - 16 * kRopeRows) { set_error("tc_rope_k: too many rows"); return ARL2_ERR_UNSUPPORTED; }
+    const cudaError_t e = launch_kernel(tc_rope_k_kernel, dim3((unsigned)((rows + 16 * kRopeRows - 1) / (16 * kRopeRows))), 256, 0, st,
+                                        static_cast<const uint4*>(k), static_cast<const uint4*>(rope_h), static_cast<uint4*>(k_rot),
+                                        (uint32_t)s.L, (uint32_t)s.H, (uint32_t)rows);
     if (e != cudaSuccess) { set_error("launch of tc_rope_k_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 1;
 }
