@@ -143,6 +143,8 @@ int tc_prepare_map(const void* w, __nv_bfloat16* w_op, int H, cudaStream_t st);
 int tc_prepare_rope(const float* cos_t, const float* sin_t, void* out, int L, cudaStream_t st);
 // k_rot = RoPE(k), bf16 [B, L, H, 128], from the packed table tc_prepare_rope wrote
 int tc_rope_k(const Shape& s, const void* k, const void* rope_h, void* k_rot, cudaStream_t st);
+// thread blocks (one per SM) that the launch of tc_step will have, and the SMs of the current device
+int tc_step_ctas(const StepArgs& a, int* ctas, int* num_sms);
 int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* state_bf16,
             cudaStream_t st);
 // partial sums on tensor cores (fills a.run_share / a.run_ntile for the finishing kernel) ...

@@ -1689,6 +1689,42 @@ tc_split_merge_kernel(const TcStepParams p)
     }
 }
 
+// The work items of a step launch and how its last wave is cut.
+void plan_items(const StepArgs& a, int num_sms, TcStepParams& p)
+{
+    p.Lk = a.Lk > 0 ? a.Lk : a.s.L;
+    p.n_q = (a.s.L + kTile - 1) / kTile;
+    p.n_kv = (p.Lk + kTile - 1) / kTile;
+    const int bh = a.s.B * a.s.H;
+    p.n_pair_items = bh * (p.n_q / 2);
+    p.n_items = p.n_pair_items + ((p.n_q & 1) ? (bh + 1) / 2 : 0);   // ragged tiles go two by two
+    const bool elem_gate = a.gate_mode == 2 && a.gate != nullptr;
+    // The last wave: `rem` items on num_sms SMs.  Cut into k key ranges, the wave takes
+    // ceil(rem k / SMs) rounds of one part each; a part costs its share of the key iterations plus
+    // what every item costs (the readout iteration, the hand-over between items) plus the exchange
+    // of the partial rows -- measured: 3.3 k clk per iteration, 10.8 k per item, about 6 k for the
+    // exchange.  Take the k that makes the wave shortest, if that is shorter than leaving it whole.
+    // (At 3.7 k, what an iteration took before the issuers took turns, 26 to 28 key tiles were still cut in three
+    // where a third costs more than it saves: 6 heads x 3300 tokens 68 us, whole 62; 29 x 3456 218, 204;
+    // 17 x 3584 139, 125.)
+    p.n_whole = p.n_items;
+    p.k_split = 1;
+    if (!elem_gate && a.split_o != nullptr) {
+        const int waves = (p.n_items + num_sms - 1) / num_sms;
+        const int rem = p.n_items - (waves - 1) * num_sms;
+        const float iter = 3.31f, fixed = 10.8f, exchange = 6.0f;
+        float best = (p.n_kv + 1) * iter + fixed;
+        for (int k = 2; k <= kMaxSplit; ++k) {
+            if (p.n_kv < 4 * k || (long)rem * k * 2 > a.split_tile_parts) break;
+            const float part = ((float)p.n_kv / k + 1.0f) * iter + fixed + exchange;
+            const float cost = (float)((rem * k + num_sms - 1) / num_sms) * part;
+            if (cost < 0.95f * best) { best = cost; p.k_split = k; }
+        }
+        if (p.k_split > 1) p.n_whole = p.n_items - rem;
+    }
+    p.n_sched = p.n_whole + (p.n_items - p.n_whole) * p.k_split;
+}
+
 std::mutex g_setup_mutex;
 DeviceSetup g_setup[kMaxDevices];
 
@@ -1744,6 +1780,15 @@ int tc_prepare_rope(const float* cos_t, const float* sin_t, void* out, int L, cu
     return 1;
 }
 
+int tc_step_ctas(const StepArgs& a, int* ctas, int* num_sms)
+{
+    if (int r = device_setup(num_sms)) return r;
+    TcStepParams p;
+    plan_items(a, *num_sms, p);
+    *ctas = p.n_sched < *num_sms ? p.n_sched : *num_sms;
+    return 0;
+}
+
 int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* state_bf16, cudaStream_t st)
 {
     int num_sms = 0;
@@ -1766,40 +1811,11 @@ int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* 
     p.out = static_cast<__nv_bfloat16*>(a.out);
     p.status = a.status;
     p.spin_limit = a.wait_limit ? a.wait_limit - 1 : kSpinLimit;
-    p.Lk = ks.L;
-    p.n_q = (a.s.L + kTile - 1) / kTile;
-    p.n_kv = (ks.L + kTile - 1) / kTile;
-    const int bh = a.s.B * a.s.H;
-    p.n_pair_items = bh * (p.n_q / 2);
-    p.n_items = p.n_pair_items + ((p.n_q & 1) ? (bh + 1) / 2 : 0);   // ragged tiles go two by two
     // two item counters alternate between launches: a launch consumes one and clears the other
     p.sched_counter = a.status + kStatusSched + (a.launch_parity & 1);
     p.sched_next = a.status + kStatusSched + ((a.launch_parity + 1) & 1);
     const bool elem_gate = p.gate_mode == 2 && p.gate != nullptr;
-    // The last wave: `rem` items on num_sms SMs.  Cut into k key ranges, the wave takes
-    // ceil(rem k / SMs) rounds of one part each; a part costs its share of the key iterations plus
-    // what every item costs (the readout iteration, the hand-over between items) plus the exchange
-    // of the partial rows -- measured: 3.3 k clk per iteration, 10.8 k per item, about 6 k for the
-    // exchange.  Take the k that makes the wave shortest, if that is shorter than leaving it whole.
-    // (At 3.7 k, what an iteration took before the issuers took turns, 26 to 28 key tiles were still cut in three
-    // where a third costs more than it saves: 6 heads x 3300 tokens 68 us, whole 62; 29 x 3456 218, 204;
-    // 17 x 3584 139, 125.)
-    p.n_whole = p.n_items;
-    p.k_split = 1;
-    if (!elem_gate && a.split_o != nullptr) {
-        const int waves = (p.n_items + num_sms - 1) / num_sms;
-        const int rem = p.n_items - (waves - 1) * num_sms;
-        const float iter = 3.31f, fixed = 10.8f, exchange = 6.0f;
-        float best = (p.n_kv + 1) * iter + fixed;
-        for (int k = 2; k <= kMaxSplit; ++k) {
-            if (p.n_kv < 4 * k || (long)rem * k * 2 > a.split_tile_parts) break;
-            const float part = ((float)p.n_kv / k + 1.0f) * iter + fixed + exchange;
-            const float cost = (float)((rem * k + num_sms - 1) / num_sms) * part;
-            if (cost < 0.95f * best) { best = cost; p.k_split = k; }
-        }
-        if (p.k_split > 1) p.n_whole = p.n_items - rem;
-    }
-    p.n_sched = p.n_whole + (p.n_items - p.n_whole) * p.k_split;
+    plan_items(a, num_sms, p);
     p.split_o = a.split_o;
     p.split_ml = a.split_ml;
     const int grid = p.n_sched < num_sms ? p.n_sched : num_sms;
