@@ -139,6 +139,7 @@ struct arl2_ctx {
     const void *wq, *wk, *wv;
     const float *rope_cos, *rope_sin;
     bool use_tc;
+    int simt_key_ctas;     // ... and the CTAs that share a unit of 16 rows
     bool simt_16_rows;     // plain-FMA step: the 16-row kernel is the faster one for this shape on this device
     uint64_t launches;
     uint32_t step_calls;   // parity selects the scheduler counter of the next step launch
@@ -240,6 +241,7 @@ int arl2_create(const arl2_config* cfg, void* d_state, void* d_workspace, size_t
     ctx->rope_cos = ctx->rope_sin = nullptr;
     ctx->use_tc = tc_supported(*cfg);
     ctx->simt_16_rows = false;
+    ctx->simt_key_ctas = 1;
     if (!ctx->use_tc) {
         int dev = 0, num_sms = 0;
         e = cudaGetDevice(&dev);
@@ -250,6 +252,7 @@ int arl2_create(const arl2_config* cfg, void* d_state, void* d_workspace, size_t
             return ARL2_ERR_CUDA;
         }
         ctx->simt_16_rows = simt_step_prefers_16_rows(ctx->shape, cfg->io_dtype, num_sms);
+        ctx->simt_key_ctas = simt_step_key_ctas(ctx->shape, num_sms);
     }
     ctx->launches = 0;
     ctx->step_calls = 0;
@@ -368,6 +371,7 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
         if (r == ARL2_OK) ++ctx->step_calls;
     } else {
         a.k_raw = step_rotates_k(ctx);
+        a.key_ctas = ctx->simt_key_ctas;
         r = account(ctx, simt_step(a, ctx->cfg.io_dtype, st));
     }
     if (e1 != nullptr) cudaEventRecord(e1, st);

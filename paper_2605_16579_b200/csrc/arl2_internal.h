@@ -47,6 +47,7 @@ struct StepArgs {
     const void* rope_h;     // [L, D/2] half2 (cos, sin) copy of the tables (tensor-core path), or nullptr
     int Lk = 0;             // > 0: K and V hold Lk tokens (a cache), [B, Lk, H, D]; 0: L
     bool k_made_before = false;   // the launch just before on the stream wrote k_rot and nothing else this step reads
+    int key_ctas = 1;       // with k_raw: CTAs that share a 16-row unit (simt_step_key_ctas)
     bool k_raw = false;     // plain-FMA path: the 16-row kernel; k_rot is the caller's K, which it rotates itself
     int gate_mode = 0;      // 0: gate [B, L, H]; 1: [B, L]; 2: [B, L, H, D]
     uint32_t wait_limit = 0;  // 0: default; n > 0: bounded waits give up after n - 1 polls (test hook)
@@ -121,6 +122,7 @@ int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, co
 // whether the 16-row step kernel is the faster one for this shape on a device of num_sms SMs.  It rotates K itself
 // (StepArgs::k_raw) and reads W_phi_q in 16-byte pieces.
 bool simt_step_prefers_16_rows(const Shape& s, int dtype, int num_sms);
+int simt_step_key_ctas(const Shape& s, int num_sms);
 int simt_step(const StepArgs& a, int dtype, cudaStream_t st);
 int simt_commit(const CommitArgs& a, int dtype, cudaStream_t st);
 int commit_reduce(const CommitArgs& a, cudaStream_t st);  // fixed-order sum + gated decay
@@ -198,20 +200,28 @@ __device__ __forceinline__ void grid_dependency_sync()
     grid_dependents_launch();
 }
 template <typename... P, typename... A>
-cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
+cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, int cluster, int threads, size_t smem, cudaStream_t st, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+template <typename... P, typename... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    return launch_cluster(kernel, grid, 1, threads, smem, st, args...);
 }
 
 }  // namespace arl2

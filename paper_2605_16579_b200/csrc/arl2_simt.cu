@@ -12,6 +12,10 @@
 //   partials in a fixed order and applies S <- sigmoid(a) S + sum.
 #include <math.h>
 
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
 #include "arl2_internal.h"
 
 namespace arl2 {
@@ -338,33 +342,48 @@ __global__ void __launch_bounds__(NT) simt_step_kernel(StepArgs a)
 // Lane (rg, kg) holds a 4 x KJ block of scores, rows 4 i + rg, keys 8 j + kg: every shared-memory read of the
 // products is a 16-byte one without bank conflicts, 8 (KJ = 4) or 6 (KJ = 2) of them per 4 columns for 64 or
 // 32 FMAs.
+//
+// Where even these units of 16 rows leave most SMs idle (simt_step_key_ctas), KS = 2 or 4 CTAs of a cluster share
+// a unit: each takes every KS-th key tile (smaller tiles, so that short sequences divide), the partial results
+// are exchanged through distributed shared memory, and each CTA finishes 16 / KS of the rows, two lanes per output
+// column halving the contraction of the other branch.  The kernel is bound by shared-memory reads of the SMs it
+// occupies: the 16 x 16 frame (2 heads, D = 64, 32 units) 13.7 us per pass on 32 SMs, 8.0 on 128; 2 heads x 500 tokens
+// (64 units, two CTAs each) 22.0 -> 15.7, at D = 128 48.4 -> 32.3, 2 x 200 at D = 128 30.0 -> 15.5.
 constexpr int SR = 16;
-template <int D>
+template <int D, int KS = 1>
 struct SmallCfg {
-    static constexpr int KT = D == 64 ? 256 : 128;     // keys per tile
+    static constexpr int KT = D == 64 ? 256 / KS : KS == 4 ? 64 : 128;     // keys per tile
+    static constexpr int KQ = KS == 1 ? 1 : 2;         // lanes per output column at the end
+    static constexpr int RR = SR / KS;                 // rows a CTA finishes
     static constexpr int KW = KT / 8, KJ = KW / 8;     // keys per warp, per lane
     static constexpr int LD = D + 4, LP = KW + 4;
-    static constexpr int kFloats = SR * LD + KT * LD + KT * D + 8 * SR * LP + 2 * 8 * SR;
+    static constexpr int kPs = 8 * SR * LP > SR * D + 2 * SR ? 8 * SR * LP : SR * D + 2 * SR;   // P, then the exchange
+    static constexpr bool kOwnW = D == 64;             // room for W_phi_q beside everything else
+    static constexpr int kFloats = SR * LD + KT * LD + KT * D + kPs + 2 * 8 * SR + D * D + (kOwnW ? D * D : 0);
 };
 
-template <int D, typename T>
-__global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
+template <int D, typename T, int KS>
+__global__ void __launch_bounds__(NT, 1) simt_step_small_kernel(StepArgs a)
 {
     grid_dependency_sync();
-    using C = SmallCfg<D>;
+    using C = SmallCfg<D, KS>;
+    constexpr int KQ = C::KQ, RR = C::RR;
     constexpr int KT = C::KT, KW = C::KW, KJ = C::KJ, LD = C::LD, LP = C::LP, CN = D / 32;
     extern __shared__ __align__(16) float smem[];
     float* Qs = smem;                  // [16][LD] rotated Q; later raw Q, then Q'
-    float* Ks = Qs + SR * LD;          // [KT][LD] rotated K tile; later the warps' O, then W_phi_q
-    float* Vs = Ks + KT * LD;          // [KT][D]  V tile; later S
+    float* Ks = Qs + SR * LD;          // [KT][LD] rotated K tile; later the warps' O, then (D = 128) W_phi_q
+    float* Vs = Ks + KT * LD;          // [KT][D]  V tile
     float* Ps = Vs + KT * D;           // [8][16][LP] probabilities, one block per warp
-    float* Ms = Ps + 8 * SR * LP;      // [8][16] reference maxima, then [8][16] row sums
+    float* Ms = Ps + C::kPs;           // [8][16] reference maxima, then [8][16] row sums
     float* Ls = Ms + 8 * SR;
+    float* Ss = Ls + 8 * SR;           // [D][D] state
+    float* Ws = C::kOwnW ? Ss + D * D : Ks;
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int rg = lane >> 3, kg = lane & 7;
     const int L = a.s.L, H = a.s.H;
-    const int i0 = blockIdx.x * SR, h = blockIdx.y, b = blockIdx.z;
+    const int rank = KS == 1 ? 0 : blockIdx.x % KS;    // this CTA in its cluster
+    const int i0 = blockIdx.x / KS * SR, h = blockIdx.y, b = blockIdx.z;
     const T* q = static_cast<const T*>(a.q);
     const T* k = static_cast<const T*>(a.k_rot);
     const T* v = static_cast<const T*>(a.v);
@@ -394,9 +413,44 @@ __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
     };
     const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 
-    for (int idx = tid; idx < SR * (D / 4); idx += NT) {
-        const int r = idx / (D / 4), c4 = idx % (D / 4);
-        *reinterpret_cast<float4*>(Qs + r * LD + c4 * 4) = i0 + r < L ? rotated4(q, i0 + r, c4) : zero4;
+    // What the branches after the loop need is fetched now: the state by asynchronous copies, the map (D = 64), the raw
+    // rows of Q, this thread's part of the rotation table and its gate in registers.
+    const float* Sh = a.state + ((size_t)b * H + h) * D * D;
+    for (int idx = tid; idx < D * D / 4; idx += NT)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(Ss + idx * 4))),
+                     "l"(Sh + idx * 4) : "memory");
+    const T* W = static_cast<const T*>(a.wq) + (size_t)h * D * D;
+    constexpr int kWPer = C::kOwnW ? D * D / 4 / NT : 1;
+    float4 wreg[kWPer];
+    if (C::kOwnW && a.wq != nullptr) {
+#pragma unroll
+        for (int i = 0; i < kWPer; ++i) wreg[i] = load4(W + (tid + i * NT) * 4);
+    }
+    constexpr int kQPer = SR * (D / 4) / NT;
+    float4 qraw[kQPer];
+#pragma unroll
+    for (int i = 0; i < kQPer; ++i) {
+        const int idx = tid + i * NT, qr = idx / (D / 4), c4 = idx % (D / 4);
+        qraw[i] = i0 + qr < L ? load4(q + (((size_t)b * L + i0 + qr) * H + h) * D + c4 * 4) : zero4;
+        *reinterpret_cast<float4*>(Qs + qr * LD + c4 * 4) = i0 + qr < L ? rotated4(q, i0 + qr, c4) : zero4;
+    }
+    // after the merge: thread = row r, columns 64 c + 4 t16 .., and which KQ-th of a contraction; a row's threads sit
+    // in one warp
+    const int kq = tid % KQ, t16 = tid / KQ & 15, r = rank * RR + tid / (16 * KQ), row = i0 + r;
+    const bool finishes = tid < RR * 16 * KQ && row < L;
+    const size_t rh = ((size_t)b * L + row) * H + h;
+    float2 cs_u[D / 64], sn_u[D / 64];
+    float gate_logit = 0.0f;
+    if (finishes) {
+        if (a.rope_cos != nullptr) {
+#pragma unroll
+            for (int c = 0; c < D / 64; ++c) {
+                const size_t at = (size_t)row * (D / 2) + c * 32 + t16 * 2;
+                cs_u[c] = *reinterpret_cast<const float2*>(a.rope_cos + at);
+                sn_u[c] = *reinterpret_cast<const float2*>(a.rope_sin + at);
+            }
+        }
+        if (a.gate_mode != 2) gate_logit = a.gate[a.gate_mode == 1 ? (size_t)b * L + row : rh];
     }
     float o[4][CN * 4];
     float mrun[4], lrun[4];
@@ -409,19 +463,26 @@ __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
     }
     float* Pw = Ps + w * SR * LP;
 
-    for (int j0 = 0; j0 < L; j0 += KT) {
+    for (int j0 = rank * KT; j0 < L; j0 += KS * KT) {
         __syncthreads();   // previous tile fully consumed
         constexpr int kPer = KT * (D / 4) / NT;
+        if constexpr (sizeof(T) == 4) {   // V beside the scores (rows past L: zeros, no bytes read)
 #pragma unroll 4
-        for (int it = 0; it < kPer; ++it) {
-            const int idx = tid + it * NT, r = idx / (D / 4), c4 = idx % (D / 4), row = j0 + r;
-            float4 kv = zero4, vv = zero4;
-            if (row < L) {
-                kv = rotated4(k, row, c4);
-                vv = load4(v + (((size_t)b * L + row) * H + h) * D + c4 * 4);
+            for (int it = 0; it < kPer; ++it) {
+                const int idx = tid + it * NT, kr = idx / (D / 4), c4 = idx % (D / 4), krow = j0 + kr;
+                const T* src = v + (((size_t)b * L + min(krow, L - 1)) * H + h) * D + c4 * 4;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                                 static_cast<uint32_t>(__cvta_generic_to_shared(Vs + kr * D + c4 * 4))),
+                             "l"(src), "r"(krow < L ? 16 : 0) : "memory");
             }
-            *reinterpret_cast<float4*>(Ks + r * LD + c4 * 4) = kv;
-            *reinterpret_cast<float4*>(Vs + r * D + c4 * 4) = vv;
+        }
+#pragma unroll 8
+        for (int it = 0; it < kPer; ++it) {
+            const int idx = tid + it * NT, kr = idx / (D / 4), c4 = idx % (D / 4), krow = j0 + kr;
+            *reinterpret_cast<float4*>(Ks + kr * LD + c4 * 4) = krow < L ? rotated4(k, krow, c4) : zero4;
+            if constexpr (sizeof(T) != 4)
+                *reinterpret_cast<float4*>(Vs + kr * D + c4 * 4) =
+                    krow < L ? load4(v + (((size_t)b * L + krow) * H + h) * D + c4 * 4) : zero4;
         }
         __syncthreads();
 
@@ -474,7 +535,8 @@ __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
 #pragma unroll
             for (int e = 0; e < CN * 4; ++e) o[i][e] *= corr;
         }
-        __syncwarp();
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();   // V (and the state) have landed
         // O += P V over this warp's keys: rows 4 i + rg, columns 32 c + 4 kg ..
         const float* vb = Vs + (w * KW) * D + kg * 4;
 #pragma unroll 2
@@ -499,9 +561,11 @@ __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
             }
         }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");   // (a CTA without keys has not waited for the state)
     __syncthreads();
     // ---- merge of the warps' results
-    float* Ow = Ks;                    // [8][16][D]
+    float* Ow = Ks;                    // [8][16][D], over the K tile (and the V tile behind it)
+    static_assert(KT * LD + KT * D >= 8 * SR * D, "the warps' O over the K and V tiles");
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int r = i * 4 + rg;
@@ -514,39 +578,80 @@ __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
             *reinterpret_cast<float4*>(Ow + (w * SR + r) * D + c * 32 + kg * 4) =
                 make_float4(o[i][c * 4], o[i][c * 4 + 1], o[i][c * 4 + 2], o[i][c * 4 + 3]);
     }
-    // (raw Q for the other branch takes the place of the rotated rows, S that of the last V tile)
-    for (int idx = tid; idx < SR * (D / 4); idx += NT) {
-        const int r = idx / (D / 4), c4 = idx % (D / 4);
-        *reinterpret_cast<float4*>(Qs + r * LD + c4 * 4) =
-            i0 + r < L ? load4(q + (((size_t)b * L + i0 + r) * H + h) * D + c4 * 4) : zero4;
+    // (raw Q for the other branch takes the place of the rotated rows)
+#pragma unroll
+    for (int i = 0; i < kQPer; ++i) {
+        const int idx = tid + i * NT, qr = idx / (D / 4), c4 = idx % (D / 4);
+        *reinterpret_cast<float4*>(Qs + qr * LD + c4 * 4) = qraw[i];
     }
-    const float* Sh = a.state + ((size_t)b * H + h) * D * D;
-#pragma unroll 4
-    for (int idx = tid; idx < D * D / 4; idx += NT)
-        *reinterpret_cast<float4*>(Vs + idx * 4) = *reinterpret_cast<const float4*>(Sh + idx * 4);
+    if (C::kOwnW && a.wq != nullptr) {
+#pragma unroll
+        for (int i = 0; i < kWPer; ++i) *reinterpret_cast<float4*>(Ws + (tid + i * NT) * 4) = wreg[i];
+    }
     __syncthreads();
-    // from here: thread = row r, columns 64 c + 4 t16 ..; the 16 threads of a row sit in one half warp
-    const int r = tid >> 4, t16 = tid & 15, row = i0 + r;
     float oi[D / 16];
     {
+        const int mr = tid >> 4, mt = tid & 15;   // row and columns 64 c + 4 mt .. of the merge
         float m_all = -INFINITY;
 #pragma unroll
-        for (int x = 0; x < 8; ++x) m_all = fmaxf(m_all, Ms[x * SR + r]);
+        for (int x = 0; x < 8; ++x) m_all = fmaxf(m_all, Ms[x * SR + mr]);
+        const float m_ref = KS > 1 && m_all == -INFINITY ? 0.0f : m_all;   // a CTA without keys: weights of 0
         float l_all = 0.0f;
 #pragma unroll
         for (int e = 0; e < D / 16; ++e) oi[e] = 0.0f;
 #pragma unroll
         for (int x = 0; x < 8; ++x) {
-            const float f = exp2f(Ms[x * SR + r] - m_all);
-            l_all = fmaf(f, Ls[x * SR + r], l_all);
+            const float f = exp2f(Ms[x * SR + mr] - m_ref);
+            l_all = fmaf(f, Ls[x * SR + mr], l_all);
 #pragma unroll
             for (int c = 0; c < D / 64; ++c) {
-                const float4 ov = *reinterpret_cast<const float4*>(Ow + (x * SR + r) * D + c * 64 + t16 * 4);
+                const float4 ov = *reinterpret_cast<const float4*>(Ow + (x * SR + mr) * D + c * 64 + mt * 4);
                 oi[c * 4 + 0] = fmaf(f, ov.x, oi[c * 4 + 0]);
                 oi[c * 4 + 1] = fmaf(f, ov.y, oi[c * 4 + 1]);
                 oi[c * 4 + 2] = fmaf(f, ov.z, oi[c * 4 + 2]);
                 oi[c * 4 + 3] = fmaf(f, ov.w, oi[c * 4 + 3]);
             }
+        }
+        if constexpr (KS > 1) {
+            // ---- the cluster's CTAs exchange their results: rows of O, then maxima and sums (over P, which is dead)
+            auto cluster = cooperative_groups::this_cluster();
+            float* Om = Ps;
+            float* Mm = Ps + SR * D;
+#pragma unroll
+            for (int c = 0; c < D / 64; ++c)
+                *reinterpret_cast<float4*>(Om + mr * D + c * 64 + mt * 4) = make_float4(oi[c * 4], oi[c * 4 + 1], oi[c * 4 + 2], oi[c * 4 + 3]);
+            if (mt == 0) {
+                Mm[mr] = m_all;
+                Mm[SR + mr] = l_all;
+            }
+            cluster.sync();
+            if (finishes) {
+                float mx[KS];
+                m_all = -INFINITY;
+#pragma unroll
+                for (int x = 0; x < KS; ++x) {
+                    mx[x] = cluster.map_shared_rank(Mm, x)[r];
+                    m_all = fmaxf(m_all, mx[x]);
+                }
+                l_all = 0.0f;
+#pragma unroll
+                for (int e = 0; e < D / 16; ++e) oi[e] = 0.0f;
+#pragma unroll
+                for (int x = 0; x < KS; ++x) {
+                    const float f = exp2f(mx[x] - m_all);
+                    l_all = fmaf(f, cluster.map_shared_rank(Mm, x)[SR + r], l_all);
+                    const float* src = cluster.map_shared_rank(Om, x) + r * D + t16 * 4;
+#pragma unroll
+                    for (int c = 0; c < D / 64; ++c) {
+                        const float4 ov = *reinterpret_cast<const float4*>(src + c * 64);
+                        oi[c * 4 + 0] = fmaf(f, ov.x, oi[c * 4 + 0]);
+                        oi[c * 4 + 1] = fmaf(f, ov.y, oi[c * 4 + 1]);
+                        oi[c * 4 + 2] = fmaf(f, ov.z, oi[c * 4 + 2]);
+                        oi[c * 4 + 3] = fmaf(f, ov.w, oi[c * 4 + 3]);
+                    }
+                }
+            }
+            asm volatile("barrier.cluster.arrive;" ::: "memory");   // this CTA has read what it needs of the others
         }
         const float inv = 1.0f / l_all;
 #pragma unroll
@@ -557,7 +662,7 @@ __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
 #pragma unroll
         for (int e = 0; e < D / 16; ++e) y[e] = 0.0f;
 #pragma unroll 4
-        for (int d = 0; d < D; d += 4) {
+        for (int d = kq * (D / KQ); d < (kq + 1) * (D / KQ); d += 4) {
             const float4 x4 = *reinterpret_cast<const float4*>(Qs + r * LD + d);
             const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
 #pragma unroll
@@ -571,61 +676,70 @@ __global__ void __launch_bounds__(NT) simt_step_small_kernel(StepArgs a)
                     y[c * 4 + 3] = fmaf(xv[e], m4.w, y[c * 4 + 3]);
                 }
         }
+        if (KQ == 2) {
+#pragma unroll
+            for (int e = 0; e < D / 16; ++e) y[e] += __shfl_xor_sync(0xffffffffu, y[e], 1);
+        }
     };
     // ---- inter branch: Q' = L2Norm(RoPE(Q W_phi_q)), then Q' S
     float u[D / 16];
     if (a.wq != nullptr) {
-        __syncthreads();               // the warps' O has been read
-        const T* W = static_cast<const T*>(a.wq) + (size_t)h * D * D;
-#pragma unroll 4
-        for (int idx = tid; idx < D * D / 4; idx += NT) *reinterpret_cast<float4*>(Ks + idx * 4) = load4(W + idx * 4);
-        __syncthreads();
-        row_times(Ks, u);
-    } else {
+        if (!C::kOwnW) {
+            __syncthreads();           // the warps' O has been read
+#pragma unroll 8
+            for (int idx = tid; idx < D * D / 4; idx += NT) *reinterpret_cast<float4*>(Ws + idx * 4) = load4(W + idx * 4);
+            __syncthreads();
+        }
+        if (tid < RR * 16 * KQ) row_times(Ws, u);   // (whole warps)
+    } else if (tid < RR * 16 * KQ) {
 #pragma unroll
         for (int c = 0; c < D / 64; ++c) {
             const float4 x4 = *reinterpret_cast<const float4*>(Qs + r * LD + c * 64 + t16 * 4);
             u[c * 4 + 0] = x4.x; u[c * 4 + 1] = x4.y; u[c * 4 + 2] = x4.z; u[c * 4 + 3] = x4.w;
         }
     }
-    float ss = 0.0f;
+    if (tid < RR * 16 * KQ) {
+        float ss = 0.0f;
 #pragma unroll
-    for (int c = 0; c < D / 64; ++c) {
-        if (a.rope_cos != nullptr && row < L) {
-            const size_t at = (size_t)row * (D / 2) + c * 32 + t16 * 2;
-            const float2 cs = *reinterpret_cast<const float2*>(a.rope_cos + at);
-            const float2 sn = *reinterpret_cast<const float2*>(a.rope_sin + at);
-            const float x0 = u[c * 4], x1 = u[c * 4 + 1], x2 = u[c * 4 + 2], x3 = u[c * 4 + 3];
-            u[c * 4 + 0] = x0 * cs.x - x1 * sn.x;
-            u[c * 4 + 1] = x0 * sn.x + x1 * cs.x;
-            u[c * 4 + 2] = x2 * cs.y - x3 * sn.y;
-            u[c * 4 + 3] = x2 * sn.y + x3 * cs.y;
+        for (int c = 0; c < D / 64; ++c) {
+            if (a.rope_cos != nullptr && row < L) {
+                const float2 cs = cs_u[c], sn = sn_u[c];
+                const float x0 = u[c * 4], x1 = u[c * 4 + 1], x2 = u[c * 4 + 2], x3 = u[c * 4 + 3];
+                u[c * 4 + 0] = x0 * cs.x - x1 * sn.x;
+                u[c * 4 + 1] = x0 * sn.x + x1 * cs.x;
+                u[c * 4 + 2] = x2 * cs.y - x3 * sn.y;
+                u[c * 4 + 3] = x2 * sn.y + x3 * cs.y;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) ss = fmaf(u[c * 4 + e], u[c * 4 + e], ss);
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) ss = fmaf(u[c * 4 + e], u[c * 4 + e], ss);
+        for (int off = 8 * KQ; off >= KQ; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+        const float rn = 1.0f / sqrtf(ss + a.s.eps);
+        __syncwarp();                      // the row's threads have read its row of Qs
+        if (kq == 0) {
+#pragma unroll
+            for (int c = 0; c < D / 64; ++c)
+                *reinterpret_cast<float4*>(Qs + r * LD + c * 64 + t16 * 4) =
+                    make_float4(u[c * 4] * rn, u[c * 4 + 1] * rn, u[c * 4 + 2] * rn, u[c * 4 + 3] * rn);
+        }
+        __syncwarp();
+        row_times(Ss, u);
     }
+    if (finishes && kq == 0) {
+        float gate = a.gate_mode == 2 ? 0.0f : sigmoidf_(gate_logit);
+        T* out = static_cast<T*>(a.out) + rh * D;
 #pragma unroll
-    for (int off = 8; off >= 1; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-    const float rn = 1.0f / sqrtf(ss + a.s.eps);
-    __syncwarp();                      // the half warp has read its row of Qs
+        for (int c = 0; c < D / 64; ++c)
 #pragma unroll
-    for (int c = 0; c < D / 64; ++c)
-        *reinterpret_cast<float4*>(Qs + r * LD + c * 64 + t16 * 4) =
-            make_float4(u[c * 4] * rn, u[c * 4 + 1] * rn, u[c * 4 + 2] * rn, u[c * 4 + 3] * rn);
-    __syncwarp();
-    row_times(Vs, u);
-    if (row >= L) return;
-    const size_t rh = ((size_t)b * L + row) * H + h;
-    float gate = a.gate_mode == 2 ? 0.0f : sigmoidf_(a.gate[a.gate_mode == 1 ? (size_t)b * L + row : rh]);
-    T* out = static_cast<T*>(a.out) + rh * D;
-#pragma unroll
-    for (int c = 0; c < D / 64; ++c)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int col = c * 64 + t16 * 4 + e;
-            if (a.gate_mode == 2) gate = sigmoidf_(a.gate[rh * D + col]);
-            from_f(out[col], oi[c * 4 + e] + gate * u[c * 4 + e]);
-        }
+            for (int e = 0; e < 4; ++e) {
+                const int col = c * 64 + t16 * 4 + e;
+                if (a.gate_mode == 2) gate = sigmoidf_(a.gate[rh * D + col]);
+                from_f(out[col], oi[c * 4 + e] + gate * u[c * 4 + e]);
+            }
+    }
+    // no CTA of a cluster ends while another may still read its shared memory
+    if constexpr (KS > 1) asm volatile("barrier.cluster.wait;" ::: "memory");
 }
 
 // partial[b, h, split] = K'^T V' over tokens [split*chunk, min(L, (split+1)*chunk)).
@@ -1154,11 +1268,18 @@ template <int D, typename T>
 int launch_step(const StepArgs& a, cudaStream_t st)
 {
     if (a.k_raw) {
-        constexpr size_t small_smem = sizeof(float) * SmallCfg<D>::kFloats;
-        if (int r = set_smem(simt_step_small_kernel<D, T>, small_smem)) return r;
-        if (int r = check_launch("simt_step_small_kernel",
-                                 launch_kernel(simt_step_small_kernel<D, T>, dim3((a.s.L + SR - 1) / SR, a.s.H, a.s.B), NT, small_smem, st, a)))
-            return r;
+        auto launch = [&](auto ks_tag) {
+            constexpr int KS = decltype(ks_tag)::value;
+            constexpr size_t small_smem = sizeof(float) * SmallCfg<D, KS>::kFloats;
+            static_assert(small_smem <= 232448, "shared memory");
+            if (int r = set_smem(simt_step_small_kernel<D, T, KS>, small_smem)) return r;
+            return check_launch("simt_step_small_kernel", launch_cluster(simt_step_small_kernel<D, T, KS>, dim3((a.s.L + SR - 1) / SR * KS, a.s.H, a.s.B),
+                                                                         KS, NT, small_smem, st, a));
+        };
+        const int r = a.key_ctas == 4   ? launch(std::integral_constant<int, 4>())
+                      : a.key_ctas == 2 ? launch(std::integral_constant<int, 2>())
+                                        : launch(std::integral_constant<int, 1>());
+        if (r) return r;
         return 1;
     }
     size_t smem = sizeof(float) * (2 * D * (BM + PAD) + BN * D + BM * (BM + PAD));
@@ -1359,6 +1480,16 @@ bool simt_step_prefers_16_rows(const Shape& s, int dtype, int num_sms)
     const float t64 = m.call64 + (per_sm64 / m.together * m.time_of[m.together - 1] + (rest ? m.time_of[rest - 1] : 0.0f)) *
                                      (m.fixed64 + m.tile64 * ((s.L + BN - 1) / BN));
     return t16 < 0.98f * t64;
+}
+
+// CTAs of a cluster that share a 16-row unit of that kernel: as many as find room beside one another (an eighth of the
+// SMs is left out of the count, as clusters do not cross the groups of SMs they are placed in).
+int simt_step_key_ctas(const Shape& s, int num_sms)
+{
+    const long units = (long)((s.L + SR - 1) / SR) * s.H * s.B;
+    for (int ks = 4; ks > 1; ks >>= 1)
+        if (8 * units * ks <= 7L * num_sms && s.L > SmallCfg<64, 4>::KT) return ks;
+    return 1;
 }
 
 int simt_step(const StepArgs& a, int dtype, cudaStream_t st)
