@@ -894,12 +894,27 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     const int row = tile * kTile + r;            // this thread's token
     const int chunk = r >> 6, jj = r & 63;       // chunk of the tile, index in the chunk
 
+    grid_dependency_sync();
+    // the gates and the rotation table are asked for before anything else: behind the first copies and MMAs, which
+    // keep the issuing warp, they held the whole CTA up by some 6 k of 44 k clk (12 heads x 4680 tokens 87.5 -> 83.1 us per
+    // pass, together with W leaving under the product for U1)
+    float alpha_logit = 0.0f, beta_logit = 0.0f;
+    uint4 cs[8];
+    if (row < L) {
+        const size_t gi = ((size_t)b * L + row) * H + h;
+        if (p.alpha != nullptr) alpha_logit = __ldg(p.alpha + gi);
+        if (p.beta != nullptr) beta_logit = __ldg(p.beta + gi);
+    }
+    if (p.rope_h != nullptr) {
+        const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16 + hf * 8) * 32 + (row & 31);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) cs[c] = __ldg(tab + c * 32);
+    }
     if (tid == 0) {
         for (int i = 0; i < kTPNumBars; ++i) mbar_init(bars + 8 * i, 1);
         *abort_flag = 0;
         fence_barrier_init();
         fence_proxy_async_smem();
-        grid_dependency_wait();
         const uint32_t bar_k = bars + 8 * kTPBarLoadK, bar_v = bars + 8 * kTPBarLoadV;
         mbar_expect_tx(bar_k, 2 * kTileBytes);
         mbar_expect_tx(bar_v, kTileBytes);
@@ -921,7 +936,6 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-    grid_dependency_sync();
 
     constexpr uint32_t kLboK = 1u << 16;
     constexpr uint32_t kLboMN = (uint32_t)(kHalfBytes >> 4) << 16;
@@ -956,31 +970,14 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
                        desc64(b_lo + (uint32_t)((c * 4 + ks) * (2048 >> 4))), idesc_kn, ks > 0);
     };
 
-    if (issuer) {
-        // ---- U_k = K W_phi_k -> columns 0-127
-        ok = wait_bar(bars + 8 * kTPBarLoadK, 0, ab, 90);
-        if (ok) {
-            tc_fence_after();
-            issue_kk(0, kTPOffK, kTPOffW);
-            mma_commit(bars + 8 * kTPBarUk);
-        }
-    }
-
     // ---- gates: log alpha_j, beta_j, cumulative decay within the chunk (tokens past L: 1 and 0)
     float la = 0.0f, be = 0.0f, cl = 0.0f;
-    uint4 cs[8];
     if (row < L) {
-        const size_t gi = ((size_t)b * L + row) * H + h;
         if (p.alpha != nullptr) {
-            const float x = __ldg(p.alpha + gi);
+            const float x = alpha_logit;
             la = x >= 0.0f ? -log1pf(expf(-x)) : x - log1pf(expf(x));
         }
-        be = p.beta != nullptr ? 1.0f / (1.0f + expf(-__ldg(p.beta + gi))) : 1.0f;
-    }
-    if (p.rope_h != nullptr) {
-        const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16 + hf * 8) * 32 + (row & 31);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) cs[c] = __ldg(tab + c * 32);
+        be = p.beta != nullptr ? 1.0f / (1.0f + expf(-beta_logit)) : 1.0f;
     }
     cl = la;   // inclusive scan over the 64 tokens of the chunk (two warps)
 #pragma unroll
@@ -993,6 +990,16 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     if (warp & 1) cl += wsum[warp - 1];
     if (hf == 0) cl_s[r] = cl;
     __syncthreads();
+    if (issuer) {
+        // ---- U_k = K W_phi_k -> columns 0-127
+        ok = wait_bar(bars + 8 * kTPBarLoadK, 0, ab, 90);
+        if (ok) {
+            tc_fence_after();
+            issue_kk(0, kTPOffK, kTPOffW);
+            mma_commit(bars + 8 * kTPBarUk);
+        }
+    }
+
     const float cl_total = cl_s[chunk * kTokC + kTokC - 1];
     const float cl_excl = cl - la;
     // log of the factor on K'_j S_0: g_{j-1} for Eq. 4 as printed, g_j when the token's prediction is made
@@ -1256,18 +1263,15 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
-    }
-    // ---- W and U1 leave as whole tiles
-    const bool all_ok = ok && alive && !*abort_flag;
-    if (issuer && all_ok) {
-        const int r0 = (int)((((size_t)b * H + h) * p.ntile + tile) * kTile);
+        // ---- it leaves as a whole tile
+        if (issuer && ok && alive && !*abort_flag) {
+            const int r0 = (int)((((size_t)b * H + h) * p.ntile + tile) * kTile);
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            tma_store_2d(&tm_w, smem_base + kTPOffK + half * kHalfBytes, half * 64, r0);
-            tma_store_2d(&tm_u1, smem_base + kTPOffV + half * kHalfBytes, half * 64, r0);
+            for (int half = 0; half < 2; ++half)
+                tma_store_2d(u == 0 ? &tm_w : &tm_u1, smem_base + (u == 0 ? kTPOffK : kTPOffV) + half * kHalfBytes, half * 64, r0);
         }
-        tma_store_wait_read();
     }
+    if (issuer) tma_store_wait_read();   // (whatever went out has been read)
     if (hf == 0 && alive && jj == kTokC - 1)
         p.gc[(((size_t)b * H + h) * p.ntile + tile) * 2 + chunk] = expf(cl_total);
     if (issuer && (!ok || *abort_flag)) {
