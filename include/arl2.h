@@ -19,8 +19,9 @@
  *     logits g: [B, L, H] fp32.  Decay logits a: [B, H] fp32.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls are
  *     asynchronous on it; ordering between calls is stream order.  (arl2_denoise_step_token_level
- *     may run part of its work on a stream of the context's own that forks from `stream` and joins it
- *     before the call returns; it is created at the first such call outside a stream capture.)
+ *     may run part of its work on a second stream that forks from `stream` and joins it before the
+ *     call returns; the context takes it at the first such call outside a stream capture, from a few that
+ *     the library keeps, and gives it back when it is destroyed.)
  *   - Every function returns an arl2_status (0 = ok, negative = error).  Argument errors
  *     are found on the host before any launch and leave S untouched.  Nothing aborts,
  *     traps or throws.  arl2_last_error() gives a thread-local message for the last error.

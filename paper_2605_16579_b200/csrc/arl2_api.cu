@@ -5,6 +5,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <mutex>
 #include <new>
 
 #include "arl2_internal.h"
@@ -130,6 +131,72 @@ Layout make_layout(const arl2_config& c)
 
 using namespace arl2;
 
+namespace {
+
+// A stream beside the caller's and the events that fork it and join it again.  Contexts borrow one at their first use and
+// give it back when they are destroyed: making one took 65 us of a context's first pass.  Work that an earlier holder left
+// on the stream only delays the next one's.
+struct Side {
+    int device = -1;
+    cudaStream_t stream = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+};
+constexpr int kMaxIdleSides = 8;
+std::mutex g_side_mutex;
+Side g_idle_sides[kMaxIdleSides];
+int g_n_idle_sides = 0;
+
+void destroy_side(Side& s)
+{
+    if (s.stream != nullptr) cudaStreamDestroy(s.stream);   // (what was launched there still runs to its end)
+    if (s.fork != nullptr) cudaEventDestroy(s.fork);
+    if (s.join != nullptr) cudaEventDestroy(s.join);
+    s = Side();
+    cudaGetLastError();
+}
+
+// One of the current device: an idle one, or a new one.
+bool borrow_side(Side& out)
+{
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
+    {
+        std::lock_guard<std::mutex> lock(g_side_mutex);
+        for (int i = 0; i < g_n_idle_sides; ++i) {
+            if (g_idle_sides[i].device != dev) continue;
+            out = g_idle_sides[i];
+            g_idle_sides[i] = g_idle_sides[--g_n_idle_sides];
+            return true;
+        }
+    }
+    Side s;
+    s.device = dev;
+    if (cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) != cudaSuccess || cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaGetLastError();
+        destroy_side(s);
+        return false;
+    }
+    out = s;
+    return true;
+}
+
+void return_side(Side& s)
+{
+    if (s.stream == nullptr) return;
+    {
+        std::lock_guard<std::mutex> lock(g_side_mutex);
+        if (g_n_idle_sides < kMaxIdleSides) {
+            g_idle_sides[g_n_idle_sides++] = s;
+            s = Side();
+            return;
+        }
+    }
+    destroy_side(s);
+}
+
+}  // namespace
+
 struct arl2_ctx {
     arl2_config cfg;
     Shape shape;
@@ -145,9 +212,7 @@ struct arl2_ctx {
     uint32_t step_calls;   // parity selects the scheduler counter of the next step launch
     int mirror;            // which of the two bf16 copies of S is current
     cudaEvent_t ev_before, ev_after;  // one-shot timing hook around the step kernel
-    // a stream of this context's own beside the caller's (arl2_denoise_step_token_level), created at its first use
-    cudaStream_t side;
-    cudaEvent_t ev_fork, ev_join;
+    Side side;             // stream beside the caller's (arl2_denoise_step_token_level), borrowed at its first use
     uint32_t wait_limit;   // 0: the kernels' default bound; n: waits give up after n - 1 polls (test hook)
     uint32_t walk_limit;   // the same for the first wait of the last thread block of arl2_commit_tokens' walk
     // projections around the core (arl2_set_projections)
@@ -445,24 +510,19 @@ bool fill_commit(arl2_ctx* ctx, CommitArgs& a, const void* d_k_clean, const void
 
 namespace {
 
-// The context's side stream, created at its first use (not while `st` is being captured).  False: there is none, and
-// the work goes to the caller's stream.
-bool have_side(arl2_ctx* ctx, cudaStream_t st)
+// Forks the context's side stream from `st` (borrowed at its first use, not while `st` is being captured).  False: there is
+// none, and the work goes to the caller's stream.
+bool fork_side(arl2_ctx* ctx, cudaStream_t st)
 {
-    if (ctx->side != nullptr) return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    if (ctx->side.stream == nullptr &&
+        (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone || !borrow_side(ctx->side))) {
         cudaGetLastError();
         return false;
     }
-    bool ok = ctx->ev_fork != nullptr || cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming) == cudaSuccess;
-    ok = ok && (ctx->ev_join != nullptr || cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) == cudaSuccess);
-    ok = ok && cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking) == cudaSuccess;
-    if (!ok) {
-        ctx->side = nullptr;
-        cudaGetLastError();
-    }
-    return ok;
+    if (cudaEventRecord(ctx->side.fork, st) == cudaSuccess && cudaStreamWaitEvent(ctx->side.stream, ctx->side.fork, 0) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
 }
 
 }  // namespace
@@ -506,21 +566,20 @@ int arl2_denoise_step_token_level(arl2_ctx* ctx, const void* d_q, const void* d_
     attach_split(ctx, plan);
     int step_ctas = 0, num_sms = 0;
     if (int r = tc_step_ctas(plan, &step_ctas, &num_sms)) return r;
-    const bool fork = !whole_heads && 4 * step_ctas <= 3 * num_sms && have_side(ctx, st) &&
-                      cudaEventRecord(ctx->ev_fork, st) == cudaSuccess && cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0) == cudaSuccess;
+    const bool fork = !whole_heads && 4 * step_ctas <= 3 * num_sms && fork_side(ctx, st);
     // 1. the intra-block softmax branch alone (closed gate) ...
     const void* k_rot = nullptr;
     int r = rotate_k(ctx, d_k, &k_rot, st);
     if (r == ARL2_OK) r = launch_step(ctx, d_q, k_rot, d_v, nullptr, d_out, st);
     // 2. ... the state at the start of every run of tiles ...
     if (!whole_heads) {
-        cudaStream_t ss = fork ? ctx->side : st;
+        cudaStream_t ss = fork ? ctx->side.stream : st;
         if (r == ARL2_OK && d_alpha_logits != nullptr)
             r = account(ctx, run_decay_weights(ctx->shape, d_alpha_logits, w, totals, share, ntile, seg.nslot, ss));
         if (r == ARL2_OK) r = account(ctx, tc_commit_partials(seg, wk_op, ss));
         if (r == ARL2_OK) r = account(ctx, tc_run_prefix(seg, d_alpha_logits != nullptr ? totals : nullptr, ss));
         // (the streams join whatever became of the launches)
-        if (fork && (cudaEventRecord(ctx->ev_join, ctx->side) != cudaSuccess || cudaStreamWaitEvent(st, ctx->ev_join, 0) != cudaSuccess) &&
+        if (fork && (cudaEventRecord(ctx->side.join, ctx->side.stream) != cudaSuccess || cudaStreamWaitEvent(st, ctx->side.join, 0) != cudaSuccess) &&
             r == ARL2_OK) {
             set_error("denoise_step_token_level: %s", cudaGetErrorString(cudaGetLastError()));
             r = ARL2_ERR_CUDA;
@@ -930,9 +989,7 @@ const char* arl2_step_kernel_name(const arl2_ctx* ctx)
 void arl2_destroy(arl2_ctx* ctx)
 {
     if (ctx == nullptr) return;
-    if (ctx->side != nullptr) cudaStreamDestroy(ctx->side);   // (what was launched there still runs to its end)
-    if (ctx->ev_fork != nullptr) cudaEventDestroy(ctx->ev_fork);
-    if (ctx->ev_join != nullptr) cudaEventDestroy(ctx->ev_join);
+    return_side(ctx->side);
     delete ctx;
 }
 
