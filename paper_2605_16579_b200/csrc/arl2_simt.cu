@@ -1458,7 +1458,8 @@ int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, co
 // The model (us: once per call, then per round a fixed part and a part per key tile; the time of 1, 2, 3 64-row
 // CTAs on an SM relative to one) was fitted to 130 shapes of 48 to 4614 tokens with 1 to 192 heads.  There it
 // picks the slower kernel nowhere by more than 8 %, in the mean by 0.2 % (always the 64-row kernel: 53 %; the 16-row
-// kernel at D = 128 and up to 156 tiles at D = 64: 3 %, 47 % at most).  At even times the 64-row kernel is taken.
+// kernel at D = 128 and up to 156 tiles at D = 64: 3 %, 47 % at most).  At even times the 64-row kernel is taken.  (The model
+// is of one CTA per unit: where clusters serve a shape, its one round goes to the 16-row kernel in any case.)
 bool simt_step_prefers_16_rows(const Shape& s, int dtype, int num_sms)
 {
     struct Model {
