@@ -19,6 +19,7 @@
 //
 // Every wait is bounded: when a limit expires the thread records ARL2_ERR_TIMEOUT in the
 // device status block, raises the CTA's abort flag and every role falls through to the exit.
+#include <type_traits>
 
 #include "tc_common.cuh"
 
@@ -832,9 +833,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 //   W = T diag(beta g) K', then U1 = T diag(beta) V': one MMA per chunk over all 128 rows, each token row
 //   read from its own chunk's result -> global: W, U1 (and Khat on the way) in bf16, chunk decays g in fp32.
 // 12 heads x 4680 tokens (444 tiles), inside the call: 66 us with one 128-thread CTA per SM, T by one 64-step
-// substitution per column and row-wise stores -> 42 us; 40 heads 205 -> 112 (each alone).  With the block products of
-// the inverse on FMAs from shared memory (7.7 of 44 k clk of a CTA) the whole call took 83.1 us, on the warp-level tensor
-// instruction 77.4; 40 heads x 3000 tokens 148.8 -> 134.2.
+// substitution per column and row-wise stores -> 42 us; 40 heads 205 -> 112 (each alone).
 // tc_token_scan_kernel: walks the chunks of a head in order (further down).
 // ---------------------------------------------------------------------------------------------
 constexpr int kTPOffK = 0;                         // raw K tile -> K' -> diag(beta g) K'
@@ -868,54 +867,6 @@ struct TcTokenParams {
     int nchunk;                // ceil(L / 64): chunks the scan walks
     int decayed;               // prediction against alpha_j S_{j-1}
 };
-
-__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-                 "{%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// x = head + remainder, both bf16 (two values at a time)
-__device__ __forceinline__ void split_bf16(float x0, float x1, uint32_t& head, uint32_t& rem)
-{
-    head = pack_bf16(x0, x1);
-    rem = pack_bf16(x0 - __uint_as_float(head << 16), x1 - __uint_as_float(head & 0xFFFF0000u));
-}
-// One warp: out(i0 .. i0 + 15, j0 .. j0 + 8 NB - 1) = sign * sum over k < N of P(i, k) Q(k, j), matrices column by column
-// (element (i, k) at [k * kLdA + i]).  On the warp-level tensor instruction with every operand split into a bf16 head and
-// remainder, three products of the four (relative error 2^-16; the result is rounded to bf16 in the end).
-template <int N, int NB>
-__device__ __forceinline__ void block_product(const float* P, const float* Q, float* out, float sign, int i0, int j0, int lane)
-{
-    const int g = lane >> 2, t2 = (lane & 3) * 2;
-    float acc[NB][4] = {};
-#pragma unroll
-    for (int ks = 0; ks < N; ks += 16) {
-        uint32_t ah[4], al[4];
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const float* src = P + (ks + t2 + (x >> 1) * 8) * kLdA + i0 + g + (x & 1) * 8;
-            split_bf16(src[0], src[kLdA], ah[x], al[x]);
-        }
-#pragma unroll
-        for (int n = 0; n < NB; ++n) {
-            const float* src = Q + (j0 + n * 8 + g) * kLdA + ks + t2;
-            const float2 q0 = *reinterpret_cast<const float2*>(src), q1 = *reinterpret_cast<const float2*>(src + 8);
-            uint32_t bh0, bl0, bh1, bl1;
-            split_bf16(q0.x, q0.y, bh0, bl0);
-            split_bf16(q1.x, q1.y, bh1, bl1);
-            mma_16816(acc[n], al, bh0, bh1);
-            mma_16816(acc[n], ah, bl0, bl1);
-            mma_16816(acc[n], ah, bh0, bh1);
-        }
-    }
-#pragma unroll
-    for (int n = 0; n < NB; ++n)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) out[(j0 + n * 8 + t2 + (x & 1)) * kLdA + i0 + g + (x >> 1) * 8] = sign * acc[n][x];
-}
 
 __global__ void __launch_bounds__(kTPThreads, 2)
 tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
@@ -1220,27 +1171,49 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
                 *reinterpret_cast<float4*>(Xd + cc * kLdA + i4 * 4) = make_float4(t[i4 * 4], t[i4 * 4 + 1], t[i4 * 4 + 2], t[i4 * 4 + 3]);
         }
         __syncthreads();
+        // out(i, j0 .. j0 + NJ) = sum over k < N of P(i, k) Q(k, j): each operand given by its first
+        // element; i runs over the lanes, k is contiguous in Q
+        auto product = [&](auto n_tag, auto nj_tag, const float* P, const float* Q, float* out, float sign, int i, int j0) {
+            constexpr int N = decltype(n_tag)::value, NJ = decltype(nj_tag)::value;
+            float acc[NJ] = {};
+#pragma unroll
+            for (int k4 = 0; k4 < N; k4 += 4) {
+                float pv[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) pv[k] = P[(k4 + k) * kLdA + i];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    const float4 q = *reinterpret_cast<const float4*>(Q + (j0 + j) * kLdA + k4);
+                    acc[j] = fmaf(pv[0], q.x, fmaf(pv[1], q.y, fmaf(pv[2], q.z, fmaf(pv[3], q.w, acc[j]))));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) out[(j0 + j) * kLdA + i] = sign * acc[j];
+        };
         {
             // blocks of 16: rows 32 m + 16 .., columns 32 m ..; the intermediate A21 T11 goes to the unused
-            // rows 0-15 of columns 32 + 16 m ..; a warp takes 8 of a block's columns
-            const int c = warp >> 2, m = warp >> 1 & 1, j0 = (warp & 1) * 8;
+            // rows 0-15 of columns 32 + 16 m ..
+            const int c = tid >> 7, m = tid >> 6 & 1, u = tid & 63;
             float* X = As + c * kTokC * kLdA;
             float* low = X + (m * 32) * kLdA + m * 32 + 16;
             float* tmp = X + (32 + m * 16) * kLdA;
-            block_product<16, 1>(low, X + (m * 32) * kLdA + m * 32, tmp, 1.0f, 0, j0, lane);
+            product(std::integral_constant<int, 16>(), std::integral_constant<int, 4>(), low, X + (m * 32) * kLdA + m * 32, tmp, 1.0f,
+                    u & 15, (u >> 4) * 4);
             __syncthreads();
-            block_product<16, 1>(X + (m * 32 + 16) * kLdA + m * 32 + 16, tmp, low, -1.0f, 0, j0, lane);
+            product(std::integral_constant<int, 16>(), std::integral_constant<int, 4>(), X + (m * 32 + 16) * kLdA + m * 32 + 16, tmp, low,
+                    -1.0f, u & 15, (u >> 4) * 4);
             __syncthreads();
         }
         {
-            // blocks of 32: rows 32 .., columns 0 ..; the intermediate in rows 0-31 of columns 32 ..; a warp takes 16 x 16
-            const int c = warp >> 2, i0 = (warp & 1) * 16, j0 = (warp >> 1 & 1) * 16;
+            // blocks of 32: rows 32 .., columns 0 ..; the intermediate in rows 0-31 of columns 32 ..
+            const int c = tid >> 7, u = tid & 127;
             float* X = As + c * kTokC * kLdA;
             float* low = X + 32;
             float* tmp = X + 32 * kLdA;
-            block_product<32, 2>(low, X, tmp, 1.0f, i0, j0, lane);
+            product(std::integral_constant<int, 32>(), std::integral_constant<int, 8>(), low, X, tmp, 1.0f, u & 31, (u >> 5) * 8);
             __syncthreads();
-            block_product<32, 2>(X + 32 * kLdA + 32, tmp, low, -1.0f, i0, j0, lane);
+            product(std::integral_constant<int, 32>(), std::integral_constant<int, 8>(), X + 32 * kLdA + 32, tmp, low, -1.0f, u & 31,
+                    (u >> 5) * 8);
             __syncthreads();
         }
         // T as a K-major swizzled operand (row = token, 64 columns), over the fp32 matrix
@@ -1356,6 +1329,14 @@ __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr)
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+                 "{%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
 template <int kSlabs, bool kShared>
 __global__ void __launch_bounds__(kSlabs * 128 + 32, kShared ? 2 : 1)
 tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_kh,
