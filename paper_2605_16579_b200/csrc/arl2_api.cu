@@ -431,8 +431,8 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
     if (ctx->use_tc) {
         r = account(ctx, tc_step(a, reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wq_op),
                                  mirror_of(ctx), st));
-        // the launch consumed one scheduler counter and cleared the other: only a launch that
-        // really went out moves on to the other one
+        // the launch uses one scheduler counter and clears the other: only a launch that really went out
+        // moves on to the other one
         if (r == ARL2_OK) ++ctx->step_calls;
     } else {
         a.k_raw = step_rotates_k(ctx);

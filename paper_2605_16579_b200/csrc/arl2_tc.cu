@@ -69,8 +69,8 @@ struct TcStepParams {
     uint32_t* status;
     uint32_t spin_limit;       // polls a bounded wait makes before it gives up
     int k_made_before;         // the kernel before this one made K and nothing else that is read or written here
-    uint32_t* sched_counter;   // this launch's item counter (zero on entry)
-    uint32_t* sched_next;      // the next launch's counter: cleared by this launch
+    uint32_t* sched_counter;   // this launch's item counter (zero on entry, and again once every item has run)
+    uint32_t* sched_next;      // the next launch's counter: cleared by this launch (the one before may have given up on a wait)
     int gate_mode;             // 0: gate logits [B, L, H]; 1: [B, L] (one per token); 2: [B, L, H, D] (per channel)
     int Lk;                    // keys per head: L, or the length of a key/value cache (Eq. 1)
     int n_q;                   // query tiles per head
@@ -616,7 +616,11 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     }
                 }
                 if (!ok) break;
-                id = (int)gridDim.x + (int)atomicAdd(p.sched_counter, 1u);
+                // Every item is followed by one draw, so the launch makes n_sched of them: the last leaves the counter as it
+                // was found, and the same launch may run again (a graph that is replayed).
+                const uint32_t drawn = atomicAdd(p.sched_counter, 1u);
+                if (drawn + 1 == (uint32_t)p.n_sched) *p.sched_counter = 0;
+                id = (int)gridDim.x + (int)drawn;
             }
             if (!ok || *abort_flag) {
                 // do not leave the CTA while bulk copies into its shared memory are in flight
@@ -1815,7 +1819,7 @@ int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* 
     p.out = static_cast<__nv_bfloat16*>(a.out);
     p.status = a.status;
     p.spin_limit = a.wait_limit ? a.wait_limit - 1 : kSpinLimit;
-    // two item counters alternate between launches: a launch consumes one and clears the other
+    // two item counters alternate between launches: a launch uses one and clears the other
     p.sched_counter = a.status + kStatusSched + (a.launch_parity & 1);
     p.sched_next = a.status + kStatusSched + ((a.launch_parity + 1) & 1);
     const bool elem_gate = p.gate_mode == 2 && p.gate != nullptr;
