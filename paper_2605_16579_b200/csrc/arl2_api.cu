@@ -102,7 +102,7 @@ Layout make_layout(const arl2_config& c)
     }
     l.partials = off;   off += align_up((size_t)c.B * c.H * l.nslot * dd * sizeof(float));
     l.partials_g = off; off += align_up((size_t)c.B * c.H * l.nslot * dd * sizeof(float));   // delta rule
-    // two bf16 operand copies of S: a tensor-core commit writes the one that is not current
+    // two bf16 operand copies of S: the delta rule reads the current one while it writes the other
     l.state_bf16 = off; off += align_up((size_t)c.B * c.H * dd * 2);
     l.state_bf16_b = off; off += align_up((size_t)c.B * c.H * dd * 2);
     l.wq_op = off;      off += align_up((size_t)c.H * dd * 2);
@@ -210,7 +210,8 @@ struct arl2_ctx {
     bool simt_16_rows;     // plain-FMA step: the 16-row kernel is the faster one for this shape on this device
     uint64_t launches;
     uint32_t step_calls;   // parity selects the scheduler counter of the next step launch
-    int mirror;            // which of the two bf16 copies of S is current
+    int mirror;            // which of the two bf16 copies of S is current (a delta-rule commit changes it)
+    bool mirror_pinned;    // ... and no longer may, since captured work holds its address
     cudaEvent_t ev_before, ev_after;  // one-shot timing hook around the step kernel
     Side side;             // stream beside the caller's (arl2_denoise_step_token_level), borrowed at its first use
     uint32_t wait_limit;   // 0: the kernels' default bound; n: waits give up after n - 1 polls (test hook)
@@ -236,6 +237,16 @@ __nv_bfloat16* mirror_of(const arl2_ctx* ctx, int which = 0)
 {
     const size_t off = ((ctx->mirror ^ which) & 1) ? ctx->lay.state_bf16_b : ctx->lay.state_bf16;
     return reinterpret_cast<__nv_bfloat16*>(ctx->ws + off);
+}
+
+// What is captured holds the address of the current mirror and may run any number of times, or never, among eager calls:
+// from then on it has to stay the current one.
+void pin_mirror_under_capture(arl2_ctx* ctx, cudaStream_t st)
+{
+    if (ctx->mirror_pinned) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+    ctx->mirror_pinned = cap != cudaStreamCaptureStatusNone;
 }
 
 // whether the plain-FMA step of this context runs on the 16-row kernel, which rotates K itself
@@ -322,6 +333,7 @@ int arl2_create(const arl2_config* cfg, void* d_state, void* d_workspace, size_t
     ctx->launches = 0;
     ctx->step_calls = 0;
     ctx->mirror = 0;
+    ctx->mirror_pinned = false;
     ctx->w_pack = ctx->w_o = nullptr;
     ctx->pack_cols = 0;
     ctx->wait_limit = cfg->flags >> ARL2_FLAG_DEBUG_WAIT_LIMIT_SHIFT;
@@ -429,6 +441,7 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
     if (e0 != nullptr) cudaEventRecord(e0, st);
     int r;
     if (ctx->use_tc) {
+        pin_mirror_under_capture(ctx, st);
         r = account(ctx, tc_step(a, reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wq_op),
                                  mirror_of(ctx), st));
         // the launch uses one scheduler counter and clears the other: only a launch that really went out
@@ -492,7 +505,7 @@ bool fill_commit(arl2_ctx* ctx, CommitArgs& a, const void* d_k_clean, const void
     a.partials = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials);
     a.partials_g = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials_g);
     a.state_bf16 = ctx->use_tc ? mirror_of(ctx) : nullptr;
-    a.state_bf16_next = ctx->use_tc ? mirror_of(ctx, 1) : nullptr;
+    a.state_bf16_next = ctx->use_tc ? mirror_of(ctx, mode == 1 ? 1 : 0) : nullptr;
     a.nsplit = ctx->lay.nsplit;
     a.nslot = ctx->lay.nslot;
     a.rope_h = (ctx->use_tc && ctx->rope_cos != nullptr) ? ctx->ws + ctx->lay.rope_h : nullptr;
@@ -687,13 +700,23 @@ int arl2_set_profile_events(arl2_ctx* ctx, void* ev_before, void* ev_after)
 
 namespace {
 
-// The second half of a tensor-core commit: the new state goes to S and to the mirror that was not
-// current, which becomes the current one.
+// The second half of a tensor-core commit: the new state goes to S and to its mirror.  The delta rule reads the whole of
+// the mirror as an operand, so it writes the other one, which becomes the current one, or is copied to it where the
+// mirror is pinned.
 int finish_commit(arl2_ctx* ctx, const CommitArgs& a, cudaStream_t st)
 {
+    pin_mirror_under_capture(ctx, st);
     int r = account(ctx, tc_commit_finish(a, st));
-    if (r == ARL2_OK) ctx->mirror ^= 1;
-    return r;
+    if (r != ARL2_OK || a.mode != 1) return r;
+    if (!ctx->mirror_pinned) {
+        ctx->mirror ^= 1;
+        return r;
+    }
+    const size_t bytes = (size_t)a.s.B * a.s.H * a.s.D * a.s.D * sizeof(__nv_bfloat16);
+    const cudaError_t e = cudaMemcpyAsync(mirror_of(ctx), a.state_bf16_next, bytes, cudaMemcpyDeviceToDevice, st);
+    if (e == cudaSuccess) return r;
+    set_error("commit_delta: %s", cudaGetErrorString(e));
+    return ARL2_ERR_CUDA;
 }
 
 // Shared by arl2_commit, arl2_commit_delta and arl2_commit_decay_tokens.
@@ -782,12 +805,14 @@ int arl2_commit_tokens(arl2_ctx* ctx, const void* d_k_clean, const void* d_v_cle
         set_error("commit_tokens: k_clean and v_clean must be 16-byte aligned");
         return ARL2_ERR_INVALID_ARG;
     }
-    if (ctx->use_tc)
+    if (ctx->use_tc) {
+        pin_mirror_under_capture(ctx, as_stream(stream));
         return account(ctx, tc_commit_tokens(
                                 a, reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wk_op),
                                 reinterpret_cast<const __nv_bfloat16*>(ctx->ws + ctx->lay.wv_op),
                                 ctx->rope_cos != nullptr ? ctx->ws + ctx->lay.rope_h : nullptr,
                                 reinterpret_cast<uint32_t*>(ctx->ws + ctx->lay.status), as_stream(stream)));
+    }
     return account(ctx, simt_commit_tokens(a, ctx->cfg.io_dtype, as_stream(stream)));
 }
 
@@ -920,6 +945,7 @@ int arl2_reset(arl2_ctx* ctx, int32_t stream_index, void* stream)
     int r = account(ctx, fill_zero(ctx->state + first, count * sizeof(float), st));
     if (r != ARL2_OK) return r;
     if (ctx->use_tc) {
+        pin_mirror_under_capture(ctx, st);
         auto* sb = mirror_of(ctx);
         r = account(ctx, fill_zero(sb + first, count * 2, st));
     }
@@ -950,10 +976,10 @@ int arl2_set_state(arl2_ctx* ctx, const float* src, void* stream)
         set_error("set_state: %s", cudaGetErrorString(e));
         return ARL2_ERR_CUDA;
     }
-    if (ctx->use_tc)
-        return account(ctx, state_to_bf16(ctx->state,
-                                          mirror_of(ctx),
-                                          n, st));
+    if (ctx->use_tc) {
+        pin_mirror_under_capture(ctx, st);
+        return account(ctx, state_to_bf16(ctx->state, mirror_of(ctx), n, st));
+    }
     return ARL2_OK;
 }
 

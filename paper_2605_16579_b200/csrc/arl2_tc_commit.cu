@@ -22,9 +22,9 @@
 // static, so the fixed-order sum of the finishing kernel is bitwise reproducible.
 //
 // tc_commit_finish_kernel: S <- alpha S + (sum of slots) W_phi_v [- (sum of G slots) S_old], fp32
-// FMA arithmetic, 16 state rows per CTA; also writes the bf16 operand copy of the new state into
-// the OTHER of two mirror buffers (the delta rule reads S_old from the current one while rows
-// are being replaced, so the mirrors alternate from commit to commit).
+// FMA arithmetic, 16 state rows per CTA; also writes the bf16 operand copy of the new state: into the
+// mirror itself, but with the delta rule into the OTHER of two buffers (it reads S_old from the
+// current one while rows are being replaced).
 //
 // Every wait is bounded (see wait_bar); a CTA that gives up records ARL2_ERR_TIMEOUT, drains its
 // copies and MMAs in flight and frees its tensor memory; the finishing kernel then leaves S alone.

@@ -60,3 +60,43 @@ def test_a_captured_step_is_replayed(B, H, L):
     layer.denoise_step(q, k, v, g, out=out)
     assert torch.equal(_bits(out), ref)
     layer.sync_status()
+
+
+@pytest.mark.parametrize("kind", ["commit", "delta", "decay", "tokens", "clean"])
+def test_a_captured_block_is_replayed(kind):
+    """Two denoise passes and the state update: every replay reads the state that the one before left."""
+    cfg, S = _cfg(2, 3, 300)
+    flags = arl2.ARL2_FLAG_TOKEN_GATES if kind == "tokens" else 0
+    q, k, v, g = (t.to(DEV) for t in workload.step_inputs(cfg, 0, 0))
+    kc, vc, a = (t.to(DEV) for t in workload.commit_inputs(cfg, 0))
+    alpha, beta = (t.to(DEV) for t in workload.token_gate_logits(cfg, 0))
+    eager, captured = _layer(cfg, S, flags), _layer(cfg, S, flags)
+
+    def block(layer, outs):
+        layer.denoise_step(q, k, v, g, out=outs[0])
+        layer.denoise_step(k, q, v, g, out=outs[1])
+        if kind == "commit":
+            layer.commit(kc, vc, a)
+        elif kind == "delta":
+            layer.commit_delta(kc, vc, a, beta)
+        elif kind == "decay":
+            layer.commit_decay_tokens(kc, vc, alpha)
+        elif kind == "tokens":
+            layer.commit_tokens(kc, vc, alpha, beta)
+        else:
+            layer.clean_pass(q, kc, vc, g, a, out=outs[2])
+
+    outs_e, outs_c = ([torch.zeros_like(q) for _ in range(3)] for _ in range(2))
+    graph = _capture(lambda: block(captured, outs_c))   # (has run nothing: the state is as it was)
+    for i in range(5):
+        block(eager, outs_e)
+        if i in (0, 4):                                  # eager calls before and after the replays
+            block(captured, outs_c)
+        else:
+            graph.replay()
+        torch.cuda.synchronize()
+        for e, c in zip(outs_e, outs_c):
+            assert torch.equal(_bits(e), _bits(c)), f"block {i}"
+        assert torch.equal(_bits(eager.state), _bits(captured.state)), f"block {i}"
+    for layer in (eager, captured):
+        layer.sync_status()
