@@ -135,64 +135,105 @@ namespace {
 
 // A stream beside the caller's and the events that fork it and join it again.  Contexts borrow one at their first use and
 // give it back when they are destroyed: making one took 65 us of a context's first pass.  Work that an earlier holder left
-// on the stream only delays the next one's.
+// on the stream only delays the next one's.  A stream that an open capture has taken in may not wait for anything
+// outside that capture (it would end in an error, and the capture with it): until the capture ends, such a stream is only
+// for calls that are part of it.
 struct Side {
     int device = -1;
     cudaStream_t stream = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
+    Side* next = nullptr;   // among the idle ones
 };
-constexpr int kMaxIdleSides = 8;
+constexpr int kMaxIdleSides = 8;   // (more only while captures hold them)
 std::mutex g_side_mutex;
-Side g_idle_sides[kMaxIdleSides];
-int g_n_idle_sides = 0;
+Side* g_idle_sides = nullptr;
 
-void destroy_side(Side& s)
+struct Capture {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusInvalidated;   // (also where it cannot be read)
+    unsigned long long id = 0;
+    bool none() const { return status == cudaStreamCaptureStatusNone; }
+};
+Capture capture_of(cudaStream_t st)
 {
-    if (s.stream != nullptr) cudaStreamDestroy(s.stream);   // (what was launched there still runs to its end)
-    if (s.fork != nullptr) cudaEventDestroy(s.fork);
-    if (s.join != nullptr) cudaEventDestroy(s.join);
-    s = Side();
+    Capture c;
+    if (cudaStreamGetCaptureInfo(st, &c.status, &c.id) != cudaSuccess) {
+        cudaGetLastError();
+        c = Capture();
+    }
+    return c;
+}
+
+// Streams and events are made and destroyed whatever this or another thread is capturing.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    bool set;
+    RelaxedCapture() { set = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess; }
+    ~RelaxedCapture()
+    {
+        if (set) cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+};
+
+void destroy_side(Side* s)
+{
+    RelaxedCapture relaxed;
+    if (s->stream != nullptr) cudaStreamDestroy(s->stream);   // (what was launched there still runs to its end)
+    if (s->fork != nullptr) cudaEventDestroy(s->fork);
+    if (s->join != nullptr) cudaEventDestroy(s->join);
+    delete s;
     cudaGetLastError();
 }
 
-// One of the current device: an idle one, or a new one.
-bool borrow_side(Side& out)
+// One of the current device: an idle one, or a new one, or nullptr.
+Side* borrow_side()
 {
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     {
         std::lock_guard<std::mutex> lock(g_side_mutex);
-        for (int i = 0; i < g_n_idle_sides; ++i) {
-            if (g_idle_sides[i].device != dev) continue;
-            out = g_idle_sides[i];
-            g_idle_sides[i] = g_idle_sides[--g_n_idle_sides];
-            return true;
+        for (Side** at = &g_idle_sides; *at != nullptr; at = &(*at)->next) {
+            Side* s = *at;
+            if (s->device != dev || !capture_of(s->stream).none()) continue;
+            *at = s->next;
+            s->next = nullptr;
+            return s;
         }
     }
-    Side s;
-    s.device = dev;
-    if (cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) != cudaSuccess || cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking) != cudaSuccess) {
+    Side* s = new (std::nothrow) Side;
+    if (s == nullptr) return nullptr;
+    s->device = dev;
+    RelaxedCapture relaxed;
+    if (cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) != cudaSuccess || cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         destroy_side(s);
-        return false;
+        return nullptr;
     }
-    out = s;
-    return true;
+    return s;
 }
 
-void return_side(Side& s)
+void return_side(Side* s)
 {
-    if (s.stream == nullptr) return;
+    if (s == nullptr) return;
+    Side* surplus = nullptr;
     {
         std::lock_guard<std::mutex> lock(g_side_mutex);
-        if (g_n_idle_sides < kMaxIdleSides) {
-            g_idle_sides[g_n_idle_sides++] = s;
-            s = Side();
-            return;
+        s->next = g_idle_sides;
+        g_idle_sides = s;
+        int idle = 0;
+        for (Side** at = &g_idle_sides; *at != nullptr;) {
+            Side* x = *at;
+            if (!capture_of(x->stream).none() || ++idle <= kMaxIdleSides) { at = &x->next; continue; }
+            *at = x->next;
+            x->next = surplus;
+            surplus = x;
         }
     }
-    destroy_side(s);
+    while (surplus != nullptr) {
+        Side* x = surplus;
+        surplus = x->next;
+        destroy_side(x);
+    }
 }
 
 }  // namespace
@@ -213,7 +254,7 @@ struct arl2_ctx {
     int mirror;            // which of the two bf16 copies of S is current (a delta-rule commit changes it)
     bool mirror_pinned;    // ... and no longer may, since captured work holds its address
     cudaEvent_t ev_before, ev_after;  // one-shot timing hook around the step kernel
-    Side side;             // stream beside the caller's (arl2_denoise_step_token_level), borrowed at its first use
+    Side* side;            // stream beside the caller's (arl2_denoise_step_token_level), borrowed at its first use
     uint32_t wait_limit;   // 0: the kernels' default bound; n: waits give up after n - 1 polls (test hook)
     uint32_t walk_limit;   // the same for the first wait of the last thread block of arl2_commit_tokens' walk
     // projections around the core (arl2_set_projections)
@@ -333,6 +374,7 @@ int arl2_create(const arl2_config* cfg, void* d_state, void* d_workspace, size_t
     ctx->launches = 0;
     ctx->step_calls = 0;
     ctx->mirror = 0;
+    ctx->side = nullptr;
     ctx->mirror_pinned = false;
     ctx->w_pack = ctx->w_o = nullptr;
     ctx->pack_cols = 0;
@@ -523,17 +565,23 @@ bool fill_commit(arl2_ctx* ctx, CommitArgs& a, const void* d_k_clean, const void
 
 namespace {
 
-// Forks the context's side stream from `st` (borrowed at its first use, not while `st` is being captured).  False: there is
-// none, and the work goes to the caller's stream.
+// Forks the context's side stream from `st` (borrowed at its first use, not while `st` is being captured; another one where
+// an open capture has taken it in that `st` is not part of).  False: there is none, and the work goes to the caller's stream.
 bool fork_side(arl2_ctx* ctx, cudaStream_t st)
 {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (ctx->side.stream == nullptr &&
-        (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone || !borrow_side(ctx->side))) {
-        cudaGetLastError();
-        return false;
+    const Capture here = capture_of(st);
+    auto usable = [&](const Side* s) {
+        const Capture c = capture_of(s->stream);
+        return c.none() || (c.status == cudaStreamCaptureStatusActive && here.status == cudaStreamCaptureStatusActive && c.id == here.id);
+    };
+    if (here.status == cudaStreamCaptureStatusInvalidated || (ctx->side == nullptr && !here.none())) return false;
+    if (ctx->side == nullptr || !usable(ctx->side)) {
+        Side* s = borrow_side();
+        if (s == nullptr) return false;
+        return_side(ctx->side);
+        ctx->side = s;
     }
-    if (cudaEventRecord(ctx->side.fork, st) == cudaSuccess && cudaStreamWaitEvent(ctx->side.stream, ctx->side.fork, 0) == cudaSuccess) return true;
+    if (cudaEventRecord(ctx->side->fork, st) == cudaSuccess && cudaStreamWaitEvent(ctx->side->stream, ctx->side->fork, 0) == cudaSuccess) return true;
     cudaGetLastError();
     return false;
 }
@@ -586,13 +634,13 @@ int arl2_denoise_step_token_level(arl2_ctx* ctx, const void* d_q, const void* d_
     if (r == ARL2_OK) r = launch_step(ctx, d_q, k_rot, d_v, nullptr, d_out, st);
     // 2. ... the state at the start of every run of tiles ...
     if (!whole_heads) {
-        cudaStream_t ss = fork ? ctx->side.stream : st;
+        cudaStream_t ss = fork ? ctx->side->stream : st;
         if (r == ARL2_OK && d_alpha_logits != nullptr)
             r = account(ctx, run_decay_weights(ctx->shape, d_alpha_logits, w, totals, share, ntile, seg.nslot, ss));
         if (r == ARL2_OK) r = account(ctx, tc_commit_partials(seg, wk_op, ss));
         if (r == ARL2_OK) r = account(ctx, tc_run_prefix(seg, d_alpha_logits != nullptr ? totals : nullptr, ss));
         // (the streams join whatever became of the launches)
-        if (fork && (cudaEventRecord(ctx->side.join, ctx->side.stream) != cudaSuccess || cudaStreamWaitEvent(st, ctx->side.join, 0) != cudaSuccess) &&
+        if (fork && (cudaEventRecord(ctx->side->join, ctx->side->stream) != cudaSuccess || cudaStreamWaitEvent(st, ctx->side->join, 0) != cudaSuccess) &&
             r == ARL2_OK) {
             set_error("denoise_step_token_level: %s", cudaGetErrorString(cudaGetLastError()));
             r = ARL2_ERR_CUDA;
