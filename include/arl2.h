@@ -20,7 +20,7 @@
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls are
  *     asynchronous on it; ordering between calls is stream order.  (arl2_denoise_step_token_level
  *     may run part of its work on a second stream that forks from `stream` and joins it before the
- *     call returns; the context takes it at the first such call outside a stream capture, from a few that
+ *     call returns and has its priority; the context takes it at the first such call outside a capture, from a few that
  *     the library keeps, and gives it back when it is destroyed.)  Calls may be captured, and what is
  *     captured may be replayed any number of times, among eager calls and other captures.
  *   - Every function returns an arl2_status (0 = ok, negative = error).  Argument errors

@@ -140,6 +140,7 @@ namespace {
 // for calls that are part of it.
 struct Side {
     int device = -1;
+    int priority = 0;       // that of the callers it works beside: at another one it would be held up, or hold others up
     cudaStream_t stream = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     Side* next = nullptr;   // among the idle ones
@@ -184,8 +185,8 @@ void destroy_side(Side* s)
     cudaGetLastError();
 }
 
-// One of the current device: an idle one, or a new one, or nullptr.
-Side* borrow_side()
+// One of the current device and this priority: an idle one, or a new one, or nullptr.
+Side* borrow_side(int priority)
 {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return nullptr; }
@@ -193,7 +194,7 @@ Side* borrow_side()
         std::lock_guard<std::mutex> lock(g_side_mutex);
         for (Side** at = &g_idle_sides; *at != nullptr; at = &(*at)->next) {
             Side* s = *at;
-            if (s->device != dev || !capture_of(s->stream).none()) continue;
+            if (s->device != dev || s->priority != priority || !capture_of(s->stream).none()) continue;
             *at = s->next;
             s->next = nullptr;
             return s;
@@ -202,9 +203,10 @@ Side* borrow_side()
     Side* s = new (std::nothrow) Side;
     if (s == nullptr) return nullptr;
     s->device = dev;
+    s->priority = priority;
     RelaxedCapture relaxed;
     if (cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) != cudaSuccess || cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaStreamCreateWithPriority(&s->stream, cudaStreamNonBlocking, priority) != cudaSuccess) {
         cudaGetLastError();
         destroy_side(s);
         return nullptr;
@@ -566,17 +568,21 @@ bool fill_commit(arl2_ctx* ctx, CommitArgs& a, const void* d_k_clean, const void
 namespace {
 
 // Forks the context's side stream from `st` (borrowed at its first use, not while `st` is being captured; another one where
-// an open capture has taken it in that `st` is not part of).  False: there is none, and the work goes to the caller's stream.
+// `st` has another priority, or an open capture that `st` is not part of has taken it in).  False: there is none, and
+// the work goes to the caller's stream.
 bool fork_side(arl2_ctx* ctx, cudaStream_t st)
 {
     const Capture here = capture_of(st);
+    int priority = 0;
+    if (cudaStreamGetPriority(st, &priority) != cudaSuccess) { cudaGetLastError(); return false; }
     auto usable = [&](const Side* s) {
+        if (s->priority != priority) return false;
         const Capture c = capture_of(s->stream);
         return c.none() || (c.status == cudaStreamCaptureStatusActive && here.status == cudaStreamCaptureStatusActive && c.id == here.id);
     };
     if (here.status == cudaStreamCaptureStatusInvalidated || (ctx->side == nullptr && !here.none())) return false;
     if (ctx->side == nullptr || !usable(ctx->side)) {
-        Side* s = borrow_side();
+        Side* s = borrow_side(priority);
         if (s == nullptr) return false;
         return_side(ctx->side);
         ctx->side = s;
