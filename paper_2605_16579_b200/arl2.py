@@ -136,6 +136,10 @@ def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+# The handle of a device's current stream; a torch without the short cut makes a Stream object of it.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
 def _stream():
     return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
 
@@ -403,10 +407,10 @@ class Layer:
         current = torch.cuda.current_device()
         index = self.device.index
         if index is None or index == current:
-            status = getattr(self._lib, name)(self._ctx, *args, torch._C._cuda_getCurrentRawStream(current))
+            status = getattr(self._lib, name)(self._ctx, *args, _raw_stream(current))
         else:
             with torch.cuda.device(index):
-                status = getattr(self._lib, name)(self._ctx, *args, torch._C._cuda_getCurrentRawStream(index))
+                status = getattr(self._lib, name)(self._ctx, *args, _raw_stream(index))
         if status != 0:
             _check(status, name)
 
