@@ -185,8 +185,9 @@ int tc_gemm(const GemmArgs& a, cudaStream_t st);
 
 void set_error(const char* fmt, ...);
 
-// Every kernel of a call goes out with programmatic stream serialisation: it may become resident while the kernel
-// before it in the stream still drains.  So each kernel calls grid_dependency_wait() before it touches memory that
+// Nearly every kernel of a call goes out with programmatic stream serialisation: it may become resident while the kernel
+// before it in the stream still drains.  (Not the plain-FMA kernels of which several CTAs fit on an SM: launch_in_order.  One
+// that lets no dependents start is followed by them at its end.)  So each of these kernels calls grid_dependency_wait() before it touches memory that
 // anything before it may write or read, and lets its own dependents start only after that (grid_dependency_sync):
 // what a kernel does ahead of its wait may then rely on everything but the kernel right before it having finished.
 // It takes 1 to 1.7 us per kernel: us per pass before and after, passes back to back: token-level pass of 12 heads x 1560

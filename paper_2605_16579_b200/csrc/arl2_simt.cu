@@ -173,7 +173,6 @@ __device__ __forceinline__ void feature_tile(float* xs, float* ws, const T* __re
 template <int D, typename T>
 __global__ void __launch_bounds__(NT) simt_step_kernel(StepArgs a)
 {
-    grid_dependency_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LD = D + PAD;       // row-major [64][D] matrices
     constexpr int LT = BM + PAD;      // transposed [D][64] matrices
@@ -746,7 +745,6 @@ __global__ void __launch_bounds__(NT, 1) simt_step_small_kernel(StepArgs a)
 template <int D, typename T>
 __global__ void __launch_bounds__(NT) simt_commit_partial_kernel(CommitArgs a)
 {
-    grid_dependency_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LD = D + PAD;
     float* Ks = smem;             // [64][LD]  K tile -> K'
@@ -876,7 +874,6 @@ constexpr int LA = kTokChunk + 4;   // row stride of the C x C matrices
 template <int D, typename T>
 __global__ void __launch_bounds__(NT) token_prepare_kernel(TokenCommitArgs a)
 {
-    grid_dependency_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LD = D + PAD;
     float* Ks = smem;                       // [64][LD]  K tile -> K'
@@ -1022,7 +1019,6 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int D, int kScanCols>
 __global__ void __launch_bounds__(NT) token_scan_kernel(TokenCommitArgs a)
 {
-    grid_dependency_sync();
     extern __shared__ __align__(16) float smem[];
     constexpr int LD = D + PAD;
     constexpr int CG = kScanCols / 4;           // float4 column groups
@@ -1189,7 +1185,6 @@ __global__ void rope_k_kernel(const T* __restrict__ k, const float* __restrict__
                               const float* __restrict__ sin_t, T* __restrict__ out, int L, int H,
                               int D, size_t total8)
 {
-    grid_dependency_sync();
     size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total8) return;
     size_t e = t * 8;
@@ -1255,6 +1250,19 @@ int set_smem(K kernel, size_t bytes)
     return 0;
 }
 
+// Ordinary launch, behind the end of the kernel before it: for the kernels of which several CTAs fit on an SM.  Let in
+// while the kernel before them drains, their CTAs pile up on the SMs that are done first or were idle; and a kernel that
+// runs for hundreds of us takes 3 to 4 % longer with the next one's CTAs waiting beside its own.  Us per pass overlapped
+// and like this: commit_tokens at D = 64, 12 x 1560 tokens 360 and 162, 12 x 4680 (bf16) 972 and 380; step in bf16 at
+// D = 64, 16 x 1000 257 and 212, 8 x 2300 512 and 447; clean pass in fp32, 12 x 777 319 and 228.  The smallest calls
+// lose the overlap (commit_tokens at D = 64, 2 x 256 tokens 51 and 56).
+template <typename... P, typename... A>
+cudaError_t launch_in_order(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    kernel<<<grid, threads, smem, st>>>(args...);
+    return cudaGetLastError();
+}
+
 int check_launch(const char* what, cudaError_t e)
 {
     if (e != cudaSuccess) {
@@ -1285,7 +1293,7 @@ int launch_step(const StepArgs& a, cudaStream_t st)
     size_t smem = sizeof(float) * (2 * D * (BM + PAD) + BN * D + BM * (BM + PAD));
     if (int r = set_smem(simt_step_kernel<D, T>, smem)) return r;
     dim3 grid((a.s.L + BM - 1) / BM, a.s.H, a.s.B);
-    if (int r = check_launch("simt_step_kernel", launch_kernel(simt_step_kernel<D, T>, grid, NT, smem, st, a))) return r;
+    if (int r = check_launch("simt_step_kernel", launch_in_order(simt_step_kernel<D, T>, grid, NT, smem, st, a))) return r;
     return 1;
 }
 
@@ -1295,7 +1303,7 @@ int launch_commit(const CommitArgs& a, cudaStream_t st)
     size_t smem = sizeof(float) * (2 * BM * (D + PAD) + BN * D);
     if (int r = set_smem(simt_commit_partial_kernel<D, T>, smem)) return r;
     dim3 grid(a.nsplit, a.s.H, a.s.B);
-    if (int r = check_launch("simt_commit_partial_kernel", launch_kernel(simt_commit_partial_kernel<D, T>, grid, NT, smem, st, a))) return r;
+    if (int r = check_launch("simt_commit_partial_kernel", launch_in_order(simt_commit_partial_kernel<D, T>, grid, NT, smem, st, a))) return r;
     return 1;
 }
 
@@ -1439,10 +1447,10 @@ int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, co
     unsigned blocks = (unsigned)((total8 + 255) / 256);
     cudaError_t e;
     if (dtype == ARL2_FP32)
-        e = launch_kernel(rope_k_kernel<float>, dim3(blocks), 256, 0, st, static_cast<const float*>(k), cos_t, sin_t,
+        e = launch_in_order(rope_k_kernel<float>, dim3(blocks), 256, 0, st, static_cast<const float*>(k), cos_t, sin_t,
                           static_cast<float*>(k_rot), s.L, s.H, s.D, total8);
     else
-        e = launch_kernel(rope_k_kernel<__nv_bfloat16>, dim3(blocks), 256, 0, st, static_cast<const __nv_bfloat16*>(k), cos_t, sin_t,
+        e = launch_in_order(rope_k_kernel<__nv_bfloat16>, dim3(blocks), 256, 0, st, static_cast<const __nv_bfloat16*>(k), cos_t, sin_t,
                           static_cast<__nv_bfloat16*>(k_rot), s.L, s.H, s.D, total8);
     if (int r = check_launch("rope_k_kernel", e)) return r;
     return 1;
@@ -1509,12 +1517,12 @@ int launch_commit_tokens(const TokenCommitArgs& a, cudaStream_t st)
     size_t smem1 = sizeof(float) * (2 * BM * (D + PAD) + BN * D + 2 * kTokChunk * LA + 3 * kTokChunk + 8);
     if (int r = set_smem(token_prepare_kernel<D, T>, smem1)) return r;
     dim3 grid1(a.nchunk, a.s.H, a.s.B);
-    if (int r = check_launch("token_prepare_kernel", launch_kernel(token_prepare_kernel<D, T>, grid1, NT, smem1, st, a))) return r;
+    if (int r = check_launch("token_prepare_kernel", launch_in_order(token_prepare_kernel<D, T>, grid1, NT, smem1, st, a))) return r;
     constexpr int kScanCols = D / 4;   // 4 CTAs per (stream, head)
     size_t smem2 = sizeof(float) * (2 * kTokChunk * (D + PAD) + 2 * kTokChunk * kScanCols + D * kScanCols);
     if (int r = set_smem(token_scan_kernel<D, kScanCols>, smem2)) return r;
     dim3 grid2(D / kScanCols, a.s.H, a.s.B);
-    if (int r = check_launch("token_scan_kernel", launch_kernel(token_scan_kernel<D, kScanCols>, grid2, NT, smem2, st, a))) return r;
+    if (int r = check_launch("token_scan_kernel", launch_in_order(token_scan_kernel<D, kScanCols>, grid2, NT, smem2, st, a))) return r;
     return 2;
 }
 
