@@ -462,10 +462,13 @@ __global__ void __launch_bounds__(NT, 1) simt_step_small_kernel(StepArgs a)
     }
     float* Pw = Ps + w * SR * LP;
 
+    // One CTA per unit walks many key tiles, and there a second barrier per tile costs more than V beside the scores gives
+    // (bf16, D = 64, 1 x 1560 81.2 us per pass with it, 76.7 without; fp32, 12 x 777 139.8 and 129.8, at D = 128 284.5 and 268.8).
+    constexpr bool kAsyncV = KS > 1 && sizeof(T) == 4;
     for (int j0 = rank * KT; j0 < L; j0 += KS * KT) {
         __syncthreads();   // previous tile fully consumed
         constexpr int kPer = KT * (D / 4) / NT;
-        if constexpr (sizeof(T) == 4) {   // V beside the scores (rows past L: zeros, no bytes read)
+        if constexpr (kAsyncV) {   // V beside the scores (rows past L: zeros, no bytes read)
 #pragma unroll 4
             for (int it = 0; it < kPer; ++it) {
                 const int idx = tid + it * NT, kr = idx / (D / 4), c4 = idx % (D / 4), krow = j0 + kr;
@@ -475,13 +478,16 @@ __global__ void __launch_bounds__(NT, 1) simt_step_small_kernel(StepArgs a)
                              "l"(src), "r"(krow < L ? 16 : 0) : "memory");
             }
         }
-#pragma unroll 8
+#pragma unroll (KS == 1 ? 4 : 8)
         for (int it = 0; it < kPer; ++it) {
             const int idx = tid + it * NT, kr = idx / (D / 4), c4 = idx % (D / 4), krow = j0 + kr;
-            *reinterpret_cast<float4*>(Ks + kr * LD + c4 * 4) = krow < L ? rotated4(k, krow, c4) : zero4;
-            if constexpr (sizeof(T) != 4)
-                *reinterpret_cast<float4*>(Vs + kr * D + c4 * 4) =
-                    krow < L ? load4(v + (((size_t)b * L + krow) * H + h) * D + c4 * 4) : zero4;
+            float4 kv = zero4, vv = zero4;
+            if (krow < L) {
+                kv = rotated4(k, krow, c4);
+                if constexpr (!kAsyncV) vv = load4(v + (((size_t)b * L + krow) * H + h) * D + c4 * 4);
+            }
+            *reinterpret_cast<float4*>(Ks + kr * LD + c4 * 4) = kv;
+            if constexpr (!kAsyncV) *reinterpret_cast<float4*>(Vs + kr * D + c4 * 4) = vv;
         }
         __syncthreads();
 
@@ -534,8 +540,12 @@ __global__ void __launch_bounds__(NT, 1) simt_step_small_kernel(StepArgs a)
 #pragma unroll
             for (int e = 0; e < CN * 4; ++e) o[i][e] *= corr;
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        __syncthreads();   // V (and the state) have landed
+        if constexpr (kAsyncV) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();   // V (and the state) have landed
+        } else {
+            __syncwarp();
+        }
         // O += P V over this warp's keys: rows 4 i + rg, columns 32 c + 4 kg ..
         const float* vb = Vs + (w * KW) * D + kg * 4;
 #pragma unroll 2
