@@ -1145,11 +1145,11 @@ __global__ void __launch_bounds__(NT) token_scan_kernel(TokenCommitArgs a)
 // S[b,h] <- sigmoid(a[b,h]) S[b,h] + sum_split partial[b,h,split], splits added in index
 // order so that the result does not depend on scheduling.  Also refreshes the bf16 operand
 // copy of S when one is kept.  One thread per 4 state elements.
-__global__ void commit_reduce_kernel(float* __restrict__ state, const float* __restrict__ partials,
-                                     const float* __restrict__ decay, int decay_direct,
+__global__ void commit_reduce_kernel(float* __restrict__ state, const float* partials,
+                                     const float* decay, int decay_direct,
                                      __nv_bfloat16* __restrict__ state_bf16, int nsplit, int DD,
                                      size_t total4, int run_share, int run_ntile, int nslot,
-                                     const uint32_t* __restrict__ status)
+                                     const uint32_t* status)
 {
     grid_dependency_sync();
     size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1191,8 +1191,8 @@ namespace {
 
 // k_rot = RoPE(k), 8 elements per thread, output in the input's dtype.
 template <typename T>
-__global__ void rope_k_kernel(const T* __restrict__ k, const float* __restrict__ cos_t,
-                              const float* __restrict__ sin_t, T* __restrict__ out, int L, int H,
+__global__ void rope_k_kernel(const T* k, const float* cos_t,
+                              const float* sin_t, T* __restrict__ out, int L, int H,
                               int D, size_t total8)
 {
     size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1325,7 +1325,7 @@ int launch_commit(const CommitArgs& a, cudaStream_t st)
 // a tile every thread owns seg consecutive tokens, the threads' sums are combined by a suffix scan
 // (warp shuffles, then the 32 warp totals through shared memory), and `carry` holds the
 // log-product of all later tiles.
-__global__ void __launch_bounds__(1024) decay_weights_kernel(const float* __restrict__ alpha,
+__global__ void __launch_bounds__(1024) decay_weights_kernel(const float* alpha,
                                                              float* __restrict__ w, float* __restrict__ total,
                                                              int L, int H, int seg)
 {
@@ -1379,7 +1379,7 @@ __global__ void __launch_bounds__(1024) decay_weights_kernel(const float* __rest
 }
 
 // Segment (run, head) of the flattened tile sequence: one block walks its tokens backwards, 256 at a time.
-__global__ void __launch_bounds__(256) run_decay_weights_kernel(const float* __restrict__ alpha, float* __restrict__ w,
+__global__ void __launch_bounds__(256) run_decay_weights_kernel(const float* alpha, float* __restrict__ w,
                                                                 float* __restrict__ total, int L, int H, int share, int ntile,
                                                                 int nslot)
 {

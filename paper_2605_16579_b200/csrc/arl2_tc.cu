@@ -229,7 +229,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
                 const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16) * 32 + (row & 31);
                 uint4 cs[16];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) cs[c] = __ldg(tab + c * 32);
+                for (int c = 0; c < 16; ++c) cs[c] = tab[c * 32];
                 if (item == 0 && !wait_bar(bars + 8 * kBarQFull, 0, ab, 10)) return;
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
@@ -330,13 +330,13 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
             // fetched early too; no gate tensor = closed gate (plain softmax attention, Eq. 1)
             const bool elem_gate = kElemGate && p.gate_mode == 2 && p.gate != nullptr;   // one gate per output channel
             const float gate_logit = (valid_row && p.gate != nullptr && !elem_gate)
-                                         ? __ldg(p.gate + (p.gate_mode == 1 ? (size_t)b * L + row : ((size_t)b * L + row) * H + h))
+                                         ? p.gate[p.gate_mode == 1 ? (size_t)b * L + row : ((size_t)b * L + row) * H + h]
                                          : -INFINITY;
             const bool rotate_u = p.rope_h != nullptr && valid_row;
             if (rotate_u) {
                 const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16) * 32 + (row & 31);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) cs[c] = __ldg(tab + c * 32);
+                for (int c = 0; c < 16; ++c) cs[c] = tab[c * 32];
             }
             if (!wait_bar(bar_s, s_cnt & 1, ab, 30 + t)) return;
             ++s_cnt;
@@ -407,7 +407,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, uint8_t* sme
                                 uint32_t w[8];
 #pragma unroll
                                 for (int i = 0; i < 4; ++i) {
-                                    const float4 gl = __ldg(reinterpret_cast<const float4*>(grow + hv * 64 + c * 32 + e * 16 + i * 4));
+                                    const float4 gl = *reinterpret_cast<const float4*>(grow + hv * 64 + c * 32 + e * 16 + i * 4);
                                     const float gv[4] = {gl.x, gl.y, gl.z, gl.w};
                                     float y[4];
 #pragma unroll
@@ -906,13 +906,13 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     uint4 cs[8];
     if (row < L) {
         const size_t gi = ((size_t)b * L + row) * H + h;
-        if (p.alpha != nullptr) alpha_logit = __ldg(p.alpha + gi);
-        if (p.beta != nullptr) beta_logit = __ldg(p.beta + gi);
+        if (p.alpha != nullptr) alpha_logit = p.alpha[gi];
+        if (p.beta != nullptr) beta_logit = p.beta[gi];
     }
     if (p.rope_h != nullptr) {
         const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16 + hf * 8) * 32 + (row & 31);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) cs[c] = __ldg(tab + c * 32);
+        for (int c = 0; c < 8; ++c) cs[c] = tab[c * 32];
     }
     if (tid == 0) {
         for (int i = 0; i < kTPNumBars; ++i) mbar_init(bars + 8 * i, 1);
@@ -1431,7 +1431,7 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
     };
     put_s();
     const float* gc = p.gc + bh * 2 * p.ntile;
-    float g_cur = lane < nchunk ? __ldg(gc + lane) : 1.0f;   // decays of 32 chunks, one per lane
+    float g_cur = lane < nchunk ? gc[lane] : 1.0f;   // decays of 32 chunks, one per lane
 
     bool dead = false;
     // On a wait that expires the warp goes on without waiting: the barriers of the group keep their
@@ -1508,7 +1508,7 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
                 *reinterpret_cast<uint32_t*>(u_s + (ge + 8 * half) * kScanLdU + wq * 16 + n * 8 + gk) = pack_bf16(lo, hi);
             }
         const float g = __shfl_sync(0xffffffffu, g_cur, c & 31);
-        if ((c & 31) == 31) g_cur = c + 1 + lane < nchunk ? __ldg(gc + c + 1 + lane) : 1.0f;
+        if ((c & 31) == 31) g_cur = c + 1 + lane < nchunk ? gc[c + 1 + lane] : 1.0f;
 #pragma unroll
         for (int n = 0; n < 4; ++n)
 #pragma unroll
@@ -1584,7 +1584,7 @@ __global__ void pack_rope_kernel(const float* __restrict__ cos_t, const float* _
 // 64-bit index divisions and the step kernel's first Q tiles requested 0.6 us later and rotated 1.2 us later: 40.2 us per
 // pass of 12 heads x 1560 tokens against 38.8, 3 x 12 x 1001 33.0 against 32.2.)
 constexpr int kRopeRows = 4;
-__global__ void __launch_bounds__(256) tc_rope_k_kernel(const uint4* __restrict__ k, const uint4* __restrict__ rope_h,
+__global__ void __launch_bounds__(256) tc_rope_k_kernel(const uint4* k, const uint4* rope_h,
                                                         uint4* __restrict__ out, uint32_t L, uint32_t H, uint32_t rows)
 {
     const uint32_t c = threadIdx.x & 15;             // vector of the 128-element row
@@ -1600,8 +1600,8 @@ __global__ void __launch_bounds__(256) tc_rope_k_kernel(const uint4* __restrict_
 #pragma unroll
     for (int i = 0; i < kRopeRows; ++i) {
         if (row0 + i * 16 < rows) {
-            raw[i] = __ldg(k + (size_t)(row0 + i * 16) * 16 + c);
-            cs[i] = __ldg(tab[i]);
+            raw[i] = k[(size_t)(row0 + i * 16) * 16 + c];
+            cs[i] = *tab[i];
         }
     }
 #pragma unroll

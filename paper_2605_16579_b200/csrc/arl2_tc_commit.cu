@@ -301,12 +301,12 @@ tc_commit_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
             if (rotate) {
                 const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16 + hf * 8) * 32 + (row & 31);
 #pragma unroll
-                for (int c = 0; c < 8; ++c) cs[c] = __ldg(tab + c * 32);
+                for (int c = 0; c < 8; ++c) cs[c] = tab[c * 32];
             }
             // per-token factor on K': the decay weight (mode 2) or the learning rate (delta rule)
             float wtok = 1.0f;
             if (kMode != 0 && p.beta != nullptr && row < L) {
-                const float x = __ldg(p.beta + ((size_t)b * L + row) * H + h);
+                const float x = p.beta[((size_t)b * L + row) * H + h];
                 wtok = kMode == 1 ? sigmoid_fast(x) : x;
             }
             if (p.k_rot != nullptr) {
@@ -523,11 +523,10 @@ __device__ __forceinline__ void fin_multiply(float (&acc)[4][4], const float* __
 
 template <int kMode>
 __global__ void __launch_bounds__(kFinThreads)
-tc_commit_finish_kernel(float* __restrict__ state, const float* __restrict__ partials,
-                        const float* __restrict__ partials_g, const __nv_bfloat16* __restrict__ wv,
-                        const float* __restrict__ decay, int decay_direct,
-                        const __nv_bfloat16* __restrict__ mirror_cur, __nv_bfloat16* __restrict__ mirror_next,
-                        int H, int share, int ntile, int nslot, const uint32_t* __restrict__ status)
+tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
+                        const float* partials_g, const __nv_bfloat16* wv,
+                        const float* decay, int decay_direct, const __nv_bfloat16* mirror_cur, __nv_bfloat16* mirror_next,
+                        int H, int share, int ntile, int nslot, const uint32_t* status)
 {
     extern __shared__ __align__(16) uint8_t fin_smem[];
     __nv_bfloat16* Ws = reinterpret_cast<__nv_bfloat16*>(fin_smem);                  // value map [m][e]
@@ -649,8 +648,8 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* __restrict__ par
 // kernel; a CTA owns 16 rows of a head and walks the head's segments in order, the sums of the next segment
 // under way while this one's are multiplied.
 __global__ void __launch_bounds__(kFinThreads)
-tc_run_prefix_kernel(float* __restrict__ slots, const float* __restrict__ state, const __nv_bfloat16* __restrict__ wv,
-                     const float* __restrict__ total, int H, int share, int ntile, int nslot)
+tc_run_prefix_kernel(float* __restrict__ slots, const float* state, const __nv_bfloat16* wv,
+                     const float* total, int H, int share, int ntile, int nslot)
 {
     extern __shared__ __align__(16) uint8_t fin_smem[];
     __nv_bfloat16* Ws = reinterpret_cast<__nv_bfloat16*>(fin_smem);
@@ -692,7 +691,7 @@ tc_run_prefix_kernel(float* __restrict__ slots, const float* __restrict__ state,
 #pragma unroll
             for (int c = 0; c < 4; ++c) *reinterpret_cast<float4*>(A + srow * kFinLdA + (warp * 4 + c) * 8 + shalf * 4) = cur[c];
             if (i + 2 < nparts) fetch(i + 1);
-            if (total != nullptr) gamma = __ldg(total + (size_t)bh * nslot + i);
+            if (total != nullptr) gamma = total[(size_t)bh * nslot + i];
         }
         __syncthreads();   // the CTA's rows of this slot have been read
         float* out = head_slots + (size_t)i * kTile * kTile + write0;

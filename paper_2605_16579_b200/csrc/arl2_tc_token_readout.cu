@@ -162,13 +162,13 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         const int bhi = g / p.ntile, b = bhi / H, h = bhi - b * H, row = (g - bhi * p.ntile) * kTile + r;
         if (row < L) {
             const size_t gi = ((size_t)b * L + row) * H + h;
-            gate_logit = __ldg(p.gate + gi);
-            if (hf == 0 && p.alpha != nullptr) alpha_logit = __ldg(p.alpha + gi);
+            gate_logit = p.gate[gi];
+            if (hf == 0 && p.alpha != nullptr) alpha_logit = p.alpha[gi];
         }
         if (p.rope_h != nullptr) {
             const uint4* tab = p.rope_h + ((size_t)(row >> 5) * 16 + hf * 8) * 32 + (row & 31);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) cs[i] = __ldg(tab + i * 32);
+            for (int i = 0; i < 8; ++i) cs[i] = tab[i * 32];
         }
     };
     fetch_row(g_begin);
