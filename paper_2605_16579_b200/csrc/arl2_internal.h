@@ -230,8 +230,10 @@ cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, int cluster, int thr
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
+    // (the error is taken out of the runtime either way: left there, it would be reported by whichever call looks next)
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    const cudaError_t last = cudaGetLastError();
+    return e != cudaSuccess ? e : last;
 }
 template <typename... P, typename... A>
 cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args)
