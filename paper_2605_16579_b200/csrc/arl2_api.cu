@@ -5,6 +5,8 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <cuda.h>
+
 #include <mutex>
 #include <new>
 
@@ -139,7 +141,7 @@ namespace {
 // outside that capture (it would end in an error, and the capture with it): until the capture ends, such a stream is only
 // for calls that are part of it.
 struct Side {
-    int device = -1;
+    unsigned long long context = 0;   // the CUDA context that owns the handles: they mean nothing in another, or after its end
     int priority = 0;       // that of the callers it works beside: at another one it would be held up, or hold others up
     cudaStream_t stream = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
@@ -148,6 +150,21 @@ struct Side {
 constexpr int kMaxIdleSides = 8;   // (more only while captures hold them)
 std::mutex g_side_mutex;
 Side* g_idle_sides = nullptr;
+
+// The current CUDA context's number, never given twice in a process; 0: there is none, or it cannot be told.
+unsigned long long current_context()
+{
+    typedef CUresult (*GetIdFn)(CUcontext, unsigned long long*);
+    static const GetIdFn get_id = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess;
+        if (!ok) cudaGetLastError();
+        return ok ? reinterpret_cast<GetIdFn>(p) : nullptr;
+    }();
+    unsigned long long id = 0;
+    return get_id != nullptr && get_id(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
 
 struct Capture {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusInvalidated;   // (also where it cannot be read)
@@ -185,16 +202,16 @@ void destroy_side(Side* s)
     cudaGetLastError();
 }
 
-// One of the current device and this priority: an idle one, or a new one, or nullptr.
+// One of the current context and this priority: an idle one, or a new one, or nullptr.
 Side* borrow_side(int priority)
 {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    const unsigned long long context = current_context();
+    if (context == 0) return nullptr;
     {
         std::lock_guard<std::mutex> lock(g_side_mutex);
         for (Side** at = &g_idle_sides; *at != nullptr; at = &(*at)->next) {
             Side* s = *at;
-            if (s->device != dev || s->priority != priority || !capture_of(s->stream).none()) continue;
+            if (s->context != context || s->priority != priority || !capture_of(s->stream).none()) continue;
             *at = s->next;
             s->next = nullptr;
             return s;
@@ -202,7 +219,7 @@ Side* borrow_side(int priority)
     }
     Side* s = new (std::nothrow) Side;
     if (s == nullptr) return nullptr;
-    s->device = dev;
+    s->context = context;
     s->priority = priority;
     RelaxedCapture relaxed;
     if (cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) != cudaSuccess || cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess ||
@@ -217,6 +234,7 @@ Side* borrow_side(int priority)
 void return_side(Side* s)
 {
     if (s == nullptr) return;
+    const unsigned long long context = current_context();   // (only this one's handles are looked at)
     Side* surplus = nullptr;
     {
         std::lock_guard<std::mutex> lock(g_side_mutex);
@@ -225,7 +243,7 @@ void return_side(Side* s)
         int idle = 0;
         for (Side** at = &g_idle_sides; *at != nullptr;) {
             Side* x = *at;
-            if (!capture_of(x->stream).none() || ++idle <= kMaxIdleSides) { at = &x->next; continue; }
+            if (x->context != context || !capture_of(x->stream).none() || ++idle <= kMaxIdleSides) { at = &x->next; continue; }
             *at = x->next;
             x->next = surplus;
             surplus = x;
