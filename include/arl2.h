@@ -20,9 +20,10 @@
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).  Calls are
  *     asynchronous on it; ordering between calls is stream order.  (arl2_denoise_step_token_level
  *     may run part of its work on a second stream that forks from `stream` and joins it before the
- *     call returns and has its priority; the context takes it at the first such call outside a capture, from a few that
- *     the library keeps, and gives it back when it is destroyed.)  Calls may be captured, and what is
- *     captured may be replayed any number of times, among eager calls and other captures.
+ *     call returns, and has its priority; the context takes it at the first such call outside a stream
+ *     capture, from a few that the library keeps, and gives it back when it is destroyed.)  Denoise
+ *     passes, commits and projections may be captured, and what is captured may be replayed any number of
+ *     times, among eager calls on the same context and other captures.
  *   - Every function returns an arl2_status (0 = ok, negative = error).  Argument errors
  *     are found on the host before any launch and leave S untouched.  Nothing aborts,
  *     traps or throws.  arl2_last_error() gives a thread-local message for the last error.

@@ -267,8 +267,8 @@ struct arl2_ctx {
     const void *wq, *wk, *wv;
     const float *rope_cos, *rope_sin;
     bool use_tc;
-    int simt_key_ctas;     // ... and the CTAs that share a unit of 16 rows
     bool simt_16_rows;     // plain-FMA step: the 16-row kernel is the faster one for this shape on this device
+    int simt_key_ctas;     // ... and the CTAs that share a unit of 16 rows
     uint64_t launches;
     uint32_t step_calls;   // parity selects the scheduler counter of the next step launch
     int mirror;            // which of the two bf16 copies of S is current (a delta-rule commit changes it)
@@ -488,7 +488,10 @@ int launch_step(arl2_ctx* ctx, const void* d_q, const void* k_rot, const void* d
     StepArgs a;
     a.s = ctx->shape;
     a.q = d_q; a.k_rot = k_rot; a.v = d_v; a.gate = d_gate_logits;
-    a.k_made_before = k_rot == ctx->ws + ctx->lay.k_rot;   // by rotate_k, or by the commit kernel of a clean pass (which does not let the step start early)
+    // By rotate_k, or by the commit kernel of a clean pass.  Both let the step in once they have waited themselves, so that
+    // all before them is complete; what the step touches ahead of its own wait (Q, the rotation table, the other item
+    // counter) must not be written by that one kernel.  Its other threads count polls while that kernel runs.
+    a.k_made_before = k_rot == ctx->ws + ctx->lay.k_rot;
     a.gate_mode = (ctx->cfg.flags & ARL2_FLAG_GATE_ELEMENTWISE) ? 2 : (ctx->cfg.flags & ARL2_FLAG_GATE_SCALAR) ? 1 : 0;
     a.state = ctx->state; a.wq = ctx->wq;
     a.rope_cos = ctx->rope_cos; a.rope_sin = ctx->rope_sin;
@@ -636,7 +639,8 @@ int arl2_denoise_step_token_level(arl2_ctx* ctx, const void* d_q, const void* d_
     // A walked tile takes about 10 us, the three launches before the walk 25 us and 1 us per tile of a run: heads
     // of no more tiles than that are walked whole, from the state itself (one tile: 35 us per pass against 60,
     // three tiles: 61 against 73; 13 tiles in runs of 2: 197 against 97).  The costs are those of heads that fit on
-    // the SMs side by side; with more heads than SMs a run is a whole head's length and heads go whole, in waves.
+    // the SMs side by side, with everything on one stream; with more heads than SMs a run is a whole head's length and heads
+    // go whole, in waves.
     const bool whole_heads = 10 * ntile <= 11 * share + 30;
     if (whole_heads) {
         seg.partials = nullptr;

@@ -205,9 +205,9 @@ __device__ __forceinline__ void grid_dependency_sync()
 }
 // Dynamic shared memory with which a CTA asks for a per_sm-th of an SM (at least what it needs): a small grid that is
 // let in while the kernel before it drains would otherwise pile up on the SMs that are done first, several CTAs to an
-// SM, while the rest of the device becomes idle.  Finishing kernel of the commits: us per pass with and without, delta
-// rule 12 heads x 4680 tokens 27.8 -> 24.9, commit 12 x 4680 23.6 -> 18.4, 40 x 4680 31.7 -> 30.5 (20.6 and 33.0 for the
-// last two when it was not let in early).
+// SM, while the rest of the device becomes idle.  Finishing kernel of the commits: us without and with, delta rule of
+// 12 heads x 4680 tokens 27.8 -> 24.9 per pass; between events around the two kernels of a commit, 12 x 4680
+// 23.6 -> 18.4, 40 x 4680 31.7 -> 30.5 (20.6 and 33.0 when it was not let in early).
 constexpr int kMaxSmemPerCta = 227 * 1024;
 inline size_t even_spread_smem(int need, int per_sm)
 {

@@ -1473,11 +1473,15 @@ int simt_rope_k(const Shape& s, int dtype, const void* k, const float* cos_t, co
 // rotation of K included) at 1, 6, 9, 11, 12, 20 and 24 heads
 //   D = 128:  72 / 236, 144 / 237, 214 / 238, 282 / 238, 285 / 460, 490 / 484, 565 / 700
 //   D = 64:   37 / 114,  72 / 117, 107 / 117, 140 / 117, 141 / 150, 242 / 155, 277 / 254
+// (of the 16-row kernel as it was: its fetches ahead of the key loop have since taken 6 to 8 % off it, 12 heads 269 and 130, and
+// clusters serve one head, 47 and 24).
 // The model (us: once per call, then per round a fixed part and a part per key tile; the time of 1, 2, 3 64-row
-// CTAs on an SM relative to one) was fitted to 130 shapes of 48 to 4614 tokens with 1 to 192 heads.  There it
-// picks the slower kernel nowhere by more than 8 %, in the mean by 0.2 % (always the 64-row kernel: 53 %; the 16-row
-// kernel at D = 128 and up to 156 tiles at D = 64: 3 %, 47 % at most).  At even times the 64-row kernel is taken.  (The model
-// is of one CTA per unit: where clusters serve a shape, its one round goes to the 16-row kernel in any case.)
+// CTAs on an SM relative to one) was fitted to 130 shapes of 48 to 4614 tokens with 1 to 192 heads, with that kernel.  With
+// the present one, over 416 shapes of 48 to 2300 tokens with 1 to 96 heads, it takes the slower kernel in the mean by
+// 0.2 % (always the 64-row kernel: 120 %, always the 16-row kernel: 5 %), but by 22 % at 40 heads x 1000 tokens
+// (fp32, D = 128: 1896 us against 1555) and by 11 to 20 % at six more: it charges the 16-row kernel too much now.  At
+// even times the 64-row kernel is taken.  (The model is of one CTA per unit: where clusters serve a shape, its one round
+// goes to the 16-row kernel in any case.)
 bool simt_step_prefers_16_rows(const Shape& s, int dtype, int num_sms)
 {
     struct Model {
@@ -1502,7 +1506,9 @@ bool simt_step_prefers_16_rows(const Shape& s, int dtype, int num_sms)
 }
 
 // CTAs of a cluster that share a 16-row unit of that kernel: as many as find room beside one another (an eighth of the
-// SMs is left out of the count, as clusters do not cross the groups of SMs they are placed in).
+// SMs is left out of the count, as clusters do not cross the groups of SMs they are placed in).  Four were not compared
+// with two just above 64 keys, where two of the four have none: 1 to 5 heads x 65 tokens 7.4 to 7.6 us in a graph (the
+// kernel before, one CTA per unit: 11.1 to 11.3).
 int simt_step_key_ctas(const Shape& s, int num_sms)
 {
     const long units = (long)((s.L + SR - 1) / SR) * s.H * s.B;

@@ -1582,7 +1582,7 @@ __global__ void pack_rope_kernel(const float* __restrict__ cos_t, const float* _
 // pairs, one 16-byte table vector each), kRopeRows rows per thread with all loads ahead of the first use.  The same table
 // rotates Q inside the step kernel.  Bound by memory, and where it is short by its latencies.  (With one row per thread,
 // 64-bit index divisions and the step kernel's first Q tiles requested 0.6 us later and rotated 1.2 us later: 40.2 us per
-// pass of 12 heads x 1560 tokens against 38.8, 3 x 12 x 1001 33.0 against 32.2.)
+// pass of 12 heads x 1560 tokens against 38.8.  The two changes were not timed apart.)
 constexpr int kRopeRows = 4;
 __global__ void __launch_bounds__(256) tc_rope_k_kernel(const uint4* k, const uint4* rope_h,
                                                         uint4* __restrict__ out, uint32_t L, uint32_t H, uint32_t rows)

@@ -432,8 +432,9 @@ tc_commit_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
 // memory; the products with the right-hand matrices (the head's value map, then S_old; both bf16)
 // run on the warp-level tensor-core instruction, one 16 x 32 block of the output per warp, with the
 // fp32 sums split into a bf16 head and a bf16 remainder (two MMAs, relative error 2^-17: far below
-// the bf16 rounding of the matrices themselves).  Every global load the CTA needs is requested
-// before the first result is used.
+// the bf16 rounding of the matrices themselves).  The first kFinMaxParts slots, the old
+// state and the matrices are requested before the first result is used; further slots, and the delta rule's second set,
+// come in a loop.
 constexpr int kFinRows = 16;
 constexpr int kFinThreads = 128;
 constexpr int kFinMaxParts = 6;     // slots of one head the unrolled loads cover; more fall back to a loop
