@@ -872,7 +872,8 @@ int arl2_commit_tokens(arl2_ctx* ctx, const void* d_k_clean, const void* d_v_cle
     a.u1 = reinterpret_cast<float*>(ctx->ws + ctx->lay.tok_u1);
     a.kh = reinterpret_cast<float*>(ctx->ws + ctx->lay.tok_kh);
     a.gc = reinterpret_cast<float*>(ctx->ws + ctx->lay.tok_gc);
-    a.next = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials);   // a [D, D] slot per head and more, not in use here
+    a.next = reinterpret_cast<float*>(ctx->ws + ctx->lay.partials);   // not in use here
+    a.next_slots = ctx->lay.nslot;
     a.nchunk = ctx->lay.nchunk;
     a.decayed = (ctx->cfg.flags & ARL2_FLAG_DELTA_DECAYED_PREDICTION) != 0;
     a.wait_limit = ctx->wait_limit;

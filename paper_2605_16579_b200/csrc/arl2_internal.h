@@ -107,7 +107,8 @@ struct TokenCommitArgs {
     float* u1;              // same shape
     float* kh;              // same shape
     float* gc;              // [B, H, nchunk] decay of a whole chunk
-    float* next;            // [B, H, D, D] fp32 scratch: the walk's result before it is published (tensor-core path)
+    float* next;            // [B, H, next_slots, D, D] fp32 scratch: the walk's result before it is published (tensor-core path)
+    int next_slots = 1;
     int nchunk;             // ceil(L / 64)
     bool decayed = false;   // each token predicts against alpha_j S_{j-1} instead of S_{j-1}
     uint32_t wait_limit = 0;   // as in StepArgs

@@ -863,12 +863,13 @@ struct TcTokenParams {
     float* gc;                 // [B, H, 2 * ntile]
     float* state;              // the walk reads it, the publishing kernel writes it and its bf16 copy
     __nv_bfloat16* state_bf16;
-    float* next;               // [B, H, 128, 128]: S after the walk, until it is published
+    float* next;               // [B, H, 2 runs - 1, 128, 128]: S after the walk (of the first run, then N and M of each further one), until it is published
     uint32_t* status;
     uint32_t spin_limit;
     uint32_t walk_limit;       // n > 0: the first wait of the walk's last CTA gives up after n - 1 polls (test hook)
     int ntile;                 // 128-token tiles; rows_pad = 128 * ntile
     int nchunk;                // ceil(L / 64): chunks the scan walks
+    int runs, run_chunks;      // runs a head's chunks are cut into, and chunks of a run (the last one may be shorter)
     int decayed;               // prediction against alpha_j S_{j-1}
 };
 
@@ -1304,7 +1305,12 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
 // The fp32 state stays in registers for the whole walk (16 per thread).  Per chunk a warp runs 16 + 16
 // instructions in four independent chains each and meets its group twice (named barriers, 128 threads);
 // the B fragments of the next chunk are fetched while this chunk's products run.  A fifth warp per CTA
-// streams the tiles through a TMA ring.  12 heads x 4680 tokens, inside the call: 162 us with one CTA per head and the
+// streams the tiles through a TMA ring.
+// Few heads leave SMs idle; kRuns cuts the chunks of a head into runs that are walked side by side.  What a run does to
+// the state it is entered with is S -> M S + N: N is the walk from the zero state, M the walk from the identity without
+// U1, so a further run has 256 columns instead of 128; tc_token_join_kernel puts the runs together.  (One group of four
+// warps for two slabs, so that both use a B fragment that was read once: 78.4 us at 12 heads x 4680 tokens instead of 76.4.)
+// 12 heads x 4680 tokens, inside the call: 162 us with one CTA per head and the
 // state in TMEM (two MMAs, two passes through registers, four CTA-wide meetings per chunk) -> 46 us (1.2 k clk per
 // chunk; the 34 KB per chunk and SM that come from L2 are about 0.65 k of that).
 constexpr int kChunkHalf = kTokC * 128;              // bytes of a 64-row, 64-column box
@@ -1341,7 +1347,7 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-template <int kSlabs, bool kShared>
+template <int kSlabs, bool kShared, bool kRuns>
 __global__ void __launch_bounds__(kSlabs * 128 + 32, kShared ? 2 : 1)
 tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_kh,
                      const __grid_constant__ CUtensorMap tm_u1, const TcTokenParams p)
@@ -1361,8 +1367,17 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int h = blockIdx.y, b = blockIdx.z;
     const size_t bh = (size_t)b * p.s.H + h;
-    const int nchunk = p.nchunk;
-    const int e0 = blockIdx.x * kSlabs * kScanSlab;      // first value column of this CTA
+    // first value column of this CTA; the run it walks, and whether these are columns of M
+    int e0 = blockIdx.x * kSlabs * kScanSlab, run = 0;
+    bool is_m = false;
+    if (kRuns && e0 >= kTile) {
+        run = 1 + (e0 - kTile) / (2 * kTile);
+        e0 = (e0 - kTile) % (2 * kTile);
+        is_m = e0 >= kTile;
+        e0 %= kTile;
+    }
+    const int chunk0 = kRuns ? run * p.run_chunks : 0;
+    const int nchunk = kRuns ? min(p.run_chunks, p.nchunk - chunk0) : p.nchunk;
 
     if (tid == 0) {
         for (int i = 0; i < kS; ++i) {
@@ -1380,7 +1395,7 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
     if (warp == kSlabs * 4) {
         // ---------------- TMA producer ----------------
         if (lane == 0) {
-            const int r0 = (int)(bh * p.ntile * kTile);
+            const int r0 = (int)(bh * p.ntile * kTile) + chunk0 * kTokC;
             bool ok = true;
             int c = 0;
             for (; c < nchunk; ++c) {
@@ -1421,7 +1436,10 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
 #pragma unroll
     for (int n = 0; n < 4; ++n)
 #pragma unroll
-        for (int x = 0; x < 4; ++x) st[n][x] = srow[(size_t)(n * 8 + (x & 1)) * kTile + (x >> 1) * 8];
+        for (int x = 0; x < 4; ++x) {
+            if (run == 0) st[n][x] = srow[(size_t)(n * 8 + (x & 1)) * kTile + (x >> 1) * 8];
+            else st[n][x] = is_m && wq * 32 + gk + n * 8 + (x & 1) == e0 + slab * kScanSlab + ge + (x >> 1) * 8 ? 1.0f : 0.0f;
+        }
     auto put_s = [&]() {
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
@@ -1430,7 +1448,8 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
         }
     };
     put_s();
-    const float* gc = p.gc + bh * 2 * p.ntile;
+    const float* gc = p.gc + bh * 2 * p.ntile + chunk0;
+    const uint32_t u1_mask = is_m ? 0u : 0xFFFFFFFFu;
     float g_cur = lane < nchunk ? gc[lane] : 1.0f;   // decays of 32 chunks, one per lane
 
     bool dead = false;
@@ -1502,7 +1521,7 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
         for (int n = 0; n < 2; ++n)
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
-                const uint32_t u1 = uf[2 * n + half];
+                const uint32_t u1 = kRuns ? uf[2 * n + half] & u1_mask : uf[2 * n + half];
                 const float lo = __uint_as_float(u1 << 16) - (y[0][n][2 * half] + y[1][n][2 * half]);
                 const float hi = __uint_as_float(u1 & 0xFFFF0000u) - (y[0][n][2 * half + 1] + y[1][n][2 * half + 1]);
                 *reinterpret_cast<uint32_t*>(u_s + (ge + 8 * half) * kScanLdU + wq * 16 + n * 8 + gk) = pack_bf16(lo, hi);
@@ -1539,6 +1558,7 @@ tc_token_scan_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_cons
     }
     if (dead) return;
     float* nrow = p.next + (srow - p.state);
+    if (kRuns) nrow += (bh * (2 * p.runs - 2) + (run == 0 ? 0 : 2 * run - 1 + (is_m ? 1 : 0))) * (size_t)(kTile * kTile);
 #pragma unroll
     for (int n = 0; n < 4; ++n)
 #pragma unroll
@@ -1559,6 +1579,78 @@ __global__ void __launch_bounds__(kPublishThreads) tc_token_publish_kernel(const
     if (err != 0u) return;
     *reinterpret_cast<float4*>(p.state + i) = v;
     *reinterpret_cast<uint2*>(p.state_bf16 + i) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+}
+
+// The same behind a walk in runs: S <- M_r S + N_r for r = 1 .. runs - 1, from the first run's S.  One CTA per
+// kJoinCols value columns of a head (columns do not mix), in fp32 FMAs: the state is not rounded between chunks, and
+// is not here.  A thread has 2 columns of 4 rows.  The kernel is one round of loads (72 KB per CTA) and 1.3 us of
+// multiplications; M of the next run is on its way while this one is used.
+constexpr int kJoinCols = 16, kJoinThreads = 256;
+constexpr int kJoinLdM = kTile + 4;   // fp32 row stride: the four rows a warp reads at a time lie in different banks
+constexpr int kJoinMatBytes = kTile * kJoinLdM * 4;
+constexpr int join_smem_bytes(int runs) { return (runs > 2 ? 2 : 1) * kJoinMatBytes + kTile * kJoinCols * 4; }
+__global__ void __launch_bounds__(kJoinThreads) tc_token_join_kernel(const TcTokenParams p)
+{
+    extern __shared__ __align__(16) float join_smem[];
+    float* Ss = join_smem + (p.runs > 2 ? 2 : 1) * kTile * kJoinLdM;
+    const int tid = threadIdx.x;
+    const size_t bh = blockIdx.x / (kTile / kJoinCols);
+    const int e0 = (int)(blockIdx.x % (kTile / kJoinCols)) * kJoinCols;
+    const int c2 = (tid & 7) * 2, r0 = tid >> 3;   // columns c2, c2 + 1 of rows r0 + 32 i
+    const float* base = p.next + bh * (2 * p.runs - 1) * (size_t)(kTile * kTile);
+    grid_dependency_sync();
+    const uint32_t err = p.status[kStatusError];
+    auto fetch_m = [&](int r) {
+        const float* M = base + (size_t)(2 * r) * kTile * kTile;
+        const uint32_t dst = smem_u32(join_smem + ((r - 1) & 1) * kTile * kJoinLdM);
+#pragma unroll
+        for (int i = 0; i < kTile * kTile / 4 / kJoinThreads; ++i) {
+            const int c = tid + i * kJoinThreads;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (uint32_t)((c >> 5) * kJoinLdM + (c & 31) * 4) * 4), "l"(M + c * 4)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch_m(1);
+    float2 S[4], out[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) S[i] = *reinterpret_cast<const float2*>(base + (size_t)(r0 + 32 * i) * kTile + e0 + c2);
+    for (int r = 1; r < p.runs; ++r) {
+        const float* N = base + (size_t)(2 * r - 1) * kTile * kTile;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) out[i] = *reinterpret_cast<const float2*>(N + (size_t)(r0 + 32 * i) * kTile + e0 + c2);
+        if (r > 1) __syncthreads();   // S and the other buffer of the run before have been read
+        if (r + 1 < p.runs) fetch_m(r + 1);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) *reinterpret_cast<float2*>(Ss + (r0 + 32 * i) * kJoinCols + c2) = S[i];
+        if (r + 1 < p.runs) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        const float* Ms = join_smem + ((r - 1) & 1) * kTile * kJoinLdM;
+#pragma unroll 4
+        for (int q = 0; q < kTile; q += 4) {
+            float2 s[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) s[x] = *reinterpret_cast<const float2*>(Ss + (q + x) * kJoinCols + c2);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 m = *reinterpret_cast<const float4*>(Ms + (r0 + 32 * i) * kJoinLdM + q);
+                out[i].x = fmaf(m.x, s[0].x, out[i].x); out[i].y = fmaf(m.x, s[0].y, out[i].y);
+                out[i].x = fmaf(m.y, s[1].x, out[i].x); out[i].y = fmaf(m.y, s[1].y, out[i].y);
+                out[i].x = fmaf(m.z, s[2].x, out[i].x); out[i].y = fmaf(m.z, s[2].y, out[i].y);
+                out[i].x = fmaf(m.w, s[3].x, out[i].x); out[i].y = fmaf(m.w, s[3].y, out[i].y);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) S[i] = out[i];
+    }
+    if (err != 0u) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const size_t at = (bh * kTile + r0 + 32 * i) * kTile + e0 + c2;
+        *reinterpret_cast<float2*>(p.state + at) = S[i];
+        *reinterpret_cast<uint32_t*>(p.state_bf16 + at) = pack_bf16(S[i].x, S[i].y);
+    }
 }
 
 // The rotation table in the form the step kernel reads: half2 (cos, sin) per pair, 16 vectors of
@@ -1743,9 +1835,12 @@ int device_setup(int* num_sms)
         if (e == cudaSuccess) e = opt_in_smem(tc_step_kernel<true, false>, kSmemBytes);
         if (e == cudaSuccess) e = opt_in_smem(tc_step_kernel<false, true>, kSmemBytes);
         if (e == cudaSuccess) e = opt_in_smem(tc_token_prepare_kernel, kTPSmemBytes);
-        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<1, false>, ScanCfg<1, false>::kSmemBytes);
-        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<2, false>, ScanCfg<2, false>::kSmemBytes);
-        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<2, true>, ScanCfg<2, true>::kSmemBytes);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<1, false, false>, ScanCfg<1, false>::kSmemBytes);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<2, false, false>, ScanCfg<2, false>::kSmemBytes);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<1, false, true>, ScanCfg<1, false>::kSmemBytes);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<2, false, true>, ScanCfg<2, false>::kSmemBytes);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_join_kernel, kMaxSmemPerCta);
+        if (e == cudaSuccess) e = opt_in_smem(tc_token_scan_kernel<2, true, false>, ScanCfg<2, true>::kSmemBytes);
         return e;
     }, num_sms);
 }
@@ -1843,6 +1938,14 @@ int tc_step(const StepArgs& a, const __nv_bfloat16* wq_op, const __nv_bfloat16* 
     return 2;
 }
 
+// What a chunk of the walk takes with one slab per SM and with two, and what runs cost on top (us; tc_token_join_kernel instead of
+// tc_token_publish_kernel): fitted to whole calls of 2 to 12 heads x 300 to 4680 tokens, each with 1 to 4 runs.
+// us per pass, one walk and with the runs this gives: 12 heads x 4680 tokens 83.3 -> 76.4 (2 runs, two slabs per SM),
+// 5 x 4680 69.0 -> 52.0 (2), 2 x 4680 60.1 -> 39.3 (3), 2 x 3 x 2000 37.1 -> 31.9 (2).  Two runs where they are not taken: 12 x 1560
+// 40.8 and 41.9, 8 x 1000 27.4 and 29.5, 2 x 600 23.6 and 24.5.
+constexpr float kWalkChunk = 0.61f, kWalkChunk2 = 0.90f, kJoinFirst = 5.0f, kJoinMore = 4.0f;
+constexpr int kMaxRuns = 4;
+
 // Eq. 4 token by token with per-token gates on the tensor-core path (bf16 I/O, D = 128).  The
 // scratch tensors of `a` (sized for the fp32 plain-FMA version) are used as bf16 here.
 int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const __nv_bfloat16* wv_op,
@@ -1875,7 +1978,19 @@ int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const
     // beyond (half the L2 traffic), two such CTAs per SM when even those do not fit beside one another (40 heads:
     // 157 -> 113 us for the walk; four slabs in one CTA took 205: its 16 warps load 139 KB of fragments per chunk).
     const long heads = (long)a.s.B * a.s.H;
-    const int slabs = heads * 8 <= num_sms ? 1 : 2;
+    // Runs of chunks walked side by side, where that is shorter than one walk (tc_token_scan_kernel).  A run more is 16 slabs
+    // per head more; the slabs have an SM each, or two share one, and the scratch has to hold 2 runs - 1 matrices per head.
+    const auto walk_ctas = [&](int runs, int per) { return heads * 8 * (2 * runs - 1) / per; };
+    p.runs = 1;
+    float best = kWalkChunk * (float)p.nchunk;
+    for (int r = 2; r <= kMaxRuns && walk_ctas(r, 2) <= num_sms && 2 * r - 1 <= a.next_slots; ++r) {
+        const float chunk = walk_ctas(r, 1) <= num_sms ? kWalkChunk : kWalkChunk2;
+        const float t = chunk * (float)((p.nchunk + r - 1) / r) + kJoinFirst + kJoinMore * (float)(r - 2);
+        if (t < 0.97f * best) { best = t; p.runs = r; }
+    }
+    p.run_chunks = (p.nchunk + p.runs - 1) / p.runs;
+    p.runs = (p.nchunk + p.run_chunks - 1) / p.run_chunks;   // (none is empty)
+    const int slabs = walk_ctas(p.runs, 1) <= num_sms ? 1 : 2;
     const bool shared_sm = heads * 4 > num_sms;
     CUtensorMap tm_k, tm_v, tm_wk, tm_wv, tm_w, tm_kh, tm_u1;
     if (int r = make_map_blhd(&tm_k, a.k, a.s)) return r;
@@ -1891,14 +2006,25 @@ int tc_commit_tokens(const TokenCommitArgs& a, const __nv_bfloat16* wk_op, const
     dim3 grid1(p.ntile, a.s.H, a.s.B);
     cudaError_t e = launch_kernel(tc_token_prepare_kernel, grid1, kTPThreads, kTPSmemBytes, st, tm_k, tm_v, tm_wk, tm_wv, out_w, out_u1, p);
     if (e != cudaSuccess) { set_error("launch of tc_token_prepare_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
-    dim3 grid2(kTile / (slabs * kScanSlab), a.s.H, a.s.B);
-    if (slabs == 1)
-        e = launch_kernel(tc_token_scan_kernel<1, false>, grid2, ScanCfg<1, false>::kThreads, ScanCfg<1, false>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
+    dim3 grid2((2 * p.runs - 1) * (kTile / (slabs * kScanSlab)), a.s.H, a.s.B);
+    if (p.runs > 1 && slabs == 1)
+        e = launch_kernel(tc_token_scan_kernel<1, false, true>, grid2, ScanCfg<1, false>::kThreads, ScanCfg<1, false>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
+    else if (p.runs > 1)
+        e = launch_kernel(tc_token_scan_kernel<2, false, true>, grid2, ScanCfg<2, false>::kThreads, ScanCfg<2, false>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
+    else if (slabs == 1)
+        e = launch_kernel(tc_token_scan_kernel<1, false, false>, grid2, ScanCfg<1, false>::kThreads, ScanCfg<1, false>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
     else if (!shared_sm)
-        e = launch_kernel(tc_token_scan_kernel<2, false>, grid2, ScanCfg<2, false>::kThreads, ScanCfg<2, false>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
+        e = launch_kernel(tc_token_scan_kernel<2, false, false>, grid2, ScanCfg<2, false>::kThreads, ScanCfg<2, false>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
     else
-        e = launch_kernel(tc_token_scan_kernel<2, true>, grid2, ScanCfg<2, true>::kThreads, ScanCfg<2, true>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
+        e = launch_kernel(tc_token_scan_kernel<2, true, false>, grid2, ScanCfg<2, true>::kThreads, ScanCfg<2, true>::kSmemBytes, st, tm_w, tm_kh, tm_u1, p);
     if (e != cudaSuccess) { set_error("launch of tc_token_scan_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
+    if (p.runs > 1) {
+        const int join_ctas = (int)heads * (kTile / kJoinCols);
+        e = launch_kernel(tc_token_join_kernel, dim3((unsigned)join_ctas), kJoinThreads,
+                          even_spread_smem(join_smem_bytes(p.runs), (join_ctas + num_sms - 1) / num_sms), st, p);
+        if (e != cudaSuccess) { set_error("launch of tc_token_join_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
+        return 3;
+    }
     e = launch_kernel(tc_token_publish_kernel, dim3((unsigned)(heads * (kTile * kTile / 4 / kPublishThreads))), kPublishThreads, 0, st, p);
     if (e != cudaSuccess) { set_error("launch of tc_token_publish_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 3;
