@@ -10,6 +10,7 @@
 //   warp 1     MMA issuer: per k-block 4 MMAs of 128 x BN x 16 per row half into TMEM accumulators
 //   warps 2-5  epilogue, one thread per output row of a half: TMEM -> registers -> bf16 -> global,
 //              32-byte stores
+// tc_gemm_pair_kernel is the same on pairs of CTAs (further down); which of them runs is decided by a cost model in tc_gemm.
 // MH = 1 keeps two accumulators (while the epilogue drains one the issuer fills the other).  MH = 2
 // uses the whole of tensor memory for one 256 x 256 tile: both halves share every B block, which
 // cuts the bytes fetched from L2 per flop by a third -- with 128-row tiles the operand fetch
@@ -69,6 +70,31 @@ __device__ __forceinline__ void tile_origin(int t, const GemmParams& p, int& m0,
     const int nt = in_band / rows;
     m0 = (band * kGBand + in_band - nt * rows) * p.tile_rows;
     n0 = nt * p.bn;
+}
+
+// 32 columns of an output row, which lie inside one segment
+__device__ __forceinline__ void store_chunk(const GemmParams& p, int row, int n, const uint32_t (&o)[32])
+{
+    if (row >= p.M || n >= p.N) return;
+    const int seg = n / p.seg_cols, col = n - seg * p.seg_cols;
+    if (seg < p.n_bf16_seg) {
+        __nv_bfloat16* dst = p.out[seg] + (size_t)row * p.ld_out + col;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            uint32_t w[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                w[i] = pack_bf16(__uint_as_float(o[e * 16 + 2 * i]), __uint_as_float(o[e * 16 + 2 * i + 1]));
+            asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + e * 16),
+                         "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                         : "memory");
+        }
+    } else {
+        float* dst = p.out_f32 + (size_t)row * p.ld_f32;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (col + i < p.f32_cols) dst[col + i] = __uint_as_float(o[i]);
+    }
 }
 
 template <int BN, int MH>
@@ -215,27 +241,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 uint32_t o[32];
                 tmem_ld32(lane_base + (MH == 1 ? buf : (uint32_t)hlf) * 256 + cc * 32, o);
                 tmem_wait_ld();
-                const int n = n0 + cc * 32;                                 // 32 columns lie inside one segment
-                if (row >= p.M || n >= p.N) continue;
-                const int seg = n / p.seg_cols, col = n - seg * p.seg_cols;
-                if (seg < p.n_bf16_seg) {
-                    __nv_bfloat16* dst = p.out[seg] + (size_t)row * p.ld_out + col;
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        uint32_t w[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            w[i] = pack_bf16(__uint_as_float(o[e * 16 + 2 * i]), __uint_as_float(o[e * 16 + 2 * i + 1]));
-                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + e * 16),
-                                     "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                                     : "memory");
-                    }
-                } else {
-                    float* dst = p.out_f32 + (size_t)row * p.ld_f32;
-#pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        if (col + i < p.f32_cols) dst[col + i] = __uint_as_float(o[i]);
-                }
+                store_chunk(p, row, n0 + cc * 32, o);
             }
             tc_fence_before();
             mbar_arrive(bars + 8 * (kGBarAccFree0 + buf));
@@ -247,6 +253,187 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, 512);
+    }
+}
+
+// The same on pairs of CTAs (clusters of two, neighbouring SMs): a tile is 256 x 256, one cta_group::2 MMA covers it, and each
+// CTA fetches its 128 rows of A and half of B's columns.  A k-block is 512 MMA clocks for 32 KB per SM instead of 48 KB
+// (the 128-row tile waits for its operands: 740 clocks), and tensor memory still holds two accumulators, so that the epilogue
+// stays hidden (with the 256-row tile of one CTA it does not).  The MMA issuer is in the pair's first CTA; that CTA's full
+// barriers count both CTAs' bytes, and its issuer's commits arrive in both.
+constexpr int kGPStages = 6;
+constexpr int kGPStageBytes = kGABytes + kGBBytes / 2;
+constexpr int kGPOffBars = kGPStages * kGPStageBytes;
+static_assert(kGPOffBars + 256 + 1024 <= kGemmSmemBytes, "shared memory of a pair's CTA");
+enum GPBar : int {
+    kGPBarFull0 = 0,
+    kGPBarEmpty0 = kGPBarFull0 + kGPStages,
+    kGPBarAccFull0 = kGPBarEmpty0 + kGPStages,
+    kGPBarAccFree0 = kGPBarAccFull0 + 2,
+    kGPBarDrain = kGPBarAccFree0 + 2,
+    kGPNumBars
+};
+// after the barriers: TMEM base, abort flag, k-blocks the producer has asked for
+static_assert(kGPNumBars * 8 + 12 <= 256, "barrier block");
+
+__global__ void __launch_bounds__(kGThreads, 1)
+tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b, const GemmParams p)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                               ~static_cast<uintptr_t>(1023));
+    const uint32_t smem_base = smem_u32(smem);
+    const uint32_t bars = smem_base + kGPOffBars;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kGPOffBars + kGPNumBars * 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + kGPOffBars + kGPNumBars * 8 + 4);
+    volatile uint32_t* asked = reinterpret_cast<volatile uint32_t*>(smem + kGPOffBars + kGPNumBars * 8 + 8);
+    const Abort ab{abort_flag, p.status, p.spin_limit};
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t rank = cluster_rank();
+    const uint32_t lead_bars = map_to_rank(bars, 0);
+    const int total = p.m_tiles * p.n_tiles;
+    const int n_kb = p.K / kGBK;
+    const int first = (int)(blockIdx.x >> 1), stride = (int)(gridDim.x >> 1);
+
+    if (tid == 0) {
+        for (int i = 0; i < kGPNumBars; ++i) mbar_init(bars + 8 * i, i == kGPBarAccFree0 || i == kGPBarAccFree0 + 1 ? 8 : 1);
+        *abort_flag = 0;
+        *asked = 0;
+        fence_barrier_init();
+        fence_proxy_async_smem();
+    }
+    __syncwarp();
+    if (warp == 1) {
+        tmem_alloc_pair(smem_u32(tmem_slot), 512);
+        tmem_relinquish_pair();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    grid_dependency_sync();
+
+    bool ok = true;
+    if (warp == 0) {
+        // ---------------- TMA producer ----------------
+        if (lane == 0) {
+            prefetch_tensormap(&tm_a);
+            prefetch_tensormap(&tm_b);
+            uint32_t n = 0;
+            for (int t = first; t < total && ok; t += stride) {
+                int m0, n0;
+                tile_origin(t, p, m0, n0);
+                m0 += (int)rank * kGBM;
+                n0 += (int)rank * 128;
+                for (int kb = 0; kb < n_kb; ++kb, ++n) {
+                    const uint32_t s = n % kGPStages;
+                    if (n >= (uint32_t)kGPStages) ok = wait_bar(bars + 8 * (kGPBarEmpty0 + s), ((n / kGPStages) - 1) & 1u, ab, 124);
+                    if (!ok) break;
+                    const uint32_t bar = lead_bars + 8 * (kGPBarFull0 + s);
+                    const uint32_t dst = smem_base + s * kGPStageBytes;
+                    if (rank == 0) mbar_expect_tx(bars + 8 * (kGPBarFull0 + s), 2 * kGPStageBytes);
+                    tma_load_2d_pair(dst, &tm_a, bar, kb * kGBK, m0);   // rows past M are fetched as zeros
+                    tma_load_2d_pair(dst + kGABytes, &tm_b, bar, n0, kb * kGBK);
+                    tma_load_2d_pair(dst + kGABytes + kGBK * 128, &tm_b, bar, n0 + 64, kb * kGBK);
+                }
+            }
+            *asked = n;
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: a whole warp in uniform control flow, one elected lane issues ----------------
+        if (rank == 0) {
+            const uint32_t lead = elect_one();
+            const uint32_t smem_base = __shfl_sync(0xffffffffu, smem_u32(smem), 0);
+            const uint32_t bars = smem_base + kGPOffBars;
+            const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+            const uint32_t desc_hi = (uint32_t)(smem_desc_sw128(0, 0) >> 32);
+            constexpr uint32_t kLboK = 1u << 16;
+            constexpr uint32_t kLboB = (uint32_t)((kGBK * 128) >> 4) << 16;     // 64-column groups of B, 8 KB apart
+            auto desc64 = [&](uint32_t lo) {
+                uint64_t d;
+                asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(desc_hi));
+                return d;
+            };
+            constexpr uint32_t idesc = idesc_bf16(2 * kGBM, 256, 0, 1);   // A K-major, B rows = contraction index
+            uint32_t s = 0, phase = 0, it = 0;
+            for (int t = first; t < total && ok; t += stride, ++it) {
+                const uint32_t buf = it & 1u;
+                if (it >= 2) ok = wait_bar_warp(bars + 8 * (kGPBarAccFree0 + buf), ((it >> 1) - 1) & 1u, ab, 125);
+                if (!ok) break;
+                tc_fence_after();   // (inside the k loop the mbarrier wait is all that operands from TMA need)
+                for (int kb = 0; kb < n_kb; ++kb) {
+                    ok = wait_bar_warp(bars + 8 * (kGPBarFull0 + s), phase, ab, 126);
+                    if (!ok) break;
+                    const uint32_t a_lo = ((smem_base + s * kGPStageBytes) >> 4) | kLboK;
+                    const uint32_t b_lo = ((smem_base + s * kGPStageBytes + kGABytes) >> 4) | kLboB;
+#pragma unroll
+                    for (int ks = 0; ks < kGBK / 16; ++ks)
+                        mma_ss_pair_if(lead, tmem_base + buf * 256, desc64(a_lo + (uint32_t)((ks * 32) >> 4)),
+                                       desc64(b_lo + (uint32_t)(ks * (2048 >> 4))), idesc, (kb > 0 || ks > 0) ? 1u : 0u);
+                    mma_commit_pair_if(lead, bars + 8 * (kGPBarEmpty0 + s));
+                    if (++s == (uint32_t)kGPStages) { s = 0; phase ^= 1u; }
+                }
+                if (ok) mma_commit_pair_if(lead, bars + 8 * (kGPBarAccFull0 + buf));
+            }
+            // tensor memory is freed and both CTAs end below: no MMA may still be running, no arrival on its way
+            mma_commit_pair_if(lead, bars + 8 * kGPBarDrain);
+            drain_bar(bars + 8 * kGPBarDrain, 0);
+        }
+    } else {
+        // ---------------- epilogue: thread = output row of this CTA's half of the tile ----------------
+        const int q = warp & 3;
+        const int r = q * 32 + lane;
+        const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
+        uint32_t it = 0;
+        for (int t = first; t < total; t += stride, ++it) {
+            const uint32_t buf = it & 1u;
+            int m0, n0;
+            tile_origin(t, p, m0, n0);
+            ok = wait_bar_warp(bars + 8 * (kGPBarAccFull0 + buf), (it >> 1) & 1u, ab, 127);
+            if (!ok) break;
+            tc_fence_after();
+#pragma unroll 1
+            for (int c = 0; c < 256 / 32; ++c) {
+                uint32_t o[32];
+                tmem_ld32(lane_base + buf * 256 + c * 32, o);
+                tmem_wait_ld();
+                store_chunk(p, m0 + (int)rank * kGBM + r, n0 + c * 32, o);
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(lead_bars + 8 * (kGPBarAccFree0 + buf));
+        }
+    }
+    __syncwarp();
+    // a wait that expired in one CTA ends the other's, too
+    if (!ok) st_cluster(map_to_rank(bars + kGPNumBars * 8 + 4, rank ^ 1u), 1u);
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();
+    if (*abort_flag) {
+        // Copies in flight are counted by the first CTA's barriers for both halves: the CTA that asked for fewer k-blocks asks for
+        // the missing ones (any 32 KB do), and the first CTA waits for all of them.
+        if (tid == 0) {
+            uint32_t n = *asked;
+            const uint32_t theirs = ld_cluster(map_to_rank(bars + kGPNumBars * 8 + 8, rank ^ 1u));
+            for (; n < theirs; ++n) {
+                const uint32_t s = n % kGPStages, bar = lead_bars + 8 * (kGPBarFull0 + s), dst = smem_base + s * kGPStageBytes;
+                if (rank == 0) mbar_expect_tx(bars + 8 * (kGPBarFull0 + s), 2 * kGPStageBytes);
+                tma_load_2d_pair(dst, &tm_a, bar, 0, 0);
+                tma_load_2d_pair(dst + kGABytes, &tm_b, bar, 0, 0);
+                tma_load_2d_pair(dst + kGABytes + kGBK * 128, &tm_b, bar, 0, 0);
+            }
+            if (rank == 0)
+                for (uint32_t m = n > (uint32_t)kGPStages ? n - kGPStages : 0; m < n; ++m)
+                    drain_bar(bars + 8 * (kGPBarFull0 + m % kGPStages), (m / kGPStages) & 1u);
+        }
+        __syncwarp();
+        cluster_sync_all();
+    }
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, 512);
     }
 }
 
@@ -280,6 +467,7 @@ int tc_gemm(const GemmArgs& a, cudaStream_t st)
             if (e == cudaSuccess) e = opt_in_smem(tc_gemm_kernel<128, 1>, kGemmSmemBytes);
             if (e == cudaSuccess) e = opt_in_smem(tc_gemm_kernel<256, 2>, kGemmSmemBytes);
             if (e == cudaSuccess) e = opt_in_smem(tc_gemm_kernel<192, 2>, kGemmSmemBytes);
+            if (e == cudaSuccess) e = opt_in_smem(tc_gemm_pair_kernel, kGemmSmemBytes);
             return e;
         }, &num_sms))
         return r;
@@ -301,9 +489,14 @@ int tc_gemm(const GemmArgs& a, cudaStream_t st)
     // contractions (K = 5120: 1430 against 1230 TFLOP/s) and not for K = 1536.  192 columns instead of 256
     // where that fills the rounds better (the 1536-wide output projection of 4680 tokens: 222 tiles of
     // 128 x 256 are two rounds on 148 SMs, the second half empty; 296 of 128 x 192 are two full ones).
+    // A pair's tile of 256 x 256 takes about 610 clocks per k-block, and its clusters about 3800 more to start and to end: us
+    // per launch with one CTA's tiles and with pairs, input projection of 12 heads x 4680 tokens 57.2 and 50.1, 8 x 12 x 1560
+    // 153.8 and 125.4, 40 x 4680 588 and 549, 12 x 1560 23.6 and 21.3, 5 x 1000 7.8 and 11.9; output projection 12 x 4680 21.9 and
+    // 21.2, 12 x 1560 12.2 and 13.3, 4 x 16 x 1001 31.4 and 34.3 (two rounds of pairs, the second nearly empty).
     // The 128-column tile serves N <= 128 only: at 128 x 128 both operands of an MMA come from shared
     // memory at its full rate, measured slower even where it fills the rounds.
     int mh = 1;
+    bool pair = false;
     p.bn = a.N <= 128 ? 128 : 256;
     if (p.bn == 256) {
         const int n_kb = a.K / kGBK;
@@ -317,6 +510,9 @@ int tc_gemm(const GemmArgs& a, cudaStream_t st)
                 if (best == 0.0f || cost < best) { best = cost; mh = cand_mh; p.bn = cand_bn; }
             }
         }
+        const long tiles = (long)((a.M + 2 * kGBM - 1) / (2 * kGBM)) * ((a.N + 255) / 256);
+        const int pairs = num_sms / 2;
+        if (pairs > 0 && a.M > kGBM && (float)((tiles + pairs - 1) / pairs) * (n_kb * 610.0f) + 3800.0f < best) { pair = true; mh = 2; p.bn = 256; }
     }
     p.tile_rows = mh * kGBM;
     p.m_tiles = (a.M + p.tile_rows - 1) / p.tile_rows;
@@ -327,6 +523,12 @@ int tc_gemm(const GemmArgs& a, cudaStream_t st)
     p.status = a.status;
     p.spin_limit = a.wait_limit ? a.wait_limit - 1 : kSpinLimit;
     const int total = p.m_tiles * p.n_tiles;
+    if (pair) {
+        const int pairs = total < num_sms / 2 ? total : num_sms / 2;
+        const cudaError_t e = launch_cluster(tc_gemm_pair_kernel, dim3((unsigned)(2 * pairs)), 2, kGThreads, kGemmSmemBytes, st, tm_a, tm_b, p);
+        if (e != cudaSuccess) { set_error("launch of tc_gemm_pair_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
+        return 1;
+    }
     const int grid = total < num_sms ? total : num_sms;
     auto kernel = mh == 2 ? (p.bn == 256 ? tc_gemm_kernel<256, 2> : tc_gemm_kernel<192, 2>)
                           : p.bn == 256 ? tc_gemm_kernel<256, 1> : p.bn == 192 ? tc_gemm_kernel<192, 1> : tc_gemm_kernel<128, 1>;
