@@ -428,16 +428,21 @@ tc_commit_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
 }
 
 // S <- alpha S + (sum_s A_s) W_phi_v [- (sum_s G_s) S_old]; one CTA per 16 state rows of a head, 128
-// threads.  The slots of a head are added in index order (each thread a 4 x 4 block) into shared
+// threads, and for the delta rule 128 more that add up and multiply the second term beside the first.  The slots of a head are added in index order (each thread a 4 x 4 block) into shared
 // memory; the products with the right-hand matrices (the head's value map, then S_old; both bf16)
 // run on the warp-level tensor-core instruction, one 16 x 32 block of the output per warp, with the
 // fp32 sums split into a bf16 head and a bf16 remainder (two MMAs, relative error 2^-17: far below
-// the bf16 rounding of the matrices themselves).  The first kFinMaxParts slots, the old
-// state and the matrices are requested before the first result is used; further slots, and the delta rule's second set,
-// come in a loop.
+// the bf16 rounding of the matrices themselves).  What it takes is latencies, so several slots (fin_parts), the old
+// state and the matrices are requested before the first result is used, and further slots as many at a time.  (One
+// by one, and the delta rule's second set and its product behind the first, the 13 slots of 12 heads x 4680 tokens were a chain
+// of 20 loads: delta rule 25.1 -> 23.6 us per pass, of 2 heads 19.4 -> 17.2; gated-linear commit 18.4 -> 18.0, per-token
+// decay 27.0 -> 26.6.  With 256 threads for a gated-linear commit as well: 12.3 -> 12.65 at 12 x 1560, 30.8 -> 31.6 at 40 x 4680.)
 constexpr int kFinRows = 16;
 constexpr int kFinThreads = 128;
-constexpr int kFinMaxParts = 6;     // slots of one head the unrolled loads cover; more fall back to a loop
+// Slots of one head whose loads go out together, and CTAs that share an SM: registers for more of one leave less of the other.
+// (6 and 8 slots with two CTAs: delta rule of 12 x 4680 24.2 us instead of 23.6, commit of 40 x 4680 32.2 instead of 30.7.)
+__host__ __device__ constexpr int fin_parts(int mode) { return mode == 1 ? 4 : 6; }
+constexpr int fin_ctas(int mode) { return mode == 1 ? 2 : 3; }
 constexpr int kFinLdM = kTile + 8;  // bf16 row stride of a right-hand matrix: 272 bytes, conflict-free 8 x 8 loads
 constexpr int kFinLdA = kTile + 8;  // fp32 row stride of the summed rows: a fragment's 8-byte reads spread over the banks
 constexpr int kFinMatBytes = kTile * kFinLdM * 2;
@@ -523,7 +528,7 @@ __device__ __forceinline__ void fin_multiply(float (&acc)[4][4], const float* __
 }
 
 template <int kMode>
-__global__ void __launch_bounds__(kFinThreads)
+__global__ void __launch_bounds__(kMode == 1 ? 2 * kFinThreads : kFinThreads, fin_ctas(kMode))
 tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
                         const float* partials_g, const __nv_bfloat16* wv,
                         const float* decay, int decay_direct, const __nv_bfloat16* mirror_cur, __nv_bfloat16* mirror_next,
@@ -534,7 +539,9 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
     float* As = reinterpret_cast<float*>(fin_smem + kFinMatBytes);                   // [16][128] summed rows
     __nv_bfloat16* Ss = reinterpret_cast<__nv_bfloat16*>(fin_smem + kFinMatBytes + kFinRowBytes);   // S_old [m][e] (delta rule)
     float* Gs = reinterpret_cast<float*>(fin_smem + 2 * kFinMatBytes + kFinRowBytes);               // its rows
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the second group of the delta rule's threads has its second term
+    const bool second = kMode == 1 && threadIdx.x >= kFinThreads;
+    const int tid = threadIdx.x & (kFinThreads - 1), lane = tid & 31, warp = tid >> 5;
     // what this thread sums: row lane / 2 of the CTA's 16, four columns (lane % 2) * 4 .. of each of
     // the column groups 4 warp .. 4 warp + 3 -- a warp then reads 512 contiguous bytes of a slot at a time
     const int srow = lane >> 1, shalf = lane & 1;
@@ -545,8 +552,8 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
     // is still draining.  What does not depend on that kernel (the value map, the current mirror) is
     // fetched first; the wait below returns once the whole preceding kernel has finished and its
     // writes are visible.
-    if (wv != nullptr) fin_load_matrix(Ws, wv + (size_t)h * kTile * kTile, tid);
-    if (kMode == 1) fin_load_matrix(Ss, mirror_cur + head, tid);
+    if (!second && wv != nullptr) fin_load_matrix(Ws, wv + (size_t)h * kTile * kTile, tid);
+    if (second) fin_load_matrix(Ss, mirror_cur + head, tid);
     const float decay_v = decay[bh];
     grid_dependency_sync();
     const uint32_t err = status != nullptr ? status[kStatusError] : 0u;
@@ -556,23 +563,30 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
     // of this thread's column groups to the next: 128 rows x 8
     const size_t slot0 = (size_t)bh * nslot * kTile * kTile + ((size_t)(warp * 4) * kTile + cta_row0 + srow) * 8 + shalf * 4;
     // ---- all loads first: the slots, the old state at the positions of this thread's output fragment
+    const float* slots = (second ? partials_g : partials) + slot0;
+    constexpr int kFinMaxParts = fin_parts(kMode);
     float4 pa[kFinMaxParts][4];
+    auto request = [&](int s0) {
 #pragma unroll
-    for (int s = 0; s < kFinMaxParts; ++s) {
-        if (s < nparts) {
+        for (int s = 0; s < kFinMaxParts; ++s) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                pa[s][i] = *reinterpret_cast<const float4*>(partials + slot0 + (size_t)s * kTile * kTile + (size_t)i * kTile * 8);
+            for (int i = 0; i < 4; ++i) {
+                if (s0 + s < nparts)
+                    pa[s][i] = *reinterpret_cast<const float4*>(slots + (size_t)(s0 + s) * kTile * kTile + (size_t)i * kTile * 8);
+            }
         }
-    }
+    };
+    request(0);
     const int g = lane >> 2, t = lane & 3;
     // output fragment: rows g and g + 8 of the CTA's 16, columns warp * 32 + 8 j + 2 t (+ 1), j = 0..3
     const size_t out0 = head + (size_t)(cta_row0 + g) * kTile + warp * 32 + 2 * t;
     float2 old[4][2];
+    if (!second) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        old[j][0] = *reinterpret_cast<const float2*>(state + out0 + j * 8);
-        old[j][1] = *reinterpret_cast<const float2*>(state + out0 + j * 8 + 8 * kTile);
+        for (int j = 0; j < 4; ++j) {
+            old[j][0] = *reinterpret_cast<const float2*>(state + out0 + j * 8);
+            old[j][1] = *reinterpret_cast<const float2*>(state + out0 + j * 8 + 8 * kTile);
+        }
     }
     if (err != 0u) {
         // a partial-sum CTA gave up on a bounded wait: S stays as it was, and so does its mirror
@@ -589,38 +603,27 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
     float4 a[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) a[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0;;) {
 #pragma unroll
-    for (int s = 0; s < kFinMaxParts; ++s) {
-        if (s < nparts) {
+        for (int s = 0; s < kFinMaxParts; ++s) {
+            if (s0 + s < nparts) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) add4(a[i], pa[s][i]);
+                for (int i = 0; i < 4; ++i) add4(a[i], pa[s][i]);
+            }
         }
+        s0 += kFinMaxParts;
+        if (s0 >= nparts) break;
+        request(s0);
     }
-    for (int s = kFinMaxParts; s < nparts; ++s) {
+    float* rows = second ? Gs : As;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            add4(a[i], *reinterpret_cast<const float4*>(partials + slot0 + (size_t)s * kTile * kTile + (size_t)i * kTile * 8));
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(As + srow * kFinLdA + (warp * 4 + i) * 8 + shalf * 4) = a[i];
-    if (kMode == 1) {
-        float4 gs[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) gs[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int s = 0; s < nparts; ++s) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                add4(gs[i], *reinterpret_cast<const float4*>(partials_g + slot0 + (size_t)s * kTile * kTile + (size_t)i * kTile * 8));
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(Gs + srow * kFinLdA + (warp * 4 + i) * 8 + shalf * 4) = gs[i];
-    }
+    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(rows + srow * kFinLdA + (warp * 4 + i) * 8 + shalf * 4) = a[i];
     fin_matrices_landed();
     __syncthreads();
     float out[4][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        if (wv == nullptr) {   // identity value map: the sums themselves
+        if (wv == nullptr && !second) {   // identity value map: the sums themselves
             const float2 lo = *reinterpret_cast<const float2*>(As + g * kFinLdA + warp * 32 + j * 8 + 2 * t);
             const float2 hi = *reinterpret_cast<const float2*>(As + (g + 8) * kFinLdA + warp * 32 + j * 8 + 2 * t);
             out[j][0] = lo.x; out[j][1] = lo.y; out[j][2] = hi.x; out[j][3] = hi.y;
@@ -628,8 +631,28 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
             out[j][0] = out[j][1] = out[j][2] = out[j][3] = 0.0f;
         }
     }
-    if (wv != nullptr) fin_multiply<false>(out, As, Ws, warp, lane);
-    if (kMode == 1) fin_multiply<true>(out, Gs, Ss, warp, lane);
+    if (kMode == 1) {
+        if (second) fin_multiply<true>(out, Gs, Ss, warp, lane);
+        else if (wv != nullptr) fin_multiply<false>(out, As, Ws, warp, lane);
+        __syncthreads();   // the second term's rows have been read: its product takes their place
+        if (second) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                *reinterpret_cast<float2*>(Gs + g * kFinLdA + warp * 32 + j * 8 + 2 * t) = make_float2(out[j][0], out[j][1]);
+                *reinterpret_cast<float2*>(Gs + (g + 8) * kFinLdA + warp * 32 + j * 8 + 2 * t) = make_float2(out[j][2], out[j][3]);
+            }
+        }
+        __syncthreads();
+        if (second) return;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 lo = *reinterpret_cast<const float2*>(Gs + g * kFinLdA + warp * 32 + j * 8 + 2 * t);
+            const float2 hi = *reinterpret_cast<const float2*>(Gs + (g + 8) * kFinLdA + warp * 32 + j * 8 + 2 * t);
+            out[j][0] += lo.x; out[j][1] += lo.y; out[j][2] += hi.x; out[j][3] += hi.y;
+        }
+    } else if (wv != nullptr) {
+        fin_multiply<false>(out, As, Ws, warp, lane);
+    }
     const float alpha = decay_direct ? decay_v : 1.0f / (1.0f + __expf(-decay_v));
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -809,7 +832,7 @@ int tc_commit_finish(const CommitArgs& a, cudaStream_t st)
     const int need = fin_smem_bytes(a.mode == 1 ? 1 : 0);
     const size_t smem = (int)grid <= 2 * (num_sms - partial_ctas) ? (size_t)need
                                                                    : even_spread_smem(need, (int)((grid + (unsigned)num_sms - 1) / (unsigned)num_sms));
-    const cudaError_t e = launch_kernel(kernel, dim3(grid), kFinThreads, smem, st, a.state, a.partials, a.partials_g,
+    const cudaError_t e = launch_kernel(kernel, dim3(grid), a.mode == 1 ? 2 * kFinThreads : kFinThreads, smem, st, a.state, a.partials, a.partials_g,
                                         static_cast<const __nv_bfloat16*>(a.wv), a.decay, a.decay_direct ? 1 : 0, a.state_bf16, a.state_bf16_next,
                                         a.s.H, a.run_share, a.run_ntile, a.nslot, a.status);
     if (e != cudaSuccess) { set_error("launch of tc_commit_finish_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
