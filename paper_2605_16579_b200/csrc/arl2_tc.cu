@@ -391,6 +391,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                 const size_t rbase = ((size_t)b * L + (valid_row ? row : 0)) * H + h;
                 __nv_bfloat16* orow = p.out + rbase * kTile;
                 const float* grow = p.gate + rbase * kTile;
+                const bool g_wide = (reinterpret_cast<uintptr_t>(p.gate) & 15) == 0;   // the logits may start at any element
 #pragma unroll 1
                 for (int hv = 0; hv < 2; ++hv) {
                     if (!wait_bar(bar_s, s_cnt & 1, ab, 32 + t)) return;
@@ -408,7 +409,8 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                                 uint32_t w[8];
 #pragma unroll
                                 for (int i = 0; i < 4; ++i) {
-                                    const float4 gl = *reinterpret_cast<const float4*>(grow + hv * 64 + c * 32 + e * 16 + i * 4);
+                                    const float* gp = grow + hv * 64 + c * 32 + e * 16 + i * 4;
+                                    const float4 gl = g_wide ? *reinterpret_cast<const float4*>(gp) : make_float4(gp[0], gp[1], gp[2], gp[3]);
                                     const float gv[4] = {gl.x, gl.y, gl.z, gl.w};
                                     float y[4];
 #pragma unroll
@@ -419,10 +421,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                                     w[i * 2] = pack_bf16(y[0], y[1]);
                                     w[i * 2 + 1] = pack_bf16(y[2], y[3]);
                                 }
-                                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
-                                                 orow + hv * 64 + c * 32 + e * 16),
-                                             "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                                             : "memory");
+                                store_row32(orow + hv * 64 + c * 32 + e * 16, w, wide_rows(p.out));
                             }
                         }
                     }
@@ -508,10 +507,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                         for (int i = 0; i < 8; ++i)
                             w[i] = pack_bf16(__uint_as_float(o[e * 16 + 2 * i]) * inv_l,
                                              __uint_as_float(o[e * 16 + 2 * i + 1]) * inv_l);
-                        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(
-                                         orow + c * 32 + e * 16),
-                                     "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                                     : "memory");
+                        store_row32(orow + c * 32 + e * 16, w, wide_rows(p.out));
                     }
                 }
             }

@@ -358,13 +358,22 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         uint32_t prev[32];
         const size_t at0 = (((size_t)b * L + (row < L ? row : 0)) * H + h) * kTile + hf * 64;
         if (row < L) {
+            if (wide_rows(p.out)) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                             : "=r"(prev[i * 8]), "=r"(prev[i * 8 + 1]), "=r"(prev[i * 8 + 2]), "=r"(prev[i * 8 + 3]),
-                               "=r"(prev[i * 8 + 4]), "=r"(prev[i * 8 + 5]), "=r"(prev[i * 8 + 6]), "=r"(prev[i * 8 + 7])
-                             : "l"(p.out + at0 + i * 16)
-                             : "memory");
+                for (int i = 0; i < 4; ++i)
+                    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                                 : "=r"(prev[i * 8]), "=r"(prev[i * 8 + 1]), "=r"(prev[i * 8 + 2]), "=r"(prev[i * 8 + 3]),
+                                   "=r"(prev[i * 8 + 4]), "=r"(prev[i * 8 + 5]), "=r"(prev[i * 8 + 6]), "=r"(prev[i * 8 + 7])
+                                 : "l"(p.out + at0 + i * 16)
+                                 : "memory");
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(prev[i * 4]), "=r"(prev[i * 4 + 1]), "=r"(prev[i * 4 + 2]), "=r"(prev[i * 4 + 3])
+                                 : "l"(p.out + at0 + i * 8)
+                                 : "memory");
+            }
         }
         alive = wait_bar(bars + 8 * kTRBarB, par, ab, 114);
         if (tid == 0 && ok && alive && g + 1 < g_end) {
@@ -394,9 +403,7 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
                     for (int m = 0; m < 8; ++m)
                         nw[m] = pack_bf16(__uint_as_float(prev[i * 8 + m] << 16) + f * __uint_as_float(o[i * 16 + 2 * m]),
                                           __uint_as_float(prev[i * 8 + m] & 0xFFFF0000u) + f * __uint_as_float(o[i * 16 + 2 * m + 1]));
-                    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p.out + at0 + i * 16), "r"(nw[0]),
-                                 "r"(nw[1]), "r"(nw[2]), "r"(nw[3]), "r"(nw[4]), "r"(nw[5]), "r"(nw[6]), "r"(nw[7])
-                                 : "memory");
+                    store_row32(p.out + at0 + i * 16, nw, wide_rows(p.out));
                 }
             }
         }
