@@ -861,9 +861,10 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
 //   Gram matrix K' K'^T -> A (fp32, column by column, over W_v);  diag(beta g) K' over K'
 //   T = (I + A)^-1 in place: the four 16 x 16 diagonal blocks of a chunk by forward substitution (thread =
 //   column), then T21 = -T22 A21 T11 for blocks of 16 and of 32 (all threads)
-//   T as a bf16 operand (over A): 128 rows x 64, each chunk's block in its own rows
-//   W = T diag(beta g) K', then U1 = T diag(beta) V': one MMA per chunk over all 128 rows, each token row
-//   read from its own chunk's result -> global: W, U1 (and Khat on the way) in bf16, chunk decays g in fp32.
+//   T as a bf16 operand (over A): 128 x 128, zero off the chunks' blocks
+//   W = T diag(beta g) K' and U1 = T diag(beta) V', T with both chunks' blocks on its diagonal (the zeros cost no MMA: with one per
+//   chunk over all 128 rows, U1 had no columns of its own and waited for W's write-out) -> global: W, U1 (and Khat on the way) in
+//   bf16, chunk decays g in fp32.
 // 12 heads x 4680 tokens (444 tiles), inside the call: 66 us with one 128-thread CTA per SM, T by one 64-step
 // substitution per column and row-wise stores -> 42 us; 40 heads 205 -> 112 (each alone).
 // tc_token_scan_kernel: walks the chunks of a head in order (further down).
@@ -992,15 +993,12 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
         for (int ks = 0; ks < 8; ++ks)
             mma_ss(tmem_base + col, desc64(a_lo + koff_k(ks)), desc64(b_lo + koff_k(ks)), idesc_kk, ks > 0);
     };
-    // columns c * 128: T (all 128 rows) times the 64 token rows of chunk c of a tile
-    auto issue_t = [&](int b_off) {
+    // D[128 x 128] = T (both chunks' blocks on its diagonal) times a tile, tokens contracted
+    auto issue_t = [&](uint32_t col, int b_off) {
         const uint32_t t_lo = ((smem_base + kTPOffW) >> 4) | kLboK, b_lo = ((smem_base + b_off) >> 4) | kLboMN;
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-                mma_ss(tmem_base + c * kTile, desc64(t_lo + (uint32_t)(ks * 32 >> 4)),
-                       desc64(b_lo + (uint32_t)((c * 4 + ks) * (2048 >> 4))), idesc_kn, ks > 0);
+        for (int ks = 0; ks < 8; ++ks)
+            mma_ss(tmem_base + col, desc64(t_lo + koff_k(ks)), desc64(b_lo + (uint32_t)(ks * (2048 >> 4))), idesc_kn, ks > 0);
     };
 
     // ---- gates: log alpha_j, beta_j, cumulative decay within the chunk (tokens past L: 1 and 0)
@@ -1040,17 +1038,18 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     const float cl_pred = p.decayed ? cl : cl_excl;
 
     // 32 columns of this thread's half row (piece q of 2) into a swizzled tile, times f
-    auto put32 = [&](int off, int q, const uint32_t (&y)[32], float f) {
+    auto put32_at = [&](int off, int half, int q, const uint32_t (&y)[32], float f) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             uint32_t w[4];
 #pragma unroll
             for (int m = 0; m < 4; ++m)
                 w[m] = pack_bf16(__uint_as_float(y[c * 8 + 2 * m]) * f, __uint_as_float(y[c * 8 + 2 * m + 1]) * f);
-            *reinterpret_cast<uint4*>(smem + off + hf * kHalfBytes + r * 128 + (((q * 4 + c) ^ (r & 7)) << 4)) =
+            *reinterpret_cast<uint4*>(smem + off + half * kHalfBytes + r * 128 + (((q * 4 + c) ^ (r & 7)) << 4)) =
                 make_uint4(w[0], w[1], w[2], w[3]);
         }
     };
+    auto put32 = [&](int off, int q, const uint32_t (&y)[32], float f) { put32_at(off, hf, q, y, f); };
     alive = wait_bar(bars + 8 * kTPBarUk, 0, ab, 96);
     if (issuer && ok && alive) {
         // the value map takes the key map's place while the rows of K' are worked out
@@ -1150,15 +1149,6 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
     alive = alive && wait_bar(bars + 8 * kTPBarG, 0, ab, 92);
     if (alive) {
         tc_fence_after();
-        // diag(beta g) K' replaces K', which the Gram matrix was the last to read
-        const float f_w = be * expf(cl_pred);
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            uint32_t y[32];
-            tmem_ld32(lane_base + hf * 64 + q * 32, y);
-            tmem_wait_ld();
-            put32(kTPOffK, q, y, f_w);
-        }
         // this token's row of A: the columns of its own chunk, strictly below the diagonal (zero elsewhere),
         // stored column by column (a warp's 32 rows side by side).  All values before the first store: the
         // compiler may not move the reads of cl_s across stores to shared memory.
@@ -1196,6 +1186,16 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
                         if (i4 * 4 + k > j) t[i4 * 4 + k] = fmaf(-av[k], t[j], t[i4 * 4 + k]);
                 }
             }
+        } else if (alive) {
+            // the other four warps meanwhile: diag(beta g) K' replaces K', which the Gram matrix was the last to read
+            const float f_w = be * expf(cl_pred);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t y[32];
+                tmem_ld32(lane_base + q * 32, y);
+                tmem_wait_ld();
+                put32_at(kTPOffK, q >> 1, q & 1, y, f_w);
+            }
         }
         __syncthreads();
         if (tid < 128) {
@@ -1205,15 +1205,20 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
         }
         __syncthreads();
         // out(i, j) = sign * sum over k0 <= k < k1 of P(i, k) Q(k, j) for i = i0 .. i0 + 3 and j = j0, j0 + JS ..: each operand given
-        // by its first element; i is contiguous in P and out, k in Q.  What binds it is the shared memory, 16 bytes
-        // per thread and load: 6 loads per 32 FMAs, and only the k where the triangular operand is not zero (the same for a
-        // warp).  With one row per thread (12 loads per 32 FMAs) and all k
-        // the products took 6.9 k of a CTA's 31 k clk, now 4.8 k: commit_tokens of 12 heads x 4680 tokens 76.4 -> 73.1 us, of 40 220 -> 206.
-        auto product = [&](auto nj_tag, auto js_tag, const float* P, const float* Q, float* out, float sign, int i0, int j0, int k0, int k1) {
-            constexpr int NJ = decltype(nj_tag)::value, JS = decltype(js_tag)::value;
+        // by its first element; i is contiguous in P and out, k in Q.  Two lanes (xor 1 << SB) share these outputs, taking every
+        // second group of four k; each ends up with half of the columns.  What binds it is the shared memory, 16 bytes
+        // per thread and load, of which a wider block needs fewer per FMA, and the chain behind one load, which the split of k
+        // halves; only the k where the triangular operand is not zero are walked (the same for a warp).
+        // The chunks' warps take their shares in opposite order, since warps w and w + 4 issue from the same quarter of the SM.
+        // Products 6.9 k of a CTA's 31 k clk with one row per thread and all k, 4.8 k with four rows and the triangles, 4.3 k so
+        // (commit_tokens of 12 heads x 4680 tokens 76.4 -> 73.1 -> 71.8 us, of 40 220 -> 206.6 -> 203.0; the last step together with the
+        // diagonal's idle warps and U1 under W, below).
+        auto product = [&](auto nj_tag, auto js_tag, auto sb_tag, const float* P, const float* Q, float* out, float sign, int i0, int j0, int k0, int k1) {
+            constexpr int NJ = decltype(nj_tag)::value, JS = decltype(js_tag)::value, SB = decltype(sb_tag)::value;
+            const bool second = (lane >> SB & 1) != 0;
             float acc[NJ][4] = {};
-#pragma unroll 4
-            for (int k4 = k0; k4 < k1; k4 += 4) {
+#pragma unroll 2
+            for (int k4 = k0 + (second ? 4 : 0); k4 < k1; k4 += 8) {
                 float4 pv[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) pv[k] = *reinterpret_cast<const float4*>(P + (k4 + k) * kLdA + i0);
@@ -1227,35 +1232,44 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
                 }
             }
 #pragma unroll
-            for (int j = 0; j < NJ; ++j)
-                *reinterpret_cast<float4*>(out + (j0 + j * JS) * kLdA + i0) = make_float4(sign * acc[j][0], sign * acc[j][1], sign * acc[j][2], sign * acc[j][3]);
+            for (int j = 0; j < NJ / 2; ++j) {
+                float y[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float give = second ? acc[j][i] : acc[NJ / 2 + j][i], keep = second ? acc[NJ / 2 + j][i] : acc[j][i];
+                    y[i] = sign * (keep + __shfl_xor_sync(0xffffffffu, give, 1 << SB));
+                }
+                *reinterpret_cast<float4*>(out + (j0 + (j + (second ? NJ / 2 : 0)) * JS) * kLdA + i0) = make_float4(y[0], y[1], y[2], y[3]);
+            }
         };
+        const int pw = (warp & 3) ^ (tid >= 128 ? 3 : 0);   // four warps per chunk
+        float* X = As + (tid >> 7) * kTokC * kLdA;
         {
             // blocks of 16: rows 32 m + 16 .., columns 32 m ..; the intermediate A21 T11 goes to the unused
-            // rows 0-15 of columns 32 + 16 m ..
-            const int c = tid >> 7, m = tid >> 6 & 1, u = tid & 63;
-            float* X = As + c * kTokC * kLdA;
+            // rows 0-15 of columns 32 + 16 m ..  Two warps per m: of columns 0-7 and 8-15 first, then of rows 0-7 and 8-15
+            const int m = pw >> 1, w = pw & 1;
             float* low = X + (m * 32) * kLdA + m * 32 + 16;
             float* tmp = X + (32 + m * 16) * kLdA;
-            const auto one = std::integral_constant<int, 1>();
-            product(one, one, low, X + (m * 32) * kLdA + m * 32, tmp, 1.0f, (u & 3) * 4, u >> 2, (u >> 5) * 8, 16);
+            const auto two = std::integral_constant<int, 2>();
+            product(two, std::integral_constant<int, 1>(), two, low, X + (m * 32) * kLdA + m * 32, tmp, 1.0f, (lane & 3) * 4, w * 8 + (lane >> 3) * 2, w * 8, 16);
             __syncthreads();
-            product(one, one, X + (m * 32 + 16) * kLdA + m * 32 + 16, tmp, low, -1.0f, (u >> 4) * 4, u & 15, 0, (u >> 5) * 8 + 8);
+            product(two, std::integral_constant<int, 8>(), std::integral_constant<int, 3>(), X + (m * 32 + 16) * kLdA + m * 32 + 16, tmp, low, -1.0f,
+                    w * 8 + (lane >> 4) * 4, lane & 7, 0, w * 8 + 8);
             __syncthreads();
         }
         {
-            // blocks of 32: rows 32 .., columns 0 ..; the intermediate in rows 0-31 of columns 32 ..
-            const int c = tid >> 7, u = tid & 127;
-            float* X = As + c * kTokC * kLdA;
+            // blocks of 32: rows 32 .., columns 0 ..; the intermediate in rows 0-31 of columns 32 ..  Four warps: of eight columns
+            // each first, then of eight rows each
             float* low = X + 32;
             float* tmp = X + 32 * kLdA;
-            const auto two = std::integral_constant<int, 2>();
-            product(two, std::integral_constant<int, 1>(), low, X, tmp, 1.0f, (u & 7) * 4, (u >> 3) * 2, (u >> 5) * 8, 32);
+            const auto four = std::integral_constant<int, 4>();
+            const auto bit3 = std::integral_constant<int, 3>();
+            product(four, std::integral_constant<int, 1>(), bit3, low, X, tmp, 1.0f, (lane & 7) * 4, pw * 8 + (lane >> 4) * 4, pw * 8, 32);
             __syncthreads();
-            product(two, std::integral_constant<int, 16>(), X + 32 * kLdA + 32, tmp, low, -1.0f, (u >> 4) * 4, u & 15, 0, (u >> 5) * 8 + 8);
+            product(four, std::integral_constant<int, 8>(), bit3, X + 32 * kLdA + 32, tmp, low, -1.0f, pw * 8 + (lane >> 4) * 4, lane & 7, 0, pw * 8 + 8);
             __syncthreads();
         }
-        // T as a K-major swizzled operand (row = token, 64 columns), over the fp32 matrix
+        // T as a K-major swizzled operand (row = token, 64 columns of the row's own chunk, zeros in the other's), over the fp32 matrix
         uint4 tv[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -1271,36 +1285,39 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
         }
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4*>(smem + kTPOffW + r * 128 + (((hf * 4 + q) ^ (r & 7)) << 4)) = tv[q];
+        for (int q = 0; q < 4; ++q) {
+            uint8_t* piece = smem + kTPOffW + r * 128 + (((hf * 4 + q) ^ (r & 7)) << 4);
+            *reinterpret_cast<uint4*>(piece + chunk * kHalfBytes) = tv[q];
+            *reinterpret_cast<uint4*>(piece + (1 - chunk) * kHalfBytes) = make_uint4(0, 0, 0, 0);
+        }
     }
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
 
-    // ---- W = T diag(beta g) K', then U1 = T diag(beta) V': chunk c's rows in columns c * 128 ..
+    // ---- W = T diag(beta g) K' -> columns 0-127, U1 = T diag(beta) V' -> columns 128-255, on its way under W's write-out
+    if (issuer && ok && !*abort_flag) {
+        tc_fence_after();
+        issue_t(0, kTPOffK);
+        mma_commit(bars + 8 * kTPBarW);
+        issue_t(kTile, kTPOffV);
+        mma_commit(bars + 8 * kTPBarU1);
+    }
 #pragma unroll 1
     for (int u = 0; u < 2; ++u) {
-        const uint32_t bar = bars + 8 * (u == 0 ? kTPBarW : kTPBarU1);
-        if (issuer && ok && !*abort_flag) {
-            tc_fence_after();
-            issue_t(u == 0 ? kTPOffK : kTPOffV);
-            mma_commit(bar);
-        }
-        alive = alive && wait_bar(bar, 0, ab, 93);
+        alive = alive && wait_bar(bars + 8 * (u == 0 ? kTPBarW : kTPBarU1), 0, ab, 93);
         if (alive) {
             tc_fence_after();
             // staged in the tile that this product was the last to read
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 uint32_t y[32];
-                tmem_ld32(lane_base + chunk * kTile + hf * 64 + q * 32, y);
+                tmem_ld32(lane_base + u * kTile + hf * 64 + q * 32, y);
                 tmem_wait_ld();
                 put32(u == 0 ? kTPOffK : kTPOffV, q, y, 1.0f);
             }
         }
         fence_proxy_async_smem();
-        tc_fence_before();
         __syncthreads();
         // ---- it leaves as a whole tile
         if (issuer && ok && alive && !*abort_flag) {
