@@ -1157,8 +1157,13 @@ tc_token_prepare_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_c
         tmem_wait_ld();
         const float* cl_c = cl_s + chunk * kTokC + hf * 32;
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
-            g[i] = __float_as_uint(hf * 32 + i < jj ? be * __expf(cl_pred - cl_c[i]) * __uint_as_float(g[i]) : 0.0f);
+        for (int i = 0; i < 32; ++i) {
+            float x = be * __expf(cl_pred - cl_c[i]) * __uint_as_float(g[i]);
+            // worked out in any case: with a branch round each exponential this pass took 2.1 k clk, now 0.8 k (2 heads x 4680
+            // tokens 37.6 -> 37.2 us, 12 heads 71.8 -> 71.3, 5 x 700 22.7 -> 22.3)
+            asm volatile("" : "+f"(x));
+            g[i] = hf * 32 + i < jj ? __float_as_uint(x) : 0u;
+        }
         float* a_out = As + (chunk * kTokC + hf * 32) * kLdA + jj;
 #pragma unroll
         for (int i = 0; i < 32; ++i) a_out[i * kLdA] = __uint_as_float(g[i]);
