@@ -41,12 +41,12 @@ namespace {
 constexpr int kTRThreads = 256;
 constexpr int kTROffWq = 0, kTROffWk = kTileBytes, kTROffWv = 2 * kTileBytes;
 constexpr int kTROffQ = 3 * kTileBytes, kTROffK = 4 * kTileBytes, kTROffV = 5 * kTileBytes;
-constexpr int kTROffS = 6 * kTileBytes;                 // bf16 copy of Shat, [d][e]
+constexpr int kTROffS = 6 * kTileBytes;                 // bf16 copy of Shat, [d][e]; then the tile's output rows
 constexpr int kTROffBars = 7 * kTileBytes;
 constexpr int kTROffGates = kTROffBars + 128;           // lg[128], then warp totals
 constexpr int kTRSmemBytes = kTROffGates + 128 * 4 + 64 + 1024;
 
-enum TRBar : int { kTRBarW = 0, kTRBarLoad, kTRBarU, kTRBarA, kTRBarB, kTRBarDrain, kTRNumBars };
+enum TRBar : int { kTRBarW = 0, kTRBarLoad, kTRBarU, kTRBarA, kTRBarB, kTRBarOut, kTRBarDrain, kTRNumBars };
 
 struct TcReadoutParams {
     Shape s;
@@ -56,7 +56,6 @@ struct TcReadoutParams {
     const float* state;        // [B, H, 128, 128] fp32, read only
     const float* entry;        // [B * H, nslot, 128 x 128]: state at the start of each segment (slot layout of the commit),
                                // or nullptr: every run is a whole head and starts from `state`
-    __nv_bfloat16* out;        // [B, L, H, 128]: receives += sigmoid(g) X
     uint32_t* status;
     uint32_t spin_limit;
     int ntile;                 // 128-token tiles per (stream, head)
@@ -68,6 +67,7 @@ __global__ void __launch_bounds__(kTRThreads, 1)
 tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                         const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_wq,
                         const __grid_constant__ CUtensorMap tm_wk, const __grid_constant__ CUtensorMap tm_wv,
+                        const __grid_constant__ CUtensorMap tm_o,   // [B, L, H, 128], boxes of 32 rows: receives += sigmoid(g) X
                         const TcReadoutParams p)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -132,7 +132,7 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             tma_load_2d(smem_base + i * kTileBytes + kHalfBytes, maps[i], bar, 64, h * kTile);
         }
     };
-    int loads = 0, map_loads = 0;
+    int loads = 0, map_loads = 0, out_loads = 0;
     if (tid == 0) {
         load_maps(g_begin / p.ntile % H);
         load_tiles(g_begin);
@@ -207,6 +207,7 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             tmem_wait_st();
             ++segs;
         }
+        if (lane == 0) tma_store_wait_read();   // the last tile's rows have left the place where Shat goes
         // ---- gates of the chunk: lg_j = sum_{m <= j} log alpha_m (tokens past L: alpha = 1)
         float la_log = 0.0f;   // log alpha of this thread's token
         if (hf == 0) {
@@ -321,6 +322,18 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             mma_commit(bars + 8 * kTRBarA);
         }
         alive = wait_bar(bars + 8 * kTRBarA, par, ab, 113);
+        if (tid == 0 && ok && alive) {
+            // Shat's operand copy has been read: what the softmax branch left in these rows comes in its place, under pass 2 and the MMAs
+            // after it, and the sums leave from there, both by TMA.  Row by row from the threads, 32 bytes at a time and
+            // asked for ahead, the epilogue took 3.0 k of a tile's 13.5 k clk (by 16, when needed, 7.9 k of 17.7 k): 40 heads x 1500 tokens
+            // 136.8 -> 131.4 us per pass, 8 x 12 x 700 116.2 -> 112.6, 12 x 1560 the same (one tile per CTA)
+            const uint32_t bar = bars + 8 * kTRBarOut;
+            mbar_expect_tx(bar, kTileBytes);
+#pragma unroll
+            for (int w = 0; w < 8; ++w)
+                tma_load_4d(smem_base + kTROffS + (w >> 2) * kHalfBytes + (w & 3) * 32 * 128, &tm_o, bar, (w >> 2) * 64, h, tl * kTile + (w & 3) * 32, b);
+            ++out_loads;
+        }
         if (alive) {
             tc_fence_after();
             // ---- pass 2: P = strictly lower triangle of SC (keys hf * 64 ..), bf16 pairs into the U_v columns
@@ -352,29 +365,6 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
             }
             mma_commit(bars + 8 * kTRBarB);
         }
-        // what the softmax branch left in this thread's half row is on its way under these MMAs, 32 bytes at a time (a whole sector:
-        // by 16, and asked for when it was needed, the epilogue took 7.9 k of a tile's 17.7 k clk, now 2.8 k: 12 heads x 1560 tokens 65.8 -> 61.6 us per pass, 8 x 12 x 700
-        // 119 -> 108)
-        uint32_t prev[32];
-        const size_t at0 = (((size_t)b * L + (row < L ? row : 0)) * H + h) * kTile + hf * 64;
-        if (row < L) {
-            if (wide_rows(p.out)) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                 : "=r"(prev[i * 8]), "=r"(prev[i * 8 + 1]), "=r"(prev[i * 8 + 2]), "=r"(prev[i * 8 + 3]),
-                                   "=r"(prev[i * 8 + 4]), "=r"(prev[i * 8 + 5]), "=r"(prev[i * 8 + 6]), "=r"(prev[i * 8 + 7])
-                                 : "l"(p.out + at0 + i * 16)
-                                 : "memory");
-            } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(prev[i * 4]), "=r"(prev[i * 4 + 1]), "=r"(prev[i * 4 + 2]), "=r"(prev[i * 4 + 3])
-                                 : "l"(p.out + at0 + i * 8)
-                                 : "memory");
-            }
-        }
         alive = wait_bar(bars + 8 * kTRBarB, par, ab, 114);
         if (tid == 0 && ok && alive && g + 1 < g_end) {
             // every MMA that read the tiles is done: the next ones land under the epilogue
@@ -387,33 +377,42 @@ tc_token_readout_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_c
         }
         const float sig = row < L ? sigmoid_fast(gate_logit) : 0.0f;
         if (g + 1 < g_end) fetch_row(g + 1);
-        if (alive) {
+        alive = alive && wait_bar(bars + 8 * kTRBarOut, par, ab, 115);
+        if (__all_sync(0xffffffffu, alive)) {
             tc_fence_after();
             // ---- epilogue: out_i += sigmoid(g_i) exp(la_i - lg_last) O_i
             uint32_t o[64];
             tmem_ld32(lane_base + kColK + hf * 64, *reinterpret_cast<uint32_t(*)[32]>(&o[0]));
             tmem_ld32(lane_base + kColK + hf * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&o[32]));
             tmem_wait_ld();
-            if (row < L) {
-                const float f = sig * __expf(la_r - lg_last);
+            const float f = sig * __expf(la_r - lg_last);
+            uint8_t* half_row = smem + kTROffS + hf * kHalfBytes + r * 128;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    uint32_t nw[8];
+            for (int i = 0; i < 8; ++i) {
+                uint4* piece = reinterpret_cast<uint4*>(half_row + ((i ^ (r & 7)) << 4));
+                const uint4 v = *piece;
+                const uint32_t prev[4] = {v.x, v.y, v.z, v.w};
+                uint32_t nw[4];
 #pragma unroll
-                    for (int m = 0; m < 8; ++m)
-                        nw[m] = pack_bf16(__uint_as_float(prev[i * 8 + m] << 16) + f * __uint_as_float(o[i * 16 + 2 * m]),
-                                          __uint_as_float(prev[i * 8 + m] & 0xFFFF0000u) + f * __uint_as_float(o[i * 16 + 2 * m + 1]));
-                    store_row32(p.out + at0 + i * 16, nw, wide_rows(p.out));
-                }
+                for (int m = 0; m < 4; ++m)
+                    nw[m] = pack_bf16(__uint_as_float(prev[m] << 16) + f * __uint_as_float(o[i * 8 + 2 * m]),
+                                      __uint_as_float(prev[m] & 0xFFFF0000u) + f * __uint_as_float(o[i * 8 + 2 * m + 1]));
+                *piece = make_uint4(nw[0], nw[1], nw[2], nw[3]);
             }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0 && row < L)   // this warp's 32 rows; those past the end stay away
+                tma_store_4d(&tm_o, smem_base + kTROffS + hf * kHalfBytes + r * 128, hf * 64, h, row, b);
         }
         tc_fence_before();
         if (__syncthreads_or(!alive)) break;   // the tiles and the gate arrays may be overwritten now
     }
+    if (lane == 0) tma_store_wait_read();
     if (tid == 0 && (!ok || *abort_flag)) {
         // leave no bulk copy in flight into this CTA's shared memory, no MMA writing tensor memory
         drain_bar(bars + 8 * kTRBarW, (uint32_t)(map_loads - 1) & 1u);
         if (loads > 0) drain_bar(bars + 8 * kTRBarLoad, (uint32_t)(loads - 1) & 1u);
+        if (out_loads > 0) drain_bar(bars + 8 * kTRBarOut, (uint32_t)(out_loads - 1) & 1u);
         mma_commit(bars + 8 * kTRBarDrain);
         drain_bar(bars + 8 * kTRBarDrain, 0);
     }
@@ -437,10 +436,11 @@ int tc_token_readout(const StepArgs& a, const float* alpha_logits, const CommitA
     if (int r = device_setup_once(g_setup_mutex, g_setup,
                                   [] { return opt_in_smem(tc_token_readout_kernel, kTRSmemBytes); }, &num_sms))
         return r;
-    CUtensorMap tm_q, tm_k, tm_v, tm_wq, tm_wk, tm_wv;
+    CUtensorMap tm_q, tm_k, tm_v, tm_wq, tm_wk, tm_wv, tm_o;
     if (int r = make_map_blhd(&tm_q, a.q, a.s)) return r;
     if (int r = make_map_blhd(&tm_k, a.k_rot, a.s)) return r;     // raw K: the feature map comes before the rotation
     if (int r = make_map_blhd(&tm_v, a.v, a.s)) return r;
+    if (int r = make_map_blhd(&tm_o, a.out, a.s, 32)) return r;
     if (int r = make_map_rows(&tm_wq, wq_op, (size_t)a.s.H * kTile)) return r;
     if (int r = make_map_rows(&tm_wk, wk_op, (size_t)a.s.H * kTile)) return r;
     if (int r = make_map_rows(&tm_wv, wv_op, (size_t)a.s.H * kTile)) return r;
@@ -451,7 +451,6 @@ int tc_token_readout(const StepArgs& a, const float* alpha_logits, const CommitA
     p.gate = a.gate;
     p.state = a.state;
     p.entry = seg.partials;
-    p.out = static_cast<__nv_bfloat16*>(a.out);
     p.status = a.status;
     p.spin_limit = a.wait_limit ? a.wait_limit - 1 : kSpinLimit;
     p.ntile = seg.run_ntile;
@@ -460,7 +459,7 @@ int tc_token_readout(const StepArgs& a, const float* alpha_logits, const CommitA
     p.total_tiles = a.s.B * a.s.H * p.ntile;
     const int grid = (p.total_tiles + p.share - 1) / p.share;
     const cudaError_t e = launch_kernel(tc_token_readout_kernel, dim3((unsigned)grid), kTRThreads, kTRSmemBytes, st, tm_q, tm_k, tm_v, tm_wq,
-                                        tm_wk, tm_wv, p);
+                                        tm_wk, tm_wv, tm_o, p);
     if (e != cudaSuccess) { set_error("launch of tc_token_readout_kernel failed: %s", cudaGetErrorString(e)); return ARL2_ERR_CUDA; }
     return 1;
 }
