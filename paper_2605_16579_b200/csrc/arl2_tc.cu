@@ -493,6 +493,28 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                 if ((r & 31) == 0) tma_store_wait_read();   // (the CTA ends soon)
                 continue;
             }
+            if (!wide_rows(p.out)) {
+                // a loop of its own: with the choice at each store, attention over a cache of 4 x 4680 tokens took 512.4 us against
+                // 509 without it (12 heads, 4680 queries); with this loop no difference is left
+#pragma unroll 1
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t o[32];
+                    tmem_ld32(o_addr + c * 32, o);
+                    tmem_wait_ld();
+                    if (valid_row) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                w[i] = pack_bf16(__uint_as_float(o[e * 8 + 2 * i]) * inv_l, __uint_as_float(o[e * 8 + 2 * i + 1]) * inv_l);
+                            *reinterpret_cast<uint4*>(orow + c * 32 + e * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                    }
+                }
+                tc_fence_before();
+                continue;
+            }
 #pragma unroll 1
             for (int c = 0; c < 4; ++c) {
                 uint32_t o[32];
@@ -507,7 +529,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                         for (int i = 0; i < 8; ++i)
                             w[i] = pack_bf16(__uint_as_float(o[e * 16 + 2 * i]) * inv_l,
                                              __uint_as_float(o[e * 16 + 2 * i + 1]) * inv_l);
-                        store_row32(orow + c * 32 + e * 16, w, wide_rows(p.out));
+                        store_row32(orow + c * 32 + e * 16, w, true);
                     }
                 }
             }
