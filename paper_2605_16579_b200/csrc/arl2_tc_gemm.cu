@@ -338,6 +338,9 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
                     tma_load_2d_pair(dst + kGABytes + kGBK * 128, &tm_b, bar, n0 + 64, kb * kGBK);
                 }
             }
+            // The stages are given back by arrivals from the first CTA: this one must not end while one is on its way.
+            for (uint32_t m = n > (uint32_t)kGPStages ? n - kGPStages : 0; m < n && ok; ++m)
+                ok = wait_bar(bars + 8 * (kGPBarEmpty0 + m % kGPStages), (m / kGPStages) & 1u, ab, 124);
             *asked = n;
         }
     } else if (warp == 1) {
@@ -376,10 +379,11 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_const
                 }
                 if (ok) mma_commit_pair_if(lead, bars + 8 * (kGPBarAccFull0 + buf));
             }
-            // tensor memory is freed and both CTAs end below: no MMA may still be running, no arrival on its way
             mma_commit_pair_if(lead, bars + 8 * kGPBarDrain);
-            drain_bar(bars + 8 * kGPBarDrain, 0);
         }
+        // Tensor memory is freed and both CTAs end below: no MMA may still be running, and this arrival, which comes to each
+        // CTA's own barrier, must not be on its way.  That one CTA has seen its own says nothing about the other's.
+        drain_bar(bars + 8 * kGPBarDrain, 0);
     } else {
         // ---------------- epilogue: thread = output row of this CTA's half of the tile ----------------
         const int q = warp & 3;
