@@ -189,6 +189,9 @@ __device__ __forceinline__ Entry item_entry(const Item& it, int n_kv, int e)
 
 // One softmax group thread: owns query row `r` of tile `t` of every item.  kElemGate compiles the
 // per-channel gate variant in (a separate kernel instantiation, so the default path is unchanged).
+// Its waits end for a whole warp alike: the lanes meet again (the vote on rescaling, the box of output rows that leaves by
+// TMA), and one that had given up alone would never come.  Attention over a cache of 4 x 4680 tokens 505 -> 508 us for it, one
+// frame of 12 heads and other shapes the same within 0.5 %.
 template <bool kElemGate, bool kSplit>
 __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtensorMap* tm_o, uint8_t* smem, uint32_t bars,
                                              uint32_t tmem_base, const Abort& ab,
@@ -211,7 +214,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
     for (uint32_t item = 0;; ++item) {
         // the first item is known without the producer: its rotation table is fetched while Q is on its way (a rotation
         // that asked for the table once Q had landed ended 1.2 us later)
-        if (item > 0 && !wait_bar(bars + 8 * kBarQFull, item & 1, ab, 10)) return;
+        if (item > 0 && !wait_bar_warp(bars + 8 * kBarQFull, item & 1, ab, 10)) return;
         const int id = item > 0 ? item_slots[item & 1] : (int)blockIdx.x;
         if (id < 0) return;
         const Item it = decode_item<kSplit>(id, p);
@@ -220,7 +223,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
         const int row = it.row0[t] + r;
         const bool valid_row = row < L;
         const bool active = t < it.ntile;
-        if (item == 0 && !active && !wait_bar(bars + 8 * kBarQFull, 0, ab, 10)) return;   // (no phase is left out)
+        if (item == 0 && !active && !wait_bar_warp(bars + 8 * kBarQFull, 0, ab, 10)) return;   // (no phase is left out)
 
         if (active) {
             // ---- Q~ = RoPE(Q): rotate this thread's row of the tile in place          (Eq. 2)
@@ -231,7 +234,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                 uint4 cs[16];
 #pragma unroll
                 for (int c = 0; c < 16; ++c) cs[c] = tab[c * 32];
-                if (item == 0 && !wait_bar(bars + 8 * kBarQFull, 0, ab, 10)) return;
+                if (item == 0 && !wait_bar_warp(bars + 8 * kBarQFull, 0, ab, 10)) return;
 #pragma unroll
                 for (int c = 0; c < 16; ++c) {
                     int off = (c >> 3) * kHalfBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4);
@@ -249,7 +252,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                     *reinterpret_cast<uint4*>(tile + off) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
                 fence_proxy_async_smem();
-            } else if (item == 0 && !wait_bar(bars + 8 * kBarQFull, 0, ab, 10)) {
+            } else if (item == 0 && !wait_bar_warp(bars + 8 * kBarQFull, 0, ab, 10)) {
                 return;
             }
             mbar_arrive(bars + 8 * (kBarQRot0 + t));
@@ -259,7 +262,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
 
             for (int jj = 0; jj < nj; ++jj) {
                 const int j = j0 + jj;
-                if (!wait_bar(bar_s, s_cnt & 1, ab, 20 + t)) return;
+                if (!wait_bar_warp(bar_s, s_cnt & 1, ab, 20 + t)) return;
                 ++s_cnt;
                 tc_fence_after();
 #pragma unroll
@@ -339,7 +342,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
 #pragma unroll
                 for (int c = 0; c < 16; ++c) cs[c] = tab[c * 32];
             }
-            if (!wait_bar(bar_s, s_cnt & 1, ab, 30 + t)) return;
+            if (!wait_bar_warp(bar_s, s_cnt & 1, ab, 30 + t)) return;
             ++s_cnt;
             tc_fence_after();
 #pragma unroll
@@ -394,7 +397,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                 const bool g_wide = (reinterpret_cast<uintptr_t>(p.gate) & 15) == 0;   // the logits may start at any element
 #pragma unroll 1
                 for (int hv = 0; hv < 2; ++hv) {
-                    if (!wait_bar(bar_s, s_cnt & 1, ab, 32 + t)) return;
+                    if (!wait_bar_warp(bar_s, s_cnt & 1, ab, 32 + t)) return;
                     ++s_cnt;
                     tc_fence_after();
 #pragma unroll 1
@@ -431,7 +434,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                 continue;
             }
             // ---- epilogue: O_t / l -> bf16 -> global                              (Eq. 6-7)
-            if (!wait_bar(bars + 8 * (kBarOFinal0 + t), of_cnt & 1, ab, 40 + t)) return;
+            if (!wait_bar_warp(bars + 8 * (kBarOFinal0 + t), of_cnt & 1, ab, 40 + t)) return;
             ++of_cnt;
             tc_fence_after();
             __nv_bfloat16* orow = p.out + (((size_t)b * L + (valid_row ? row : 0)) * H + h) * kTile;
