@@ -622,7 +622,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
             const uint32_t bar_q = bars + 8 * kBarQFull;
             uint32_t n = 0;       // ring entries produced so far (all items)
             bool ok = true;
-            int q_item = 0;       // item whose Q tiles were requested last
+            int q_item = 0;       // the last phase of bar_q that was armed: an item's Q tiles, or the end of the items
             int id = (int)blockIdx.x;
             for (uint32_t item = 0; ok; ++item) {
                 if (item > 0) ok = wait_bar(bars + 8 * kBarQFree, (item - 1) & 1, ab, 50);
@@ -630,6 +630,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 if (id >= p.n_sched) {
                     item_slots[item & 1] = -1;
                     mbar_arrive(bar_q);
+                    q_item = (int)item;
                     break;
                 }
                 const Item it = decode_item<kSplit>(id, p);
@@ -675,12 +676,11 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 if (drawn + 1 == (uint32_t)p.n_sched) *p.sched_counter = 0;
                 id = (int)gridDim.x + (int)drawn;
             }
-            if (!ok || *abort_flag) {
-                // do not leave the CTA while bulk copies into its shared memory are in flight
-                drain_bar(bar_q, (uint32_t)q_item & 1);
-                for (uint32_t m = (n > (uint32_t)kStages ? n - kStages : 0); m < n; ++m)
-                    drain_bar(bars + 8 * (kBarFull0 + m % kStages), (m / kStages) & 1);
-            }
+            // Do not leave the CTA while bulk copies into its shared memory are in flight.  Whatever became of the waits here: a
+            // role that copies were for may give up after this one is through.
+            drain_bar(bar_q, (uint32_t)q_item & 1);
+            for (uint32_t m = (n > (uint32_t)kStages ? n - kStages : 0); m < n; ++m)
+                drain_bar(bars + 8 * (kBarFull0 + m % kStages), (m / kStages) & 1);
         }
     } else if (warp == 9 || warp == 10) {
         // ---------------- MMA issuers: warp 9 drives query tile 0, warp 10 tile 1 ----------------
@@ -858,11 +858,10 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                 cons += shared ? 1 : ntile;
             }
             (void)of_cnt;
-            if (!ok || __any_sync(0xffffffffu, *abort_flag)) {
-                // tensor memory is freed below: none of this thread's MMAs may still be running
-                mma_commit_if(lead, bars + 8 * (kBarDrain0 + t));
-                drain_bar(bars + 8 * (kBarDrain0 + t), 0);
-            }
+            // tensor memory is freed below: none of this thread's MMAs may still be running, even if the softmax group gives up on
+            // them after this
+            mma_commit_if(lead, bars + 8 * (kBarDrain0 + t));
+            drain_bar(bars + 8 * (kBarDrain0 + t), 0);
         }
     }
 

@@ -187,12 +187,10 @@ tc_commit_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                 // once the first stage would land only after a third of that burst
                 if (k == 0 && n_my > 1) ok = wait_bar(bars + 8 * (kCBarStageFull0 + 0), 0u, ab, 79);
             }
-            if (!ok || *abort_flag) {
-                // do not leave the CTA while bulk copies into its shared memory are in flight
-                if (n_w > 0) drain_bar(bars + 8 * kCBarWFull, (uint32_t)(n_w - 1) & 1u);
-                for (int m = (issued > kS ? issued - kS : 0); m < issued; ++m)
-                    drain_bar(bars + 8 * (kCBarStageFull0 + m % kS), (uint32_t)(m / kS) & 1u);
-            }
+            // do not leave the CTA while bulk copies into its shared memory are in flight, whether or not a wait has expired yet
+            drain_bar(bars + 8 * kCBarWFull, (uint32_t)(n_w - 1) & 1u);
+            for (int m = (issued > kS ? issued - kS : 0); m < issued; ++m)
+                drain_bar(bars + 8 * (kCBarStageFull0 + m % kS), (uint32_t)(m / kS) & 1u);
         }
     } else if (warp == 1 || warp == kCThreads / 32 - 1) {
         // ---------------- two MMA issuers ----------------
@@ -271,12 +269,11 @@ tc_commit_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant
                     }
                 }
             }
-            if (!ok || __any_sync(0xffffffffu, *abort_flag)) {
-                // tensor memory is freed below: none of this thread's MMAs may still be running
-                const uint32_t bar_drain = bars + 8 * (warp == 1 ? kCBarDrain0 : kCBarDrain1);
-                mma_commit_if(lead, bar_drain);
-                drain_bar(bar_drain, 0);
-            }
+            // tensor memory is freed below: none of this thread's MMAs may still be running, even if the token threads give up on
+            // them after this
+            const uint32_t bar_drain = bars + 8 * (warp == 1 ? kCBarDrain0 : kCBarDrain1);
+            mma_commit_if(lead, bar_drain);
+            drain_bar(bar_drain, 0);
         }
     } else {
         // ---------------- token threads: (row r, half hf) of every tile of the run ----------------

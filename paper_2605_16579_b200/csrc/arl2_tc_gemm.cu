@@ -164,10 +164,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                         tma_load_2d(dst + MH * kGABytes + g * (kGBK * 128), &tm_b, bar, n0 + g * 64, kb * kGBK);
                 }
             }
-            if (!ok || *abort_flag) {
-                for (uint32_t m = (n > (uint32_t)kGStages ? n - kGStages : 0); m < n; ++m)
-                    drain_bar(bars + 8 * (kGBarFull0 + m % kGStages), (m / kGStages) & 1u);
-            }
+            // no copy may be under way when the CTA ends, and no MMA (below), whether or not a wait has expired yet
+            for (uint32_t m = (n > (uint32_t)kGStages ? n - kGStages : 0); m < n; ++m)
+                drain_bar(bars + 8 * (kGBarFull0 + m % kGStages), (m / kGStages) & 1u);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
@@ -214,10 +213,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 }
                 if (ok) mma_commit(bars + 8 * (kGBarAccFull0 + buf));
             }
-            if (!ok || *abort_flag) {
-                mma_commit(bars + 8 * kGBarDrain);
-                drain_bar(bars + 8 * kGBarDrain, 0);
-            }
+            mma_commit(bars + 8 * kGBarDrain);
+            drain_bar(bars + 8 * kGBarDrain, 0);
         }
     } else {
         // ---------------- epilogue: thread = output row of the tile ----------------
