@@ -187,8 +187,8 @@ __device__ __forceinline__ Entry item_entry(const Item& it, int n_kv, int e)
     return en;
 }
 
-// One softmax group thread: owns query row `r` of tile `t` of every item.  kElemGate compiles the
-// per-channel gate variant in (a separate kernel instantiation, so the default path is unchanged).
+// One softmax group thread: owns query row `r` of tile `t` of every item.  kElemGate: one gate
+// per output channel, which only launches with such gates take (a kernel instantiation of its own, with that epilogue alone).
 // Its waits end for a whole warp alike: the lanes meet again (the vote on rescaling, the box of output rows that leaves by
 // TMA), and one that had given up alone would never come.  Attention over a cache of 4 x 4680 tokens 505 -> 508 us for it, one
 // frame of 12 heads and other shapes the same within 0.5 %.
@@ -332,8 +332,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
             // the row's rotation table is fetched while the MMA is still running
             uint4 cs[16];
             // fetched early too; no gate tensor = closed gate (plain softmax attention, Eq. 1)
-            const bool elem_gate = kElemGate && p.gate_mode == 2 && p.gate != nullptr;   // one gate per output channel
-            const float gate_logit = (valid_row && p.gate != nullptr && !elem_gate)
+            const float gate_logit = (valid_row && p.gate != nullptr && !kElemGate)
                                          ? p.gate[p.gate_mode == 1 ? (size_t)b * L + row : ((size_t)b * L + row) * H + h]
                                          : -INFINITY;
             const bool rotate_u = p.rope_h != nullptr && valid_row;
@@ -376,7 +375,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                 const float gate = valid_row ? sigmoid_fast(gate_logit) : 0.0f;
                 // scaled by the row sum so that the common 1/l of the epilogue leaves gate * Q' S;
                 // with per-channel gates the readout is kept apart and gated in the epilogue
-                const float f = elem_gate ? rsqrtf(ss + p.s.eps) : rsqrtf(ss + p.s.eps) * gate * l_sum;
+                const float f = kElemGate ? rsqrtf(ss + p.s.eps) : rsqrtf(ss + p.s.eps) * gate * l_sum;
 #pragma unroll
                 for (int c = 0; c < 64; ++c)
                     sreg[c] = pack_bf16(__uint_as_float(sreg[2 * c]) * f, __uint_as_float(sreg[2 * c + 1]) * f);
@@ -387,14 +386,17 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
             tc_fence_before();
             mbar_arrive(bar_p);
 
-            if (elem_gate) {
+            if constexpr (kElemGate) {
                 // ---- per-channel gates: X = Q' S arrives 64 channels at a time in columns 64-127 of
                 // S_t; out = O_t / l + sigmoid(G) X.  O_t is final: its last MMA preceded U's.
                 const float inv_l = 1.0f / l_sum;
                 const size_t rbase = ((size_t)b * L + (valid_row ? row : 0)) * H + h;
                 __nv_bfloat16* orow = p.out + rbase * kTile;
                 const float* grow = p.gate + rbase * kTile;
-                const bool g_wide = (reinterpret_cast<uintptr_t>(p.gate) & 15) == 0;   // the logits may start at any element
+                // The logits may start at any element and the output rows on any 16 bytes: decided once per 32 channels.  At each
+                // access, 40 heads x 1560 tokens took 114.1 us against 113.4 without the choice; so, and without the other
+                // epilogues in this instantiation, 112.2 (12 x 1560: 55.6, 55.0 and 54.6).
+                const bool wide = (reinterpret_cast<uintptr_t>(p.gate) & 15) == 0 && wide_rows(p.out);
 #pragma unroll 1
                 for (int hv = 0; hv < 2; ++hv) {
                     if (!wait_bar_warp(bar_s, s_cnt & 1, ab, 32 + t)) return;
@@ -406,14 +408,14 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                         tmem_ld32(s_addr + 64 + c * 32, x);
                         tmem_ld32(o_addr + hv * 64 + c * 32, o);
                         tmem_wait_ld();
-                        if (valid_row) {
+                        const int at = hv * 64 + c * 32;
+                        if (valid_row && wide) {
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
                                 uint32_t w[8];
 #pragma unroll
                                 for (int i = 0; i < 4; ++i) {
-                                    const float* gp = grow + hv * 64 + c * 32 + e * 16 + i * 4;
-                                    const float4 gl = g_wide ? *reinterpret_cast<const float4*>(gp) : make_float4(gp[0], gp[1], gp[2], gp[3]);
+                                    const float4 gl = *reinterpret_cast<const float4*>(grow + at + e * 16 + i * 4);
                                     const float gv[4] = {gl.x, gl.y, gl.z, gl.w};
                                     float y[4];
 #pragma unroll
@@ -424,7 +426,20 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                                     w[i * 2] = pack_bf16(y[0], y[1]);
                                     w[i * 2 + 1] = pack_bf16(y[2], y[3]);
                                 }
-                                store_row32(orow + hv * 64 + c * 32 + e * 16, w, wide_rows(p.out));
+                                store_row32(orow + at + e * 16, w);
+                            }
+                        } else if (valid_row) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                uint32_t w[4];
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    const int n = e * 8 + i * 2;
+                                    const float* gp = grow + at + n;
+                                    w[i] = pack_bf16(__uint_as_float(o[n]) * inv_l + sigmoid_fast(gp[0]) * __uint_as_float(x[n]),
+                                                     __uint_as_float(o[n + 1]) * inv_l + sigmoid_fast(gp[1]) * __uint_as_float(x[n + 1]));
+                                }
+                                *reinterpret_cast<uint4*>(orow + at + e * 8) = make_uint4(w[0], w[1], w[2], w[3]);
                             }
                         }
                     }
@@ -532,7 +547,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                         for (int i = 0; i < 8; ++i)
                             w[i] = pack_bf16(__uint_as_float(o[e * 16 + 2 * i]) * inv_l,
                                              __uint_as_float(o[e * 16 + 2 * i + 1]) * inv_l);
-                        store_row32(orow + c * 32 + e * 16, w, true);
+                        store_row32(orow + c * 32 + e * 16, w);
                     }
                 }
             }
@@ -828,7 +843,7 @@ tc_step_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__
                     ++p_cnt;
                     if (!ok) break;
                     tc_fence_after();
-                    if (kElemGate && p.gate_mode == 2 && p.gate != nullptr) {
+                    if constexpr (kElemGate) {
                         // per-channel gates: X = Q' S kept apart from O_t, 64 channels at a time into
                         // columns 64-127 of S_t (Q' sits in columns 0-63)
                         constexpr uint32_t idesc_x = idesc_bf16(kTile, 64, 0, 1);

@@ -61,20 +61,16 @@ __device__ __forceinline__ void drain_bar(uint32_t bar, uint32_t parity)
         if (mbar_try_wait(bar, parity)) return;
 }
 
-// 32 bytes of an output row, a whole sector.  A caller's tensor need only start on a 16-byte boundary; `wide` (the same for
-// every row of the tensor, rows being 256 bytes) says that it starts on a 32-byte one.
+// A caller's tensor need only start on a 16-byte boundary; this says that it starts on a 32-byte one (the same for every row
+// of the tensor, rows being 256 bytes).
 __device__ __forceinline__ bool wide_rows(const void* base) { return (reinterpret_cast<uintptr_t>(base) & 31) == 0; }
 
-__device__ __forceinline__ void store_row32(void* dst, const uint32_t (&w)[8], bool wide)
+// 32 bytes of an output row of such a tensor, a whole sector
+__device__ __forceinline__ void store_row32(void* dst, const uint32_t (&w)[8])
 {
-    if (wide) {
-        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
-                     "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                     : "memory");
-    } else {
-        static_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        static_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    }
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
+                 "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
 }
 
 __device__ __forceinline__ float sigmoid_fast(float x) { return 1.0f / (1.0f + __expf(-x)); }
