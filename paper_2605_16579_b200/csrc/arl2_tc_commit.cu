@@ -438,8 +438,16 @@ constexpr int kFinRows = 16;
 constexpr int kFinThreads = 128;
 // Slots of one head whose loads go out together, and CTAs that share an SM: registers for more of one leave less of the other.
 // (6 and 8 slots with two CTAs: delta rule of 12 x 4680 24.2 us instead of 23.6, commit of 40 x 4680 32.2 instead of 30.7.)
+// kMany (gated-linear rule): at most 128 registers instead of 147, so that a fourth CTA fits.  Where more than three want onto an
+// SM that saves a wave: us per pass with 147 and with 128, commit of 3 x 24 x 218 tokens 14.5 and 13.1, 8 x 8 x 202 13.5 and 12.9,
+// 3 x 24 x 3995 46.1 and 44.2, 8 x 40 x 489 52.4 and 51.1, 4 x 14 x 1000 20.2 and 19.4; with fewer CTAs it is the slower one (12 x 1560
+// 12.0 and 12.4, 2 x 4680 12.2 and 12.6) or the same (40 x 4680).  With per-token decay the next call's first kernel is
+// let in beside these CTAs, and its blocks of 1024 threads fit beside two of them only so: 4 x 8 x 351 20.1 and 16.9,
+// 4 x 8 x 512 18.9 and 15.7, 2 x 40 x 461 29.1 and 27.5; where an SM has one CTA at most there is room in any case (2 x 4680
+// 18.8 and 19.3).
 __host__ __device__ constexpr int fin_parts(int mode) { return mode == 1 ? 4 : 6; }
-constexpr int fin_ctas(int mode) { return mode == 1 ? 2 : 3; }
+constexpr int kFinMore = 4;   // slots at a time after the first ones, where registers are for four CTAs per SM
+constexpr int fin_ctas(int mode, bool many) { return mode == 1 ? 2 : many ? 4 : 3; }
 constexpr int kFinLdM = kTile + 8;  // bf16 row stride of a right-hand matrix: 272 bytes, conflict-free 8 x 8 loads
 constexpr int kFinLdA = kTile + 8;  // fp32 row stride of the summed rows: a fragment's 8-byte reads spread over the banks
 constexpr int kFinMatBytes = kTile * kFinLdM * 2;
@@ -524,8 +532,8 @@ __device__ __forceinline__ void fin_multiply(float (&acc)[4][4], const float* __
     }
 }
 
-template <int kMode>
-__global__ void __launch_bounds__(kMode == 1 ? 2 * kFinThreads : kFinThreads, fin_ctas(kMode))
+template <int kMode, bool kMany>
+__global__ void __launch_bounds__(kMode == 1 ? 2 * kFinThreads : kFinThreads, fin_ctas(kMode, kMany))
 tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
                         const float* partials_g, const __nv_bfloat16* wv,
                         const float* decay, int decay_direct, const __nv_bfloat16* mirror_cur, __nv_bfloat16* mirror_next,
@@ -563,17 +571,18 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
     const float* slots = (second ? partials_g : partials) + slot0;
     constexpr int kFinMaxParts = fin_parts(kMode);
     float4 pa[kFinMaxParts][4];
-    auto request = [&](int s0) {
+    auto request = [&](auto& to, int s0) {
+        constexpr int kN = sizeof(to) / sizeof(to[0]);
 #pragma unroll
-        for (int s = 0; s < kFinMaxParts; ++s) {
+        for (int s = 0; s < kN; ++s) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 if (s0 + s < nparts)
-                    pa[s][i] = *reinterpret_cast<const float4*>(slots + (size_t)(s0 + s) * kTile * kTile + (size_t)i * kTile * 8);
+                    to[s][i] = *reinterpret_cast<const float4*>(slots + (size_t)(s0 + s) * kTile * kTile + (size_t)i * kTile * 8);
             }
         }
     };
-    request(0);
+    request(pa, 0);
     const int g = lane >> 2, t = lane & 3;
     // output fragment: rows g and g + 8 of the CTA's 16, columns warp * 32 + 8 j + 2 t (+ 1), j = 0..3
     const size_t out0 = head + (size_t)(cta_row0 + g) * kTile + warp * 32 + 2 * t;
@@ -600,17 +609,31 @@ tc_commit_finish_kernel(float* __restrict__ state, const float* partials,
     float4 a[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) a[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0;;) {
+    auto add = [&](const auto& from, int s0) {
+        constexpr int kN = sizeof(from) / sizeof(from[0]);
 #pragma unroll
-        for (int s = 0; s < kFinMaxParts; ++s) {
+        for (int s = 0; s < kN; ++s) {
             if (s0 + s < nparts) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) add4(a[i], pa[s][i]);
+                for (int i = 0; i < 4; ++i) add4(a[i], from[s][i]);
             }
         }
-        s0 += kFinMaxParts;
-        if (s0 >= nparts) break;
-        request(s0);
+    };
+    if constexpr (kMany) {
+        add(pa, 0);
+#pragma unroll 1
+        for (int s0 = kFinMaxParts; s0 < nparts; s0 += kFinMore) {
+            float4 more[kFinMore][4];
+            request(more, s0);
+            add(more, s0);
+        }
+    } else {
+        for (int s0 = 0;;) {
+            add(pa, s0);
+            s0 += kFinMaxParts;
+            if (s0 >= nparts) break;
+            request(pa, s0);
+        }
     }
     float* rows = second ? Gs : As;
 #pragma unroll
@@ -751,8 +774,9 @@ int device_setup(int* num_sms)
         cudaError_t e = opt_in_smem(tc_commit_kernel<0>, kCommitSmemBytes);
         if (e == cudaSuccess) e = opt_in_smem(tc_commit_kernel<1>, kCommitSmemBytes);
         if (e == cudaSuccess) e = opt_in_smem(tc_commit_kernel<2>, kCommitSmemBytes);
-        if (e == cudaSuccess) e = opt_in_smem(tc_commit_finish_kernel<0>, kMaxSmemPerCta);
-        if (e == cudaSuccess) e = opt_in_smem(tc_commit_finish_kernel<1>, kMaxSmemPerCta);
+        if (e == cudaSuccess) e = opt_in_smem(tc_commit_finish_kernel<0, false>, kMaxSmemPerCta);
+        if (e == cudaSuccess) e = opt_in_smem(tc_commit_finish_kernel<0, true>, kMaxSmemPerCta);
+        if (e == cudaSuccess) e = opt_in_smem(tc_commit_finish_kernel<1, false>, kMaxSmemPerCta);
         if (e == cudaSuccess) e = opt_in_smem(tc_run_prefix_kernel, kPrefixSmemBytes);
         return e;
     }, num_sms);
@@ -819,7 +843,6 @@ int tc_commit_partials(CommitArgs& a, const __nv_bfloat16* wk_op, cudaStream_t s
 
 int tc_commit_finish(const CommitArgs& a, cudaStream_t st)
 {
-    auto kernel = a.mode == 1 ? tc_commit_finish_kernel<1> : tc_commit_finish_kernel<0>;
     int num_sms = 0;
     if (int r = device_setup(&num_sms)) return r;
     // (SMs that the partial sums leave idle throughout have the CTAs waiting there: any number to an SM, 12.1 us per pass of
@@ -829,6 +852,8 @@ int tc_commit_finish(const CommitArgs& a, cudaStream_t st)
     const int need = fin_smem_bytes(a.mode == 1 ? 1 : 0);
     const size_t smem = (int)grid <= 2 * (num_sms - partial_ctas) ? (size_t)need
                                                                    : even_spread_smem(need, (int)((grid + (unsigned)num_sms - 1) / (unsigned)num_sms));
+    // (lines and figures: fin_parts)
+    auto kernel = a.mode == 1 ? tc_commit_finish_kernel<1, false> : (int)grid > (a.mode == 2 ? 1 : 3) * num_sms ? tc_commit_finish_kernel<0, true> : tc_commit_finish_kernel<0, false>;
     const cudaError_t e = launch_kernel(kernel, dim3(grid), a.mode == 1 ? 2 * kFinThreads : kFinThreads, smem, st, a.state, a.partials, a.partials_g,
                                         static_cast<const __nv_bfloat16*>(a.wv), a.decay, a.decay_direct ? 1 : 0, a.state_bf16, a.state_bf16_next,
                                         a.s.H, a.run_share, a.run_ntile, a.nslot, a.status);
