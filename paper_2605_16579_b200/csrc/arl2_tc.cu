@@ -480,11 +480,14 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
                 continue;
             }
             const float inv_l = 1.0f / l_sum;
-            if (p.one_item) {
+            if (p.one_item && it.row0[t] + 96 < L) {
                 // A row per thread makes a warp's stores 32 bytes of 32 rows each, which the load/store unit takes one by one: 3.8 k
                 // clk for the two tiles, now 2.5 k.  Where no further item's Q is on its way, the rows go over this tile's Q
                 // (every score MMA is done) and leave by TMA, 32 rows per warp; rows past L are cut off by the tensor map.
-                // 12 heads x 1560 tokens 38.8 -> 38.3 us per pass, 3 x 12 x 1001 31.8 -> 31.3.
+                // us per pass with row stores and so: 12 heads x 1560 tokens 38.7 and 38.3, 3 x 12 x 1001 32.6 and 32.4, 12 x 512 18.3
+                // and 17.9, 2 x 384 17.7 and 17.5.  Only tiles in which all four warps have rows: the TMA's own latency is
+                // there for a few rows, too, whose stores would be through sooner (12 x 300, 44 rows in the last tile,
+                // 16.9 and 17.3; 12 x 330, 74 rows, 17.3 and 17.5).
                 uint8_t* tile = smem + kOffQ + t * kTileBytes;
 #pragma unroll 1
                 for (int c = 0; c < 4; ++c) {

@@ -1,4 +1,5 @@
-"""Output rows of the step kernel where every CTA has one work item: they leave 32 at a time, and rows past the end do not."""
+"""Output rows of the step kernel where every CTA has one work item: those of a tile with more than 96 leave 32 at a time, those
+of a shorter one row by row, and rows past the end do not."""
 import pytest
 
 from paper_2605_16579_b200 import workload
