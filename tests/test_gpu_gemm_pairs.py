@@ -3,6 +3,7 @@ last column tile with the gate logits, and a wait that expires."""
 import pytest
 import torch
 
+from graph_util import captured_kernels
 from paper_2605_16579_b200 import arl2
 
 pytestmark = pytest.mark.gpu
@@ -36,13 +37,27 @@ def _check(got, x, w, bf16):
     assert bool(((got - ref).abs() <= bound).all())
 
 
-# 1536 = 6 tiles exactly; then a tile whose second CTA has no row, both with rows, one row; two streams
-@pytest.mark.parametrize("B,L", [(1, 1536), (1, 1560), (1, 1665), (1, 1793), (2, 1560)])
-def test_input_projection_on_pairs(B, L):
-    H = 12
+def _on_pairs(call):
+    """Which of the kernels serves the call (the rule goes by a cost model: a size that it serves otherwise tests nothing here)."""
+    (name, grid, _, cluster), = captured_kernels(call)
+    pairs = "tc_gemm_pair_kernel" in name
+    assert cluster == (2 if pairs else 1) and (not pairs or grid[0] % 2 == 0)
+    return pairs
+
+
+# On pairs: 12 tiles of 256 rows exactly; one whose first CTA has a row and the second none; 48 rows; the second CTA has one
+# row; two streams; 5 heads (the gate logits' columns begin in the middle of a tile).  Beside the rule's line: 256 x 256 tiles of one
+# CTA, and 128 x 256.
+@pytest.mark.parametrize("B,H,L,pairs", [(1, 12, 3072, True), (1, 12, 3073, True), (1, 12, 3120, True), (1, 12, 3201, True),
+                                         (2, 12, 1560, True), (1, 5, 6241, True), (1, 12, 1536, False), (1, 12, 1560, False),
+                                         (1, 12, 1665, False), (1, 12, 1793, False)])
+def test_input_projection_on_pairs(B, H, L, pairs):
     layer, (w_q, w_k, w_v, w_g, _), x = _layer(B, H, L, 31)
     (q, eq), (k, ek), (v, ev) = (_guarded((B, L, H, 128), torch.bfloat16) for _ in range(3))
     g, eg = _guarded((B, L, H), torch.float32)
+    assert _on_pairs(lambda: layer.project_in(x, q, k, v, g)) == pairs
+    for t in (q, k, v, g):
+        t.fill_(float("nan"))
     layer.project_in(x, q, k, v, g)
     layer.sync_status()
     for got, w in ((q, w_q), (k, w_k), (v, w_v)):
@@ -51,10 +66,14 @@ def test_input_projection_on_pairs(B, L):
     assert all(bool(torch.isnan(e).all()) for e in (eq, ek, ev, eg))
 
 
-def test_output_projection_on_pairs():
-    B, H, L = 8, 12, 1560
+# whole tiles, and one row in the last tile
+@pytest.mark.parametrize("B,L", [(8, 1560), (8, 1536), (1, 12289)])
+def test_output_projection_on_pairs(B, L):
+    H = 12
     layer, w, o = _layer(B, H, L, 32)
     y, end = _guarded((B, L, H * 128), torch.bfloat16)
+    assert _on_pairs(lambda: layer.project_out(o.view(B, L, H, 128), y))
+    y.fill_(float("nan"))
     layer.project_out(o.view(B, L, H, 128), y)
     layer.sync_status()
     _check(y, o, w[4], True)
@@ -62,14 +81,24 @@ def test_output_projection_on_pairs():
 
 
 def test_a_wait_that_expires_on_pairs():
-    layer, w, x = _layer(1, 12, 1560, 33)
+    """Every wait at once (0 polls), and at different points of the two CTAs of a pair: they end together, with as many k-blocks
+    asked for by one as by the other, and the launches after them are whole."""
+    layer, w, x = _layer(1, 12, 3120, 33)
     want = [t.clone() for t in layer.project_in(x)]
-    layer.debug_set_wait_limit(0)
-    layer.project_in(x)
-    with pytest.raises(arl2.Arl2Error):
+    assert _on_pairs(lambda: layer.project_in(x, *[torch.empty_like(t) for t in want]))
+    expired = []
+    for polls in list(range(17)) * 2:
+        layer.debug_set_wait_limit(polls)
+        got = layer.project_in(x)
+        try:
+            layer.sync_status()
+            for a, b in zip(got, want):
+                assert torch.equal(a, b)
+        except arl2.Arl2Error:
+            expired.append(polls)
         layer.sync_status()
-    layer.sync_status()
-    layer.debug_set_wait_limit(-1)
-    for a, b in zip(layer.project_in(x), want):
-        assert torch.equal(a, b)
-    layer.sync_status()
+        layer.debug_set_wait_limit(-1)
+        for a, b in zip(layer.project_in(x), want):
+            assert torch.equal(a, b)
+        layer.sync_status()
+    assert expired.count(0) == 2 and len(expired) > 2
