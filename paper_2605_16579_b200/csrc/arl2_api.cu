@@ -636,11 +636,12 @@ int arl2_denoise_step_token_level(arl2_ctx* ctx, const void* d_q, const void* d_
         return ARL2_ERR_INVALID_ARG;
     int share = 0, ntile = 0;
     if (int r = tc_commit_run_share(ctx->shape, seg.nslot, &share, &ntile)) return r;
-    // A walked tile takes about 10 us, the three launches before the walk 25 us and 1 us per tile of a run: heads
-    // of no more tiles than that are walked whole, from the state itself (one tile: 35 us per pass against 60,
-    // three tiles: 61 against 73; 13 tiles in runs of 2: 197 against 97).  The costs are those of heads that fit on
-    // the SMs side by side, with everything on one stream; with more heads than SMs a run is a whole head's length and heads
-    // go whole, in waves.
+    // Heads of few tiles are walked whole, from the state itself.  The line counts 10 us for a walked tile, 25 for the three
+    // launches before the walk and 1 per tile of a run, which is what they took one after the other on one stream.  us per
+    // pass whole and in runs now, 12 heads: one tile 26 and 37, two 36 and 37, three 45 and 40, four 54 and 41, five 64 and
+    // 44, six 73 and 44, 13 tiles 144 and 62; 8 x 12 heads of three tiles 52 and 64, 4 x 40 of three 100 and 107.  So a few heads of
+    // three to five tiles would be quicker in runs, and the line errs on the side of the whole heads; with more heads than
+    // SMs a run is a whole head's length and heads go whole, in waves.
     const bool whole_heads = 10 * ntile <= 11 * share + 30;
     if (whole_heads) {
         seg.partials = nullptr;

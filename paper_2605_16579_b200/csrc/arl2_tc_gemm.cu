@@ -492,8 +492,11 @@ int tc_gemm(const GemmArgs& a, cudaStream_t st)
     // 128 x 256 are two rounds on 148 SMs, the second half empty; 296 of 128 x 192 are two full ones).
     // A pair's tile of 256 x 256 takes about 610 clocks per k-block, and its clusters about 3800 more to start and to end: us
     // per launch with one CTA's tiles and with pairs, input projection of 12 heads x 4680 tokens 57.2 and 50.1, 8 x 12 x 1560
-    // 153.8 and 125.4, 40 x 4680 588 and 549, 12 x 1560 23.6 and 21.3, 5 x 1000 7.8 and 11.9; output projection 12 x 4680 21.9 and
-    // 21.2, 12 x 1560 12.2 and 13.3, 4 x 16 x 1001 31.4 and 34.3 (two rounds of pairs, the second nearly empty).
+    // 153.8 and 125.4, 40 x 4680 588 and 549, 5 x 1000 7.8 and 11.9; output projection 8 x 12 x 1560 54 and 49, 12 x 1560 12.2 and 13.2,
+    // 24 x 4680 75 and 83.  The one-CTA shapes are charged nothing for their own start and last epilogue, so where the rounds
+    // are few the model keeps them on shapes that were quicker on pairs: input projection of 12 x 1560 22.9 and 21.0,
+    // 12 x 2002 30.7 and 27.5, 16 x 1560 42.6 and 39.6, 40 x 700 122 and 100; output projection 4 x 16 x 1001 34.4 and 31.7,
+    // 40 x 1560 73 and 70, 12 x 4680 the same on both.
     // The 128-column tile serves N <= 128 only: at 128 x 128 both operands of an MMA come from shared
     // memory at its full rate, measured slower even where it fills the rounds.
     int mh = 1;

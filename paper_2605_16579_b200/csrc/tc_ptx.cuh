@@ -1,5 +1,5 @@
 // Thin inline-PTX wrappers for the sm_100a features the tensor-core kernels use:
-// mbarrier, TMA tiled loads (no multicast anywhere), tcgen05 MMA / commit / TMEM access.
+// mbarrier, TMA tiled loads (none with multicast), tcgen05 MMA / commit / TMEM access.
 #pragma once
 
 #include <cuda.h>
