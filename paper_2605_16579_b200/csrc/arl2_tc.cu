@@ -189,9 +189,11 @@ __device__ __forceinline__ Entry item_entry(const Item& it, int n_kv, int e)
 
 // One softmax group thread: owns query row `r` of tile `t` of every item.  kElemGate: one gate
 // per output channel, which only launches with such gates take (a kernel instantiation of its own, with that epilogue alone).
-// Its waits end for a whole warp alike: the lanes meet again (the vote on rescaling, the box of output rows that leaves by
-// TMA), and one that had given up alone would never come.  Attention over a cache of 4 x 4680 tokens 505 -> 508 us for it, one
-// frame of 12 heads and other shapes the same within 0.5 %.
+// No lane leaves it alone when a wait expires: the lanes meet again (the vote on rescaling, the box of output rows that leaves by
+// TMA), and the others would wait for it for good.  In the key loop the role goes on instead; the error is recorded, the waits
+// after it end at once, and the next one behind the loop ends the role for the whole warp.  Lanes that left by themselves,
+// a whole-warp wait in the loop too, and this: 40 heads x 4680 tokens 454, 461, 457 us, 8 x 12 x 4680 1071, 1084, 1076, attention over a
+// cache of 4 x 4680 tokens 498, 499, 502; shorter ones the same.
 template <bool kElemGate, bool kSplit>
 __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtensorMap* tm_o, uint8_t* smem, uint32_t bars,
                                              uint32_t tmem_base, const Abort& ab,
@@ -262,7 +264,7 @@ __device__ __forceinline__ void softmax_role(const TcStepParams& p, const CUtens
 
             for (int jj = 0; jj < nj; ++jj) {
                 const int j = j0 + jj;
-                if (!wait_bar_warp(bar_s, s_cnt & 1, ab, 20 + t)) return;
+                (void)wait_bar(bar_s, s_cnt & 1, ab, 20 + t);   // (where it expired, the loop goes on over whatever is there)
                 ++s_cnt;
                 tc_fence_after();
 #pragma unroll
